@@ -233,3 +233,54 @@ def tolerance(case):
     # Products are exact in FP32, sums are FP32, the result is rounded once to FP16 (2^-11 relative at most).  Against the
     # same products summed in FP64 the cases show rel 2.1e-4 and max 5.1e-4; FP8 codes and scales are the same bit for bit.
     return {"rel": 8e-4, "max": 2e-3}
+
+
+def _weights(w, enc, mode):
+    """The weights a linear multiplies with, in FP64: all bits in full mode, those the persistent byte keeps in fast mode."""
+    if mode == dps.DPS_MODE_FAST:
+        keep = 7 if enc in (dps.DPS_ENC_E4M3, dps.DPS_ENC_E4M3_RN) else 8      # low bits of the word the byte leaves out
+        half = 1 << (keep - 1) if enc in (dps.DPS_ENC_E4M3_RN, dps.DPS_ENC_E5M2_RN) else 0
+        bits = (w.view(torch.int16).to(torch.int32) + half) >> keep << keep
+        w = bits.to(torch.int16).view(torch.float16)
+    return w.double()
+
+
+def exact(case, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(int(seed))
+    kind = case["kind"]
+    if kind == "load":      # bytes, the same in every implementation
+        return None
+    if kind == "moe":
+        e, t, h, f = case["experts"], case["tokens"], case["hidden"], case["ffn"]
+        mode = MODES[case["mode"]]
+        first = torch.randint(0, e, (t,), generator=gen, device="cuda")
+        second = (first + 1 + torch.randint(0, e - 1, (t,), generator=gen, device="cuda")) % e
+        expert = torch.stack([first, second], 1).reshape(-1)
+        x = [_normal((t, h), gen).double().repeat_interleave(2, 0), _normal((2 * t, f), gen).double()]
+        out = []
+        for i, (n, k) in enumerate(((2 * f, h), (h, f))):
+            y = torch.empty((2 * t, n), dtype=torch.float64, device="cuda")
+            for j in range(e):
+                w = _weights(_normal((n, k), gen, 0.02), dps.DPS_ENC_E4M3 if j % 4 != 3 else dps.DPS_ENC_E5M2, mode)
+                rows = (expert == j).nonzero().view(-1)
+                y[rows] = x[i][rows] @ w.T
+            out.append(y)
+        return tuple(out)
+    enc = ENCODINGS[case["enc"]]
+    if kind == "single":
+        x, w = _normal((case["tokens"], case["k"]), gen).double(), _normal((case["n"], case["k"]), gen, 0.02)
+        return [x @ _weights(w, enc, mode).T for mode in (dps.DPS_MODE_FAST, dps.DPS_MODE_FULL)]
+    out = []
+    for _ in range(case.get("layers", 1)):
+        for n, k in _linears(case):
+            x, w = _normal((case["tokens"], k), gen), _normal((n, k), gen, 0.02)
+            if kind != "fp8act":
+                out.append(x.double() @ _weights(w, enc, MODES[case["mode"]]).T)
+                continue
+            # the codes and the scales are FP32 by definition; the product of the codes is what has a 64-bit value
+            top = x.float().abs().amax(1)
+            scale = torch.where(top > 0, top / torch.full_like(top, 448.0), torch.ones_like(top))      # (a scalar divisor is turned into a factor)
+            codes = (x.float() / scale[:, None]).to(torch.float8_e4m3fn).double()
+            out.append((None, None, scale.double()[:, None] * (codes @ _weights(w, enc, dps.DPS_MODE_FAST).T)))
+    return out
