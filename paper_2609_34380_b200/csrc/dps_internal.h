@@ -37,6 +37,10 @@ struct PerDeviceOnce {
 // max over the tensor of (word & 0x7FFF), written with atomicMax into *stat (caller zeroes it).
 cudaError_t launch_magnitude_stat(const uint16_t* w, int64_t n, unsigned* stat, cudaStream_t stream);
 cudaError_t launch_split(const uint16_t* w, uint8_t* p, uint8_t* r, int64_t n, int enc, cudaStream_t stream);
+// The AUTO split in one pass: E4M3 planes, or, if *flag and *host (mapped host memory) read `call` afterwards,
+// planes that are incomplete because a word is out of E4M3's AUTO range.
+cudaError_t launch_split_auto(const uint16_t* w, uint8_t* p, uint8_t* r, int64_t n, unsigned* flag, unsigned* host,
+                              unsigned call, cudaStream_t stream);
 cudaError_t launch_reconstruct(const uint8_t* p, const uint8_t* r, uint16_t* w, int64_t n, int enc,
                                cudaStream_t stream);
 
