@@ -1685,12 +1685,13 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     CUtensorMap mp, mr, mx;
     constexpr int kBlockK = block_k(FULL, TN);
     constexpr CUtensorMapSwizzle kPlaneSwizzle = kBlockK == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    constexpr CUtensorMapL2promotion kPromotion = TN <= 64 ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
     if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kTileRows, kBlockK,
-                     kPlaneSwizzle))
+                     kPlaneSwizzle, kPromotion))
         return cudaErrorInvalidValue;
     if (FULL) {
         if (!make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kTileRows, kBlockK,
-                         kPlaneSwizzle))
+                         kPlaneSwizzle, kPromotion))
             return cudaErrorInvalidValue;
     } else {
         mr = mp;
@@ -1950,11 +1951,11 @@ cudaError_t launch_grouped_tn(const uint32_t* e5m2_mask, const void* x_sorted, c
     constexpr int kBlockK = block_k(FULL, TN, RB);
     constexpr CUtensorMapSwizzle kPlaneSwizzle = kBlockK == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)E * (uint64_t)N, (uint64_t)K, kTileRows * RB,
-                     kBlockK, kPlaneSwizzle))
+                     kBlockK, kPlaneSwizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
         return cudaErrorInvalidValue;
     if (FULL) {
         if (!make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)E * (uint64_t)N, (uint64_t)K, kTileRows * RB,
-                         kBlockK, kPlaneSwizzle))
+                         kBlockK, kPlaneSwizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
             return cudaErrorInvalidValue;
     } else {
         mr = mp;
