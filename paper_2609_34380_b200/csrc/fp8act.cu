@@ -11,13 +11,16 @@
 // taken): scale[m] = max_k |x[m][k]| / 448 (1 for an all-zero token), q = E4M3(x / scale), round to
 // nearest even, saturating; y[m][n] = scale[m] * sum_k q[m][k] * W_fast[n][k].
 //
-// Kernel: tiles of 128 weight rows x 256 tokens, K in blocks of 128 bytes, one persistent CTA per
-// SM.  Warp 0 TMA producer (P tile 128 x 128 B, activation tile 256 x 128 B, 128-byte swizzle), warp 1
-// MMA issuer (two accumulators in tensor memory), warps 2-5 epilogue (TMEM -> scale -> FP16 ->
-// shared-memory buffer -> 16-byte stores), overlapped with the next tile's MMAs.
+// Kernel: tiles of 256 weight rows x up to 256 tokens, K in blocks of 128 bytes, one persistent CTA PAIR
+// (cta_group::2) per two SMs.  In each CTA: warp 0 TMA producer (its 128 rows of P, its half of the
+// tokens, 128-byte swizzle), warp 1 MMA issuer (in the first CTA, for both; two accumulators in tensor
+// memory), warps 2-5 epilogue of its 128 rows (TMEM -> scale -> FP16 -> shared-memory buffer ->
+// 16-byte stores), overlapped with the next tile's MMAs.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
+
+#include <cstdlib>
 
 #include "dps_internal.h"
 #include "sm100.cuh"
@@ -110,12 +113,13 @@ quantize_activations_kernel(const uint4* __restrict__ x, uint2* __restrict__ q, 
 }
 
 // ---- FP8 x FP8 linear ---------------------------------------------------------------------------
-constexpr int kRows = 128;      // weight rows per tile (UMMA M)
+constexpr int kRows = 128;      // weight rows per CTA; a pair's tile has 256 (UMMA M)
 constexpr int kBlockBytes = 128;                                  // K per stage (one swizzle atom of bytes)
 constexpr int kThreads = 192;
-// Tokens per tile (UMMA N): 256, or 128 when 256-token tiles would leave SMs without one.
-__host__ __device__ constexpr int stage_bytes_fp8(int tokens) { return (kRows + tokens) * kBlockBytes; }   // 48 / 32 KB
-__host__ __device__ constexpr int stages_fp8(int tokens) { return tokens == 256 ? 4 : 6; }
+constexpr int kMaxTokens = 256;                                   // tokens per tile (UMMA N): any multiple of 16 up to this
+constexpr int kStageBytes = (kRows + kMaxTokens / 2) * kBlockBytes;   // 32 KB: this CTA's rows, its half of the tokens
+constexpr int kStages = 6;
+constexpr uint32_t kTmemCols = 2 * kMaxTokens;                    // two accumulators
 
 // Instruction descriptor for kind::f8f6f4: FP32 accumulator, K-major operands; formats 0 = E4M3, 1 = E5M2.
 __host__ __device__ constexpr uint32_t idesc_f8(int m, int n, int a_format, int b_format) {
@@ -123,14 +127,15 @@ __host__ __device__ constexpr uint32_t idesc_f8(int m, int n, int a_format, int 
            ((uint32_t)(m >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem], FP8 operands; issued by ONE thread.
-__device__ __forceinline__ void umma_f8_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                           uint32_t accumulate) {
+// D[tmem] (+)= A[smem] * B[smem] over a CTA pair, FP8 operands; issued by ONE thread of the pair's first CTA.
+// Descriptors and addresses hold for both CTAs: each brings its 128 rows of A and its half of B's rows.
+__device__ __forceinline__ void umma_f8_ss_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -138,41 +143,44 @@ struct Fp8Params {
     __half* y;
     const float* scale;
     int M, N, K;
+    int tokens;    // per tile
     int e5m2;      // the persistent plane is E5M2 (else E4M3, whose bytes read as FP8 are 2^8 times the weights)
     int* status;
 };
 
 constexpr int kEpiCols = 32;                                      // token columns per epilogue chunk
-constexpr int kEpiBytes = kEpiCols * kRows * 2;                   // 8 KB buffer behind the ring
+constexpr int kEpiBytes = kEpiCols * kRows * 2 + 4 * kMaxTokens * 4;   // behind the ring: four warps' chunks (2 KB each) and scales
 
-// Persistent: one CTA per SM walks the tiles (groups of 8 row tiles x all token tiles).  Two
-// accumulators of 256 columns fill tensor memory, so the MMA warp starts the next tile while the
-// four epilogue warps drain the previous one -- at FP8 rates the epilogue of a 128 x 256 tile is a
-// fifth of the tile's MMA time.  The epilogue goes through a small buffer, 32 token columns at a
-// time: the stage ring never idles.
-template <int kTokens>
+// Persistent: one CTA pair per two SMs walks the tiles (groups of 8 row tiles x all token tiles).  What bounds the
+// main loop is not the tensor pipe but what an SM can pull out of L2, about 50 bytes a clock: a CTA by itself with
+// a 128 x 256 tile needs 48 KB per 512 tensor cycles, a pair with a 256 x 256 tile 32 KB per CTA, since each CTA
+// fetches half of the tokens and the tensor cores of both read both halves.  Four Llama-7B linears at 512 / 2048 /
+// 8192 tokens: 147 / 413 / 1562 us with single CTAs, 123 / 361 / 1428 us with pairs (2.35 PFLOP/s; from about 2000
+// tokens on the 1000 W power cap holds the clock down).
+// Two accumulators of 256 columns fill tensor memory, so the MMA warp starts the next tile while the four
+// epilogue warps of each CTA drain the previous one.  The epilogue goes through a small buffer, 32 token columns
+// at a time: the stage ring never idles.
 __global__ void __launch_bounds__(kThreads, 1)
 fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_x,
                      const Fp8Params prm) {
-    constexpr int kStageBytes = stage_bytes_fp8(kTokens);
-    constexpr int kStages = stages_fp8(kTokens);
-    constexpr uint32_t kTmemCols = 2 * kTokens;   // two accumulators
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_full[kStages];
+    __shared__ __align__(8) uint64_t bar_full[kStages];     // the first CTA's count for both
     __shared__ __align__(8) uint64_t bar_empty[kStages];
     __shared__ __align__(8) uint64_t bar_d_full[2];
-    __shared__ __align__(8) uint64_t bar_d_empty[2];
+    __shared__ __align__(8) uint64_t bar_d_empty[2];        // the first CTA's count for both
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;    // set by an epilogue warp whose wait timed out; the four leave together
 
     grid_launch_dependents();
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t epi_base = smem_base + (uint32_t)(kStages * kStageBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row_tiles = (prm.N + kRows - 1) / kRows, tok_tiles = (prm.M + kTokens - 1) / kTokens;
+    const int rank = (int)cluster_ctarank();
+    const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
+    const int tokens = prm.tokens;
+    const int row_tiles = (prm.N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (prm.M + tokens - 1) / tokens;
     const int total = row_tiles * tok_tiles;
     const int num_kb = (prm.K + kBlockBytes - 1) / kBlockBytes;
-    auto tile_origin = [&](int lin, int& n0, int& m0) {
+    auto tile_origin = [&](int lin, int& n0, int& m0) {     // this CTA's first row, the pair's first token
         int row_tile = lin, tok_tile = 0;
         if (tok_tiles > 1) {
             constexpr int kRowGroup = 8;
@@ -182,8 +190,8 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
             row_tile = group * kRowGroup + within % rows_here;
             tok_tile = within / rows_here;
         }
-        n0 = row_tile * kRows;
-        m0 = tok_tile * kTokens;
+        n0 = (2 * row_tile + rank) * kRows;
+        m0 = tok_tile * tokens;
     };
 
     if (threadIdx.x == 0) {
@@ -193,58 +201,72 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(smem_u32(&bar_d_full[a]), 1);
-            mbar_init(smem_u32(&bar_d_empty[a]), 4);   // one arrival per epilogue warp
+            mbar_init(smem_u32(&bar_d_empty[a]), 8);   // one arrival per epilogue warp of the pair
         }
-        abort_flag = 0;
         fence_barrier_init();
         prefetch_tensormap(&map_p);
         prefetch_tensormap(&map_x);
     }
-    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), kTmemCols);
+    if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_slot), kTmemCols);
     tc_fence_before_sync();
     __syncthreads();
+    cluster_sync_all();           // the other CTA's barriers exist
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
 
     bool ok = true;
     if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        grid_dependency_wait();   // the activation codes come from the quantisation kernel
+        // ---------------- TMA producer: this CTA's rows and its half of the tokens ----------------
+        const uint32_t half_tokens = (uint32_t)tokens / 2;
+        const uint32_t pair_bytes = 2u * (kRows + half_tokens) * kBlockBytes;
+        auto load_plane = [&](int s, int i, int n0) {
+            // (the second CTA's bytes may land before this: the phase still waits for the one arrival)
+            if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_full[s]), pair_bytes);
+            tma_load_2d_pair(smem_base + (uint32_t)s * kStageBytes, &map_p, map_to_cta(smem_u32(&bar_full[s]), 0u),
+                             i * kBlockBytes, n0);
+        };
+        // the plane is model state: its first stages are requested before the preceding kernel (the quantisation,
+        // whose codes and scales this kernel reads) has ended
+        const int ahead = min(num_kb, kStages);
+        int n0, m0;
+        tile_origin(pair, n0, m0);
+        if (elect_one())
+            for (int i = 0; i < ahead; ++i) load_plane(i, i, n0);
+        __syncwarp();
+        grid_dependency_wait();
         int s = 0;
         uint32_t ph = 0;
-        for (int lin = blockIdx.x; lin < total && ok; lin += gridDim.x) {
-            int n0, m0;
+        for (int lin = pair; lin < total && ok; lin += pairs) {
             tile_origin(lin, n0, m0);
+            m0 += rank * (int)half_tokens;
             for (int i = 0; i < num_kb && ok; ++i, s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0)) {
                 ok = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 if (elect_one()) {
-                    const uint32_t full = smem_u32(&bar_full[s]);
-                    const uint32_t dst = smem_base + (uint32_t)s * kStageBytes;
-                    mbar_arrive_expect_tx(full, (uint32_t)kStageBytes);
-                    tma_load_2d(dst, &map_p, full, i * kBlockBytes, n0);
-                    tma_load_2d(dst + kRows * kBlockBytes, &map_x, full, i * kBlockBytes, m0);
+                    if (lin != pair || i >= ahead) load_plane(s, i, n0);
+                    tma_load_2d_pair(smem_base + (uint32_t)(s * kStageBytes + kRows * kBlockBytes), &map_x,
+                                     map_to_cta(smem_u32(&bar_full[s]), 0u), i * kBlockBytes, m0);
                 }
                 __syncwarp();
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
-        const uint32_t idesc = idesc_f8(kRows, kTokens, prm.e5m2 ? 1 : 0, 0);
+        // ---------------- MMA issuer: the pair's first CTA ----------------
+        const uint32_t idesc = idesc_f8(2 * kRows, tokens, prm.e5m2 ? 1 : 0, 0);
         int s = 0, it = 0;
         uint32_t ph = 0;
-        for (int lin = blockIdx.x; lin < total && ok; lin += gridDim.x, ++it) {
+        for (int lin = pair; rank == 0 && lin < total && ok; lin += pairs, ++it) {
             const int acc = it & 1;
-            if (it >= 2) {   // the tile before last used this accumulator: its epilogue must have read it out
-                ok = mbar_wait(smem_u32(&bar_d_empty[acc]), (uint32_t)((it >> 1) - 1) & 1u);
+            if (it >= 2) {   // the tile before last used this accumulator: both epilogues must have read it out
+                ok = mbar_wait_cluster(smem_u32(&bar_d_empty[acc]), (uint32_t)((it >> 1) - 1) & 1u);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 tc_fence_after_sync();
             }
-            const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kTokens);
+            const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kMaxTokens);
             for (int i = 0; i < num_kb && ok; ++i, s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0)) {
-                ok = mbar_wait(smem_u32(&bar_full[s]), ph);
+                ok = mbar_wait_cluster(smem_u32(&bar_full[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 tc_fence_after_sync();
@@ -253,87 +275,101 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
                     const uint64_t adesc = umma_desc_k_sw128(abase), bdesc = umma_desc_k_sw128(abase + kRows * kBlockBytes);
 #pragma unroll
                     for (int j = 0; j < kBlockBytes / 32; ++j)   // 32 K elements = 32 bytes per instruction
-                        umma_f8_ss(tmem_d, adesc + (uint64_t)(j * 2), bdesc + (uint64_t)(j * 2), idesc,
-                                   (i > 0 || j > 0) ? 1u : 0u);
-                    umma_commit(smem_u32(&bar_empty[s]));
-                    if (i == num_kb - 1) umma_commit(smem_u32(&bar_d_full[acc]));
+                        umma_f8_ss_pair(tmem_d, adesc + (uint64_t)(j * 2), bdesc + (uint64_t)(j * 2), idesc,
+                                        (i > 0 || j > 0) ? 1u : 0u);
+                    umma_commit_pair(smem_u32(&bar_empty[s]));
+                    if (i == num_kb - 1) umma_commit_pair(smem_u32(&bar_d_full[acc]));
                 }
                 __syncwarp();
             }
         }
     } else {
         // ---------------- epilogue: D[row][token] * scale[token] -> FP16 -> y[token][n0 + row] ----------------
+        // Every warp by itself, without barriers among the four: its 32 rows are 64 contiguous bytes of a token's y,
+        // whole sectors.  32 token columns go through 2 KB of shared memory of its own, [token][row].  (With barriers
+        // among the four warps and the scales fetched per thread and column, a tile of 256 tokens took 6 us more than its
+        // MMAs at 4096 columns: QKV at 2048 tokens 101 against 89 us.)
         const int q = warp & 3;                          // TMEM lane quarter this warp may touch
-        const int row = q * 32 + lane;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const float wscale = prm.e5m2 ? 1.0f : 0.00390625f;   // E4M3 bytes read as FP8 are 2^8 times the weights
-        const int et = (int)threadIdx.x - 64;            // index among the 128 epilogue threads
+        const uint32_t buf = epi_base + (uint32_t)(q * kEpiCols * 64);
+        float* scales = reinterpret_cast<float*>(smem_raw + (epi_base - smem_u32(smem_raw)) + 4 * kEpiCols * 64) + q * kMaxTokens;
         int it = 0;
-        for (int lin = blockIdx.x; lin < total; lin += gridDim.x, ++it) {
+        for (int lin = pair; lin < total; lin += pairs, ++it) {
             int n0, m0;
             tile_origin(lin, n0, m0);
             const int acc = it & 1;
-            const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kTokens);
-            const int ncols = min(kTokens, prm.M - m0);
-            if (ok) ok = mbar_wait(smem_u32(&bar_d_full[acc]), (uint32_t)(it >> 1) & 1u);
+            const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kMaxTokens) + lane_base;
+            const int ncols = min(tokens, prm.M - m0);
+            ok = mbar_wait_cluster(smem_u32(&bar_d_full[acc]), (uint32_t)(it >> 1) & 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
-            if (ok) tc_fence_after_sync();
-            else abort_flag = 1;
-            // same trip count in all four warps (it depends on the tile only): the barriers always match
+            if (!ok) break;
+            tc_fence_after_sync();
+            // (written by the preceding kernel; the accumulator could not be complete before it was)
+            for (int c = lane; c < ncols; c += 32) scales[c] = prm.scale[m0 + c] * wscale;
+            __syncwarp();
+            const int row0 = n0 + q * 32;                // this warp's first row
+            __half* yrow = prm.y + (int64_t)(m0 + (lane >> 2)) * prm.N + row0 + (lane & 3) * 8;
+            const bool row_in = row0 + (lane & 3) * 8 < prm.N;   // N is a multiple of 8
             for (int c0 = 0; c0 < ncols; c0 += kEpiCols) {
-                if (ok) {
-#pragma unroll
-                    for (int h = 0; h < kEpiCols / 16; ++h) {
-                        const int cb = c0 + 16 * h;
-                        if (cb >= ncols) break;
-                        uint32_t v[16];
-                        tmem_ld_32x32b_x16(tmem_d + lane_base + (uint32_t)cb, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int c = cb + j;
-                            const float sc = c < ncols ? prm.scale[m0 + c] * wscale : 0.f;
-                            const __half hv = __float2half_rn(__uint_as_float(v[j]) * sc);
-                            const uint32_t addr = epi_base + (uint32_t)(((c - c0) * kRows + row) * 2);
-                            asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(__half_as_ushort(hv)) : "memory");
-                        }
-                    }
-                }
+                uint32_t v[32];
+                tmem_ld_32x32b_x32(tmem_d + (uint32_t)c0, v);
+                tmem_wait_ld();
                 if (c0 + kEpiCols >= ncols) {            // last chunk read: the accumulator is free again
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bar_d_empty[acc]));
+                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_d_empty[acc]), 0u));
                 }
-                named_barrier_sync(1, 128);
-                if (ok) {
-                    constexpr int kChunks = kRows / 8;   // 16-byte pieces of one token's rows
-                    const int cols_here = min(kEpiCols, ncols - c0);
-                    for (int item = et; item < cols_here * kChunks; item += 128) {
-                        const int c = item / kChunks, qq = item % kChunks;
-                        const int n = n0 + qq * 8;
-                        if (n >= prm.N) continue;        // N is a multiple of 8
-                        uint4 val;
-                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
-                                     : "r"(epi_base + (uint32_t)((c * kRows + qq * 8) * 2)));
-                        *reinterpret_cast<uint4*>(prm.y + (int64_t)(m0 + c0 + c) * prm.N + n) = val;
-                    }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const __half hv = __float2half_rn(__uint_as_float(v[j]) * scales[c0 + j]);   // columns past ncols are not stored
+                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(buf + (uint32_t)(j * 64 + lane * 2)), "h"(__half_as_ushort(hv))
+                                 : "memory");
                 }
-                named_barrier_sync(1, 128);              // the buffer is free for the next chunk
-            }
-            if (*reinterpret_cast<volatile int*>(&abort_flag)) {   // read after the tile's last barrier: the same in all four warps
-                ok = false;
-                break;
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {            // 8 tokens x 64 bytes per instruction
+                    const int c = c0 + 8 * i + (lane >> 2);
+                    uint4 val;
+                    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+                                 : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
+                                 : "r"(buf + (uint32_t)(i * 512 + lane * 16)));
+                    if (row_in && c < ncols) *reinterpret_cast<uint4*>(yrow + (int64_t)(c0 + 8 * i) * prm.N) = val;
+                }
+                __syncwarp();                            // the buffer is free for the next chunk
             }
         }
     }
     if (!ok) atomicExch(prm.status, (int)DPS_ERR_CUDA);
     tc_fence_before_sync();
     __syncthreads();
+    cluster_sync_all();           // nobody frees tensor memory or leaves while the pair still works
     if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc_pair(tmem_base, kTmemCols);
     }
+}
+
+// Tokens per tile.  A round of tiles over the pairs takes as long as its slowest member, so the number of token tiles
+// is chosen to make the sum over the rounds small.  Measured per K block on Llama-7B QKV, 512 tokens: 0.24 / 0.30 / 0.41 /
+// 0.48 us with tiles of 64 / 128 / 192 / 256 tokens, i.e. proportional to 128 + tokens (a CTA's share of what comes out
+// of L2 is 128 rows and half of the tokens, its tensor time grows with the tokens).
+// DPS_FP8_TOKENS=16..256 overrides (tuning knob).
+int pick_tokens(int64_t M, int64_t N, int pairs) {
+    static const int forced = [] {
+        const char* e = getenv("DPS_FP8_TOKENS");
+        return e ? atoi(e) / 16 * 16 : 0;
+    }();
+    if (forced >= 16 && forced <= kMaxTokens) return forced;
+    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows);
+    int64_t best = 16, best_cost = INT64_MAX;
+    for (int64_t t = (M + kMaxTokens - 1) / kMaxTokens, end = 2 * t + 6; t <= end; ++t) {
+        const int64_t tokens = ((M + t - 1) / t + 15) / 16 * 16;
+        const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens), rounds = (tiles + pairs - 1) / pairs;
+        const int64_t cost = rounds * (128 + tokens);
+        if (cost < best_cost) { best_cost = cost; best = tokens; }
+    }
+    return (int)best;
 }
 
 }  // namespace
@@ -355,21 +391,20 @@ cudaError_t launch_quantize_activations(const void* x, uint8_t* q, float* scale,
     return e;
 }
 
-namespace {
-template <int kTokens>
-cudaError_t launch_fp8_tokens(int enc, const uint8_t* q, const float* scale, const uint8_t* p, void* y, int64_t M, int64_t N,
-                              int64_t K, int* status, cudaStream_t stream) {
-    static PerDeviceOnce setup;     // per instantiation and per device
-    const size_t smem = (size_t)stages_fp8(kTokens) * stage_bytes_fp8(kTokens) + kEpiBytes + 1024;
-    auto kernel = fp8act_linear_kernel<kTokens>;
+cudaError_t launch_linear_fp8act(int enc, const uint8_t* q, const float* scale, const uint8_t* p, void* y, int64_t M,
+                                 int64_t N, int64_t K, int* status, cudaStream_t stream) {
+    static PerDeviceOnce setup;     // per device
+    const size_t smem = (size_t)kStages * kStageBytes + kEpiBytes + 1024;
     {
         const cudaError_t e = setup.run(
-            [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+            [&] { return cudaFuncSetAttribute(fp8act_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
         if (e != cudaSuccess) return e;
     }
+    const int pairs = sm_count() / 2;
+    const int tokens = pick_tokens(M, N, pairs);
     CUtensorMap mp, mx;
     if (!make_byte_map_sw128(&mp, p, (uint64_t)N, (uint64_t)K, kRows) ||
-        !make_byte_map_sw128(&mx, q, (uint64_t)M, (uint64_t)K, kTokens))
+        !make_byte_map_sw128(&mx, q, (uint64_t)M, (uint64_t)K, (uint32_t)tokens / 2))
         return cudaErrorInvalidValue;
     Fp8Params prm;
     prm.y = static_cast<__half*>(y);
@@ -377,31 +412,27 @@ cudaError_t launch_fp8_tokens(int enc, const uint8_t* q, const float* scale, con
     prm.M = (int)M;
     prm.N = (int)N;
     prm.K = (int)K;
+    prm.tokens = tokens;
     prm.e5m2 = enc == DPS_ENC_E5M2;
     prm.status = status;
-    const int64_t tiles = ((N + kRows - 1) / kRows) * ((M + kTokens - 1) / kTokens);
+    const int64_t tiles = ((N + 2 * kRows - 1) / (2 * kRows)) * ((M + tokens - 1) / tokens);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(tiles < sm_count() ? tiles : sm_count()), 1, 1);   // one CTA per SM walks the tiles
+    cfg.gridDim = dim3((unsigned)(2 * (tiles < pairs ? tiles : pairs)), 1, 1);   // one pair per two SMs walks the tiles
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mp, mx, prm);
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fp8act_linear_kernel, mp, mx, prm);
     count_launch();
     return e;
-}
-}  // namespace
-
-cudaError_t launch_linear_fp8act(int enc, const uint8_t* q, const float* scale, const uint8_t* p, void* y, int64_t M,
-                                 int64_t N, int64_t K, int* status, cudaStream_t stream) {
-    // 256-token tiles unless they would leave SMs without a tile (few weight rows, few tokens)
-    const int64_t tiles256 = ((N + kRows - 1) / kRows) * ((M + 255) / 256);
-    if (tiles256 < sm_count() && M > 128) return launch_fp8_tokens<128>(enc, q, scale, p, y, M, N, K, status, stream);
-    return launch_fp8_tokens<256>(enc, q, scale, p, y, M, N, K, status, stream);
 }
 
 }  // namespace dps
