@@ -73,6 +73,7 @@ int forced_path() {
         if (!strcmp(v, "gemv")) return 1;
         if (!strcmp(v, "umma")) return 2;
         if (!strcmp(v, "stream")) return 3;
+        if (!strcmp(v, "pair")) return 4;
         return 0;
     }();
     return path;
@@ -138,6 +139,14 @@ int sm_count() {
 using namespace dps;
 
 namespace {
+// 65-128 tokens: two 64-token decode tiles per 128 weight rows (K split over a cluster) instead of CTA pairs with 256-row
+// tiles, where the latter would leave most SMs idle and the weights are few enough to be streamed out of L2 and rebuilt
+// twice.  Measured, fast / full mode, 96-128 tokens: 4096 x 4096 10.4 / 14.1 us against 12.8 / 14.1-15.9, 2048 x 2048
+// 6.9 / 7.4 against 9.3 / 10.7, 6144 x 1024 6.9 / 8.2 against 7.9 / 9.1; 3088 x 8336 in full mode 25.2 against 20.0,
+// 4632 x 3088 16.6 / 23.1 against 12.4 / 14.5, 12288 x 4096 20.2 / 39.9 against 16.2 / 24.1.
+bool decode_tiles_for_128(bool full, int64_t M, int64_t N, int64_t K) {
+    return M <= 128 && ((N <= 4096 && N * K <= ((int64_t)1 << (full ? 24 : 26))) || N * K <= ((int64_t)1 << 23));
+}
 bool known_encoding(int32_t enc) {
     return enc == DPS_ENC_E4M3 || enc == DPS_ENC_E5M2 || enc == DPS_ENC_E4M3_RN || enc == DPS_ENC_E5M2_RN;
 }
@@ -258,16 +267,21 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     // and hidden-8192 shapes, in both modes: the tensor-core kernel's set-up and cluster reduction
     // cost a few microseconds per launch, its TMA stream is faster once running; it wins from 2^25
     // weights on (by 0-20 %), the streaming kernel below (4096 x 4096: by 15-30 %).  Beyond 16
-    // tokens the tcgen05 tiles take over.  (The CUDA-core GEMV is kept as a cross-check.)
+    // tokens the tcgen05 tiles take over, beyond 64 tokens CTA pairs (four Llama-7B linears, fast / full mode: 64 tokens
+    // 62 / 97 us with the tiles, 75 / 109 with pairs; 96 tokens 84 / 134 against 74 / 107).  (The CUDA-core GEMV is
+    // kept as a cross-check.)
     const bool stream_mid = N * K < ((int64_t)1 << 25);
     const int path = forced_path();
     cudaError_t err;
     if (path == 1) err = launch_gemv(mode, enc, x, w_persist, r, y, M, N, K, stream);
     else if (path == 2) err = launch_umma_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
+    else if (path == 4) err = launch_pair_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
     else if (path == 3 || M <= 8 || (M <= 16 && stream_mid)) {
         if (M > 16) return DPS_ERR_UNSUPPORTED;      // (only reachable with DPS_FORCE_PATH=stream)
         err = launch_decode_mma(mode, enc, x, w_persist, r, y, M, N, K, stream);
-    } else err = launch_umma_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
+    } else if (M > 64 && !decode_tiles_for_128(mode == DPS_MODE_FULL, M, N, K))
+        err = launch_pair_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
+    else err = launch_umma_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
     return err == cudaSuccess ? DPS_OK : DPS_ERR_CUDA;
 }
 

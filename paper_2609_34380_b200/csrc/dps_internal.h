@@ -57,6 +57,10 @@ cudaError_t launch_decode_mma(int mode, int enc, const void* x, const uint8_t* p
 cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y,
                                int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream);
 
+// Dense linear on CTA pairs (any M; meant for many tokens).
+cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
+                               int64_t N, int64_t K, int* status, cudaStream_t stream);
+
 // Grouped linear on the tensor-core path.  e5m2_mask: 64 words, bit e of the first 32 set for an E5M2
 // expert, of the last 32 for a rounded nest.  x_sorted: [A][K] activations grouped by expert;
 // tiles / num_tiles / sorted_rows: device tables built by the routing pre-pass; tn: token-tile

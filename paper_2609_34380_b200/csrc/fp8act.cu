@@ -259,14 +259,14 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
         for (int lin = pair; rank == 0 && lin < total && ok; lin += pairs, ++it) {
             const int acc = it & 1;
             if (it >= 2) {   // the tile before last used this accumulator: both epilogues must have read it out
-                ok = mbar_wait_cluster(smem_u32(&bar_d_empty[acc]), (uint32_t)((it >> 1) - 1) & 1u);
+                ok = mbar_wait(smem_u32(&bar_d_empty[acc]), (uint32_t)((it >> 1) - 1) & 1u);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 tc_fence_after_sync();
             }
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kMaxTokens);
             for (int i = 0; i < num_kb && ok; ++i, s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0)) {
-                ok = mbar_wait_cluster(smem_u32(&bar_full[s]), ph);
+                ok = mbar_wait(smem_u32(&bar_full[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 tc_fence_after_sync();
@@ -301,7 +301,7 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
             const int acc = it & 1;
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kMaxTokens) + lane_base;
             const int ncols = min(tokens, prm.M - m0);
-            ok = mbar_wait_cluster(smem_u32(&bar_d_full[acc]), (uint32_t)(it >> 1) & 1u);
+            ok = mbar_wait(smem_u32(&bar_d_full[acc]), (uint32_t)(it >> 1) & 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after_sync();

@@ -1,0 +1,599 @@
+// Dense linear layer for many tokens: tcgen05.mma over CTA PAIRS (cta_group::2), the rebuilt weights as the A operand in
+// tensor memory, the activations as the B operand in the shared memory of both CTAs.
+//
+// Paper: "Scheduler: Dual-Precision Execution" -- full mode combines the FP8 tensor with the residual tensor into the
+// original FP16 values during computation; fast mode uses the FP8 tensor alone.
+//
+// What bounds a prefill main loop on this part is what an SM can pull out of L2, about 50 bytes a clock, and in full mode
+// its shared memory (128 bytes a clock).  A CTA by itself with a 128 x 256 tile needs 48 KB (full mode) per 64 columns of K
+// and 512 tensor cycles; a CTA of a pair with a (2 x 128) x 256 tile needs 32 KB, because it fetches half of the tokens
+// and the tensor cores of both SMs read both halves.
+//
+// Tile: 256 weight rows x `tokens` tokens (a multiple of 16, chosen per launch), K walked in steps of 128.  Persistent: a pair
+// per two SMs walks the tiles.  Roles of a CTA (24 warps):
+//   warp 0       plane producer: units of 128 rows x 128 columns of P (and R) into a ring; a unit is handed back as soon as
+//                the zip warps have it in registers, so the ring holds nothing that waits for the tensor core
+//   warp 2       activation producer: this CTA's half of the tile's tokens into slots, a K step at a time (64 columns at a
+//                time the loop took 880 cycles per step)
+//   warp 3       waits for a step's activations and reports them to the first CTA
+//   warps 8-23   zip warps: plane bytes -> FP16 in registers -> tensor memory.  Eight take a step (a quarter of the rows and a
+//                half of the columns each), eight the next one.  A step is a chain of latencies in a warp (1400 cycles for
+//                64 columns: waits of 150 each even when nothing has to be waited for, loads and conversion 600), not
+//                arithmetic: eight warps in all made 650 cycles per 64 columns
+//   warp 1       (first CTA) issues the MMAs of the pair: one wait, eight MMAs and one commit per step, about 600 cycles;
+//                with a barrier of its own for the activations and another commit for the A slots, in steps of 64 columns,
+//                it took 650 per step however few tokens there were
+//   warps 4-7    epilogue of this CTA's rows: each warp takes its 32 rows by itself (64 contiguous bytes of a token's y)
+// Against single CTAs, the four Llama-7B linears together, fast / full mode: 256 tokens 140 / 183 -> 114 / 150 us, 512
+// 209 / 269 -> 174 / 237, 2048 715 / 889 -> 644 / 739, 8192 2696 / 3500 -> 2598 / 3007 (there the power cap holds the clock
+// near 1.4 GHz).
+// The arrivals on the other CTA's barriers carry no cluster-scope release: what they order is tensor memory
+// (tcgen05.fence) and shared memory; with the release a step took twice as long.
+#include <cuda_fp16.h>
+
+#include <cstdio>
+#include <cstdlib>
+
+#include "bits.cuh"
+#include "dps_internal.h"
+#include "sm100.cuh"
+#include "tensor_map.h"
+
+namespace dps {
+
+namespace {
+
+using namespace sm100;
+
+constexpr int kRows = 128;                 // weight rows of a row block in one CTA
+constexpr int kUnitK = 128;                // columns of K in a plane unit
+constexpr int kMaxUnits = 12, kMaxXSlots = 8;
+constexpr int kASteps = 4;                 // K steps the A ring holds
+constexpr int kACols = kUnitK / 2;         // tensor memory of one of them
+constexpr int kAccCols = 512 - kASteps * kACols;
+constexpr int kDone = 8;                   // ring of barriers that report completed K steps
+constexpr int kThreads = 768;
+constexpr int kMaxSplit = 4;               // pairs of a cluster (eight CTAs, the portable limit)
+constexpr int kEpiCols = 32;               // token columns per epilogue chunk
+constexpr int kEpiBytes = 4 * kEpiCols * 64;
+constexpr int kSmemBytes = 222 * 1024;     // ring + slots + epilogue chunks + alignment
+
+__host__ __device__ constexpr int unit_bytes(bool full) { return kRows * kUnitK * (full ? 2 : 1); }
+
+struct PairParams {
+    __half* y;
+    int M, N, K;
+    int tokens;        // per tile
+    int tail_tokens;   // per piece of a tile of the last, partial round
+    int tail_parts;    // pieces such a tile is cut into (1: not cut)
+    int units, x_slots;
+    int split;         // K split: pairs of a cluster that share a tile, each a range of its K steps (then one tile per cluster)
+    int* status;
+};
+
+// D[tmem] (+)= A[tmem] * B[smem] over a CTA pair; issued by ONE thread of the pair's first CTA.  Addresses and descriptor
+// hold for both CTAs: each brings its 128 rows of A and its half of B's rows.
+__device__ __forceinline__ void umma_f16_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+
+// Tensor memory: accumulators first (two tiles' worth where they fit, so that the next tile's MMAs overlap the epilogue),
+// then the A slots.
+struct Work {
+    int row_tile, m0;       // tile row index, first token
+    int tokens, ncols;      // MMA columns, columns that exist
+    bool piece;             // a piece of a tile of the last round
+};
+
+template <int ENC, bool FULL>
+__global__ void __launch_bounds__(kThreads, 1)
+umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r,
+                 const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_xt, const PairParams prm) {
+    constexpr int kUnit = unit_bytes(FULL);
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bar_p_full[kMaxUnits], bar_p_empty[kMaxUnits];
+    __shared__ __align__(8) uint64_t bar_x_full[kMaxXSlots];
+    __shared__ __align__(8) uint64_t bar_a_full[kASteps];       // the first CTA's: A and activations of both are ready
+    __shared__ __align__(8) uint64_t bar_done[kDone];           // the MMAs of a K step are complete
+    __shared__ __align__(8) uint64_t bar_d_full[2];
+    __shared__ __align__(8) uint64_t bar_d_empty[2];            // the first CTA's count for both
+    __shared__ uint32_t tmem_base_slot;
+
+    grid_launch_dependents();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int split = prm.split;
+    const uint32_t first = cluster_ctarank() & ~1u;             // cluster rank of the pair's first CTA
+    const int rank = (int)(cluster_ctarank() & 1u), ks = (int)(first >> 1);
+    const int pair = (int)blockIdx.x / (2 * split), pairs = (int)gridDim.x / (2 * split);   // (split > 1: the cluster)
+    const int units = prm.units, x_slots = prm.x_slots;
+    const int x_atom = prm.tokens / 2 * 128, x_bytes = 2 * x_atom;   // 64 columns of K; a slot, 128
+    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t x_base = smem_base + (uint32_t)(units * kUnit);
+    const uint32_t epi_base = x_base + (uint32_t)(x_slots * x_bytes);
+    const int row_tiles = (prm.N + 2 * kRows - 1) / (2 * kRows);
+    const int tok_tiles = (prm.M + prm.tokens - 1) / prm.tokens;
+    const int total = row_tiles * tok_tiles;
+    const int t_main = prm.tail_parts > 1 ? total - total % pairs : total;
+    const int all_steps = (prm.K + kUnitK - 1) / kUnitK;        // K steps of a tile ...
+    const int step0 = all_steps * ks / split;                   // ... and this pair's of them
+    const int steps_k = all_steps * (ks + 1) / split - step0;
+
+    // Work item `i` of this pair: whole tiles, then at most one piece of a tile of the last round.
+    auto work = [&](int i, Work& w) -> bool {
+        int lin = pair + i * pairs, part = 0;
+        w.piece = false;
+        if (lin >= t_main) {
+            if (lin - pair != t_main || prm.tail_parts <= 1) return false;
+            lin = t_main + pair / prm.tail_parts;
+            part = pair % prm.tail_parts;
+            if (lin >= total) return false;
+            w.piece = true;
+        }
+        int tok_tile = 0;
+        w.row_tile = lin;
+        if (tok_tiles > 1) {
+            // groups of 8 row tiles x all token tiles: the planes and activation tiles in use stay in L2
+            constexpr int kRowGroup = 8;
+            const int per_group = kRowGroup * tok_tiles;
+            const int group = lin / per_group, within = lin % per_group;
+            const int rows_here = min(kRowGroup, row_tiles - group * kRowGroup);
+            w.row_tile = group * kRowGroup + within % rows_here;
+            tok_tile = within / rows_here;
+        }
+        w.tokens = w.piece ? prm.tail_tokens : prm.tokens;
+        const int end = min(prm.M, (tok_tile + 1) * prm.tokens);
+        w.m0 = tok_tile * prm.tokens + part * prm.tail_tokens;
+        w.ncols = min(w.tokens, end - w.m0);
+        return w.ncols > 0;      // a piece past the last token is the end: nothing follows a piece
+    };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < units; ++s) {
+            mbar_init(smem_u32(&bar_p_full[s]), 1);
+            mbar_init(smem_u32(&bar_p_empty[s]), 8);            // the zip warps that take the step
+        }
+        for (int s = 0; s < x_slots; ++s) mbar_init(smem_u32(&bar_x_full[s]), 1);
+        for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 9);   // both CTAs' eight zip warps and warp 3
+        for (int a = 0; a < kDone; ++a) mbar_init(smem_u32(&bar_done[a]), 1);
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(smem_u32(&bar_d_full[a]), 1);
+            mbar_init(smem_u32(&bar_d_empty[a]), 8);            // the epilogue warps of both CTAs
+        }
+        fence_barrier_init();
+        prefetch_tensormap(&map_p);
+        if (FULL) prefetch_tensormap(&map_r);
+        prefetch_tensormap(&map_x);
+    }
+    if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_slot), 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    cluster_sync_all();           // the other CTA's barriers exist
+    tc_fence_after_sync();
+    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t tmem_a = tmem_base + kAccCols;
+    // accumulators: one or two tiles' worth
+    const int accs = 2 * prm.tokens <= kAccCols ? 2 : 1;
+
+    // K steps are counted over all tiles of the pair (t).  A waiter for step t cannot take an older phase of
+    // bar_done[t % kDone] for it: it has seen a step later than t - kDone before.
+    auto wait_done = [&](uint32_t t) { return mbar_wait(smem_u32(&bar_done[t % kDone]), (t / kDone) & 1u); };
+
+    bool ok = true;
+    Work w;
+    if (warp == 0) {
+        // ---------------- plane producer (model state: does not wait for the preceding kernel) ----------------
+        int s = 0;
+        uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
+        for (int i = 0; ok && work(i, w); ++i) {
+            const int row = (2 * w.row_tile + rank) * kRows;
+            for (int u = 0; u < steps_k && ok; ++u, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
+                ok = mbar_wait(smem_u32(&bar_p_empty[s]), ph);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                                if (!ok) break;
+                if (elect_one()) {
+                    const uint32_t full = smem_u32(&bar_p_full[s]), dst = smem_base + (uint32_t)(s * kUnit);
+                    mbar_arrive_expect_tx(full, (uint32_t)kUnit);
+                    tma_load_2d(dst, &map_p, full, (step0 + u) * kUnitK, row);
+                    if (FULL) tma_load_2d(dst + kRows * kUnitK, &map_r, full, (step0 + u) * kUnitK, row);
+                }
+                __syncwarp();
+            }
+        }
+    } else if (warp == 2) {
+        // ---------------- activation producer: this CTA's half of the tokens ----------------
+        grid_dependency_wait();
+        int s = 0;
+        uint32_t t = 0;
+        for (int i = 0; ok && work(i, w); ++i) {
+            const int half = w.tokens / 2;
+            const int m0 = w.m0 + rank * half;
+            const CUtensorMap* map = w.piece ? &map_xt : &map_x;
+            for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == x_slots) ? 0 : s + 1) {
+                if (t >= (uint32_t)x_slots) ok = wait_done(t - (uint32_t)x_slots);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                if (elect_one()) {
+                    const uint32_t full = smem_u32(&bar_x_full[s]), dst = x_base + (uint32_t)(s * x_bytes);
+                    mbar_arrive_expect_tx(full, (uint32_t)(2 * half * 128));
+                    tma_load_2d(dst, map, full, (step0 + j) * kUnitK, m0);
+                    tma_load_2d(dst + (uint32_t)x_atom, map, full, (step0 + j) * kUnitK + 64, m0);
+                }
+                __syncwarp();
+            }
+        }
+    } else if (warp == 3) {
+        // ---------------- reports the activations of a K step to the first CTA ----------------
+        int s = 0;
+        uint32_t ph = 0, t = 0;
+        for (int i = 0; ok && work(i, w); ++i) {
+            for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == x_slots) ? 0 : s + 1, ph ^= (s == 0)) {
+                if (t >= kASteps) ok = wait_done(t - kASteps);    // else the arrival might count for that step
+                if (ok) ok = mbar_wait(smem_u32(&bar_x_full[s]), ph);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (ok && lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_a_full[t % kASteps]), first));
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: the pair's first CTA ----------------
+        int xs = 0;
+        uint32_t t = 0;
+        for (int i = 0; rank == 0 && ok && work(i, w); ++i) {
+            const uint32_t idesc = umma_idesc_f16(2 * kRows, w.tokens);
+            const int acc = accs == 2 ? i & 1 : 0, use = accs == 2 ? i >> 1 : i;
+            const uint32_t tmem_d = tmem_base + (uint32_t)(acc * prm.tokens);
+            if (use > 0) {   // the tile before must have been read out of the accumulator by both CTAs
+                ok = mbar_wait(smem_u32(&bar_d_empty[acc]), (uint32_t)(use - 1) & 1u);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                                if (!ok) break;
+                tc_fence_after_sync();
+            }
+            for (int j = 0; j < steps_k && ok; ++j, ++t) {
+                const uint32_t a = t % kASteps;
+                const uint64_t bdesc0 = umma_desc_k_sw128(x_base + (uint32_t)(xs * x_bytes));
+                const uint64_t bdesc1 = bdesc0 + (uint64_t)(x_atom >> 4);
+                const bool second = (step0 + j) * kUnitK + 64 < prm.K;        // (behind the end of K both operands are zero)
+                ok = mbar_wait(smem_u32(&bar_a_full[a]), (t / kASteps) & 1u);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                                if (!ok) break;
+                tc_fence_after_sync();
+                if (elect_one()) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)                     // 16 columns of K = 32 bytes of the 128-byte swizzle atom
+                        umma_f16_ts_pair(tmem_d, tmem_a + a * kACols + q * 8, bdesc0 + (uint64_t)(q * 2), idesc,
+                                         (j > 0 || q > 0) ? 1u : 0u);
+                    if (second) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            umma_f16_ts_pair(tmem_d, tmem_a + a * kACols + 32 + q * 8, bdesc1 + (uint64_t)(q * 2), idesc, 1u);
+                    }
+                    umma_commit_pair(smem_u32(&bar_done[t % kDone]), first);
+                    if (j == steps_k - 1) umma_commit_pair(smem_u32(&bar_d_full[acc]), first);
+                }
+                __syncwarp();
+                xs = xs + 1 == x_slots ? 0 : xs + 1;
+            }
+        }
+    } else if (warp >= 8) {
+        // ---------------- zip warps: planes -> FP16 -> tensor memory ----------------
+        const int set = (warp - 8) >> 3, half = ((warp - 8) >> 2) & 1;   // K steps of this parity; columns 64 half ... of a step
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        const uint32_t sw = (uint32_t)(row & 7);                // TMA swizzle: 16-byte chunk index ^= row % 8
+        uint32_t s = 0, ph = 0, t = 0;
+        for (int i = 0; ok && work(i, w); ++i) {
+            for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == (uint32_t)units) ? 0 : s + 1, ph ^= (s == 0)) {
+                if ((int)(t & 1u) != set) continue;             // (an even number of units: a unit's readers are always the same)
+                ok = mbar_wait(smem_u32(&bar_p_full[s]), ph);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                                if (!ok) break;
+                const uint32_t prow = smem_base + s * kUnit + (uint32_t)(row * kUnitK);
+                uint32_t h[32];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t off = ((uint32_t)(4 * half + c) ^ sw) * 16u;
+                    const uint4 pv = lds128(prow + off);
+                    const uint4 rv = FULL ? lds128(prow + kRows * kUnitK + off) : make_uint4(0, 0, 0, 0);
+                    uint32_t h8[8];
+                    if (FULL) join16<ENC, FULL>(pv, rv, h8);
+                    else fast16<ENC>(pv, h8);   // E4M3: 2^8 times the weights, undone in the epilogue
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) h[c * 8 + q] = h8[q];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_p_empty[s]));
+                const uint32_t a = t % kASteps;
+                if (t >= kASteps) ok = wait_done(t - kASteps);  // the MMAs that read the slot before
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                                if (!ok) break;
+                tc_fence_after_sync();
+                tmem_st_32x32b_x32(tmem_a + lane_base + a * kACols + (uint32_t)(half * 32), h);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_a_full[a]), first));
+            }
+        }
+    } else {
+        // ---------------- epilogue: D[row][token] -> FP16 -> y[token][row], every warp its 32 rows ----------------
+        const int q = warp & 3;
+        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        const uint32_t buf = epi_base + (uint32_t)(q * kEpiCols * 64);
+        const float out_scale = (!FULL && base_enc(ENC) == kEncE4M3) ? 0.00390625f : 1.0f;
+        for (int i = 0; work(i, w); ++i) {
+            const int acc = accs == 2 ? i & 1 : 0, use = accs == 2 ? i >> 1 : i;
+            ok = mbar_wait(smem_u32(&bar_d_full[acc]), (uint32_t)use & 1u);
+            ok = __all_sync(0xFFFFFFFFu, ok);
+                        if (!ok) break;
+            tc_fence_after_sync();
+            const uint32_t tmem_d = tmem_base + lane_base + (uint32_t)(acc * prm.tokens);
+            if (split > 1) {
+                // a range of K: the FP32 partial tile goes to shared memory, [token][row], over the rings -- the tile's MMAs are
+                // complete, nothing is in flight any more -- and is summed after the role loops
+                for (int c0 = 0; c0 < w.ncols; c0 += kEpiCols) {
+                    uint32_t v[32];
+                    tmem_ld_32x32b_x32(tmem_d + (uint32_t)c0, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (c0 + j < w.ncols)
+                            asm volatile("st.shared.f32 [%0], %1;" ::"r"(smem_base + (uint32_t)(((c0 + j) * kRows + q * 32 + lane) * 4)),
+                                         "f"(__uint_as_float(v[j]) * out_scale)
+                                         : "memory");
+                }
+                break;
+            }
+            const int n = (2 * w.row_tile + rank) * kRows + q * 32 + (lane & 3) * 8;
+            __half* yrow = prm.y + (int64_t)(w.m0 + (lane >> 2)) * prm.N + n;
+            for (int c0 = 0; c0 < w.ncols; c0 += kEpiCols) {
+                uint32_t v[32];
+                tmem_ld_32x32b_x32(tmem_d + (uint32_t)c0, v);
+                tmem_wait_ld();
+                if (c0 + kEpiCols >= w.ncols) {          // last chunk read: the accumulator is free again
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_d_empty[acc]), first));
+                }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const __half hv = __float2half_rn(__uint_as_float(v[j]) * out_scale);
+                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(buf + (uint32_t)(j * 64 + lane * 2)),
+                                 "h"(__half_as_ushort(hv))
+                                 : "memory");
+                }
+                __syncwarp();
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {            // 8 tokens x 64 bytes per instruction; N is a multiple of 8
+                    const uint4 val = lds128(buf + (uint32_t)(t * 512 + lane * 16));
+                    if (n < prm.N && c0 + 8 * t + (lane >> 2) < w.ncols)
+                        *reinterpret_cast<uint4*>(yrow + (int64_t)(c0 + 8 * t) * prm.N) = val;
+                }
+                __syncwarp();                            // the buffer is free for the next chunk
+            }
+        }
+    }
+    if (!ok) atomicExch(prm.status, (int)DPS_ERR_CUDA);
+    if (split > 1) {
+        // The cluster's partial tiles, summed in the order of their K ranges: pair ks takes every split-th token, each CTA its
+        // own 128 rows (the same in all pairs), consecutive threads consecutive 8-row pieces.
+        __syncthreads();
+        cluster_sync_all();
+        if (work(0, w)) {
+            const int n0 = (2 * w.row_tile + rank) * kRows;
+            const int mine = (w.ncols - ks + split - 1) / split;
+            for (int idx = (int)threadIdx.x; idx < mine * (kRows / 8); idx += kThreads) {
+                const int c = ks + split * (idx / (kRows / 8)), n = n0 + (idx % (kRows / 8)) * 8;
+                if (n >= prm.N) continue;                // N is a multiple of 8
+                const uint32_t local = smem_base + (uint32_t)((c * kRows + (idx % (kRows / 8)) * 8) * 4);
+                float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int p = 0; p < split; ++p) {
+                    const uint32_t from = map_to_cta(local, (uint32_t)(2 * p + rank));
+                    const float4 a = ld_cluster_v4_f32(from), b = ld_cluster_v4_f32(from + 16u);
+                    sum[0] += a.x; sum[1] += a.y; sum[2] += a.z; sum[3] += a.w;
+                    sum[4] += b.x; sum[5] += b.y; sum[6] += b.z; sum[7] += b.w;
+                }
+                uint32_t out[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __half2 h = __floats2half2_rn(sum[2 * k], sum[2 * k + 1]);
+                    out[k] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+                *reinterpret_cast<uint4*>(prm.y + (int64_t)(w.m0 + c) * prm.N + n) = make_uint4(out[0], out[1], out[2], out[3]);
+            }
+        }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    cluster_sync_all();           // nobody frees tensor memory or leaves while the pair still works
+    if (warp == 1) {
+        tc_fence_after_sync();
+        tmem_dealloc_pair(tmem_base, 512);
+    }
+}
+
+// ---- host side ---------------------------------------------------------------------------------
+
+struct Plan {
+    int tokens = 256, tail_parts = 1, tail_tokens = 256, split = 1;
+    double cost = 0;
+};
+
+// Time of one K step of a tile in ns, all pairs at work: measured with 74 and 148 tiles of one width (18944 and 37888 rows,
+// 8192 columns; in full mode, up to 128 tokens, on planes that come out of L2) every 32 tokens, between them in proportion.
+double step_ns(bool full, int tokens) {
+    static const double fast_ns[9] = {370, 370, 415, 480, 535, 610, 685, 750, 850};
+    static const double full_ns[9] = {500, 500, 520, 600, 680, 800, 1000, 1040, 1100};
+    const double* t = full ? full_ns : fast_ns;
+    const int i = tokens >= 256 ? 7 : tokens / 32;
+    return t[i] + (t[i + 1] - t[i]) * (tokens - 32 * i) / 32.0;
+}
+
+// A round of tiles over the pairs takes as long as one tile, so the number of token tiles is chosen to make the sum over the
+// rounds small; the tiles of a last, partial round are cut into pieces of the tokens if that shortens it.  Few tiles: up to
+// four pairs share each, a range of K each; capacity[s] = clusters of s pairs that are resident at once.
+// DPS_PAIR_TOKENS=16..256 and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
+Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) {
+    static const int forced = [] { const char* e = getenv("DPS_PAIR_TOKENS"); return e ? atoi(e) / 16 * 16 : 0; }();
+    static const int forced_split = [] { const char* e = getenv("DPS_PAIR_SPLIT"); return e ? atoi(e) : 0; }();
+    const int64_t steps = (K + kUnitK - 1) / kUnitK, pairs = capacity[1];
+    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), t0 = (M + 255) / 256;
+    Plan best;
+    for (int64_t t = t0; t <= 2 * t0 + 4; ++t) {
+        int64_t tokens = ((M + t - 1) / t + 15) / 16 * 16;
+        if (forced >= 16 && forced <= 256) tokens = forced;
+        const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens);
+        for (int split = 1; split <= kMaxSplit; ++split) {
+            if (split > 1 && (tiles > capacity[split] || steps < 2 * split)) continue;
+            if (forced_split && split != forced_split && !(split == 1 && (tiles > capacity[forced_split] || steps < 2 * forced_split)))
+                continue;
+            const int64_t rounds = tiles / pairs, tail = split > 1 ? 1 : tiles % pairs;
+            Plan p;
+            p.split = split;
+            p.tokens = p.tail_tokens = (int)tokens;
+            // between tiles: with one accumulator the MMAs wait until it has been read out
+            const double drain = 2 * tokens <= kAccCols ? 100.0 : 3.0 * (double)tokens;
+            const double cost1 = step_ns(full, (int)tokens);
+            p.cost = (double)rounds * ((double)steps * cost1 + drain) + 4.0 * (double)tokens;
+            if (split > 1) {
+                // the sum over the cluster, measured: 1 us + 30 ns per token
+                p.cost = (double)((steps + split - 1) / split) * cost1 + 1000.0 + 30.0 * (double)tokens;
+            } else if (tail > 0) {
+                double last = (double)steps * cost1;
+                for (int parts = 2; rounds > 0 && parts <= 8 && parts * tail <= pairs && 16 * parts <= tokens; ++parts) {
+                    const int tt = (int)(((tokens + parts - 1) / parts + 15) / 16 * 16);
+                    const double c = 1.2 * (double)steps * step_ns(full, tt) + drain;   // (the pieces stream the planes again)
+                    if (c < 0.9 * last) { last = c; p.tail_parts = parts; p.tail_tokens = tt; }
+                }
+                p.cost += last;
+            }
+            if (best.cost == 0 || p.cost < best.cost) best = p;
+        }
+    }
+    return best;
+}
+
+template <int ENC, bool FULL>
+cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K, int* status,
+                       cudaStream_t stream) {
+    auto kernel = umma_pair_kernel<ENC, FULL>;
+    // Clusters of s pairs that are resident at once, per device (they must fit inside a GPC): filled by the first call on a
+    // device, read only after that set-up has returned.
+    static int capacity_of[kMaxDevices][kMaxSplit + 1] = {};
+    static PerDeviceOnce setup;     // per instantiation and per device
+    int dev = 0;
+    {
+        const cudaError_t e = setup.run([&] {
+            int d = 0;
+            cudaGetDevice(&d);
+            const cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+            if (a != cudaSuccess) return a;
+            for (int s = 1; s <= kMaxSplit; ++s) {
+                cudaLaunchConfig_t q = {};
+                q.gridDim = dim3((unsigned)(2 * s), 1, 1);
+                q.blockDim = dim3(kThreads, 1, 1);
+                q.dynamicSmemBytes = kSmemBytes;
+                cudaLaunchAttribute qa[1];
+                qa[0].id = cudaLaunchAttributeClusterDimension;
+                qa[0].val.clusterDim.x = (unsigned)(2 * s);
+                qa[0].val.clusterDim.y = 1;
+                qa[0].val.clusterDim.z = 1;
+                q.attrs = qa;
+                q.numAttrs = 1;
+                int clusters = 0;
+                if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &q) != cudaSuccess) clusters = 0;
+                capacity_of[d][s] = clusters;
+            }
+            (void)cudaGetLastError();
+            if (capacity_of[d][1] <= 0) capacity_of[d][1] = sm_count() / 2;
+            return cudaSuccess;
+        }, &dev);
+        if (e != cudaSuccess) return e;
+    }
+    const Plan plan = make_plan(FULL, M, N, K, capacity_of[dev]);
+    const int pairs = capacity_of[dev][1];
+    CUtensorMap mp, mr, mx, mxt;
+    if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kRows, kUnitK,
+                     CU_TENSOR_MAP_SWIZZLE_128B))
+        return cudaErrorInvalidValue;
+    mr = mp;
+    if (FULL && !make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kRows, kUnitK,
+                             CU_TENSOR_MAP_SWIZZLE_128B))
+        return cudaErrorInvalidValue;
+    if (!make_map_2d(&mx, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K, (uint32_t)plan.tokens / 2, 64,
+                     CU_TENSOR_MAP_SWIZZLE_128B))
+        return cudaErrorInvalidValue;
+    mxt = mx;
+    if (plan.tail_parts > 1 && !make_map_2d(&mxt, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K,
+                                            (uint32_t)plan.tail_tokens / 2, 64, CU_TENSOR_MAP_SWIZZLE_128B))
+        return cudaErrorInvalidValue;
+    PairParams prm = {};
+    prm.y = static_cast<__half*>(y);
+    prm.M = (int)M;
+    prm.N = (int)N;
+    prm.K = (int)K;
+    prm.tokens = plan.tokens;
+    prm.tail_tokens = plan.tail_tokens;
+    prm.tail_parts = plan.tail_parts;
+    prm.split = plan.split;
+    prm.status = status;
+    // Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
+    // (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024), more if four plane units still fit;
+    // the planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are
+    // all seen by the same zip warps.
+    const int x_bytes = plan.tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
+    int xs = (room - 4 * unit_bytes(FULL)) / x_bytes;
+    xs = xs < 4 ? 4 : xs > kMaxXSlots ? kMaxXSlots : xs;
+    const int units = (room - xs * x_bytes) / unit_bytes(FULL);
+    prm.x_slots = xs;
+    prm.units = units > kMaxUnits ? kMaxUnits : units & ~1;
+    const int64_t tiles = ((N + 2 * kRows - 1) / (2 * kRows)) * ((M + plan.tokens - 1) / plan.tokens);
+    if (getenv("DPS_DEBUG"))
+        fprintf(stderr, "[dps] pair full=%d M=%lld N=%lld K=%lld tokens=%d tiles=%lld tail=%dx%d split=%d (%d %d %d %d) units=%d x_slots=%d\n", (int)FULL,
+                (long long)M, (long long)N, (long long)K, plan.tokens, (long long)tiles, plan.tail_parts, plan.tail_tokens,
+                plan.split, capacity_of[dev][1], capacity_of[dev][2], capacity_of[dev][3], capacity_of[dev][4], prm.units, xs);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(plan.split > 1 ? 2 * plan.split * tiles : 2 * (tiles < pairs ? tiles : pairs)), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)(2 * plan.split);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mp, mr, mx, mxt, prm);
+    count_launch();
+    return e;
+}
+
+}  // namespace
+
+cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
+                               int64_t N, int64_t K, int* status, cudaStream_t stream) {
+    const bool full = mode == DPS_MODE_FULL;
+    if (!full) enc = base_enc(enc);   // fast mode reads the persistent byte of a rounded nest like any other
+    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, M, N, K, status, stream);
+    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, M, N, K, status, stream);
+    if (enc == kEncE4M3)
+        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, M, N, K, status, stream)
+                    : launch_enc<kEncE4M3, false>(x, p, r, y, M, N, K, status, stream);
+    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, M, N, K, status, stream)
+                : launch_enc<kEncE5M2, false>(x, p, r, y, M, N, K, status, stream);
+}
+
+}  // namespace dps

@@ -10,6 +10,7 @@ namespace dps {
 namespace sm100 {
 
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
+constexpr uint32_t kTryWaitNs = 20000;   // how long one try_wait may suspend the warp
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -48,10 +49,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity)
+        : "r"(bar), "r"(parity), "r"(kTryWaitNs)
         : "memory");
     return ok != 0;
 }
@@ -81,29 +82,6 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, u
 // The wait every kernel uses: gives up after kWaitLimitNs.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return mbar_wait_limit(bar, parity, kWaitLimitNs);
-}
-
-// The same for a barrier that the other CTA of a pair arrives on: what it did before is visible afterwards.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
-    auto attempt = [&] {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        return ok != 0;
-    };
-    if (attempt()) return true;
-    const unsigned long long t0 = global_timer_ns();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 1024; ++i)
-            if (attempt()) return true;
-        if (global_timer_ns() - t0 > kWaitLimitNs) return false;
-    }
 }
 
 // ---- TMA -----------------------------------------------------------------------------------
@@ -241,10 +219,11 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 
 // The pair's version, issued by one thread of the pair's first CTA: arrives on the barrier at this offset in BOTH CTAs
 // once every MMA issued so far by this thread has completed in both.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+// `first`: the cluster rank of the pair's first CTA.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t first = 0) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-        "h"((uint16_t)3)
+        "h"((uint16_t)(3u << first))
         : "memory");
 }
 
@@ -269,7 +248,7 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
 }
 // Arrives on an mbarrier of the cluster (a shared::cluster address).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
