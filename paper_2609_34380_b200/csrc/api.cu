@@ -262,15 +262,17 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     if (st != DPS_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const uint8_t* r = (mode == DPS_MODE_FULL) ? w_resid : nullptr;  // fast mode never sees the pointer
-    // A handful of tokens makes the layer a pure weight stream: up to 8 tokens (one MMA column group)
-    // the register-streaming kernel serves it.  For 9-16 tokens the choice was measured on Llama-7B
-    // and hidden-8192 shapes, in both modes: the tensor-core kernel's set-up and cluster reduction
-    // cost a few microseconds per launch, its TMA stream is faster once running; it wins from 2^25
-    // weights on (by 0-20 %), the streaming kernel below (4096 x 4096: by 15-30 %).  Beyond 16
-    // tokens the tcgen05 tiles take over, beyond 64 tokens CTA pairs (four Llama-7B linears, fast / full mode: 64 tokens
-    // 62 / 97 us with the tiles, 75 / 109 with pairs; 96 tokens 84 / 134 against 74 / 107).  (The CUDA-core GEMV is
-    // kept as a cross-check.)
-    const bool stream_mid = N * K < ((int64_t)1 << 25);
+    // A handful of tokens makes the layer a pure weight stream: up to 8 tokens (one MMA column group) the
+    // register-streaming kernel serves it.  For 9-16 tokens that kernel is the faster one for a single small matrix (4096 x
+    // 4096: 4.9 us against 7.0), but not for a layer: it lives on a large L1, the tensor-core tiles on a large
+    // shared memory, and an SM that changes its split drains first.  Four linears in turn at 12-13 tokens, streaming kernel
+    // / tiles / the one or the other by N K < 2^25, which was the rule: hidden 3088 in full mode 57 / 46 / 98 us, 2048 in
+    // fast mode 23.0 / 22.6 / 38, 4096 in full mode (16 tokens) 86 / 83 / 91; 1024 14.7 / 17.7, 512 9.3 / 13.2.  The smaller
+    // side of the matrix is the hidden size in all four, so a rule on it keeps a layer in one family.
+    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens CTA pairs (four Llama-7B linears, fast / full mode: 64
+    // tokens 62 / 97 us with the tiles, 75 / 109 with pairs; 96 tokens 84 / 134 against 74 / 107).  (The CUDA-core GEMV
+    // is kept as a cross-check.)
+    const bool stream_mid = (N < K ? N : K) <= 1536;
     const int path = forced_path();
     cudaError_t err;
     if (path == 1) err = launch_gemv(mode, enc, x, w_persist, r, y, M, N, K, stream);
