@@ -217,26 +217,13 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
     bool ok = true;
     if (warp == 0) {
         // ---------------- TMA producer: this CTA's rows and its half of the tokens ----------------
-        const uint32_t half_tokens = (uint32_t)tokens / 2;
-        const uint32_t pair_bytes = 2u * (kRows + half_tokens) * kBlockBytes;
-        auto load_plane = [&](int s, int i, int n0) {
-            // (the second CTA's bytes may land before this: the phase still waits for the one arrival)
-            if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_full[s]), pair_bytes);
-            tma_load_2d_pair(smem_base + (uint32_t)s * kStageBytes, &map_p, map_to_cta(smem_u32(&bar_full[s]), 0u),
-                             i * kBlockBytes, n0);
-        };
-        // the plane is model state: its first stages are requested before the preceding kernel (the quantisation,
-        // whose codes and scales this kernel reads) has ended
-        const int ahead = min(num_kb, kStages);
-        int n0, m0;
-        tile_origin(pair, n0, m0);
-        if (elect_one())
-            for (int i = 0; i < ahead; ++i) load_plane(i, i, n0);
-        __syncwarp();
-        grid_dependency_wait();
+        grid_dependency_wait();   // the activation codes come from the quantisation kernel
         int s = 0;
         uint32_t ph = 0;
+        const uint32_t half_tokens = (uint32_t)tokens / 2;
+        const uint32_t pair_bytes = 2u * (kRows + half_tokens) * kBlockBytes;
         for (int lin = pair; lin < total && ok; lin += pairs) {
+            int n0, m0;
             tile_origin(lin, n0, m0);
             m0 += rank * (int)half_tokens;
             for (int i = 0; i < num_kb && ok; ++i, s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0)) {
@@ -244,9 +231,12 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 if (elect_one()) {
-                    if (lin != pair || i >= ahead) load_plane(s, i, n0);
-                    tma_load_2d_pair(smem_base + (uint32_t)(s * kStageBytes + kRows * kBlockBytes), &map_x,
-                                     map_to_cta(smem_u32(&bar_full[s]), 0u), i * kBlockBytes, m0);
+                    const uint32_t full = map_to_cta(smem_u32(&bar_full[s]), 0u);
+                    const uint32_t dst = smem_base + (uint32_t)s * kStageBytes;
+                    // (the second CTA's bytes may land before this: the phase still waits for the one arrival)
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_full[s]), pair_bytes);
+                    tma_load_2d_pair(dst, &map_p, full, i * kBlockBytes, n0);
+                    tma_load_2d_pair(dst + kRows * kBlockBytes, &map_x, full, i * kBlockBytes, m0);
                 }
                 __syncwarp();
             }
@@ -363,7 +353,7 @@ int pick_tokens(int64_t M, int64_t N, int pairs) {
     if (forced >= 16 && forced <= kMaxTokens) return forced;
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows);
     int64_t best = 16, best_cost = INT64_MAX;
-    for (int64_t t = (M + kMaxTokens - 1) / kMaxTokens, end = 2 * t + 6; t <= end; ++t) {
+    for (int64_t t = (M + kMaxTokens - 1) / kMaxTokens, end = t + (t < 10 ? t + 6 : 16); t <= end; ++t) {
         const int64_t tokens = ((M + t - 1) / t + 15) / 16 * 16;
         const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens), rounds = (tiles + pairs - 1) / pairs;
         const int64_t cost = rounds * (128 + tokens);

@@ -449,7 +449,7 @@ Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) 
     const int64_t steps = (K + kUnitK - 1) / kUnitK, pairs = capacity[1];
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), t0 = (M + 255) / 256;
     Plan best;
-    for (int64_t t = t0; t <= 2 * t0 + 4; ++t) {
+    for (int64_t t = t0, end = t0 + (t0 < 12 ? t0 + 4 : 16); t <= end; ++t) {
         int64_t tokens = ((M + t - 1) / t + 15) / 16 * 16;
         if (forced >= 16 && forced <= 256) tokens = forced;
         const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens);
