@@ -61,6 +61,12 @@ cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* 
 cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
                                int64_t N, int64_t K, int* status, cudaStream_t stream);
 
+// Grouped linear on CTA pairs: arguments as below, `masks` the e5m2_mask array; pair_grouped_tokens: its token-tile width.
+int pair_grouped_tokens(int64_t A, int32_t E);
+cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y,
+                                int64_t A, int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,
+                                const int32_t* sorted_rows, int max_tiles, int* status, cudaStream_t stream);
+
 // Grouped linear on the tensor-core path.  e5m2_mask: 64 words, bit e of the first 32 set for an E5M2
 // expert, of the last 32 for a rounded nest.  x_sorted: [A][K] activations grouped by expert;
 // tiles / num_tiles / sorted_rows: device tables built by the routing pre-pass; tn: token-tile

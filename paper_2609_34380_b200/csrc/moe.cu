@@ -62,49 +62,92 @@ __device__ __forceinline__ bool row_valid(const int32_t* token_of_row, const int
     return e >= 0 && e < E && t >= 0 && t < T;
 }
 
-// One CTA.  Warp w owns experts w, w+32, ...; for each it walks all rows in order, so the
-// grouping is stable without any atomics.  Invalid rows belong to no group and raise the
-// status word.
+// One CTA.  Invalid rows belong to no group and raise the status word.  Rows are counted per expert with integer atomics
+// (the counts do not depend on their order); the grouping itself is stable without any: rows are placed 1024 at a time, a
+// row's position among its expert's rows being that of the rows placed before, of the warps before its own (a table of
+// counts per warp and expert, scanned by one thread per expert) and of the lanes before its own.  Latency-bound, one SM:
+// 4.7 us for 32 rows of 32 experts.  More than kTableExperts experts (the table's size): one warp per expert walks all rows.
+constexpr int kTableExperts = 256;
+
 __global__ void __launch_bounds__(kRouteThreads)
 moe_route_kernel(const int32_t* __restrict__ token_of_row, const int32_t* __restrict__ expert_of_row, int A, int T,
                  int E, int tile_tokens, int32_t* counts, int32_t* offsets, int32_t* sorted_rows,
                  int32_t* num_tiles, int4* tiles, int* status) {
     __shared__ int s_cnt[kMaxExperts];
     __shared__ int s_off[kMaxExperts];
+    __shared__ int s_table[kRouteThreads / 32][kTableExperts];
     // the gather and the grouped kernel may be made resident now; both wait for their predecessor
     // (griddepcontrol.wait) before they read anything this kernel writes
     sm100::grid_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < E; e += kRouteThreads) s_cnt[e] = 0;
+    __syncthreads();
+    sm100::grid_dependency_wait();      // the routing and, through an earlier call, the workspace are earlier kernels'
     int bad = 0;
-    for (int a = tid; a < A; a += kRouteThreads) bad |= !row_valid(token_of_row, expert_of_row, a, T, E);
+    for (int a = tid; a < A; a += kRouteThreads) {
+        if (row_valid(token_of_row, expert_of_row, a, T, E)) atomicAdd(&s_cnt[expert_of_row[a]], 1);
+        else bad = 1;
+    }
     if (__syncthreads_or(bad) && tid == 0) atomicExch(status, (int)DPS_ERR_DATA);
-    for (int e = warp; e < E; e += kRouteThreads / 32) {
-        int c = 0;
-        for (int base = 0; base < A; base += 32) {
-            const int a = base + lane;
-            const bool hit = a < A && expert_of_row[a] == e && row_valid(token_of_row, expert_of_row, a, T, E);
-            c += __popc(__ballot_sync(0xFFFFFFFFu, hit));
-        }
-        if (lane == 0) s_cnt[e] = c;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int run = 0, nt = 0;
-        for (int e = 0; e < E; ++e) {
-            s_off[e] = run;
-            offsets[e] = run;
-            counts[e] = s_cnt[e];
-            for (int first = 0; first < s_cnt[e]; first += tile_tokens) {
-                const int rows = s_cnt[e] - first < tile_tokens ? s_cnt[e] - first : tile_tokens;
-                tiles[nt++] = make_int4(e, run + first, rows, 0);
+    if (warp == 0) {
+        // first position and first tile of every expert
+        int rows = 0, nt = 0;
+        for (int base = 0; base < E; base += 32) {
+            const int e = base + lane;
+            const int c = e < E ? s_cnt[e] : 0, k = (c + tile_tokens - 1) / tile_tokens;
+            int ci = c, ki = k;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int cu = __shfl_up_sync(0xFFFFFFFFu, ci, o), ku = __shfl_up_sync(0xFFFFFFFFu, ki, o);
+                if (lane >= o) {
+                    ci += cu;
+                    ki += ku;
+                }
             }
-            run += s_cnt[e];
+            if (e < E) {
+                const int off = rows + ci - c;
+                s_off[e] = off;
+                offsets[e] = off;
+                counts[e] = c;
+                int t = nt + ki - k;
+                for (int first = 0; first < c; first += tile_tokens)
+                    tiles[t++] = make_int4(e, off + first, c - first < tile_tokens ? c - first : tile_tokens, 0);
+            }
+            rows += __shfl_sync(0xFFFFFFFFu, ci, 31);
+            nt += __shfl_sync(0xFFFFFFFFu, ki, 31);
         }
-        offsets[E] = run;
-        num_tiles[0] = nt;
-        num_tiles[1] = run;  // number of valid rows
+        if (lane == 0) {
+            offsets[E] = rows;
+            num_tiles[0] = nt;
+            num_tiles[1] = rows;  // number of valid rows
+        }
     }
     __syncthreads();
+    if (E <= kTableExperts) {
+        for (int base = 0; base < A; base += kRouteThreads) {
+            for (int i = tid; i < (kRouteThreads / 32) * E; i += kRouteThreads) s_table[i / E][i % E] = 0;
+            __syncthreads();
+            const int a = base + tid;
+            const bool valid = a < A && row_valid(token_of_row, expert_of_row, a, T, E);
+            const int e = valid ? expert_of_row[a] : -1;
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, e);
+            const int before = __popc(same & ((1u << lane) - 1u));
+            if (valid && before == 0) s_table[warp][e] = __popc(same);
+            __syncthreads();
+            if (tid < E) {
+                int run = s_off[tid];
+                for (int w = 0; w < kRouteThreads / 32; ++w) {
+                    const int c = s_table[w][tid];
+                    s_table[w][tid] = run;
+                    run += c;
+                }
+                s_off[tid] = run;
+            }
+            __syncthreads();
+            if (valid) sorted_rows[s_table[warp][e] + before] = a;
+            __syncthreads();
+        }
+        return;
+    }
     for (int e = warp; e < E; e += kRouteThreads / 32) {
         int pos = s_off[e];
         for (int base = 0; base < A; base += 32) {
@@ -146,12 +189,28 @@ cudaError_t launch_moe(int mode, const int32_t* enc_host, const void* x, const i
                        int64_t T, int64_t N, int64_t K, int32_t E, void* workspace, int* status,
                        cudaStream_t stream) {
     const Workspace w = carve(workspace, A, E, K);
-    const int tn = grouped_tile_tokens(A, E);
-    moe_route_kernel<<<1, kRouteThreads, 0, stream>>>(token_of_row, expert_of_row, (int)A, (int)T, E, tn, w.counts,
-                                                      w.offsets, w.sorted_rows, w.num_tiles, w.tiles, status);
-    count_launch();
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
+    // CTA pairs from 48 rows per expert on; below, 128-row tiles of two CTAs per SM, which divide few experts' rows more
+    // evenly (measured per call, gate/up + down: Mixtral experts, 64 tokens, fast mode 284 us with the tiles against 290 with
+    // pairs, 4 tokens in full mode 219 / 229; 256 tokens 314 / 309 in fast and 532 / 512 in full mode, 1024 tokens 758 / 675,
+    // 2048 in full mode 2167 / 1969).
+    const bool pairs = A >= 48 * (int64_t)E;
+    const int tn = pairs ? pair_grouped_tokens(A, E) : grouped_tile_tokens(A, E);
+    cudaError_t err;
+    {   // programmatic dependent launch, as the two kernels behind it: each waits before its first read
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, 1, 1);
+        cfg.blockDim = dim3(kRouteThreads, 1, 1);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        err = cudaLaunchKernelEx(&cfg, moe_route_kernel, token_of_row, expert_of_row, (int)A, (int)T, (int)E, tn, w.counts,
+                                 w.offsets, w.sorted_rows, w.num_tiles, w.tiles, status);
+        count_launch();
+        if (err != cudaSuccess) return err;
+    }
     const int gather_grid = (int)(A < 4096 ? A : 4096);
     {   // programmatic dependent launch: resident while the routing kernel runs, waits before its first read
         cudaLaunchConfig_t cfg = {};
@@ -180,6 +239,9 @@ cudaError_t launch_moe(int mode, const int32_t* enc_host, const void* x, const i
     }
     // an upper bound on the number of token tiles that needs no device round trip
     const int max_tiles = (int)((A + tn - 1) / tn + E);
+    if (pairs)
+        return launch_pair_grouped(mode, mask, w.x_sorted, p, r, y, A, N, K, E, tn, w.tiles, w.num_tiles, w.sorted_rows,
+                                   max_tiles < w.max_tiles ? max_tiles : (int)w.max_tiles, status, stream);
     return launch_umma_grouped(mode, mask, w.x_sorted, p, r, y, A, N, K, E, tn, w.tiles, w.num_tiles, w.sorted_rows,
                                max_tiles < w.max_tiles ? max_tiles : (int)w.max_tiles, status, stream);
 }

@@ -31,6 +31,7 @@
 // (tcgen05.fence) and shared memory; with the release a step took twice as long.
 #include <cuda_fp16.h>
 
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 
@@ -92,15 +93,44 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 // Tensor memory: accumulators first (two tiles' worth where they fit, so that the next tile's MMAs overlap the epilogue),
 // then the A slots.
 struct Work {
-    int row_tile, m0;       // tile row index, first token
+    int row_tile, m0;       // tile row index, first token (grouped: first sorted row)
     int tokens, ncols;      // MMA columns, columns that exist
+    int plane_row0;         // grouped: first plane row of the expert in the [E * N][K] view
     bool piece;             // a piece of a tile of the last round
+    bool e5m2, rounded;     // grouped: the expert's encoding
 };
 
+// Grouped (MoE) launches: token tiles built on the device by the routing pre-pass, (expert, first sorted row, rows, unused).
+struct PairGroups {
+    const int4* tiles;
+    const int32_t* num_tiles;
+    const int32_t* sorted_rows;   // sorted position -> caller's row id
+    uint32_t e5m2[32];            // bit e set: expert e is E5M2 (truncated or rounded)
+    uint32_t rounded[32];         // bit e set: expert e is a rounded nest (full mode only; fast mode reads P alike)
+};
+
+// 64 columns of one row (half a unit): plane bytes -> packed FP16 pairs.
 template <int ENC, bool FULL>
+__device__ __forceinline__ void rebuild(uint32_t prow, int half, uint32_t sw, uint32_t (&h)[32]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t off = ((uint32_t)(4 * half + c) ^ sw) * 16u;
+        const uint4 pv = lds128(prow + off);
+        const uint4 rv = FULL ? lds128(prow + kRows * kUnitK + off) : make_uint4(0, 0, 0, 0);
+        uint32_t h8[8];
+        if (FULL) join16<ENC, FULL>(pv, rv, h8);
+        else fast16<ENC>(pv, h8);   // E4M3: 2^8 times the weights, undone in the epilogue
+#pragma unroll
+        for (int q = 0; q < 8; ++q) h[c * 8 + q] = h8[q];
+    }
+}
+
+// GROUPED: a work item is a row tile of one expert x one of its token tiles; ENC is not used, the encoding is the expert's.
+template <int ENC, bool FULL, bool GROUPED>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r,
-                 const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_xt, const PairParams prm) {
+                 const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_xt, const PairParams prm,
+                 const PairGroups gp) {
     constexpr int kUnit = unit_bytes(FULL);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_p_full[kMaxUnits], bar_p_empty[kMaxUnits];
@@ -123,7 +153,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     const uint32_t x_base = smem_base + (uint32_t)(units * kUnit);
     const uint32_t epi_base = x_base + (uint32_t)(x_slots * x_bytes);
     const int row_tiles = (prm.N + 2 * kRows - 1) / (2 * kRows);
-    const int tok_tiles = (prm.M + prm.tokens - 1) / prm.tokens;
+    if (GROUPED) grid_dependency_wait();                        // the tile list comes from the routing pre-pass
+    const int tok_tiles = GROUPED ? *gp.num_tiles : (prm.M + prm.tokens - 1) / prm.tokens;
     const int total = row_tiles * tok_tiles;
     const int t_main = prm.tail_parts > 1 ? total - total % pairs : total;
     const int all_steps = (prm.K + kUnitK - 1) / kUnitK;        // K steps of a tile ...
@@ -134,6 +165,19 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     auto work = [&](int i, Work& w) -> bool {
         int lin = pair + i * pairs, part = 0;
         w.piece = false;
+        if (GROUPED) {
+            if (lin >= total) return false;
+            const int4 g = gp.tiles[lin / row_tiles];
+            w.row_tile = lin % row_tiles;
+            w.m0 = g.y;
+            w.ncols = g.z;
+            w.tokens = (g.z + 15) & ~15;
+            w.plane_row0 = g.x * prm.N;
+            w.e5m2 = (gp.e5m2[g.x >> 5] >> (g.x & 31)) & 1u;
+            w.rounded = FULL && ((gp.rounded[g.x >> 5] >> (g.x & 31)) & 1u);
+            return true;
+        }
+        w.plane_row0 = 0;
         if (lin >= t_main) {
             if (lin - pair != t_main || prm.tail_parts <= 1) return false;
             lin = t_main + pair / prm.tail_parts;
@@ -197,7 +241,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         int s = 0;
         uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
         for (int i = 0; ok && work(i, w); ++i) {
-            const int row = (2 * w.row_tile + rank) * kRows;
+            const int row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
             for (int u = 0; u < steps_k && ok; ++u, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
                 ok = mbar_wait(smem_u32(&bar_p_empty[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
@@ -219,14 +263,17 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         for (int i = 0; ok && work(i, w); ++i) {
             const int half = w.tokens / 2;
             const int m0 = w.m0 + rank * half;
-            const CUtensorMap* map = w.piece ? &map_xt : &map_x;
+            // (grouped: boxes of a quarter of the tile's tokens when they do)
+            const bool small = GROUPED ? 4 * half <= prm.tokens && prm.tokens >= 32 : w.piece;
+            const CUtensorMap* map = small ? &map_xt : &map_x;
+            const int box = GROUPED ? (small ? prm.tokens / 4 : prm.tokens / 2) : half;
             for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == x_slots) ? 0 : s + 1) {
                 if (t >= (uint32_t)x_slots) ok = wait_done(t - (uint32_t)x_slots);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 if (elect_one()) {
                     const uint32_t full = smem_u32(&bar_x_full[s]), dst = x_base + (uint32_t)(s * x_bytes);
-                    mbar_arrive_expect_tx(full, (uint32_t)(2 * half * 128));
+                    mbar_arrive_expect_tx(full, (uint32_t)(2 * box * 128));
                     tma_load_2d(dst, map, full, (step0 + j) * kUnitK, m0);
                     tma_load_2d(dst + (uint32_t)x_atom, map, full, (step0 + j) * kUnitK + 64, m0);
                 }
@@ -300,16 +347,14 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                                 if (!ok) break;
                 const uint32_t prow = smem_base + s * kUnit + (uint32_t)(row * kUnitK);
                 uint32_t h[32];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint32_t off = ((uint32_t)(4 * half + c) ^ sw) * 16u;
-                    const uint4 pv = lds128(prow + off);
-                    const uint4 rv = FULL ? lds128(prow + kRows * kUnitK + off) : make_uint4(0, 0, 0, 0);
-                    uint32_t h8[8];
-                    if (FULL) join16<ENC, FULL>(pv, rv, h8);
-                    else fast16<ENC>(pv, h8);   // E4M3: 2^8 times the weights, undone in the epilogue
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) h[c * 8 + q] = h8[q];
+                if constexpr (!GROUPED) {
+                    rebuild<ENC, FULL>(prow, half, sw, h);
+                } else if (FULL && w.rounded) {
+                    if (w.e5m2) rebuild<kEncE5M2R, FULL>(prow, half, sw, h);
+                    else rebuild<kEncE4M3R, FULL>(prow, half, sw, h);
+                } else {
+                    if (w.e5m2) rebuild<kEncE5M2, FULL>(prow, half, sw, h);
+                    else rebuild<kEncE4M3, FULL>(prow, half, sw, h);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_p_empty[s]));
@@ -330,8 +375,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         const int q = warp & 3;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const uint32_t buf = epi_base + (uint32_t)(q * kEpiCols * 64);
-        const float out_scale = (!FULL && base_enc(ENC) == kEncE4M3) ? 0.00390625f : 1.0f;
         for (int i = 0; work(i, w); ++i) {
+            const float out_scale = (!FULL && (GROUPED ? !w.e5m2 : base_enc(ENC) == kEncE4M3)) ? 0.00390625f : 1.0f;
+            // grouped: the callers' row ids of the chunk's tokens, one per lane, a chunk ahead of their use
+            int32_t ids = GROUPED && lane < w.ncols ? gp.sorted_rows[w.m0 + lane] : 0;
             const int acc = accs == 2 ? i & 1 : 0, use = accs == 2 ? i >> 1 : i;
             ok = mbar_wait(smem_u32(&bar_d_full[acc]), (uint32_t)use & 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
@@ -355,10 +402,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 break;
             }
             const int n = (2 * w.row_tile + rank) * kRows + q * 32 + (lane & 3) * 8;
-            __half* yrow = prm.y + (int64_t)(w.m0 + (lane >> 2)) * prm.N + n;
+            __half* yrow = prm.y + (GROUPED ? (int64_t)n : (int64_t)(w.m0 + (lane >> 2)) * prm.N + n);
             for (int c0 = 0; c0 < w.ncols; c0 += kEpiCols) {
                 uint32_t v[32];
                 tmem_ld_32x32b_x32(tmem_d + (uint32_t)c0, v);
+                int32_t next_ids = 0;
+                if (GROUPED && c0 + kEpiCols + lane < w.ncols) next_ids = gp.sorted_rows[w.m0 + c0 + kEpiCols + lane];
                 tmem_wait_ld();
                 if (c0 + kEpiCols >= w.ncols) {          // last chunk read: the accumulator is free again
                     tc_fence_before_sync();
@@ -376,9 +425,11 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {            // 8 tokens x 64 bytes per instruction; N is a multiple of 8
                     const uint4 val = lds128(buf + (uint32_t)(t * 512 + lane * 16));
+                    const int64_t m = GROUPED ? __shfl_sync(0xFFFFFFFFu, ids, 8 * t + (lane >> 2)) : c0 + 8 * t;
                     if (n < prm.N && c0 + 8 * t + (lane >> 2) < w.ncols)
-                        *reinterpret_cast<uint4*>(yrow + (int64_t)(c0 + 8 * t) * prm.N) = val;
+                        *reinterpret_cast<uint4*>(yrow + m * prm.N) = val;
                 }
+                ids = next_ids;
                 __syncwarp();                            // the buffer is free for the next chunk
             }
         }
@@ -483,10 +534,23 @@ Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) 
     return best;
 }
 
+// Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
+// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024), more if four plane units still fit; the
+// planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen
+// by the same zip warps.
+void size_rings(bool full, int tokens, PairParams& prm) {
+    const int x_bytes = tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
+    int xs = (room - 4 * unit_bytes(full)) / x_bytes;
+    xs = xs < 4 ? 4 : xs > kMaxXSlots ? kMaxXSlots : xs;
+    const int units = (room - xs * x_bytes) / unit_bytes(full);
+    prm.x_slots = xs;
+    prm.units = units > kMaxUnits ? kMaxUnits : units & ~1;
+}
+
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K, int* status,
                        cudaStream_t stream) {
-    auto kernel = umma_pair_kernel<ENC, FULL>;
+    auto kernel = umma_pair_kernel<ENC, FULL, false>;
     // Clusters of s pairs that are resident at once, per device (they must fit inside a GPC): filled by the first call on a
     // device, read only after that set-up has returned.
     static int capacity_of[kMaxDevices][kMaxSplit + 1] = {};
@@ -547,21 +611,12 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     prm.tail_parts = plan.tail_parts;
     prm.split = plan.split;
     prm.status = status;
-    // Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
-    // (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024), more if four plane units still fit;
-    // the planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are
-    // all seen by the same zip warps.
-    const int x_bytes = plan.tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
-    int xs = (room - 4 * unit_bytes(FULL)) / x_bytes;
-    xs = xs < 4 ? 4 : xs > kMaxXSlots ? kMaxXSlots : xs;
-    const int units = (room - xs * x_bytes) / unit_bytes(FULL);
-    prm.x_slots = xs;
-    prm.units = units > kMaxUnits ? kMaxUnits : units & ~1;
+    size_rings(FULL, plan.tokens, prm);
     const int64_t tiles = ((N + 2 * kRows - 1) / (2 * kRows)) * ((M + plan.tokens - 1) / plan.tokens);
     if (getenv("DPS_DEBUG"))
         fprintf(stderr, "[dps] pair full=%d M=%lld N=%lld K=%lld tokens=%d tiles=%lld tail=%dx%d split=%d (%d %d %d %d) units=%d x_slots=%d\n", (int)FULL,
                 (long long)M, (long long)N, (long long)K, plan.tokens, (long long)tiles, plan.tail_parts, plan.tail_tokens,
-                plan.split, capacity_of[dev][1], capacity_of[dev][2], capacity_of[dev][3], capacity_of[dev][4], prm.units, xs);
+                plan.split, capacity_of[dev][1], capacity_of[dev][2], capacity_of[dev][3], capacity_of[dev][4], prm.units, prm.x_slots);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(plan.split > 1 ? 2 * plan.split * tiles : 2 * (tiles < pairs ? tiles : pairs)), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -576,12 +631,98 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mp, mr, mx, mxt, prm);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mp, mr, mx, mxt, prm, PairGroups{});
+    count_launch();
+    return e;
+}
+
+template <bool FULL>
+cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y, int64_t A,
+                           int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,
+                           const int32_t* sorted_rows, int max_tiles, int* status, cudaStream_t stream) {
+    auto kernel = umma_pair_kernel<0, FULL, true>;
+    static PerDeviceOnce setup;     // per instantiation and per device
+    {
+        const cudaError_t e = setup.run(
+            [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); });
+        if (e != cudaSuccess) return e;
+    }
+    CUtensorMap mp, mr, mx, mxt;
+    if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)E * (uint64_t)N, (uint64_t)K, kRows, kUnitK,
+                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
+        return cudaErrorInvalidValue;
+    mr = mp;
+    if (FULL && !make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)E * (uint64_t)N, (uint64_t)K, kRows, kUnitK,
+                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
+        return cudaErrorInvalidValue;
+    if (!make_map_2d(&mx, x_sorted, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)A, (uint64_t)K, (uint32_t)tn / 2, 64,
+                     CU_TENSOR_MAP_SWIZZLE_128B))
+        return cudaErrorInvalidValue;
+    mxt = mx;
+    if (tn >= 32 && !make_map_2d(&mxt, x_sorted, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)A, (uint64_t)K, (uint32_t)tn / 4, 64,
+                                 CU_TENSOR_MAP_SWIZZLE_128B))
+        return cudaErrorInvalidValue;
+    PairParams prm = {};
+    prm.y = static_cast<__half*>(y);
+    prm.M = (int)A;
+    prm.N = (int)N;
+    prm.K = (int)K;
+    prm.tokens = prm.tail_tokens = tn;
+    prm.tail_parts = 1;
+    prm.split = 1;
+    prm.status = status;
+    size_rings(FULL, tn, prm);
+    PairGroups gp;
+    gp.tiles = static_cast<const int4*>(tiles);
+    gp.num_tiles = num_tiles;
+    gp.sorted_rows = sorted_rows;
+    for (int i = 0; i < 32; ++i) {   // the caller's array holds the E5M2 bits, then the rounded-nest bits
+        gp.e5m2[i] = masks[i];
+        gp.rounded[i] = FULL ? masks[32 + i] : 0u;
+    }
+    const int64_t upper = ((N + 2 * kRows - 1) / (2 * kRows)) * max_tiles, pairs = sm_count() / 2;
+    if (getenv("DPS_DEBUG"))
+        fprintf(stderr, "[dps] pair grouped full=%d A=%lld N=%lld K=%lld E=%d tokens=%d tiles<=%lld units=%d x_slots=%d\n", (int)FULL,
+                (long long)A, (long long)N, (long long)K, (int)E, tn, (long long)upper, prm.units, prm.x_slots);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * (upper < pairs ? upper : pairs)), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mp, mr, mx, mxt, prm, gp);
     count_launch();
     return e;
 }
 
 }  // namespace
+
+// Token-tile width of grouped launches: an expert with a quarter, or two and a half standard deviations of an even routing,
+// more rows than the average still fits the average's number of tiles.
+int pair_grouped_tokens(int64_t A, int32_t E) {
+    const double avg = (double)A / E, spread = 2.5 * sqrt(avg);
+    const double want = avg + (spread > 0.25 * avg ? spread : 0.25 * avg);
+    const int tiles = (int)ceil(want / 256.0);
+    const int tokens = (int)(ceil(want / tiles / 16.0)) * 16;
+    return tokens < 16 ? 16 : tokens > 256 ? 256 : tokens;
+}
+
+cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y,
+                                int64_t A, int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,
+                                const int32_t* sorted_rows, int max_tiles, int* status, cudaStream_t stream) {
+    return mode == DPS_MODE_FULL ? launch_grouped<true>(masks, x_sorted, p, r, y, A, N, K, E, tn, tiles, num_tiles, sorted_rows,
+                                                        max_tiles, status, stream)
+                                 : launch_grouped<false>(masks, x_sorted, p, r, y, A, N, K, E, tn, tiles, num_tiles, sorted_rows,
+                                                         max_tiles, status, stream);
+}
 
 cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
                                int64_t N, int64_t K, int* status, cudaStream_t stream) {
