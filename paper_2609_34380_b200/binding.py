@@ -7,6 +7,7 @@ no CPU or PyTorch fallback.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 from pathlib import Path
 from typing import Optional, Sequence, Tuple
 
@@ -45,6 +46,8 @@ ABI = {
 }
 
 _lib = None
+FASTCALL_PATH = Path(__file__).resolve().parent / "_fastcall.so"
+_fast_linear = None     # native marshalling of dps_linear (csrc/fastcall.cpp); set when the library is loaded, if it was built
 
 
 class DpsError(RuntimeError):
@@ -67,7 +70,23 @@ def library() -> ctypes.CDLL:
             fn.restype = res
             fn.argtypes = args
         _lib = lib
+        _load_fastcall(lib)
     return _lib
+
+
+def _load_fastcall(lib: ctypes.CDLL) -> None:
+    """The same call with less host work; without the module every call takes the ctypes path below."""
+    global _fast_linear
+    if not FASTCALL_PATH.exists():
+        return
+    try:
+        spec = importlib.util.spec_from_file_location("_fastcall", FASTCALL_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+    except ImportError:         # built against another PyTorch
+        return
+    module.set_linear(ctypes.cast(lib.dps_linear, ctypes.c_void_p).value)
+    _fast_linear = module.linear
 
 
 def status_string(status: int) -> str:
@@ -79,8 +98,15 @@ def _check(status: int, what: str) -> None:
         raise DpsError(status, what)
 
 
+# The current stream's handle without building a torch.cuda.Stream object around it for every call.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -88,13 +114,13 @@ def _stream(stream) -> int:
 def _dev(t: Optional[torch.Tensor], dtype, what: str) -> Optional[int]:
     if t is None:
         return None
+    if t.is_cuda and t.dtype is dtype and t.is_contiguous():
+        return t.data_ptr()
     if not t.is_cuda:
         raise ValueError(f"{what} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{what} must be {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
-        raise ValueError(f"{what} must be contiguous")
-    return t.data_ptr()
+    raise ValueError(f"{what} must be contiguous")
 
 
 def dps_split_weights(w_fp16: torch.Tensor, enc: int = DPS_ENC_AUTO, w_persist: Optional[torch.Tensor] = None,
@@ -129,6 +155,10 @@ def dps_reconstruct(w_persist: torch.Tensor, w_resid: Optional[torch.Tensor], en
 def dps_linear(mode: int, enc: int, x: torch.Tensor, w_persist: torch.Tensor, w_resid: Optional[torch.Tensor],
                y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """y[M][N] = x[M][K] * W_eff^T from the planes, in fast or full mode."""
+    if stream is None and _fast_linear is not None:
+        out = _fast_linear(mode, enc, x, w_persist, w_resid, y)
+        if out is not None:     # None: not a plain case, or refused; the path below runs it or says why
+            return out
     M, K = x.shape
     N, K2 = w_persist.shape
     if K != K2:

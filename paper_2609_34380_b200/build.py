@@ -8,12 +8,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libdps.so"
+FASTCALL = PKG / "_fastcall.so"
 INCLUDE = PKG.parent / "include"
 
 NVCC_FLAGS = [
@@ -73,5 +75,31 @@ def build_library(force: bool = False, verbose: bool = False) -> Path:
     return LIB
 
 
+def build_fastcall(force: bool = False) -> Path:
+    """Compile csrc/fastcall.cpp, the CPython entry of dps_linear, against the installed PyTorch."""
+    import torch
+    from torch.utils.cpp_extension import include_paths, library_paths
+
+    src = CSRC / "fastcall.cpp"
+    if not force and FASTCALL.exists() and FASTCALL.stat().st_mtime >= src.stat().st_mtime:
+        return FASTCALL
+    tmp = FASTCALL.with_suffix(f".tmp{os.getpid()}.so")
+    cuda = Path(_nvcc()).resolve().parent.parent / "include"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for inc in [*include_paths(), sysconfig.get_paths()["include"], str(cuda)]:
+        cmd += ["-isystem", inc]
+    cmd += [str(src), "-o", str(tmp)]
+    for lib in library_paths():
+        cmd += ["-L", lib, f"-Wl,-rpath,{lib}"]
+    cmd += ["-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"g++ failed for {src.name}:\n{res.stdout}\n{res.stderr}")
+    os.replace(tmp, FASTCALL)
+    return FASTCALL
+
+
 if __name__ == "__main__":
+    print(build_fastcall(force="--force" in sys.argv))
     print(build_library(force="--force" in sys.argv, verbose="-v" in sys.argv))
