@@ -79,13 +79,11 @@ __device__ __forceinline__ void to_half_pairs(const uint4& p, const uint4& r, ui
     else join16<ENC, FULL>(p, r, h);
 }
 
+// SHORT: K is U rounds and perhaps a ragged end, less than a batch of the long variant; all of it is one batch.
 // HALF: the CTA owns 8 weight rows instead of 16 (the upper half of every MMA tile is zero).  It
 // doubles the number of CTAs for matrices with few rows; the MMA work wasted is irrelevant here.
-// Three CTAs per SM for the variant that fits them (full mode, 8 tokens, two rounds in flight:
-// 80 registers); one register more and the allocation granularity drops it to two CTAs, which
-// was measured 10 % slower on the wide Llama-7B layers.
-template <int ENC, bool FULL, int NT, int U, bool HALF>
-__global__ void __launch_bounds__(kThreads, (FULL && NT == 1 && U == 2) ? 3 : 2)
+template <int ENC, bool FULL, int NT, int U, bool SHORT, bool HALF>
+__global__ void __launch_bounds__(kThreads, 2)
 decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp,
                   __half* __restrict__ y, int M, int64_t N, int64_t K, int prefetch_steps,
                   int prefetch_ctas, int trace_slot) {
@@ -173,7 +171,7 @@ decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, c
         };
 
         int r0 = 0;
-        for (; r0 + U <= full_rounds; r0 += U) {          // U rounds in flight, immediate offsets
+        for (; SHORT ? r0 == 0 : r0 + U <= full_rounds; r0 += U) {   // U rounds in flight, immediate offsets
             const int base = r0 * kRoundK;
             uint4 wp_lo[U], wp_hi[U], wr_lo[U], wr_hi[U];
 #pragma unroll
@@ -184,6 +182,17 @@ decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, c
                 if (FULL) {
                     wr_lo[u] = ldg_stream(r_lo + base + u * kRoundK);
                     if (!HALF) wr_hi[u] = ldg_stream(r_hi + base + u * kRoundK);
+                }
+            }
+            const int kt = U * kRoundK;                   // SHORT: the ragged end of K
+            const bool tail = SHORT && has_tail && kt + kl < K;
+            uint4 tp_lo = make_uint4(0, 0, 0, 0), tp_hi = tp_lo, tr_lo = tp_lo, tr_hi = tp_lo;
+            if (tail) {
+                tp_lo = ldg_stream(p_lo + kt);
+                if (!HALF) tp_hi = ldg_stream(p_hi + kt);
+                if (FULL) {
+                    tr_lo = ldg_stream(r_lo + kt);
+                    if (!HALF) tr_hi = ldg_stream(r_hi + kt);
                 }
             }
             // Everything but the planes may come from the preceding kernel: wait for it here, with the
@@ -200,14 +209,20 @@ decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, c
             for (int u = 0; u < U; ++u) load_x(xb[u], base + u * kRoundK, true);
 #pragma unroll
             for (int u = 0; u < U; ++u) multiply(wp_lo[u], wp_hi[u], wr_lo[u], wr_hi[u], xb[u]);
+            // warp-uniform skip (the MMA needs the whole warp); lanes past K multiply zeros
+            if (SHORT && has_tail && kt + warp * 64 < K) {
+                uint4 xt[NT][2];
+                load_x(xt, kt, tail);
+                multiply(tp_lo, tp_hi, tr_lo, tr_hi, xt);
+            }
         }
         const int total_rounds = full_rounds + (has_tail ? 1 : 0);
         // Leftover rounds and the ragged end of K: predicated batches (of at most 128 bytes per lane, which
         // keeps the predicated copy of the loop body free of register spills), never one round at
         // a time -- a lone round costs a full DRAM latency.
         constexpr int UT = FULL ? 2 : (U > 4 ? 4 : U);
-        if (r0 == 0) sm100::grid_dependency_wait();   // K shorter than one full batch: nothing was loaded ahead
-        for (; r0 < total_rounds; r0 += UT) {
+        if (!SHORT && r0 == 0) sm100::grid_dependency_wait();   // K shorter than one round: nothing was loaded ahead
+        for (; !SHORT && r0 < total_rounds; r0 += UT) {
             uint4 wp_lo[UT], wp_hi[UT], wr_lo[UT], wr_hi[UT];
             uint4 xb[UT][NT][2];
 #pragma unroll
@@ -262,7 +277,7 @@ decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, c
     }
 }
 
-template <int ENC, bool FULL, int NT, int U, bool HALF>
+template <int ENC, bool FULL, int NT, int U, bool SHORT, bool HALF>
 cudaError_t launch_one(const __half* x, const uint8_t* p, const uint8_t* r, __half* y, int M, int64_t N, int64_t K,
                        cudaStream_t stream) {
     constexpr int kRows = HALF ? 8 : kRowsPerBlock;
@@ -299,35 +314,48 @@ cudaError_t launch_one(const __half* x, const uint8_t* p, const uint8_t* r, __ha
     static int trace_launches = 0;
     trace_slot = trace_launches++;
 #endif
-    cudaError_t e = cudaLaunchKernelEx(&cfg, decode_mma_kernel<ENC, FULL, NT, U, HALF>, x, p, r, y, M, N, K,
+    cudaError_t e = cudaLaunchKernelEx(&cfg, decode_mma_kernel<ENC, FULL, NT, U, SHORT, HALF>, x, p, r, y, M, N, K,
                                        prefetch_steps, prefetch_ctas, trace_slot);
     count_launch();
     return e;
 }
 
-template <int ENC, bool FULL>
-cudaError_t launch_enc(const __half* x, const uint8_t* p, const uint8_t* r, __half* y, int M, int64_t N, int64_t K,
-                       cudaStream_t stream) {
+template <int ENC, bool FULL, int NT, int U>
+cudaError_t launch_short(int rounds, const __half* x, const uint8_t* p, const uint8_t* r, __half* y, int M, int64_t N,
+                         int64_t K, cudaStream_t stream) {
+    if constexpr (U > 1)
+        if (rounds < U) return launch_short<ENC, FULL, NT, U - 1>(rounds, x, p, r, y, M, N, K, stream);
+    return launch_one<ENC, FULL, NT, U, true, false>(x, p, r, y, M, N, K, stream);
+}
+
+template <int ENC, bool FULL, int NT>
+cudaError_t launch_tokens(const __half* x, const uint8_t* p, const uint8_t* r, __half* y, int M, int64_t N, int64_t K,
+                          cudaStream_t stream) {
     // Rounds in flight per lane: 256 bytes (fast mode: 8 rounds of one plane; full mode: 4 rounds of
     // two), two CTAs per SM.  Half as much with three CTAs per SM in full mode was the default until the
     // first batch of weight loads moved in front of the dependency wait; since then the deeper
     // batches measure 2-26 % faster on every Llama-7B and hidden-8192 shape but one (QKV, full mode,
-    // 8 tokens: -3 %).  DPS_STREAM_U2=0 selects the shallower batches (tuning knob).
+    // 8 tokens: -3 %).
+    // A matrix whose K is less than that is one batch of its own length, the ragged end included: in predicated batches of
+    // half as many rounds, which serve the leftover of longer ones, nothing was loaded ahead of the dependency and each
+    // batch cost a DRAM latency.  Four linears in turn, us before / after: hidden 1024, 8 tokens, fast mode 12.2 / 11.3, full mode
+    // (4 tokens) 15.3 / 13.7; 2048, 2 tokens, fast mode 19.0 / 17.6; 3088, 1 token, fast mode 30.8 / 29.1.  (The same with several
+    // even batches instead of full ones and a leftover lost up to 15 % on longer K.)
     // Half-height blocks were measured slower for every Llama-7B shape (the kernel is bound by
     // instruction issue, and they double the MMA and activation-load instructions per weight), so
     // they stay off.
-    static const int u_forced = [] {
-        const char* e = getenv("DPS_STREAM_U2");
-        return e ? atoi(e) : -1;
-    }();
-    constexpr int U = FULL ? 2 : 4;
-    const bool wide_batches = u_forced >= 0 ? u_forced != 0 : true;
-    if (wide_batches) {
-        if (M <= 8) return launch_one<ENC, FULL, 1, 2 * U, false>(x, p, r, y, M, N, K, stream);
-        if (M <= 16) return launch_one<ENC, FULL, 2, 2 * U, false>(x, p, r, y, M, N, K, stream);
-    }
-    if (M <= 8) return launch_one<ENC, FULL, 1, U, false>(x, p, r, y, M, N, K, stream);
-    return launch_one<ENC, FULL, 2, U, false>(x, p, r, y, M, N, K, stream);   // (callers never pass more than 16 tokens)
+    constexpr int kMost = FULL ? 4 : 8;
+    const int64_t full_rounds = K / kRoundK;
+    if (full_rounds > 0 && full_rounds < kMost)
+        return launch_short<ENC, FULL, NT, kMost - 1>((int)full_rounds, x, p, r, y, M, N, K, stream);
+    return launch_one<ENC, FULL, NT, kMost, false, false>(x, p, r, y, M, N, K, stream);
+}
+
+template <int ENC, bool FULL>
+cudaError_t launch_enc(const __half* x, const uint8_t* p, const uint8_t* r, __half* y, int M, int64_t N, int64_t K,
+                       cudaStream_t stream) {
+    return M <= 8 ? launch_tokens<ENC, FULL, 1>(x, p, r, y, M, N, K, stream)
+                  : launch_tokens<ENC, FULL, 2>(x, p, r, y, M, N, K, stream);   // (callers never pass more than 16 tokens)
 }
 
 }  // namespace
