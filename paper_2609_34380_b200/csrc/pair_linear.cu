@@ -14,8 +14,9 @@
 //   warp 0       plane producer: units of 128 rows x 128 columns of P (and R) into a ring; a unit is handed back as soon as
 //                the zip warps have it in registers, so the ring holds nothing that waits for the tensor core
 //   warp 2       activation producer: this CTA's half of the tile's tokens into slots, a K step at a time (64 columns at a
-//                time the loop took 880 cycles per step)
-//   warp 3       waits for a step's activations and reports them to the first CTA
+//                time the loop took 880 cycles per step); the bytes of both CTAs are counted on the first CTA's barrier,
+//                where the MMAs that read both halves are issued
+//   warp 3       (first CTA) waits for both halves of a step's activations and reports them to the MMA warp
 //   warps 8-23   zip warps: plane bytes -> FP16 in registers -> tensor memory.  Eight take a step (a quarter of the rows and a
 //                half of the columns each), eight the next one.  A step is a chain of latencies in a warp (1400 cycles for
 //                64 columns: waits of 150 each even when nothing has to be waited for, loads and conversion 600), not
@@ -27,8 +28,9 @@
 // Against single CTAs, the four Llama-7B linears together, fast / full mode: 256 tokens 140 / 183 -> 114 / 150 us, 512
 // 209 / 269 -> 174 / 237, 2048 715 / 889 -> 644 / 739, 8192 2696 / 3500 -> 2598 / 3007 (there the power cap holds the clock
 // near 1.4 GHz).
-// The arrivals on the other CTA's barriers carry no cluster-scope release: what they order is tensor memory
-// (tcgen05.fence) and shared memory; with the release a step took twice as long.
+// The arrivals on the other CTA's barriers carry no cluster-scope release (with it a step took twice as long): what they
+// order is tensor memory only, by the tcgen05 fences on both sides.  Nothing that a CTA or its copy engine wrote to shared
+// memory is handed over by them: the activations of the second CTA complete on the first one's barrier.
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -134,7 +136,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     constexpr int kUnit = unit_bytes(FULL);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_p_full[kMaxUnits], bar_p_empty[kMaxUnits];
-    __shared__ __align__(8) uint64_t bar_x_full[kMaxXSlots];
+    __shared__ __align__(8) uint64_t bar_x_full[kMaxXSlots];    // the first CTA's count the bytes of both
     __shared__ __align__(8) uint64_t bar_a_full[kASteps];       // the first CTA's: A and activations of both are ready
     __shared__ __align__(8) uint64_t bar_done[kDone];           // the MMAs of a K step are complete
     __shared__ __align__(8) uint64_t bar_d_full[2];
@@ -209,7 +211,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             mbar_init(smem_u32(&bar_p_empty[s]), 8);            // the zip warps that take the step
         }
         for (int s = 0; s < x_slots; ++s) mbar_init(smem_u32(&bar_x_full[s]), 1);
-        for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 9);   // both CTAs' eight zip warps and warp 3
+        for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 8 + 1);   // both CTAs' eight zip warps, warp 3
         for (int a = 0; a < kDone; ++a) mbar_init(smem_u32(&bar_done[a]), 1);
         for (int a = 0; a < 2; ++a) {
             mbar_init(smem_u32(&bar_d_full[a]), 1);
@@ -272,24 +274,25 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 if (elect_one()) {
-                    const uint32_t full = smem_u32(&bar_x_full[s]), dst = x_base + (uint32_t)(s * x_bytes);
-                    mbar_arrive_expect_tx(full, (uint32_t)(2 * box * 128));
-                    tma_load_2d(dst, map, full, (step0 + j) * kUnitK, m0);
-                    tma_load_2d(dst + (uint32_t)x_atom, map, full, (step0 + j) * kUnitK + 64, m0);
+                    const uint32_t full = map_to_cta(smem_u32(&bar_x_full[s]), first), dst = x_base + (uint32_t)(s * x_bytes);
+                    // (the second CTA's bytes may land before this: the phase still waits for the one arrival)
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_x_full[s]), (uint32_t)(2 * 2 * box * 128));
+                    tma_load_2d_pair(dst, map, full, (step0 + j) * kUnitK, m0);
+                    tma_load_2d_pair(dst + (uint32_t)x_atom, map, full, (step0 + j) * kUnitK + 64, m0);
                 }
                 __syncwarp();
             }
         }
     } else if (warp == 3) {
-        // ---------------- reports the activations of a K step to the first CTA ----------------
+        // ---------------- reports the activations of a K step, both halves: the pair's first CTA ----------------
         int s = 0;
         uint32_t ph = 0, t = 0;
-        for (int i = 0; ok && work(i, w); ++i) {
+        for (int i = 0; rank == 0 && ok && work(i, w); ++i) {
             for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == x_slots) ? 0 : s + 1, ph ^= (s == 0)) {
                 if (t >= kASteps) ok = wait_done(t - kASteps);    // else the arrival might count for that step
                 if (ok) ok = mbar_wait(smem_u32(&bar_x_full[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                if (ok && lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_a_full[t % kASteps]), first));
+                if (ok && lane == 0) mbar_arrive(smem_u32(&bar_a_full[t % kASteps]));
             }
         }
     } else if (warp == 1) {
