@@ -9,7 +9,7 @@
 // and 512 tensor cycles; a CTA of a pair with a (2 x 128) x 256 tile needs 32 KB, because it fetches half of the tokens
 // and the tensor cores of both SMs read both halves.
 //
-// Tile: 256 weight rows x `tokens` tokens (a multiple of 16, chosen per launch), K walked in steps of 128.  Persistent: a pair
+// Tile: 256 weight rows x `tokens` tokens (a multiple of kTokenStep, chosen per launch), K walked in steps of 128.  Persistent: a pair
 // per two SMs walks the tiles.  Roles of a CTA (24 warps):
 //   warp 0       plane producer: units of 128 rows x 128 columns of P (and R) into a ring; a unit is handed back as soon as
 //                the zip warps have it in registers, so the ring holds nothing that waits for the tensor core
@@ -33,12 +33,12 @@
 // memory is handed over by them: the activations of the second CTA complete on the first one's barrier.
 #include <cuda_fp16.h>
 
-#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 
 #include "bits.cuh"
 #include "dps_internal.h"
+#include "pair_plan.h"
 #include "sm100.cuh"
 #include "tensor_map.h"
 
@@ -48,20 +48,11 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kRows = 128;                 // weight rows of a row block in one CTA
-constexpr int kUnitK = 128;                // columns of K in a plane unit
-constexpr int kMaxUnits = 12, kMaxXSlots = 8;
-constexpr int kASteps = 4;                 // K steps the A ring holds
-constexpr int kACols = kUnitK / 2;         // tensor memory of one of them
-constexpr int kAccCols = 512 - kASteps * kACols;
+using namespace pair_plan;
+
+constexpr int kACols = kUnitK / 2;         // tensor memory of one K step of A
 constexpr int kDone = 8;                   // ring of barriers that report completed K steps
 constexpr int kThreads = 768;
-constexpr int kMaxSplit = 4;               // pairs of a cluster (eight CTAs, the portable limit)
-constexpr int kEpiCols = 32;               // token columns per epilogue chunk
-constexpr int kEpiBytes = 4 * kEpiCols * 64;
-constexpr int kSmemBytes = 222 * 1024;     // ring + slots + epilogue chunks + alignment
-
-__host__ __device__ constexpr int unit_bytes(bool full) { return kRows * kUnitK * (full ? 2 : 1); }
 
 struct PairParams {
     __half* y;
@@ -173,7 +164,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             w.row_tile = lin % row_tiles;
             w.m0 = g.y;
             w.ncols = g.z;
-            w.tokens = (g.z + 15) & ~15;
+            w.tokens = (g.z + kTokenStep - 1) / kTokenStep * kTokenStep;
             w.plane_row0 = g.x * prm.N;
             w.e5m2 = (gp.e5m2[g.x >> 5] >> (g.x & 31)) & 1u;
             w.rounded = FULL && ((gp.rounded[g.x >> 5] >> (g.x & 31)) & 1u);
@@ -266,7 +257,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             const int half = w.tokens / 2;
             const int m0 = w.m0 + rank * half;
             // (grouped: boxes of a quarter of the tile's tokens when they do)
-            const bool small = GROUPED ? 4 * half <= prm.tokens && prm.tokens >= 32 : w.piece;
+            const bool small = GROUPED ? 4 * half <= prm.tokens : w.piece;
             const CUtensorMap* map = small ? &map_xt : &map_x;
             const int box = GROUPED ? (small ? prm.tokens / 4 : prm.tokens / 2) : half;
             for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == x_slots) ? 0 : s + 1) {
@@ -478,78 +469,6 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 
 // ---- host side ---------------------------------------------------------------------------------
 
-struct Plan {
-    int tokens = 256, tail_parts = 1, tail_tokens = 256, split = 1;
-    double cost = 0;
-};
-
-// Time of one K step of a tile in ns, all pairs at work: measured with 74 and 148 tiles of one width (18944 and 37888 rows,
-// 8192 columns; in full mode, up to 128 tokens, on planes that come out of L2) every 32 tokens, between them in proportion.
-double step_ns(bool full, int tokens) {
-    static const double fast_ns[9] = {370, 370, 415, 480, 535, 610, 685, 750, 850};
-    static const double full_ns[9] = {500, 500, 520, 600, 680, 800, 1000, 1040, 1100};
-    const double* t = full ? full_ns : fast_ns;
-    const int i = tokens >= 256 ? 7 : tokens / 32;
-    return t[i] + (t[i + 1] - t[i]) * (tokens - 32 * i) / 32.0;
-}
-
-// A round of tiles over the pairs takes as long as one tile, so the number of token tiles is chosen to make the sum over the
-// rounds small; the tiles of a last, partial round are cut into pieces of the tokens if that shortens it.  Few tiles: up to
-// four pairs share each, a range of K each; capacity[s] = clusters of s pairs that are resident at once.
-// DPS_PAIR_TOKENS=16..256 and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
-Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) {
-    static const int forced = [] { const char* e = getenv("DPS_PAIR_TOKENS"); return e ? atoi(e) / 16 * 16 : 0; }();
-    static const int forced_split = [] { const char* e = getenv("DPS_PAIR_SPLIT"); return e ? atoi(e) : 0; }();
-    const int64_t steps = (K + kUnitK - 1) / kUnitK, pairs = capacity[1];
-    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), t0 = (M + 255) / 256;
-    Plan best;
-    for (int64_t t = t0, end = t0 + (t0 < 12 ? t0 + 4 : 16); t <= end; ++t) {
-        int64_t tokens = ((M + t - 1) / t + 15) / 16 * 16;
-        if (forced >= 16 && forced <= 256) tokens = forced;
-        const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens);
-        for (int split = 1; split <= kMaxSplit; ++split) {
-            if (split > 1 && (tiles > capacity[split] || steps < 2 * split)) continue;
-            if (forced_split && split != forced_split && !(split == 1 && (tiles > capacity[forced_split] || steps < 2 * forced_split)))
-                continue;
-            const int64_t rounds = tiles / pairs, tail = split > 1 ? 1 : tiles % pairs;
-            Plan p;
-            p.split = split;
-            p.tokens = p.tail_tokens = (int)tokens;
-            // between tiles: with one accumulator the MMAs wait until it has been read out
-            const double drain = 2 * tokens <= kAccCols ? 100.0 : 3.0 * (double)tokens;
-            const double cost1 = step_ns(full, (int)tokens);
-            p.cost = (double)rounds * ((double)steps * cost1 + drain) + 4.0 * (double)tokens;
-            if (split > 1) {
-                // the sum over the cluster, measured: 1 us + 30 ns per token
-                p.cost = (double)((steps + split - 1) / split) * cost1 + 1000.0 + 30.0 * (double)tokens;
-            } else if (tail > 0) {
-                double last = (double)steps * cost1;
-                for (int parts = 2; rounds > 0 && parts <= 8 && parts * tail <= pairs && 16 * parts <= tokens; ++parts) {
-                    const int tt = (int)(((tokens + parts - 1) / parts + 15) / 16 * 16);
-                    const double c = 1.2 * (double)steps * step_ns(full, tt) + drain;   // (the pieces stream the planes again)
-                    if (c < 0.9 * last) { last = c; p.tail_parts = parts; p.tail_tokens = tt; }
-                }
-                p.cost += last;
-            }
-            if (best.cost == 0 || p.cost < best.cost) best = p;
-        }
-    }
-    return best;
-}
-
-// Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
-// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024), more if four plane units still fit; the
-// planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen
-// by the same zip warps.
-void size_rings(bool full, int tokens, PairParams& prm) {
-    const int x_bytes = tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
-    int xs = (room - 4 * unit_bytes(full)) / x_bytes;
-    xs = xs < 4 ? 4 : xs > kMaxXSlots ? kMaxXSlots : xs;
-    const int units = (room - xs * x_bytes) / unit_bytes(full);
-    prm.x_slots = xs;
-    prm.units = units > kMaxUnits ? kMaxUnits : units & ~1;
-}
-
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K, int* status,
                        cudaStream_t stream) {
@@ -614,7 +533,9 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     prm.tail_parts = plan.tail_parts;
     prm.split = plan.split;
     prm.status = status;
-    size_rings(FULL, plan.tokens, prm);
+    const Rings rings = size_rings(FULL, plan.tokens);
+    prm.units = rings.units;
+    prm.x_slots = rings.x_slots;
     const int64_t tiles = ((N + 2 * kRows - 1) / (2 * kRows)) * ((M + plan.tokens - 1) / plan.tokens);
     if (getenv("DPS_DEBUG"))
         fprintf(stderr, "[dps] pair full=%d M=%lld N=%lld K=%lld tokens=%d tiles=%lld tail=%dx%d split=%d (%d %d %d %d) units=%d x_slots=%d\n", (int)FULL,
@@ -661,9 +582,8 @@ cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const ui
     if (!make_map_2d(&mx, x_sorted, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)A, (uint64_t)K, (uint32_t)tn / 2, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
-    mxt = mx;
-    if (tn >= 32 && !make_map_2d(&mxt, x_sorted, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)A, (uint64_t)K, (uint32_t)tn / 4, 64,
-                                 CU_TENSOR_MAP_SWIZZLE_128B))
+    if (!make_map_2d(&mxt, x_sorted, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)A, (uint64_t)K, (uint32_t)tn / 4, 64,
+                     CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
     PairParams prm = {};
     prm.y = static_cast<__half*>(y);
@@ -674,7 +594,9 @@ cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const ui
     prm.tail_parts = 1;
     prm.split = 1;
     prm.status = status;
-    size_rings(FULL, tn, prm);
+    const Rings rings = size_rings(FULL, tn);
+    prm.units = rings.units;
+    prm.x_slots = rings.x_slots;
     PairGroups gp;
     gp.tiles = static_cast<const int4*>(tiles);
     gp.num_tiles = num_tiles;
@@ -708,15 +630,7 @@ cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const ui
 
 }  // namespace
 
-// Token-tile width of grouped launches: an expert with a quarter, or two and a half standard deviations of an even routing,
-// more rows than the average still fits the average's number of tiles.
-int pair_grouped_tokens(int64_t A, int32_t E) {
-    const double avg = (double)A / E, spread = 2.5 * sqrt(avg);
-    const double want = avg + (spread > 0.25 * avg ? spread : 0.25 * avg);
-    const int tiles = (int)ceil(want / 256.0);
-    const int tokens = (int)(ceil(want / tiles / 16.0)) * 16;
-    return tokens < 16 ? 16 : tokens > 256 ? 256 : tokens;
-}
+int pair_grouped_tokens(int64_t A, int32_t E) { return grouped_tokens(A, E); }
 
 cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y,
                                 int64_t A, int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,

@@ -1,0 +1,113 @@
+// Tile plan of the CTA-pair linear (pair_linear.cu): plain host arithmetic, no CUDA, so that it can be checked over every size.
+#pragma once
+#include <cmath>
+#include <cstdint>
+#include <cstdlib>
+
+namespace dps {
+namespace pair_plan {
+
+constexpr int kRows = 128;                 // weight rows of a row block in one CTA
+constexpr int kUnitK = 128;                // columns of K in a plane unit
+constexpr int kMaxUnits = 12, kMaxXSlots = 8;
+constexpr int kASteps = 4;                 // K steps the A ring in tensor memory holds
+constexpr int kAccCols = 512 - kASteps * (kUnitK / 2);
+constexpr int kMaxSplit = 4;               // pairs of a cluster (eight CTAs, the portable limit)
+constexpr int kEpiCols = 32;               // token columns per epilogue chunk
+constexpr int kEpiBytes = 4 * kEpiCols * 64;
+constexpr int kSmemBytes = 222 * 1024;     // ring + slots + epilogue chunks + alignment
+
+// Token widths are multiples of 32: CUTLASS's atom for this instruction, SM100_MMA_F16BF16_2x1SM_TS (A in tensor memory, two
+// CTAs), admits N = 32, 64 .. 256 and nothing between; only the form with A in shared memory goes in steps of 16.
+constexpr int kTokenStep = 32;
+constexpr int kMaxTokens = 256;
+
+constexpr int unit_bytes(bool full) { return kRows * kUnitK * (full ? 2 : 1); }
+
+struct Rings {
+    int units, x_slots;
+};
+
+struct Plan {
+    int tokens = 256, tail_parts = 1, tail_tokens = 256, split = 1;
+    double cost = 0;
+};
+
+// Time of one K step of a tile in ns, all pairs at work: measured with 74 and 148 tiles of one width (18944 and 37888 rows,
+// 8192 columns; in full mode, up to 128 tokens, on planes that come out of L2) every 32 tokens, between them in proportion.
+inline double step_ns(bool full, int tokens) {
+    static const double fast_ns[9] = {370, 370, 415, 480, 535, 610, 685, 750, 850};
+    static const double full_ns[9] = {500, 500, 520, 600, 680, 800, 1000, 1040, 1100};
+    const double* t = full ? full_ns : fast_ns;
+    const int i = tokens >= 256 ? 7 : tokens / 32;
+    return t[i] + (t[i + 1] - t[i]) * (tokens - 32 * i) / 32.0;
+}
+
+// A round of tiles over the pairs takes as long as one tile, so the number of token tiles is chosen to make the sum over the
+// rounds small; the tiles of a last, partial round are cut into pieces of the tokens if that shortens it.  Few tiles: up to
+// four pairs share each, a range of K each; capacity[s] = clusters of s pairs that are resident at once.
+// DPS_PAIR_TOKENS=1..256 (rounded up to a width there is) and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
+inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) {
+    static const int forced = [] { const char* e = getenv("DPS_PAIR_TOKENS"); return e ? (atoi(e) + kTokenStep - 1) / kTokenStep * kTokenStep : 0; }();
+    static const int forced_split = [] { const char* e = getenv("DPS_PAIR_SPLIT"); return e ? atoi(e) : 0; }();
+    const int64_t steps = (K + kUnitK - 1) / kUnitK, pairs = capacity[1];
+    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), t0 = (M + 255) / 256;
+    Plan best;
+    for (int64_t t = t0, end = t0 + (t0 < 12 ? t0 + 4 : 16); t <= end; ++t) {
+        int64_t tokens = ((M + t - 1) / t + kTokenStep - 1) / kTokenStep * kTokenStep;
+        if (forced >= kTokenStep && forced <= kMaxTokens) tokens = forced;
+        const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens);
+        for (int split = 1; split <= kMaxSplit; ++split) {
+            if (split > 1 && (tiles > capacity[split] || steps < 2 * split)) continue;
+            if (forced_split && split != forced_split && !(split == 1 && (tiles > capacity[forced_split] || steps < 2 * forced_split)))
+                continue;
+            const int64_t rounds = tiles / pairs, tail = split > 1 ? 1 : tiles % pairs;
+            Plan p;
+            p.split = split;
+            p.tokens = p.tail_tokens = (int)tokens;
+            // between tiles: with one accumulator the MMAs wait until it has been read out
+            const double drain = 2 * tokens <= kAccCols ? 100.0 : 3.0 * (double)tokens;
+            const double cost1 = step_ns(full, (int)tokens);
+            p.cost = (double)rounds * ((double)steps * cost1 + drain) + 4.0 * (double)tokens;
+            if (split > 1) {
+                // the sum over the cluster, measured: 1 us + 30 ns per token
+                p.cost = (double)((steps + split - 1) / split) * cost1 + 1000.0 + 30.0 * (double)tokens;
+            } else if (tail > 0) {
+                double last = (double)steps * cost1;
+                for (int parts = 2; rounds > 0 && parts <= 8 && parts * tail <= pairs && kTokenStep * parts <= tokens; ++parts) {
+                    const int tt = (int)(((tokens + parts - 1) / parts + kTokenStep - 1) / kTokenStep * kTokenStep);
+                    const double c = 1.2 * (double)steps * step_ns(full, tt) + drain;   // (the pieces stream the planes again)
+                    if (c < 0.9 * last) { last = c; p.tail_parts = parts; p.tail_tokens = tt; }
+                }
+                p.cost += last;
+            }
+            if (best.cost == 0 || p.cost < best.cost) best = p;
+        }
+    }
+    return best;
+}
+
+// Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
+// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024), more if four plane units still fit; the
+// planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen
+// by the same zip warps.
+inline Rings size_rings(bool full, int tokens) {
+    const int x_bytes = tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
+    int xs = (room - 4 * unit_bytes(full)) / x_bytes;
+    xs = xs < 4 ? 4 : xs > kMaxXSlots ? kMaxXSlots : xs;
+    const int units = (room - xs * x_bytes) / unit_bytes(full);
+    return {units > kMaxUnits ? kMaxUnits : units & ~1, xs};
+}
+
+// Token-tile width of grouped launches: an expert with a quarter, or two and a half standard deviations of an even routing,
+// more rows than the average still fits the average's number of tiles.
+inline int grouped_tokens(int64_t A, int32_t E) {
+    const double avg = (double)A / E, spread = 2.5 * sqrt(avg);
+    const double want = avg + (spread > 0.25 * avg ? spread : 0.25 * avg);
+    const int tiles = (int)ceil(want / 256.0);
+    const int tokens = (int)ceil(want / tiles / kTokenStep) * kTokenStep;
+    return tokens < kTokenStep ? kTokenStep : tokens > kMaxTokens ? kMaxTokens : tokens;
+}
+
+}  // namespace pair_plan
+}  // namespace dps
