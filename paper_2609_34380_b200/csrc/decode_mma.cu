@@ -82,11 +82,11 @@ __device__ __forceinline__ void to_half_pairs(const uint4& p, const uint4& r, ui
 // SHORT: K is U rounds and perhaps a ragged end, less than a batch of the long variant; all of it is one batch.
 // HALF: the CTA owns 8 weight rows instead of 16 (the upper half of every MMA tile is zero).  It
 // doubles the number of CTAs for matrices with few rows; the MMA work wasted is irrelevant here.
+// x without __restrict__: its writer may still run when a CTA starts, so it must not go through the non-coherent path.
 template <int ENC, bool FULL, int NT, int U, bool SHORT, bool HALF>
 __global__ void __launch_bounds__(kThreads, 2)
-decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp,
-                  __half* __restrict__ y, int M, int64_t N, int64_t K, int prefetch_steps,
-                  int prefetch_ctas, int trace_slot) {
+decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp, __half* y, int M, int64_t N,
+                  int64_t K, int prefetch_steps, int prefetch_ctas, int trace_slot) {
     constexpr float kScale = (ENC == kEncE4M3 && !FULL) ? 0.00390625f : 1.0f;  // 2^-8, exact
     __shared__ float red[kWarps][kRowsPerBlock][NT * 8 + 1];
     sm100::grid_launch_dependents();

@@ -53,9 +53,9 @@ __device__ __forceinline__ uint2 quantize8(const uint4& v, float sc) {
     return make_uint2(out[0], out[1]);
 }
 
+// (x without __restrict__: its writer may still run when a CTA starts)
 __global__ void __launch_bounds__(kQuantThreads)
-quantize_activations_kernel(const uint4* __restrict__ x, uint2* __restrict__ q, float* __restrict__ scale, int64_t k8,
-                            int* status) {
+quantize_activations_kernel(const uint4* x, uint2* q, float* scale, int64_t k8, int* status) {
     __shared__ float s_max[kQuantThreads / 32];
     __shared__ float s_scale;
     grid_launch_dependents();

@@ -9,8 +9,8 @@ namespace {
 
 template <int ENC, bool FULL, int MT>
 __global__ void __launch_bounds__(kGemvThreads, 2)
-gemv_dense_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp,
-                  __half* __restrict__ y, int m_count, int64_t N, int64_t K, int rows_per_cta, int red_stride) {
+gemv_dense_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp, __half* y, int m_count,
+                  int64_t N, int64_t K, int rows_per_cta, int red_stride) {
     extern __shared__ float red[];
     sm100::grid_launch_dependents();  // let the next kernel's CTAs take the slots this grid frees
     sm100::grid_dependency_wait();    // activations (and possibly planes) come from the preceding kernel

@@ -70,9 +70,8 @@ __device__ __forceinline__ bool row_valid(const int32_t* token_of_row, const int
 constexpr int kTableExperts = 256;
 
 __global__ void __launch_bounds__(kRouteThreads)
-moe_route_kernel(const int32_t* __restrict__ token_of_row, const int32_t* __restrict__ expert_of_row, int A, int T,
-                 int E, int tile_tokens, int32_t* counts, int32_t* offsets, int32_t* sorted_rows,
-                 int32_t* num_tiles, int4* tiles, int* status) {
+moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E, int tile_tokens,
+                 int32_t* counts, int32_t* offsets, int32_t* sorted_rows, int32_t* num_tiles, int4* tiles, int* status) {
     __shared__ int s_cnt[kMaxExperts];
     __shared__ int s_off[kMaxExperts];
     __shared__ int s_table[kRouteThreads / 32][kTableExperts];
@@ -161,10 +160,11 @@ moe_route_kernel(const int32_t* __restrict__ token_of_row, const int32_t* __rest
 }
 
 // x_sorted[i][:] = x[token(sorted_rows[i])][:] for the valid rows; 16 bytes per thread.
+// No __restrict__ here and in the routing kernel: both are resident while the kernels that write what they read still run,
+// and a pointer marked so may be read through the non-coherent path, which wants data that nobody writes meanwhile.
 __global__ void __launch_bounds__(256)
-moe_gather_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ token_of_row,
-                  const int32_t* __restrict__ sorted_rows, const int32_t* __restrict__ num_tiles,
-                  uint4* __restrict__ x_sorted, int64_t k16) {
+moe_gather_kernel(const uint4* x, const int32_t* token_of_row, const int32_t* sorted_rows, const int32_t* num_tiles,
+                  uint4* x_sorted, int64_t k16) {
     sm100::grid_launch_dependents();
     sm100::grid_dependency_wait();   // sorted_rows and num_tiles come from the routing kernel
     const int valid = num_tiles[1];
