@@ -157,7 +157,9 @@ def dps_linear(mode: int, enc: int, x: torch.Tensor, w_persist: torch.Tensor, w_
     """y[M][N] = x[M][K] * W_eff^T from the planes, in fast or full mode."""
     if stream is None and _fast_linear is not None:
         out = _fast_linear(mode, enc, x, w_persist, w_resid, y)
-        if out is not None:     # None: not a plain case, or refused; the path below runs it or says why
+        if out.__class__ is int:    # refused
+            _check(out, "dps_linear")
+        if out is not None:         # None: not a plain case; the path below runs it or says why
             return out
     M, K = x.shape
     N, K2 = w_persist.shape

@@ -1,7 +1,9 @@
 // CPython entry for the call that a decoder makes most, dps_linear: argument checks, output allocation and the current stream
 // in native code, then the same C ABI function of libdps.so.  Small layers are bound by the host: a call of a 512 x 512 layer takes 13.0 us through ctypes, 4.6 us through here.
-// Anything out of the ordinary (another tensor type, a wrong dtype, a shape that does not fit, a status other than 0)
-// returns None, and the caller takes the ctypes path, which says what is wrong.
+// Anything out of the ordinary (another tensor type, a wrong dtype, a shape that does not fit) returns None, and the caller
+// takes the ctypes path, which says what is wrong.  A status other than 0 is returned as an int: the call was made once, and
+// is not made again.  The GIL is released around the allocation and the call, as ctypes and PyTorch's operators do: either may
+// block (a full launch queue, a first call's set-up), and what they wait for may need Python.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -12,6 +14,11 @@ namespace {
 
 using LinearFn = int (*)(int32_t, int32_t, const void*, const uint8_t*, const uint8_t*, void*, int64_t, int64_t, int64_t, void*);
 LinearFn g_linear = nullptr;
+
+struct WithoutGil {
+    PyThreadState* state = PyEval_SaveThread();
+    ~WithoutGil() { PyEval_RestoreThread(state); }
+};
 
 // set_linear(address of dps_linear)
 PyObject* set_linear(PyObject*, PyObject* arg) {
@@ -24,7 +31,7 @@ bool plain(const at::Tensor& t, at::ScalarType type) {
     return t.is_cuda() && t.scalar_type() == type && t.layout() == at::kStrided && t.is_contiguous();
 }
 
-// linear(mode, enc, x, w_persist, w_resid or None, y or None) -> y, or None: use the other path
+// linear(mode, enc, x, w_persist, w_resid or None, y or None) -> y, or a status that is not 0, or None: use the other path
 PyObject* linear(PyObject*, PyObject* const* args, Py_ssize_t n) {
     if (n != 6 || g_linear == nullptr || !PyLong_Check(args[0]) || !PyLong_Check(args[1])) Py_RETURN_NONE;
     if (!THPVariable_CheckExact(args[2]) || !THPVariable_CheckExact(args[3])) Py_RETURN_NONE;
@@ -47,17 +54,23 @@ PyObject* linear(PyObject*, PyObject* const* args, Py_ssize_t n) {
             r = t.const_data_ptr<uint8_t>();
         }
         const int64_t m = x.size(0), rows = p.size(0), k = x.size(1);
+        const void* px = x.const_data_ptr();
+        const uint8_t* pp = p.const_data_ptr<uint8_t>();
         PyObject* out = args[5];
         at::Tensor y;
         if (out != Py_None) {
             y = THPVariable_Unpack(out);
             if (!plain(y, at::kHalf)) Py_RETURN_NONE;
-        } else {
-            y = at::empty({m, rows}, at::TensorOptions().dtype(at::kHalf).device(x.device()));
         }
-        const int status = g_linear((int32_t)mode, (int32_t)enc, x.const_data_ptr(), p.const_data_ptr<uint8_t>(), r,
-                                    y.mutable_data_ptr(), m, rows, k, c10::cuda::getCurrentCUDAStream().stream());
-        if (status != 0) Py_RETURN_NONE;
+        int status = 0;
+        {
+            const auto device = x.device();
+            WithoutGil nogil;   // (the caller's frame holds the argument tensors)
+            if (!y.defined()) y = at::empty({m, rows}, at::TensorOptions().dtype(at::kHalf).device(device));
+            status = g_linear((int32_t)mode, (int32_t)enc, px, pp, r, y.mutable_data_ptr(), m, rows, k,
+                              c10::cuda::getCurrentCUDAStream().stream());
+        }
+        if (status != 0) return PyLong_FromLong(status);
         if (out != Py_None) {
             Py_INCREF(out);
             return out;

@@ -1,4 +1,8 @@
 """The native marshalling of dps_linear: what it does not take goes the ctypes way and is refused there as before."""
+import ctypes
+import threading
+import time
+
 import pytest
 import torch
 
@@ -46,3 +50,71 @@ def test_same_results_and_same_refusals():
                        ((0, enc, x.t().contiguous().t(), p, r), ValueError)]:
         with pytest.raises(error):
             dps.dps_linear(*bad)
+
+
+@pytest.fixture
+def plain_call():
+    """A call that the native entry takes, and a way to put another function in the place of the library's; undone afterwards."""
+    w = workloads.weights(136, 144, 1, device="cuda:0")
+    p, r, enc = dps.dps_split_weights(w)
+    x = workloads.activations(5, 144, 2, device="cuda:0")
+    assert binding._fast_linear is not None
+    set_linear = binding._fast_linear.__self__.set_linear
+    yield (enc, x, p, r), lambda fn: set_linear(ctypes.cast(fn, ctypes.c_void_p).value)
+    set_linear(ctypes.cast(binding.library().dps_linear, ctypes.c_void_p).value)
+
+
+@pytest.mark.gpu
+def test_plain_calls_are_taken_and_go_to_the_current_stream(plain_call):
+    (enc, x, p, r), _ = plain_call
+    y = binding._fast_linear(dps.DPS_MODE_FULL, enc, x, p, r, None)
+    assert isinstance(y, torch.Tensor)
+    out = torch.zeros_like(y)
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=side):            # a launch on another stream is not in the graph
+        assert binding._fast_linear(dps.DPS_MODE_FULL, enc, x, p, r, out) is out
+    torch.cuda.synchronize()
+    assert bool((out == 0).all())
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, y)
+
+
+@pytest.mark.gpu
+def test_other_threads_run_while_the_call_blocks(plain_call):
+    (enc, x, p, r), put = plain_call
+    put(ctypes.CDLL(None).sleep)                          # sleep(mode) seconds, then status 0
+    ticks, stop = [], threading.Event()
+
+    def tick():
+        while not stop.wait(0.01):
+            ticks.append(time.monotonic())
+    thread = threading.Thread(target=tick)
+    thread.start()
+    try:
+        begin = time.monotonic()
+        assert isinstance(dps.dps_linear(1, enc, x, p, r), torch.Tensor)
+        end = time.monotonic()
+    finally:
+        stop.set()
+        thread.join()
+    assert end - begin > 0.9
+    assert sum(begin + 0.1 < t < end - 0.1 for t in ticks) > 20
+
+
+@pytest.mark.gpu
+def test_a_failed_call_is_reported_and_not_made_again(plain_call):
+    (enc, x, p, r), put = plain_call
+    calls = []
+
+    def fails(*args):
+        calls.append(args)
+        return binding.DPS_ERR_CUDA
+    fn = ctypes.CFUNCTYPE(ctypes.c_int, *binding.library().dps_linear.argtypes)(fails)
+    put(fn)
+    before = dps.dps_launch_count()
+    with pytest.raises(dps.DpsError) as caught:
+        dps.dps_linear(dps.DPS_MODE_FULL, enc, x, p, r)
+    assert caught.value.status == binding.DPS_ERR_CUDA
+    assert len(calls) == 1 and dps.dps_launch_count() == before
