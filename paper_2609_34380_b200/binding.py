@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import importlib.util
+import sysconfig
 from pathlib import Path
 from typing import Optional, Sequence, Tuple
 
@@ -46,7 +47,17 @@ ABI = {
 }
 
 _lib = None
-FASTCALL_PATH = Path(__file__).resolve().parent / "_fastcall.so"
+
+
+def fastcall_path() -> Path:
+    """Where the native marshalling for the PyTorch and Python of this process lives: it reads tensors by their C++
+    layout, so a binary built against another version must not be taken for it."""
+    return Path(__file__).resolve().parent / (f"_fastcall-{torch.__version__}-{str(torch.version.git_version)[:8]}-"
+                                              f"{sysconfig.get_config_var('SOABI')}.so")
+
+
+FASTCALL_PATH = fastcall_path()
+
 _fast_linear = None     # native marshalling of dps_linear (csrc/fastcall.cpp); set when the library is loaded, if it was built
 
 
@@ -77,13 +88,14 @@ def library() -> ctypes.CDLL:
 def _load_fastcall(lib: ctypes.CDLL) -> None:
     """The same call with less host work; without the module every call takes the ctypes path below."""
     global _fast_linear
-    if not FASTCALL_PATH.exists():
+    path = fastcall_path()
+    if not path.exists():       # not built, or built for another PyTorch or Python
         return
     try:
-        spec = importlib.util.spec_from_file_location("_fastcall", FASTCALL_PATH)
+        spec = importlib.util.spec_from_file_location("_fastcall", path)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)
-    except ImportError:         # built against another PyTorch
+    except ImportError:
         return
     module.set_linear(ctypes.cast(lib.dps_linear, ctypes.c_void_p).value)
     _fast_linear = module.linear

@@ -15,7 +15,6 @@ from pathlib import Path
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libdps.so"
-FASTCALL = PKG / "_fastcall.so"
 INCLUDE = PKG.parent / "include"
 
 NVCC_FLAGS = [
@@ -80,10 +79,15 @@ def build_fastcall(force: bool = False) -> Path:
     import torch
     from torch.utils.cpp_extension import include_paths, library_paths
 
-    src = CSRC / "fastcall.cpp"
-    if not force and FASTCALL.exists() and FASTCALL.stat().st_mtime >= src.stat().st_mtime:
-        return FASTCALL
-    tmp = FASTCALL.with_suffix(f".tmp{os.getpid()}.so")
+    from .binding import fastcall_path
+
+    src, out = CSRC / "fastcall.cpp", fastcall_path()
+    for other in PKG.glob("_fastcall*.so"):         # other versions' modules
+        if other != out:
+            other.unlink(missing_ok=True)
+    if not force and out.exists() and out.stat().st_mtime >= src.stat().st_mtime:
+        return out
+    tmp = out.with_name(f"fastcall.tmp{os.getpid()}.so")
     cuda = Path(_nvcc()).resolve().parent.parent / "include"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
@@ -96,8 +100,8 @@ def build_fastcall(force: bool = False) -> Path:
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"g++ failed for {src.name}:\n{res.stdout}\n{res.stderr}")
-    os.replace(tmp, FASTCALL)
-    return FASTCALL
+    os.replace(tmp, out)
+    return out
 
 
 if __name__ == "__main__":

@@ -118,3 +118,15 @@ def test_a_failed_call_is_reported_and_not_made_again(plain_call):
         dps.dps_linear(dps.DPS_MODE_FULL, enc, x, p, r)
     assert caught.value.status == binding.DPS_ERR_CUDA
     assert len(calls) == 1 and dps.dps_launch_count() == before
+
+
+def test_a_module_of_another_version_is_not_taken(monkeypatch):
+    build.build_fastcall()
+    lib = binding.library()
+    monkeypatch.setattr(binding, "_fast_linear", None)
+    monkeypatch.setattr(torch, "__version__", "2.99.0")
+    binding._load_fastcall(lib)
+    assert binding._fast_linear is None
+    monkeypatch.undo()
+    binding._load_fastcall(lib)
+    assert binding._fast_linear is not None
