@@ -1,11 +1,12 @@
 """GPU: the dense linear on CTA pairs against the oracle, at the edges of its tiles: rows within the first CTA of a pair, just
 into the second, beyond a whole tile; one token to several token tiles; K below, at and above one plane unit and the ring;
-more tiles than pairs, with a last round cut into pieces.
+more tiles than pairs; a last round cut into pieces.
 
 DPS_FORCE_PATH / DPS_PAIR_TOKENS / DPS_PAIR_SPLIT pin the family, the tile width and the K split; the library reads them once
 per process, so each forced run is a child process: this file executed as a script.
 """
 import os
+import re
 import subprocess
 import sys
 
@@ -44,6 +45,22 @@ def _run(shapes):
                 count += 1
     assert dps.dps_stream_status() == dps.DPS_OK
     print(f"all {count} cases passed")
+
+
+# 80 tiles of 256 tokens: one round and 6 to 14 tiles more on 74 to 66 pairs, each cut into at least 4 pieces; the last token
+# tile has 108 tokens, which end inside a piece
+CUT = (2440, 1040, 1900)
+
+
+@pytest.mark.gpu
+def test_last_round_in_pieces_in_child_process():
+    env = dict(os.environ, DPS_FORCE_PATH="pair", DPS_PAIR_TOKENS="256", DPS_PAIR_SPLIT="1", DPS_DEBUG="1", PYTHONPATH=REPO)
+    out = subprocess.run([sys.executable, os.path.abspath(__file__), ",".join(map(str, CUT))], cwd=REPO, env=env,
+                         capture_output=True, text=True, timeout=900)
+    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
+    assert "all 6 cases passed" in out.stdout
+    parts = [int(p) for p in re.findall(r"\[dps\] pair full=.*? tail=(\d+)x", out.stderr)]
+    assert len(parts) == 12 and min(parts) > 1, out.stderr[-2000:]
 
 
 @pytest.mark.gpu

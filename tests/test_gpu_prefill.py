@@ -62,10 +62,8 @@ def test_prefill_determinism():
 
 @pytest.mark.parametrize("enc_req", [dps.DPS_ENC_AUTO, dps.DPS_ENC_E5M2])
 def test_persistent_kernel_ragged_shapes_every_output(enc_req):
-    """More tiles than SMs with a short last round, ragged in every direction: N = 2056 (17 row
-    tiles, the last with 8 rows), K = 1104 (a partial last K block, an odd number of blocks to halve),
-    M = 2500 (partial last token tile).  Full mode walks 170 tiles of 256 tokens, fast mode 180
-    two-row-block tiles; in both the last round is shared out as halves of K.  Every output is checked."""
+    """Two rounds of tiles, ragged in every direction: N = 2056 (nine tiles of 256 rows, the last with 8), K = 1104 (a partial
+    last K step), M = 2500 (a partial last token tile).  Every output is checked."""
     N, K, M = 2056, 1104, 2500
     w = workloads.weights(N, K, 611, device=DEV)
     p, r, enc, p_ref, r_ref = split_both(w, enc_req, DEV)

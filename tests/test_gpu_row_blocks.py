@@ -1,9 +1,8 @@
-"""GPU parity of the two-row-block tiles (256 weight rows per CTA) and of the persistent kernel on
-small, ragged shapes.
+"""GPU parity of dense and grouped linears on small, ragged shapes: with the kernels that the library picks, and with other
+families, tile widths and K splits forced.
 
-The launchers pick those only for large problems; the tuning knobs DPS_DENSE_RB, DPS_GROUPED_RB and
-DPS_PERSIST force them.  The library reads its knobs once per process, so each forced run is a child
-process: this file executed as a script compares against the oracle and prints one line per case.
+The library reads its knobs (DPS_FORCE_PATH, DPS_FORCE_SPLIT, DPS_PAIR_TOKENS, DPS_PAIR_SPLIT) once per process, so each
+forced run is a child process: this file executed as a script compares against the oracle and prints one line per case.
 """
 import os
 import subprocess
@@ -24,7 +23,7 @@ def _cases():
     from tests.helpers import assert_close_to_oracle, split_both, to_np_words
 
     dev = "cuda:0"
-    # dense: N not a multiple of 256 (second row block ragged or absent), K with a ragged last block,
+    # dense: N not a multiple of 256 (a pair's second row block ragged or absent), K with a ragged last block,
     # token counts that leave a partial last token tile
     for (N, K, M) in [(640, 1088, 200), (128, 512, 65), (904, 2064, 300), (392, 272, 577)]:
         for forced_enc in (dps.DPS_ENC_AUTO, dps.DPS_ENC_E5M2):
@@ -36,7 +35,8 @@ def _cases():
                 ref = oracle.linear(mode, enc, to_np_words(x), p_ref, r_ref, threads=8)
                 assert_close_to_oracle(y, ref, f"dense N={N} K={K} M={M} enc={enc} mode={mode}")
                 print(f"ok dense N={N} K={K} M={M} enc={enc} mode={mode}")
-    # grouped: experts with 0, few and more than one tile of rows; N ragged against 256
+    # grouped: experts with 0, few and more than one tile of rows; N ragged against 256; 45 and 100 rows per expert, on the
+    # tiles of one CTA and on CTA pairs
     for (E, N, K, T) in [(4, 384, 1040, 90), (3, 136, 528, 150)]:
         ps, rs, encs, p_refs, r_refs = [], [], [], [], []
         for e in range(E):
@@ -62,46 +62,32 @@ def _cases():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("persist", ["0", "2"])      # one CTA per tile / persistent kernel forced
-def test_forced_two_row_blocks_in_child_process(persist):
-    env = dict(os.environ, DPS_DENSE_RB="2", DPS_GROUPED_RB="2", DPS_PERSIST=persist, PYTHONPATH=REPO)
+@pytest.mark.parametrize("knobs", [
+    {},
+    {"DPS_FORCE_PATH": "pair", "DPS_PAIR_TOKENS": "192", "DPS_PAIR_SPLIT": "1"},
+    {"DPS_FORCE_PATH": "pair", "DPS_PAIR_TOKENS": "256", "DPS_PAIR_SPLIT": "1"},
+    {"DPS_FORCE_PATH": "pair", "DPS_PAIR_TOKENS": "256", "DPS_PAIR_SPLIT": "2"},
+    {"DPS_FORCE_PATH": "umma", "DPS_FORCE_SPLIT": "1"},
+    {"DPS_FORCE_PATH": "umma", "DPS_FORCE_SPLIT": "3"},
+], ids=["default", "pair192", "pair256", "pair256_split2", "umma", "umma_split3"])
+def test_ragged_shapes_in_child_process(knobs):
+    env = dict(os.environ, DPS_DEBUG="1", PYTHONPATH=REPO, **knobs)
     out = subprocess.run([sys.executable, os.path.abspath(__file__)], cwd=REPO, env=env, capture_output=True,
                          text=True, timeout=600)
     assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
     assert "all row-block cases passed" in out.stdout
     assert out.stdout.count("ok dense") == 16 and out.stdout.count("ok grouped") == 4
-
-
-@pytest.mark.gpu
-@pytest.mark.parametrize("persist", ["0", "2"])
-def test_forced_192_token_two_row_block_tiles_in_child_process(persist):
-    """Fast mode, 256 rows x 192 tokens per CTA (the launcher picks it from two rounds of such tiles on): here
-    forced on shapes with a ragged second row block, a ragged last K block and a short last token tile."""
-    env = dict(os.environ, DPS_DENSE_RB="2", DPS_RB2_TN="192", DPS_PERSIST=persist, PYTHONPATH=REPO)
-    out = subprocess.run([sys.executable, os.path.abspath(__file__)], cwd=REPO, env=env, capture_output=True,
-                         text=True, timeout=600)
-    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
-    assert "all row-block cases passed" in out.stdout
-
-
-@pytest.mark.gpu
-def test_forced_k_halves_for_every_tile_in_child_process():
-    """Few 256-token tiles: two CTAs per tile, each with one half of K (forced; 1 to 8 tiles here)."""
-    env = dict(os.environ, DPS_PAIR_ALL="2", DPS_FORCE_TN="256", PYTHONPATH=REPO)
-    out = subprocess.run([sys.executable, os.path.abspath(__file__)], cwd=REPO, env=env, capture_output=True,
-                         text=True, timeout=600)
-    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
-    assert "all row-block cases passed" in out.stdout
-
-
-@pytest.mark.gpu
-def test_forced_persistent_kernel_with_default_tiles_in_child_process():
-    """256-token tiles (forced: the shapes here are small) walked by the persistent kernel."""
-    env = dict(os.environ, DPS_PERSIST="2", DPS_FORCE_TN="256", PYTHONPATH=REPO)
-    out = subprocess.run([sys.executable, os.path.abspath(__file__)], cwd=REPO, env=env, capture_output=True,
-                         text=True, timeout=600)
-    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
-    assert "all row-block cases passed" in out.stdout
+    # what was asked for is what ran
+    launches = [line for line in out.stderr.splitlines() if line.startswith("[dps]") and "grouped" not in line]
+    assert len(launches) == 16
+    path, tokens, split = (knobs.get(k) for k in ("DPS_FORCE_PATH", "DPS_PAIR_TOKENS", "DPS_PAIR_SPLIT"))
+    if path:
+        assert all(line.startswith(f"[dps] {path} ") for line in launches)
+    if tokens:
+        assert all(f"tokens={tokens} " in line for line in launches)
+    split = split or knobs.get("DPS_FORCE_SPLIT")
+    if split:       # (a K of fewer steps than the split needs keeps a smaller one)
+        assert sum(f"split={split} " in line for line in launches) >= 12
 
 
 if __name__ == "__main__":
