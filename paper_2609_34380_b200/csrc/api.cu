@@ -65,7 +65,7 @@ DeviceInfo* device_info() {
     return &d;
 }
 
-// Tuning / debugging knob: DPS_FORCE_PATH=gemv, =umma or =stream pins the dense kernel family.
+// Tuning / debugging knob: DPS_FORCE_PATH=gemv, =umma, =stream or =pair pins the dense kernel family.
 int forced_path() {
     static const int path = [] {
         const char* v = getenv("DPS_FORCE_PATH");

@@ -80,10 +80,8 @@ __device__ __forceinline__ void to_half_pairs(const uint4& p, const uint4& r, ui
 }
 
 // SHORT: K is U rounds and perhaps a ragged end, less than a batch of the long variant; all of it is one batch.
-// HALF: the CTA owns 8 weight rows instead of 16 (the upper half of every MMA tile is zero).  It
-// doubles the number of CTAs for matrices with few rows; the MMA work wasted is irrelevant here.
 // x without __restrict__: its writer may still run when a CTA starts, so it must not go through the non-coherent path.
-template <int ENC, bool FULL, int NT, int U, bool SHORT, bool HALF>
+template <int ENC, bool FULL, int NT, int U, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp, __half* y, int M, int64_t N,
                   int64_t K, int prefetch_steps, int prefetch_ctas, int trace_slot) {
@@ -97,8 +95,8 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
     // of its rows behind that batch, so that the DRAM pipe keeps working through the other
     // kernel's tail.  Thread i takes row i / 16 and every 16th 128-byte line of it.
     if (prefetch_steps > 0 && (int)blockIdx.x < prefetch_ctas) {
-        const int64_t prow = (int64_t)blockIdx.x * (HALF ? 8 : kRowsPerBlock) + (threadIdx.x >> 4);
-        if (prow < N && (!HALF || (threadIdx.x >> 4) < 8)) {
+        const int64_t prow = (int64_t)blockIdx.x * kRowsPerBlock + (threadIdx.x >> 4);
+        if (prow < N) {
             const int64_t first = (int64_t)U * kRoundK;   // bytes of a row the first batch loads itself
             const int64_t pbase = prow * K + first + (threadIdx.x & 15) * 128;
             for (int j = 0; j < prefetch_steps; ++j) {
@@ -112,7 +110,6 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    constexpr int kRows = HALF ? 8 : kRowsPerBlock;
     const int full_rounds = (int)(K / kRoundK);           // rounds in which every lane is inside K
     const bool has_tail = (K % kRoundK) != 0;
     const int kl = warp * 64 + t * 16;                    // this lane's byte offset inside a round
@@ -126,7 +123,7 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
     {   // one row block per CTA: the hardware block scheduler balances the SMs
         const int64_t rb = blockIdx.x;
         // rows past N are clamped for the loads and dropped at the store
-        const int64_t row_lo = rb * kRows + g, row_hi = row_lo + 8;
+        const int64_t row_lo = rb * kRowsPerBlock + g, row_hi = row_lo + 8;
         const uint8_t* p_lo = P + (row_lo < N ? row_lo : N - 1) * K + kl;
         const uint8_t* p_hi = P + (row_hi < N ? row_hi : N - 1) * K + kl;
         const uint8_t* r_lo = FULL ? Rp + (row_lo < N ? row_lo : N - 1) * K + kl : nullptr;
@@ -151,12 +148,7 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
                             const uint4 (&xb)[NT][2]) {
             uint32_t a_lo[8], a_hi[8];
             to_half_pairs<ENC, FULL>(wp_lo, wr_lo, a_lo);
-            if (HALF) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) a_hi[i] = 0u;
-            } else {
-                to_half_pairs<ENC, FULL>(wp_hi, wr_hi, a_hi);
-            }
+            to_half_pairs<ENC, FULL>(wp_hi, wr_hi, a_hi);
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
                 const uint4 b0 = xb[n][0], b1 = xb[n][1];
@@ -178,10 +170,10 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
             for (int u = 0; u < U; ++u) {
                 wp_hi[u] = wr_lo[u] = wr_hi[u] = make_uint4(0, 0, 0, 0);
                 wp_lo[u] = ldg_stream(p_lo + base + u * kRoundK);
-                if (!HALF) wp_hi[u] = ldg_stream(p_hi + base + u * kRoundK);
+                wp_hi[u] = ldg_stream(p_hi + base + u * kRoundK);
                 if (FULL) {
                     wr_lo[u] = ldg_stream(r_lo + base + u * kRoundK);
-                    if (!HALF) wr_hi[u] = ldg_stream(r_hi + base + u * kRoundK);
+                    wr_hi[u] = ldg_stream(r_hi + base + u * kRoundK);
                 }
             }
             const int kt = U * kRoundK;                   // SHORT: the ragged end of K
@@ -189,10 +181,10 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
             uint4 tp_lo = make_uint4(0, 0, 0, 0), tp_hi = tp_lo, tr_lo = tp_lo, tr_hi = tp_lo;
             if (tail) {
                 tp_lo = ldg_stream(p_lo + kt);
-                if (!HALF) tp_hi = ldg_stream(p_hi + kt);
+                tp_hi = ldg_stream(p_hi + kt);
                 if (FULL) {
                     tr_lo = ldg_stream(r_lo + kt);
-                    if (!HALF) tr_hi = ldg_stream(r_hi + kt);
+                    tr_hi = ldg_stream(r_hi + kt);
                 }
             }
             // Everything but the planes may come from the preceding kernel: wait for it here, with the
@@ -232,10 +224,10 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
                 wp_lo[u] = wp_hi[u] = wr_lo[u] = wr_hi[u] = make_uint4(0, 0, 0, 0);
                 if (in) {
                     wp_lo[u] = ldg_stream(p_lo + base);
-                    if (!HALF) wp_hi[u] = ldg_stream(p_hi + base);
+                    wp_hi[u] = ldg_stream(p_hi + base);
                     if (FULL) {
                         wr_lo[u] = ldg_stream(r_lo + base);
-                        if (!HALF) wr_hi[u] = ldg_stream(r_hi + base);
+                        wr_hi[u] = ldg_stream(r_hi + base);
                     }
                 }
                 load_x(xb[u], base, in);
@@ -256,15 +248,13 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
         for (int n = 0; n < NT; ++n) {
             red[warp][g][n * 8 + 2 * t] = acc[n][0];
             red[warp][g][n * 8 + 2 * t + 1] = acc[n][1];
-            if (!HALF) {
-                red[warp][g + 8][n * 8 + 2 * t] = acc[n][2];
-                red[warp][g + 8][n * 8 + 2 * t + 1] = acc[n][3];
-            }
+            red[warp][g + 8][n * 8 + 2 * t] = acc[n][2];
+            red[warp][g + 8][n * 8 + 2 * t + 1] = acc[n][3];
         }
         __syncthreads();
-        for (int o = threadIdx.x; o < kRows * NT * 8; o += kThreads) {
-            const int tok = o / kRows, row = o % kRows;
-            const int64_t n_out = rb * kRows + row;
+        for (int o = threadIdx.x; o < kRowsPerBlock * NT * 8; o += kThreads) {
+            const int tok = o / kRowsPerBlock, row = o % kRowsPerBlock;
+            const int64_t n_out = rb * kRowsPerBlock + row;
             if (tok < M && n_out < N) {
                 float s = 0.f;
 #pragma unroll
@@ -277,11 +267,10 @@ decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t*
     }
 }
 
-template <int ENC, bool FULL, int NT, int U, bool SHORT, bool HALF>
+template <int ENC, bool FULL, int NT, int U, bool SHORT>
 cudaError_t launch_one(const __half* x, const uint8_t* p, const uint8_t* r, __half* y, int M, int64_t N, int64_t K,
                        cudaStream_t stream) {
-    constexpr int kRows = HALF ? 8 : kRowsPerBlock;
-    const int64_t grid = (N + kRows - 1) / kRows;
+    const int64_t grid = (N + kRowsPerBlock - 1) / kRowsPerBlock;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -314,7 +303,7 @@ cudaError_t launch_one(const __half* x, const uint8_t* p, const uint8_t* r, __ha
     static int trace_launches = 0;
     trace_slot = trace_launches++;
 #endif
-    cudaError_t e = cudaLaunchKernelEx(&cfg, decode_mma_kernel<ENC, FULL, NT, U, SHORT, HALF>, x, p, r, y, M, N, K,
+    cudaError_t e = cudaLaunchKernelEx(&cfg, decode_mma_kernel<ENC, FULL, NT, U, SHORT>, x, p, r, y, M, N, K,
                                        prefetch_steps, prefetch_ctas, trace_slot);
     count_launch();
     return e;
@@ -325,7 +314,7 @@ cudaError_t launch_short(int rounds, const __half* x, const uint8_t* p, const ui
                          int64_t K, cudaStream_t stream) {
     if constexpr (U > 1)
         if (rounds < U) return launch_short<ENC, FULL, NT, U - 1>(rounds, x, p, r, y, M, N, K, stream);
-    return launch_one<ENC, FULL, NT, U, true, false>(x, p, r, y, M, N, K, stream);
+    return launch_one<ENC, FULL, NT, U, true>(x, p, r, y, M, N, K, stream);
 }
 
 template <int ENC, bool FULL, int NT>
@@ -341,14 +330,13 @@ cudaError_t launch_tokens(const __half* x, const uint8_t* p, const uint8_t* r, _
     // batch cost a DRAM latency.  Four linears in turn, us before / after: hidden 1024, 8 tokens, fast mode 12.2 / 11.3, full mode
     // (4 tokens) 15.3 / 13.7; 2048, 2 tokens, fast mode 19.0 / 17.6; 3088, 1 token, fast mode 30.8 / 29.1.  (The same with several
     // even batches instead of full ones and a leftover lost up to 15 % on longer K.)
-    // Half-height blocks were measured slower for every Llama-7B shape (the kernel is bound by
-    // instruction issue, and they double the MMA and activation-load instructions per weight), so
-    // they stay off.
+    // Blocks of 8 rows instead of 16 were measured slower for every Llama-7B shape (the kernel is bound by instruction
+    // issue, and they double the MMA and activation-load instructions per weight).
     constexpr int kMost = FULL ? 4 : 8;
     const int64_t full_rounds = K / kRoundK;
     if (full_rounds > 0 && full_rounds < kMost)
         return launch_short<ENC, FULL, NT, kMost - 1>((int)full_rounds, x, p, r, y, M, N, K, stream);
-    return launch_one<ENC, FULL, NT, kMost, false, false>(x, p, r, y, M, N, K, stream);
+    return launch_one<ENC, FULL, NT, kMost, false>(x, p, r, y, M, N, K, stream);
 }
 
 template <int ENC, bool FULL>

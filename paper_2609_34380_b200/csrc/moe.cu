@@ -3,8 +3,8 @@
 // asymmetric switching" -- GroupedGEMM kernels with nested reconstruction serve MoE models.
 //
 // Steps, all enqueued on the caller's stream without synchronising:
-//   1. route   (one CTA): validate rows, count rows per expert, group row ids by expert in
-//               ascending row order (stable, no atomics), and cut every group into token tiles.
+//   1. route   (one CTA): validate rows, count rows per expert (integer atomics), group row ids by
+//               expert in ascending row order (stable), and cut every group into token tiles.
 //   2. gather  : x_sorted[i][:] = x[token(sorted_rows[i])][:], so that each expert's activations
 //               are one contiguous matrix a TMA tile load can address.
 //   3. grouped tensor-core kernel over (weight-row tile, token tile): every expert's planes are

@@ -238,7 +238,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             for (int u = 0; u < steps_k && ok; ++u, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
                 ok = mbar_wait(smem_u32(&bar_p_empty[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                                if (!ok) break;
+                if (!ok) break;
                 if (elect_one()) {
                     const uint32_t full = smem_u32(&bar_p_full[s]), dst = smem_base + (uint32_t)(s * kUnit);
                     mbar_arrive_expect_tx(full, (uint32_t)kUnit);
@@ -297,7 +297,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             if (use > 0) {   // the tile before must have been read out of the accumulator by both CTAs
                 ok = mbar_wait(smem_u32(&bar_d_empty[acc]), (uint32_t)(use - 1) & 1u);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                                if (!ok) break;
+                if (!ok) break;
                 tc_fence_after_sync();
             }
             for (int j = 0; j < steps_k && ok; ++j, ++t) {
@@ -307,7 +307,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 const bool second = (step0 + j) * kUnitK + 64 < prm.K;        // (behind the end of K both operands are zero)
                 ok = mbar_wait(smem_u32(&bar_a_full[a]), (t / kASteps) & 1u);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                                if (!ok) break;
+                if (!ok) break;
                 tc_fence_after_sync();
                 if (elect_one()) {
 #pragma unroll
@@ -338,7 +338,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 if ((int)(t & 1u) != set) continue;             // (an even number of units: a unit's readers are always the same)
                 ok = mbar_wait(smem_u32(&bar_p_full[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                                if (!ok) break;
+                if (!ok) break;
                 const uint32_t prow = smem_base + s * kUnit + (uint32_t)(row * kUnitK);
                 uint32_t h[32];
                 if constexpr (!GROUPED) {
@@ -355,7 +355,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 const uint32_t a = t % kASteps;
                 if (t >= kASteps) ok = wait_done(t - kASteps);  // the MMAs that read the slot before
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                                if (!ok) break;
+                if (!ok) break;
                 tc_fence_after_sync();
                 tmem_st_32x32b_x32(tmem_a + lane_base + a * kACols + (uint32_t)(half * 32), h);
                 tmem_wait_st();
@@ -376,7 +376,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             const int acc = accs == 2 ? i & 1 : 0, use = accs == 2 ? i >> 1 : i;
             ok = mbar_wait(smem_u32(&bar_d_full[acc]), (uint32_t)use & 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
-                        if (!ok) break;
+            if (!ok) break;
             tc_fence_after_sync();
             const uint32_t tmem_d = tmem_base + lane_base + (uint32_t)(acc * prm.tokens);
             if (split > 1) {

@@ -96,13 +96,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
-                                            int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-        : "memory");
-}
 
 // Prefetch of a 2-D tile into L2 only (no shared-memory destination, no completion to wait for).
 __device__ __forceinline__ void tma_prefetch_l2_2d(const CUtensorMap* map, int c0, int c1) {
@@ -111,8 +104,7 @@ __device__ __forceinline__ void tma_prefetch_l2_2d(const CUtensorMap* map, int c
                  : "memory");
 }
 
-// ---- tensor memory -------------------------------------------------------------------------
-// CTA pair (cluster of two, cta_group::2): the load's bytes are counted on an mbarrier that may be the other CTA's;
+// CTA pair (cta_group::2): the load's bytes are counted on an mbarrier that may be the other CTA's;
 // `bar` is a shared::cluster address (map_to_cta), dst this CTA's own shared memory.  No multicast.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
     asm volatile(
@@ -121,6 +113,7 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+// ---- tensor memory -------------------------------------------------------------------------
 // Executed by one full warp.  ncols: power of two in [32, 512].
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
@@ -217,9 +210,8 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
                  : "memory");
 }
 
-// The pair's version, issued by one thread of the pair's first CTA: arrives on the barrier at this offset in BOTH CTAs
-// once every MMA issued so far by this thread has completed in both.
-// `first`: the cluster rank of the pair's first CTA.
+// The pair's version, issued by one thread of the pair's first CTA (cluster rank `first`): arrives on the barrier at this
+// offset in BOTH CTAs once every MMA issued so far by this thread has completed in both.
 __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t first = 0) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
@@ -231,11 +223,6 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t first = 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_nctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return r;
 }
 __device__ __forceinline__ void cluster_sync_all() {
@@ -250,19 +237,10 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
 __device__ __forceinline__ void st_cluster_v4_f32(uint32_t addr, float4 v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                  : "memory");
 }
-__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ float4 ld_cluster_v4_f32(uint32_t addr) {
     float4 v;
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -273,9 +251,6 @@ __device__ __forceinline__ float4 ld_cluster_v4_f32(uint32_t addr) {
 }
 
 // ---- programmatic dependent launch ---------------------------------------------------------------
-// launch_dependents: the next kernel in the stream (if launched with programmatic stream
-// serialization) may begin once every CTA of this grid has executed this or exited.
-// wait: blocks until the preceding grid has completed and its memory operations are visible.
 // Ask for one line of global memory to be brought into L2.  L2 is the point of coherence for this
 // GPU's own writes, so a line requested before an earlier kernel has finished writing it is still
 // read correctly afterwards.
@@ -287,6 +262,9 @@ __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+// launch_dependents: the next kernel in the stream (if launched with programmatic stream
+// serialization) may begin once every CTA of this grid has executed this or exited.
+// wait: blocks until the preceding grid has completed and its memory operations are visible.
 __device__ __forceinline__ void grid_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

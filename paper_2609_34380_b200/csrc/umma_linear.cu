@@ -187,9 +187,6 @@ struct UmmaParams {
     int red_offset;  // byte offset (from the aligned base of dynamic smem) of the split-K mailbox
     int x_offset;    // byte offset of the activation slots (tiles whose activations do not ride in the stages)
     int x_slots;     // activation slots (tiles that keep the activations apart from the plane ring)
-    int pair_min;    // ring depth from which stages are filled two at a time
-    int tail_parts;  // persistent dense launches: the tiles of the last, partial round are cut into this many
-                     // token ranges (1, 2 or 4), each a work item of its own
     int* status;
 #ifdef DPS_TRACE
     int trace_slot;  // which half of the CTA time table this launch writes
@@ -209,20 +206,13 @@ struct ZipCtx {
     uint64_t *bar_full, *bar_empty, *bar_a_full, *bar_a_empty;
 };
 
-// Ring position of a zip warp; carried from tile to tile by the persistent kernel.
-struct ZipState {
-    int s = 0;                // stage of the next K block
-    uint32_t s_parity = 0;    // phase parity of that stage
-    int cnt = 0;              // K blocks this warp's group has rebuilt so far
-};
-
 // Zip loop of one warp: for each of its K blocks, wait for the planes to land and for the A slot
 // to be free, rebuild 128 FP16 weights of this thread's row from the plane bytes and store them
 // into tensor memory.  Returns false if a wait timed out.
 //
 // EARLY: the stage holds planes only, so it is handed back as soon as this warp has it in registers.
 template <int ENC, bool FULL, int TN, bool EARLY = false>
-__device__ __forceinline__ bool zip_blocks(const ZipCtx& z, ZipState& st) {
+__device__ __forceinline__ bool zip_blocks(const ZipCtx& z) {
     constexpr int kBlockK = block_k(FULL, TN);
     constexpr int kACols = kBlockK / 2;
     constexpr int kPlaneStageBytes = plane_stage_bytes(FULL, TN);
@@ -234,11 +224,10 @@ __device__ __forceinline__ bool zip_blocks(const ZipCtx& z, ZipState& st) {
     // it uses in turn.
     constexpr int kTotalSlots = a_slots_max(FULL, TN);
     const int my_slots = (kTotalSlots - z.group + 1) / 2;   // 1 or 2
-    int s = st.s;
-    uint32_t s_parity = st.s_parity;   // phase parity of stage s
-    int cnt = st.cnt;                  // K blocks this group has rebuilt so far
-    int i = 0;
-    for (; i < z.num_kb && ok; ++i, s = (s + 1 == z.num_stages) ? 0 : s + 1, s_parity ^= (s == 0)) {
+    int s = 0;
+    uint32_t s_parity = 0;             // phase parity of stage s
+    int cnt = 0;                       // K blocks this group has rebuilt so far
+    for (int i = 0; i < z.num_kb && ok; ++i, s = (s + 1 == z.num_stages) ? 0 : s + 1, s_parity ^= (s == 0)) {
         if ((s & 1) != z.group) continue;
         const int turn = my_slots == 2 ? (cnt & 1) : 0;
         const int a = z.group + 2 * turn;
@@ -297,9 +286,6 @@ __device__ __forceinline__ bool zip_blocks(const ZipCtx& z, ZipState& st) {
         }
         if (z.warp == 2 + 4 * z.group) DPS_STAMP(8, i);
     }
-    st.s = s;
-    st.s_parity = s_parity;
-    st.cnt = cnt;
     return ok;
 }
 
@@ -430,8 +416,6 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     bool ok = true;
     if (warp == 0) {
         // ---------------- TMA producer (whole warp converged, one elected lane issues) ----------------
-        // Optionally (tuning knob, off by default) stages are filled two at a time.
-        const bool pair = (num_stages >= prm.pair_min) && (num_stages % 2 == 0);
         // First pass over the ring.  The planes are model state: (dense launches) their loads are
         // issued BEFORE the dependency wait, so that the ring fills while the preceding kernel
         // drains; only the activations -- that kernel's output in a decoder -- wait for it.  A
@@ -494,12 +478,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         int s = first == num_stages ? 0 : first;
         uint32_t ph = first == num_stages ? 1u : 0u;
         for (int i = first; !kXS && i < num_kb && ok; ++i, s = (s + 1 == num_stages) ? 0 : s + 1, ph ^= (s == 0)) {
-            if (!pair || (i & 1) == 0) {
-                ok = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u);
-                if (ok && pair && (i & 1) == 0 && i + 1 < num_kb) {     // pairs never wrap: the ring depth is even
-                    ok = mbar_wait(smem_u32(&bar_empty[s + 1]), ph ^ 1u);
-                }
-            }
+            ok = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             DPS_STAMP(0, i);
@@ -638,16 +617,14 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         // grouped launches: the callers' row ids of the tile's tokens, fetched before the zip loop (which
         // hides the latency) rather than in front of every store of the epilogue
         if (GROUPED && (int)threadIdx.x - 64 < tile_tokens) s_rows[threadIdx.x - 64] = gp.sorted_rows[m0 + (int)threadIdx.x - 64];
-        if (GROUPED && !(ENC == kEncE4M3 || ENC == kEncE5M2)) {
+        if constexpr (GROUPED) {
             // encoding known only at run time (one per expert): uniform branch per CTA
-            ZipState zst;
             if (FULL && rounded)
-                ok = e5m2 ? zip_blocks<kEncE5M2R, FULL, TN>(zc, zst) : zip_blocks<kEncE4M3R, FULL, TN>(zc, zst);
+                ok = e5m2 ? zip_blocks<kEncE5M2R, FULL, TN>(zc) : zip_blocks<kEncE4M3R, FULL, TN>(zc);
             else
-                ok = e5m2 ? zip_blocks<kEncE5M2, FULL, TN>(zc, zst) : zip_blocks<kEncE4M3, FULL, TN>(zc, zst);
+                ok = e5m2 ? zip_blocks<kEncE5M2, FULL, TN>(zc) : zip_blocks<kEncE4M3, FULL, TN>(zc);
         } else {
-            ZipState zst;
-            ok = zip_blocks<ENC, FULL, TN, kXS>(zc, zst);
+            ok = zip_blocks<ENC, FULL, TN, kXS>(zc);
         }
         // E4M3 fast mode multiplied with 2^8 times the weights (hardware FP8 conversion)
         const float out_scale = (!FULL && !e5m2) ? 0.00390625f : 1.0f;
@@ -779,18 +756,6 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
 
 // ---- host side ---------------------------------------------------------------------------------
 
-// Tuning knob: DPS_PAIR_MIN=<depth> sets the (even) ring depth from which two stages are filled at a
-// time, so that two boxes cover 256 adjacent bytes of every weight row.  Off by default: with rings
-// of 5-7 stages it was measured equal or slower (up to 20 % on a 6-deep full-mode ring) than
-// refilling every stage as soon as it is free.
-int pair_min_depth() {
-    static const int v = [] {
-        const char* e = getenv("DPS_PAIR_MIN");
-        return e ? atoi(e) : 1000;
-    }();
-    return v;
-}
-
 // Tuning / debugging knob: DPS_FORCE_SPLIT=<1..8> pins the K split.
 int forced_split() {
     static const int v = [] {
@@ -828,21 +793,10 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     constexpr int kMailMax = (TN + kMaxSplit) * kTileRows * 4;  // mailbox, worst case
     // Ring depth for a given mailbox size: whatever fits (stage s is rebuilt by zip group s % 2, so
     // odd depths work; they just give the first group one stage more).
-    static const int deep_forced = [] {
-        const char* e = getenv("DPS_FORCE_DEEP");
-        return e ? atoi(e) : -1;
-    }();
-    // One CTA per SM with a ring twice as deep when the tiles cannot fill two CTA slots per SM anyway.
-    const bool deep = deep_forced >= 0 ? deep_forced != 0 : false;
-    const int smem_total = deep ? 216 * 1024 : kSmemTotal;
-    static const int max_stages = [] {   // DPS_MAX_STAGES=<n>: tuning knob, caps the ring depth
-        const char* e = getenv("DPS_MAX_STAGES");
-        return e ? atoi(e) : 8;
-    }();
     auto ring_depth = [&](int mail_bytes) {
         const int x_ring = (mail_bytes > 0 ? kXSlots : kXSlotsAlone) * kXTile;
-        int d = (smem_total - mail_bytes - x_ring) / kStage;
-        if (d > max_stages) d = max_stages;
+        int d = (kSmemTotal - mail_bytes - x_ring) / kStage;
+        if (d > 8) d = 8;
         if (d < 2) d = 2;
         return d;
     };
@@ -920,7 +874,6 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     const int total_kb = (int)((K + kBlockK - 1) / kBlockK);
     int split = forced_split();
     if (split <= 0) split = choose_split(row_tiles * tok_tiles, total_kb, capacity, FULL ? 5 : 4);
-    if (deep) split = 1;
     if (split > total_kb) split = total_kb;
     if (split > kMaxSplit) split = kMaxSplit;
     // the mailbox exists only when K is split, and then has its exact size
@@ -946,7 +899,6 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     prm.x_slots = xs_n;
     prm.red_offset = stages * kStage + x_ring;
     prm.status = status;
-    prm.pair_min = pair_min_depth();
 #ifdef DPS_TRACE
     static int trace_launches = 0;
     prm.trace_slot = (trace_launches++) & 1;
@@ -1050,7 +1002,6 @@ cudaError_t launch_grouped_tn(const uint32_t* e5m2_mask, const void* x_sorted, c
     prm.split = 1;
     prm.red_offset = 0;
     prm.status = status;
-    prm.pair_min = pair_min_depth();
     GroupedParams gp;
     gp.tiles = static_cast<const int4*>(tiles);
     gp.num_tiles = num_tiles;
