@@ -80,11 +80,15 @@ __device__ __forceinline__ void to_half_pairs(const uint4& p, const uint4& r, ui
 }
 
 // SHORT: K is U rounds and perhaps a ragged end, less than a batch of the long variant; all of it is one batch.
-// x without __restrict__: its writer may still run when a CTA starts, so it must not go through the non-coherent path.
+// x is read through the non-coherent path although its writer may still run when a CTA starts: the lines it leaves in L1 serve
+// the CTAs that follow on the SM.  A coherent load's lines do not survive the next CTA's dependency wait, and four Llama-7B
+// layers at 1 token in fast and 8 tokens in full mode took 178 and 328 us instead of 166 and 298.  A line read before x was
+// complete cannot be met here: every read comes after the wait, L1 is emptied when a grid starts on the SM, and the grid after
+// x's writer starts when the one before that writer, the last that may have read the buffer's old contents, has exited.
 template <int ENC, bool FULL, int NT, int U, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 2)
-decode_mma_kernel(const __half* x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp, __half* y, int M, int64_t N,
-                  int64_t K, int prefetch_steps, int prefetch_ctas, int trace_slot) {
+decode_mma_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ P, const uint8_t* __restrict__ Rp,
+                  __half* __restrict__ y, int M, int64_t N, int64_t K, int prefetch_steps, int prefetch_ctas, int trace_slot) {
     constexpr float kScale = (ENC == kEncE4M3 && !FULL) ? 0.00390625f : 1.0f;  // 2^-8, exact
     __shared__ float red[kWarps][kRowsPerBlock][NT * 8 + 1];
     sm100::grid_launch_dependents();
