@@ -268,11 +268,17 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     // shared memory, and an SM that changes its split drains first.  Four linears in turn at 12-13 tokens, streaming kernel
     // / tiles / the one or the other by N K < 2^25, which was the rule: hidden 3088 in full mode 57 / 46 / 98 us, 2048 in
     // fast mode 23.0 / 22.6 / 38, 4096 in full mode (16 tokens) 86 / 83 / 91; 1024 14.7 / 17.7, 512 9.3 / 13.2.  The smaller
-    // side of the matrix is the hidden size in all four, so a rule on it keeps a layer in one family.
+    // side of the matrix is the hidden size in all four, so a rule on it keeps a layer in one family.  Matrices of 2^25 weights
+    // and more with a small side, output heads, are the tiles' all the same (9 tokens, streaming kernel / tiles): 128256 x 1024
+    // by itself 45.8 / 35.0 us in fast and 60.0 / 52.3 in full mode, behind twelve layers of hidden size 1024 198 / 184 and 260 / 246
+    // for all; 57344 x 1536 behind eight layers 156 / 148 and 220 / 218.  (By itself, in full mode, 35.6 / 39.4.)
+    // What the rule costs: a matrix beyond it that is called by itself.  2048 x 2048, 9 tokens, takes 4.5 us in fast and 5.4 in
+    // full mode, the streaming kernel 3.4 and 3.9; 4096 x 4096 6.7 and 9.3 against 5.7 and 8.8.  With other programs' kernels
+    // between the linears every launch of the tiles pays for the change of split, about 2 us: 2048 x 2048 7.0 against 4.2.
     // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens CTA pairs (four Llama-7B linears, fast / full mode: 64
     // tokens 62 / 97 us with the tiles, 75 / 109 with pairs; 96 tokens 84 / 134 against 74 / 107).  (The CUDA-core GEMV
     // is kept as a cross-check.)
-    const bool stream_mid = (N < K ? N : K) <= 1536;
+    const bool stream_mid = (N < K ? N : K) <= 1536 && N * K < ((int64_t)1 << 25);
     const int path = forced_path();
     cudaError_t err;
     if (path == 1) err = launch_gemv(mode, enc, x, w_persist, r, y, M, N, K, stream);

@@ -1,4 +1,4 @@
-"""GPU: 9-16 tokens on both sides of the rule that picks the kernel family by the smaller side of the matrix (1536)."""
+"""GPU: 9-16 tokens on both sides of the rule that picks the kernel family: the smaller side of the matrix (1536) and its size (2^25)."""
 import pytest
 import torch
 
@@ -22,4 +22,20 @@ def test_both_families(N, K):
                 ref = oracle.linear(mode, enc, to_np_words(x), p_ref, r_ref, threads=8)
                 assert_close_to_oracle(y, ref, f"N={N} K={K} M={M} enc={enc} mode={mode}")
                 assert torch.equal(y, dps.dps_linear(mode, enc, x, p, r if mode else None))
+    assert dps.dps_stream_status() == dps.DPS_OK
+
+
+def test_wide_flat_matrices_are_the_tiles(monkeypatch, capfd):
+    """Just below and just above 2^25 weights with a side of 256: the tiles print a launch line, the streaming kernel does not."""
+    monkeypatch.setenv("DPS_DEBUG", "1")
+    K, M = 256, 9
+    for N, tiles in ((131064, False), (131072, True)):
+        p, r, enc, p_ref, r_ref = split_both(workloads.weights(N, K, 63, device=DEV), dps.DPS_ENC_AUTO, DEV)
+        x = workloads.activations(M, K, 64, device=DEV)
+        for mode in (dps.DPS_MODE_FAST, dps.DPS_MODE_FULL):
+            capfd.readouterr()
+            y = dps.dps_linear(mode, enc, x, p, r)
+            assert ("[dps] umma " in capfd.readouterr().err) == tiles
+            ref = oracle.linear(mode, enc, to_np_words(x), p_ref, r_ref, threads=8)
+            assert_close_to_oracle(y, ref, f"N={N} mode={mode}")
     assert dps.dps_stream_status() == dps.DPS_OK
