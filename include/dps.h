@@ -27,7 +27,8 @@
  *     be written by the kernel launched immediately before dps_linear / dps_moe_linear
  *     on the same stream.  Planes written by dps_split_weights, by a copy
  *     (cudaMemcpyAsync) or by any kernel further back in the stream are safe:
- *     dps_split_weights ends with a fence launch for exactly this reason.
+ *     dps_split_weights has either finished when it returns (AUTO answering E4M3) or
+ *     ends with a fence launch, for exactly this reason.
  *   - Pointers are DEVICE pointers unless a parameter says "host".  The caller owns
  *     every buffer; the library never allocates or frees device memory.
  *   - cuda_stream is a cudaStream_t passed as void* (NULL = the default stream).  Work
@@ -102,9 +103,11 @@ typedef enum {
  * w_fp16: device, rows*cols FP16 words.  w_persist, w_resid: device, rows*cols bytes each.
  * enc_inout: HOST int32.  On entry DPS_ENC_AUTO, DPS_ENC_AUTO_RN or one of the four encodings; on return
  * the encoding that was used.
- *   AUTO  -> E4M3 iff every word has b[14] == 0 and max|w| <= 1.75, else E5M2.  The
- *            statistics pass needs its result on the host, so this variant SYNCHRONISES
- *            the stream (splitting is load-time work).
+ *   AUTO  -> E4M3 iff every word has b[14] == 0 and max|w| <= 1.75, else E5M2.  The tensor
+ *            is split as E4M3 and looked over in one pass, and split again as E5M2 if a word
+ *            is out of range.  The host has to learn which, so this variant SYNCHRONISES the
+ *            stream (splitting is load-time work).  The first such call on a device keeps one
+ *            page-locked host word; make it outside any stream capture.
  *   E4M3  -> also synchronises: the tensor is checked first, and if any word has b[14] set
  *            or would produce the byte 0x7F/0xFF the call returns DPS_ERR_DATA with both
  *            planes untouched.
