@@ -232,6 +232,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     Work w;
     if (warp == 0) {
         // ---------------- plane producer (model state: does not wait for the preceding kernel) ----------------
+        // Four Llama-7B linears in a chain, fast / full mode, against a producer that waits first: 72 tokens 74.1 / 105 us
+        // against 75.6 / 109, 128 tokens 82.0 / 111.8 against 82.3 / 113.7, 512 tokens 167.5 / 215 against 167.9 / 217.
         int s = 0;
         uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
         uint32_t issued = 0;
