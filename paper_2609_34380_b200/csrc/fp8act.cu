@@ -169,7 +169,6 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
     __shared__ __align__(8) uint64_t bar_d_full[2];
     __shared__ __align__(8) uint64_t bar_d_empty[2];        // the first CTA's count for both
     __shared__ uint32_t tmem_base_slot;
-    __shared__ uint32_t issued_stages;                      // this CTA's producer's (read after a failure)
 
     grid_launch_dependents();
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -220,7 +219,7 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
         // ---------------- TMA producer: this CTA's rows and its half of the tokens ----------------
         grid_dependency_wait();   // the activation codes come from the quantisation kernel
         int s = 0;
-        uint32_t ph = 0, issued = 0;
+        uint32_t ph = 0;
         const uint32_t half_tokens = (uint32_t)tokens / 2;
         const uint32_t pair_bytes = 2u * (kRows + half_tokens) * kBlockBytes;
         for (int lin = pair; lin < total && ok; lin += pairs) {
@@ -240,10 +239,8 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
                     tma_load_2d_pair(dst + kRows * kBlockBytes, &map_x, full, i * kBlockBytes, m0);
                 }
                 __syncwarp();
-                ++issued;
             }
         }
-        issued_stages = issued;
     } else if (warp == 1) {
         // ---------------- MMA issuer: the pair's first CTA ----------------
         const uint32_t idesc = idesc_f8(2 * kRows, tokens, prm.e5m2 ? 1 : 0, 0);
@@ -335,8 +332,7 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
     }
     if (!ok) atomicExch(prm.status, (int)DPS_ERR_CUDA);
     tc_fence_before_sync();
-    // (the first CTA's barriers count both CTAs' bytes; the second CTA leaves with it)
-    if (__syncthreads_or(!ok) && warp == 0 && rank == 0) drain_copies(bar_full, issued_stages, kStages);
+    __syncthreads();
     cluster_sync_all();           // nobody frees tensor memory or leaves while the pair still works
     if (warp == 1) {
         tc_fence_after_sync();

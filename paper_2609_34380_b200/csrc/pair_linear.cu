@@ -133,7 +133,6 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     __shared__ __align__(8) uint64_t bar_d_full[2];
     __shared__ __align__(8) uint64_t bar_d_empty[2];            // the first CTA's count for both
     __shared__ uint32_t tmem_base_slot;
-    __shared__ uint32_t issued_units, issued_x;                 // copies of this CTA's producers (read after a failure)
 
     grid_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -236,7 +235,6 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         // against 75.6 / 109, 128 tokens 82.0 / 111.8 against 82.3 / 113.7, 512 tokens 167.5 / 215 against 167.9 / 217.
         int s = 0;
         uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
-        uint32_t issued = 0;
         for (int i = 0; ok && work(i, w); ++i) {
             const int row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
             for (int u = 0; u < steps_k && ok; ++u, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
@@ -250,10 +248,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                     if (FULL) tma_load_2d(dst + kRows * kUnitK, &map_r, full, (step0 + u) * kUnitK, row);
                 }
                 __syncwarp();
-                ++issued;
             }
         }
-        issued_units = issued;
     } else if (warp == 2) {
         // ---------------- activation producer: this CTA's half of the tokens ----------------
         grid_dependency_wait();
@@ -280,7 +276,6 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 __syncwarp();
             }
         }
-        issued_x = t;
     } else if (warp == 3) {
         // ---------------- reports the activations of a K step, both halves: the pair's first CTA ----------------
         int s = 0;
@@ -466,11 +461,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         }
     }
     tc_fence_before_sync();
-    if (__syncthreads_or(!ok)) {
-        if (warp == 0) drain_copies(bar_p_full, issued_units, (uint32_t)units);
-        // (the first CTA's barriers count both CTAs' activations; the second CTA leaves with it)
-        if (warp == 2 && rank == 0) drain_copies(bar_x_full, issued_x, (uint32_t)x_slots);
-    }
+    __syncthreads();
     cluster_sync_all();           // nobody frees tensor memory or leaves while the pair still works
     if (warp == 1) {
         tc_fence_after_sync();

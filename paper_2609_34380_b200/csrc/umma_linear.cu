@@ -316,7 +316,6 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     __shared__ __align__(8) uint64_t bar_x_empty[kMaxXSlots];
     __shared__ __align__(8) uint64_t bar_dep;
     __shared__ uint32_t tmem_base_slot;
-    __shared__ uint32_t issued_stages, issued_x;   // the producer's copies (read after a failure)
     __shared__ int s_rows[GROUPED ? TN : 1];   // grouped launches: row ids of the tile's tokens
 
     grid_launch_dependents();  // the next kernel's prologue may overlap this kernel's tail
@@ -478,7 +477,6 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         // activations of K block i).
         int s = first == num_stages ? 0 : first;
         uint32_t ph = first == num_stages ? 1u : 0u;
-        int issued = first;
         for (int i = first; !kXS && i < num_kb && ok; ++i, s = (s + 1 == num_stages) ? 0 : s + 1, ph ^= (s == 0)) {
             ok = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
@@ -489,9 +487,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 load_x(i, s);
             }
             __syncwarp();
-            ++issued;
         }
-        if (!kXS) issued_stages = (uint32_t)issued;
         // Steady state with activation slots: two streams with different consumers.  A plane stage is free as
         // soon as its zip group holds it in registers; an activation slot is free when the MMAs that read it
         // are complete, several K blocks later.  One loop serves both by PROBING (test_wait never suspends)
@@ -539,8 +535,6 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                     else if (now - t0 > kWaitLimitNs) ok = false;
                 }
             }
-            issued_stages = (uint32_t)ip;
-            issued_x = (uint32_t)ix;
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (whole warp converged, one elected lane issues) ----------------
@@ -752,10 +746,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     }
     DPS_CTA_STAMP(6);
     tc_fence_before_sync();
-    if (__syncthreads_or(!ok) && warp == 0) {
-        drain_copies(bar_full, issued_stages, (uint32_t)num_stages);
-        if (kXS) drain_copies(bar_x_full, issued_x, (uint32_t)xs_n);
-    }
+    __syncthreads();
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, kCols);
