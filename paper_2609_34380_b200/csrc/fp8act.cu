@@ -219,7 +219,7 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
         // ---------------- TMA producer: this CTA's rows and its half of the tokens ----------------
         grid_dependency_wait();   // the activation codes come from the quantisation kernel
         int s = 0;
-        uint32_t ph = 0;
+        uint32_t ph = 0, issued = 0;
         const uint32_t half_tokens = (uint32_t)tokens / 2;
         const uint32_t pair_bytes = 2u * (kRows + half_tokens) * kBlockBytes;
         for (int lin = pair; lin < total && ok; lin += pairs) {
@@ -239,8 +239,11 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
                     tma_load_2d_pair(dst + kRows * kBlockBytes, &map_x, full, i * kBlockBytes, m0);
                 }
                 __syncwarp();
+                ++issued;
             }
         }
+        // (the first CTA's barriers count both CTAs' bytes, the second CTA leaves with it)
+        if (rank == 0) drain_copies(bar_full, issued, kStages);
     } else if (warp == 1) {
         // ---------------- MMA issuer: the pair's first CTA ----------------
         const uint32_t idesc = idesc_f8(2 * kRows, tokens, prm.e5m2 ? 1 : 0, 0);

@@ -235,6 +235,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         // against 75.6 / 109, 128 tokens 82.0 / 111.8 against 82.3 / 113.7, 512 tokens 167.5 / 215 against 167.9 / 217.
         int s = 0;
         uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
+        uint32_t issued = 0;
         for (int i = 0; ok && work(i, w); ++i) {
             const int row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
             for (int u = 0; u < steps_k && ok; ++u, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
@@ -248,8 +249,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                     if (FULL) tma_load_2d(dst + kRows * kUnitK, &map_r, full, (step0 + u) * kUnitK, row);
                 }
                 __syncwarp();
+                ++issued;
             }
         }
+        drain_copies(bar_p_full, issued, (uint32_t)units);
     } else if (warp == 2) {
         // ---------------- activation producer: this CTA's half of the tokens ----------------
         grid_dependency_wait();
@@ -276,6 +279,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 __syncwarp();
             }
         }
+        // (t: steps issued; the first CTA's barriers count both CTAs' bytes, the second CTA leaves with it)
+        if (rank == 0) drain_copies(bar_x_full, t, (uint32_t)x_slots);
     } else if (warp == 3) {
         // ---------------- reports the activations of a K step, both halves: the pair's first CTA ----------------
         int s = 0;

@@ -477,6 +477,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         // activations of K block i).
         int s = first == num_stages ? 0 : first;
         uint32_t ph = first == num_stages ? 1u : 0u;
+        int issued = first;
         for (int i = first; !kXS && i < num_kb && ok; ++i, s = (s + 1 == num_stages) ? 0 : s + 1, ph ^= (s == 0)) {
             ok = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u);
             ok = __all_sync(0xFFFFFFFFu, ok);
@@ -487,7 +488,9 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 load_x(i, s);
             }
             __syncwarp();
+            ++issued;
         }
+        if (!kXS) drain_copies(bar_full, (uint32_t)issued, (uint32_t)num_stages);
         // Steady state with activation slots: two streams with different consumers.  A plane stage is free as
         // soon as its zip group holds it in registers; an activation slot is free when the MMAs that read it
         // are complete, several K blocks later.  One loop serves both by PROBING (test_wait never suspends)
@@ -535,6 +538,8 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                     else if (now - t0 > kWaitLimitNs) ok = false;
                 }
             }
+            drain_copies(bar_full, (uint32_t)ip, (uint32_t)num_stages);
+            drain_copies(bar_x_full, (uint32_t)ix, (uint32_t)xs_n);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (whole warp converged, one elected lane issues) ----------------
