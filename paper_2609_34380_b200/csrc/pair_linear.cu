@@ -63,6 +63,9 @@ struct PairParams {
     int tail_parts;    // pieces such a tile is cut into (1: not cut)
     int units, x_slots;
     int split;         // K split: pairs of a cluster that share a tile, each a range of its K steps (then one tile per cluster)
+    // What every warp would have to divide for in front of the first load: pairs in the grid (with a split, clusters), row tiles,
+    // (not grouped) token tiles and the tiles of whole rounds, and the K steps' quotient and remainder by the split.
+    int pairs, row_tiles, tok_tiles, t_main, steps_each, steps_over;
     int* status;
 };
 
@@ -140,20 +143,18 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     const int split = prm.split;
     const uint32_t first = cluster_ctarank() & ~1u;             // cluster rank of the pair's first CTA
     const int rank = (int)(cluster_ctarank() & 1u), ks = (int)(first >> 1);
-    const int pair = (int)blockIdx.x / (2 * split), pairs = (int)gridDim.x / (2 * split);   // (split > 1: the cluster)
+    const int pair = (int)cluster_id(), pairs = prm.pairs;      // (split > 1: the cluster)
     const int units = prm.units, x_slots = prm.x_slots;
     const int x_atom = prm.tokens / 2 * 128, x_bytes = 2 * x_atom;   // 64 columns of K; a slot, 128
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t x_base = smem_base + (uint32_t)(units * kUnit);
     const uint32_t epi_base = x_base + (uint32_t)(x_slots * x_bytes);
-    const int row_tiles = (prm.N + 2 * kRows - 1) / (2 * kRows);
+    const int row_tiles = prm.row_tiles;
     if (GROUPED) grid_dependency_wait();                        // the tile list comes from the routing pre-pass
-    const int tok_tiles = GROUPED ? *gp.num_tiles : (prm.M + prm.tokens - 1) / prm.tokens;
-    const int total = row_tiles * tok_tiles;
-    const int t_main = prm.tail_parts > 1 ? total - total % pairs : total;
-    const int all_steps = (prm.K + kUnitK - 1) / kUnitK;        // K steps of a tile ...
-    const int step0 = all_steps * ks / split;                   // ... and this pair's of them
-    const int steps_k = all_steps * (ks + 1) / split - step0;
+    const int tok_tiles = GROUPED ? *gp.num_tiles : prm.tok_tiles;
+    const int total = row_tiles * tok_tiles, t_main = GROUPED ? total : prm.t_main;
+    const int step0 = ks * prm.steps_each + min(ks, prm.steps_over);      // this pair's K steps of a tile
+    const int steps_k = prm.steps_each + (ks < prm.steps_over ? 1 : 0);
 
     // Work item `i` of this pair: whole tiles, then at most one piece of a tile of the last round.
     auto work = [&](int i, Work& w) -> bool {
@@ -197,11 +198,35 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         return w.ncols > 0;      // a piece past the last token is the end: nothing follows a piece
     };
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < units; ++s) {
-            mbar_init(smem_u32(&bar_p_full[s]), 1);
-            mbar_init(smem_u32(&bar_p_empty[s]), 8);            // the zip warps that take the step
+    auto load_unit = [&](int s, int step, int row) {            // by one thread
+        const uint32_t full = smem_u32(&bar_p_full[s]), dst = smem_base + (uint32_t)(s * kUnit);
+        mbar_arrive_expect_tx(full, (uint32_t)kUnit);
+        tma_load_2d(dst, &map_p, full, step * kUnitK, row);
+        if (FULL) tma_load_2d(dst + kRows * kUnitK, &map_r, full, step * kUnitK, row);
+    };
+    Work w;
+    int loaded = 0;               // units loaded ahead of the roles (by warp 0)
+    if (warp == 0) {
+        if (lane == 0) {
+            for (int s = 0; s < units; ++s) {
+                mbar_init(smem_u32(&bar_p_full[s]), 1);
+                mbar_init(smem_u32(&bar_p_empty[s]), 8);            // the zip warps that take the step
+            }
+            fence_barrier_init();
+            fence_async_proxy();
         }
+        __syncwarp();
+        // The planes are model state, and their barriers this CTA's own: the ring fills while tensor memory is allocated and the
+        // pair meets.  With the divisions left to the host, four linears in a chain, fast / full mode: Llama-7B 64
+        // tokens 67.6 / 98.8 -> 65.1 / 95.5 us, 128 80.3 / 108.5 -> 76.5 / 104.9, 256 103.3 / 139.8 -> 100.8 / 138; 2048-wide layers, 128
+        // tokens, 42.1 / 49.3 -> 40.7 / 46.9 (the split's sum, 1-3 % of launches that have one, is in these).
+        if (work(0, w)) {
+            loaded = min(units, steps_k);
+            if (elect_one())
+                for (int s = 0; s < loaded; ++s) load_unit(s, step0 + s, w.plane_row0 + (2 * w.row_tile + rank) * kRows);
+            __syncwarp();
+        }
+    } else if (warp == 2 && lane == 0) {
         for (int s = 0; s < x_slots; ++s) mbar_init(smem_u32(&bar_x_full[s]), 1);
         for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 8 + 1);   // both CTAs' eight zip warps, warp 3
         for (int a = 0; a < kDone; ++a) mbar_init(smem_u32(&bar_done[a]), 1);
@@ -210,8 +235,6 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             mbar_init(smem_u32(&bar_d_empty[a]), 8);            // the epilogue warps of both CTAs
         }
         fence_barrier_init();
-        prefetch_tensormap(&map_p);
-        if (FULL) prefetch_tensormap(&map_r);
         prefetch_tensormap(&map_x);
     }
     if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_slot), 512);
@@ -229,7 +252,6 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     auto wait_done = [&](uint32_t t) { return mbar_wait(smem_u32(&bar_done[t % kDone]), (t / kDone) & 1u); };
 
     bool ok = true;
-    Work w;
     if (warp == 0) {
         // ---------------- plane producer (model state: does not wait for the preceding kernel) ----------------
         // Four Llama-7B linears in a chain, fast / full mode, against a producer that waits first: 72 tokens 74.1 / 105 us
@@ -239,18 +261,13 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         uint32_t issued = 0;
         for (int i = 0; ok && work(i, w); ++i) {
             const int row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
-            for (int u = 0; u < steps_k && ok; ++u, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
+            for (int u = 0; u < steps_k && ok; ++u, ++issued, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
+                if (issued < (uint32_t)loaded) continue;
                 ok = mbar_wait(smem_u32(&bar_p_empty[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                if (elect_one()) {
-                    const uint32_t full = smem_u32(&bar_p_full[s]), dst = smem_base + (uint32_t)(s * kUnit);
-                    mbar_arrive_expect_tx(full, (uint32_t)kUnit);
-                    tma_load_2d(dst, &map_p, full, (step0 + u) * kUnitK, row);
-                    if (FULL) tma_load_2d(dst + kRows * kUnitK, &map_r, full, (step0 + u) * kUnitK, row);
-                }
+                if (elect_one()) load_unit(s, step0 + u, row);
                 __syncwarp();
-                ++issued;
             }
         }
         drain_copies(bar_p_full, issued, (uint32_t)units);
@@ -313,8 +330,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 const uint64_t bdesc0 = umma_desc_k_sw128(x_base + (uint32_t)(xs * x_bytes));
                 const uint64_t bdesc1 = bdesc0 + (uint64_t)(x_atom >> 4);
                 const bool second = (step0 + j) * kUnitK + 64 < prm.K;        // (behind the end of K both operands are zero)
-                ok = mbar_wait(smem_u32(&bar_a_full[a]), (t / kASteps) & 1u);
-                ok = __all_sync(0xFFFFFFFFu, ok);
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bar_a_full[a]), (t / kASteps) & 1u));
                 if (!ok) break;
                 tc_fence_after_sync();
                 if (elect_one()) {
@@ -340,12 +356,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         const int row = (warp & 3) * 32 + lane;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t sw = (uint32_t)(row & 7);                // TMA swizzle: 16-byte chunk index ^= row % 8
-        uint32_t s = 0, ph = 0, t = 0;
+        // t: the step; s, ph: its unit (an even number of units: a unit's readers are always the same)
+        uint32_t s = (uint32_t)set, ph = 0, t = (uint32_t)set, done = 0;
         for (int i = 0; ok && work(i, w); ++i) {
-            for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == (uint32_t)units) ? 0 : s + 1, ph ^= (s == 0)) {
-                if ((int)(t & 1u) != set) continue;             // (an even number of units: a unit's readers are always the same)
-                ok = mbar_wait(smem_u32(&bar_p_full[s]), ph);
-                ok = __all_sync(0xFFFFFFFFu, ok);
+            done += (uint32_t)steps_k;                          // steps up to the end of this tile
+            for (; t < done; t += 2) {
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bar_p_full[s]), ph));
                 if (!ok) break;
                 const uint32_t prow = smem_base + s * kUnit + (uint32_t)(row * kUnitK);
                 uint32_t h[32];
@@ -360,9 +376,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_p_empty[s]));
+                s += 2;
+                if (s >= (uint32_t)units) s -= (uint32_t)units, ph ^= 1u;
                 const uint32_t a = t % kASteps;
-                if (t >= kASteps) ok = wait_done(t - kASteps);  // the MMAs that read the slot before
-                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (t >= kASteps) ok = __all_sync(0xFFFFFFFFu, wait_done(t - kASteps));  // the MMAs that read the slot before
                 if (!ok) break;
                 tc_fence_after_sync();
                 tmem_st_32x32b_x32(tmem_a + lane_base + a * kACols + (uint32_t)(half * 32), h);
@@ -563,13 +580,21 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     const Rings rings = size_rings(FULL, plan.tokens);
     prm.units = rings.units;
     prm.x_slots = rings.x_slots;
-    const int64_t tiles = ((N + 2 * kRows - 1) / (2 * kRows)) * ((M + plan.tokens - 1) / plan.tokens);
+    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
+    const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
+    const int64_t steps = (K + kUnitK - 1) / kUnitK;
+    prm.pairs = (int)grid_pairs;
+    prm.row_tiles = (int)row_tiles;
+    prm.tok_tiles = (int)tok_tiles;
+    prm.t_main = (int)(plan.tail_parts > 1 ? tiles - tiles % grid_pairs : tiles);
+    prm.steps_each = (int)(steps / plan.split);
+    prm.steps_over = (int)(steps % plan.split);
     if (getenv("DPS_DEBUG"))
         fprintf(stderr, "[dps] pair full=%d M=%lld N=%lld K=%lld tokens=%d tiles=%lld tail=%dx%d split=%d (%d %d %d %d) units=%d x_slots=%d\n", (int)FULL,
                 (long long)M, (long long)N, (long long)K, plan.tokens, (long long)tiles, plan.tail_parts, plan.tail_tokens,
                 plan.split, capacity_of[dev][1], capacity_of[dev][2], capacity_of[dev][3], capacity_of[dev][4], prm.units, prm.x_slots);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(plan.split > 1 ? 2 * plan.split * tiles : 2 * (tiles < pairs ? tiles : pairs)), 1, 1);
+    cfg.gridDim = dim3((unsigned)(2 * plan.split * grid_pairs), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
@@ -632,12 +657,16 @@ cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const ui
         gp.e5m2[i] = masks[i];
         gp.rounded[i] = FULL ? masks[32 + i] : 0u;
     }
-    const int64_t upper = ((N + 2 * kRows - 1) / (2 * kRows)) * max_tiles, pairs = sm_count() / 2;
+    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), upper = row_tiles * max_tiles;
+    const int64_t pairs = upper < sm_count() / 2 ? upper : sm_count() / 2;
+    prm.pairs = (int)pairs;
+    prm.row_tiles = (int)row_tiles;
+    prm.steps_each = (int)((K + kUnitK - 1) / kUnitK);
     if (getenv("DPS_DEBUG"))
         fprintf(stderr, "[dps] pair grouped full=%d A=%lld N=%lld K=%lld E=%d tokens=%d tiles<=%lld units=%d x_slots=%d\n", (int)FULL,
                 (long long)A, (long long)N, (long long)K, (int)E, tn, (long long)upper, prm.units, prm.x_slots);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * (upper < pairs ? upper : pairs)), 1, 1);
+    cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
