@@ -62,6 +62,7 @@ struct PairParams {
     int tail_tokens;   // per piece of a tile of the last, partial round
     int tail_parts;    // pieces such a tile is cut into (1: not cut)
     int units, x_slots;
+    int ahead;         // plane units asked of L2 in front of their loads
     int split;         // K split: pairs of a cluster that share a tile, each a range of its K steps (then one tile per cluster)
     // What every warp would have to divide for in front of the first load: pairs in the grid (with a split, clusters), row tiles,
     // (not grouped) token tiles and the tiles of whole rounds, and the K steps' quotient and remainder by the split.
@@ -204,6 +205,11 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         tma_load_2d(dst, &map_p, full, step * kUnitK, row);
         if (FULL) tma_load_2d(dst + kRows * kUnitK, &map_r, full, step * kUnitK, row);
     };
+    auto ask = [&](int step, int row) {                         // the same unit into L2 only
+        tma_prefetch_l2_2d(&map_p, step * kUnitK, row);
+        if (FULL) tma_prefetch_l2_2d(&map_r, step * kUnitK, row);
+    };
+    const int ahead = FULL ? prm.ahead : 0;
     Work w;
     int loaded = 0;               // units loaded ahead of the roles (by warp 0)
     if (warp == 0) {
@@ -222,8 +228,11 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         // tokens, 42.1 / 49.3 -> 40.7 / 46.9 (the split's sum, 1-3 % of launches that have one, is in these).
         if (work(0, w)) {
             loaded = min(units, steps_k);
-            if (elect_one())
-                for (int s = 0; s < loaded; ++s) load_unit(s, step0 + s, w.plane_row0 + (2 * w.row_tile + rank) * kRows);
+            if (elect_one()) {
+                const int row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
+                for (int s = 0; s < loaded; ++s) load_unit(s, step0 + s, row);
+                for (int s = loaded; s < min(loaded + ahead, steps_k); ++s) ask(step0 + s, row);
+            }
             __syncwarp();
         }
     } else if (warp == 2 && lane == 0) {
@@ -259,14 +268,24 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         int s = 0;
         uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
         uint32_t issued = 0;
-        for (int i = 0; ok && work(i, w); ++i) {
+        bool more = work(0, w);
+        for (int i = 0; ok && more; ++i) {
             const int row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
+            more = work(i + 1, w);
+            const int next_row = w.plane_row0 + (2 * w.row_tile + rank) * kRows;
             for (int u = 0; u < steps_k && ok; ++u, ++issued, s = (s + 1 == units) ? 0 : s + 1, ph ^= (s == 0)) {
                 if (issued < (uint32_t)loaded) continue;
                 ok = mbar_wait(smem_u32(&bar_p_empty[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                if (elect_one()) load_unit(s, step0 + u, row);
+                if (elect_one()) {
+                    load_unit(s, step0 + u, row);
+                    if (ahead > 0) {
+                        const int v = u + ahead - steps_k;       // that many steps into the next tile
+                        if (v < 0) ask(step0 + u + ahead, row);
+                        else if (more && v < steps_k) ask(step0 + v, next_row);
+                    }
+                }
                 __syncwarp();
             }
         }
@@ -580,6 +599,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     const Rings rings = size_rings(FULL, plan.tokens);
     prm.units = rings.units;
     prm.x_slots = rings.x_slots;
+    prm.ahead = ahead_units(FULL, M, rings);
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
     const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
     const int64_t steps = (K + kUnitK - 1) / kUnitK;

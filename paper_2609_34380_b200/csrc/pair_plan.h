@@ -99,6 +99,14 @@ inline Rings size_rings(bool full, int tokens) {
     return {units > kMaxUnits ? kMaxUnits : units & ~1, xs};
 }
 
+// Plane units asked of L2 ahead of their loads.  A ring of two units (full mode, tiles of 192 tokens and more) has 64 KB per SM in
+// flight at best, and memory's latency takes more: the three units behind it are asked for too.  Up to 512 tokens, where every pair
+// streams planes of its own; with more token tiles several pairs read the same planes and it gained nothing.  Four linears in a
+// chain, full mode, without / with 3 / 4 / 6 units, us: Llama-7B 192 tokens 132.8 / 121.5 / 122.2 / 124.2, 256 141 / 133.9 / 134.2 /
+// 135.8, 512 222 / 216.8 / 216.7 / 217.1; 8192-wide 256 tokens 481 / 434 / 443 / 456.  Rings of four units lose by it: 12288 x 4096 at
+// 128 tokens 24.7 / - / 25.5 in full mode, 256 tokens in fast mode 26.8 / - / 27.3.
+inline int ahead_units(bool full, int64_t M, const Rings& rings) { return full && rings.units == 2 && M <= 512 ? 3 : 0; }
+
 // Token-tile width of grouped launches: an expert with a quarter, or two and a half standard deviations of an even routing,
 // more rows than the average still fits the average's number of tiles.
 inline int grouped_tokens(int64_t A, int32_t E) {
