@@ -3,6 +3,7 @@
 // asymmetric switching" -- GroupedGEMM kernels with nested reconstruction serve MoE models.
 //
 // Steps, all enqueued on the caller's stream without synchronising:
+//   (up to 1024 rows: 1 and 2 in one launch, see moe_rank_gather_kernel)
 //   1. route   (one CTA): validate rows, count rows per expert (integer atomics), group row ids by
 //               expert in ascending row order (stable), and cut every group into token tiles.
 //   2. gather  : x_sorted[i][:] = x[token(sorted_rows[i])][:], so that each expert's activations
@@ -69,27 +70,19 @@ __device__ __forceinline__ bool row_valid(const int32_t* token_of_row, const int
 // 4.7 us for 32 rows of 32 experts.  More than kTableExperts experts (the table's size): one warp per expert walks all rows.
 constexpr int kTableExperts = 256;
 
-__global__ void __launch_bounds__(kRouteThreads)
-moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E, int tile_tokens,
-                 int32_t* counts, int32_t* offsets, int32_t* sorted_rows, int32_t* num_tiles, int4* tiles, int* status) {
-    __shared__ int s_cnt[kMaxExperts];
-    __shared__ int s_off[kMaxExperts];
-    __shared__ int s_table[kRouteThreads / 32][kTableExperts];
-    // the gather and the grouped kernel may be made resident now; both wait for their predecessor
-    // (griddepcontrol.wait) before they read anything this kernel writes
-    sm100::grid_launch_dependents();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int e = tid; e < E; e += kRouteThreads) s_cnt[e] = 0;
-    __syncthreads();
-    sm100::grid_dependency_wait();      // the routing and, through an earlier call, the workspace are earlier kernels'
+// By the whole block: rows per expert (s_cnt, E entries, zero on entry), then by its first warp the first position and the
+// first tile of every expert, the tile list and the totals.  s_off (where not null): the first positions.
+__device__ __forceinline__ void list_tiles(const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E,
+                                           int tile_tokens, int* s_cnt, int* s_off, int32_t* counts, int32_t* offsets,
+                                           int32_t* num_tiles, int4* tiles, int* status) {
+    const int tid = threadIdx.x, lane = tid & 31;
     int bad = 0;
-    for (int a = tid; a < A; a += kRouteThreads) {
+    for (int a = tid; a < A; a += (int)blockDim.x) {
         if (row_valid(token_of_row, expert_of_row, a, T, E)) atomicAdd(&s_cnt[expert_of_row[a]], 1);
         else bad = 1;
     }
     if (__syncthreads_or(bad) && tid == 0) atomicExch(status, (int)DPS_ERR_DATA);
-    if (warp == 0) {
-        // first position and first tile of every expert
+    if (tid < 32) {
         int rows = 0, nt = 0;
         for (int base = 0; base < E; base += 32) {
             const int e = base + lane;
@@ -104,7 +97,7 @@ moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int 
             }
             if (e < E) {
                 const int off = rows + ci - c;
-                s_off[e] = off;
+                if (s_off != nullptr) s_off[e] = off;
                 offsets[e] = off;
                 counts[e] = c;
                 int t = nt + ki - k;
@@ -120,6 +113,22 @@ moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int 
             num_tiles[1] = rows;  // number of valid rows
         }
     }
+}
+
+__global__ void __launch_bounds__(kRouteThreads)
+moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E, int tile_tokens,
+                 int32_t* counts, int32_t* offsets, int32_t* sorted_rows, int32_t* num_tiles, int4* tiles, int* status) {
+    __shared__ int s_cnt[kMaxExperts];
+    __shared__ int s_off[kMaxExperts];
+    __shared__ int s_table[kRouteThreads / 32][kTableExperts];
+    // the gather and the grouped kernel may be made resident now; both wait for their predecessor
+    // (griddepcontrol.wait) before they read anything this kernel writes
+    sm100::grid_launch_dependents();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < E; e += kRouteThreads) s_cnt[e] = 0;
+    __syncthreads();
+    sm100::grid_dependency_wait();      // the routing and, through an earlier call, the workspace are earlier kernels'
+    list_tiles(token_of_row, expert_of_row, A, T, E, tile_tokens, s_cnt, s_off, counts, offsets, num_tiles, tiles, status);
     __syncthreads();
     if (E <= kTableExperts) {
         for (int base = 0; base < A; base += kRouteThreads) {
@@ -177,6 +186,62 @@ moe_gather_kernel(const uint4* x, const int32_t* token_of_row, const int32_t* so
     }
 }
 
+// Routing and gather in one launch, for up to kRankRows rows: every row has a block of its own, which finds the row's position
+// among the sorted rows by itself -- the number of valid rows of smaller experts, and of its own expert in front of it -- and
+// copies the activations there; one more block makes the tile list.  Two launches, each a chain of latencies that the next waits
+// for, become one.  The positions cost A comparisons per row, which is the longer way for many rows.  A whole call with hardly any
+// weights (256 rows x 4096, 8 experts / 256 x 2048, 64 experts), two launches against one, us: 2 rows 16.8 / 12.2 against 14.4 / 9.8,
+// 128 rows 17.1 / 13.6 against 15.0 / 11.0, 512 20.6 / 14.6 against 20.4 / 12.6, 1024 23.8 / 15.4 against 24.0 / 14.2, 2048 27.1 / 20.8
+// against 31.2 / 23.3, 4096 37.6 / 28.2 against 56.7 / 47.0.
+constexpr int kRankRows = 1024;
+constexpr int kRankThreads = 256;
+
+__global__ void __launch_bounds__(kRankThreads)
+moe_rank_gather_kernel(const uint4* x, const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E,
+                       int tile_tokens, int32_t* counts, int32_t* offsets, int32_t* sorted_rows, int32_t* num_tiles, int4* tiles,
+                       uint4* x_sorted, int64_t k16, int* status) {
+    __shared__ int s_cnt[kMaxExperts];
+    __shared__ int s_sum[kRankThreads / 32];
+    sm100::grid_launch_dependents();
+    const int tid = threadIdx.x;
+    if (blockIdx.x == 0) {
+        for (int e = tid; e < E; e += kRankThreads) s_cnt[e] = 0;
+        __syncthreads();
+        sm100::grid_dependency_wait();
+        list_tiles(token_of_row, expert_of_row, A, T, E, tile_tokens, s_cnt, nullptr, counts, offsets, num_tiles, tiles, status);
+        return;
+    }
+    const int a = (int)blockIdx.x - 1;
+    sm100::grid_dependency_wait();      // the routing and, through an earlier call, the workspace are earlier kernels'
+    if (!row_valid(token_of_row, expert_of_row, a, T, E)) return;       // (block 0 reports it)
+    const int e = expert_of_row[a];
+    const int64_t tok = token_of_row ? token_of_row[a] : a;
+    const uint4* src = x + tok * k16;
+    constexpr int kAhead = 4;           // pieces of the row requested before its position is known
+    uint4 v[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+        if (tid + i * kRankThreads < k16) v[i] = src[tid + i * kRankThreads];
+    int before = 0;
+#pragma unroll 4
+    for (int b = tid; b < A; b += kRankThreads) {
+        const int other = expert_of_row[b];
+        before += (other < e || (other == e && b < a)) && row_valid(token_of_row, expert_of_row, b, T, E);
+    }
+    before = __reduce_add_sync(0xFFFFFFFFu, before);
+    if ((tid & 31) == 0) s_sum[tid >> 5] = before;
+    __syncthreads();
+    int pos = 0;
+#pragma unroll
+    for (int i = 0; i < kRankThreads / 32; ++i) pos += s_sum[i];
+    if (tid == 0) sorted_rows[pos] = a;
+    uint4* dst = x_sorted + (int64_t)pos * k16;
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+        if (tid + i * kRankThreads < k16) dst[tid + i * kRankThreads] = v[i];
+    for (int64_t c = tid + kAhead * kRankThreads; c < k16; c += kRankThreads) dst[c] = src[c];
+}
+
 }  // namespace
 
 size_t moe_workspace_bytes(int64_t A, int32_t E, int64_t K) {
@@ -196,35 +261,35 @@ cudaError_t launch_moe(int mode, const int32_t* enc_host, const void* x, const i
     const bool pairs = A >= 48 * (int64_t)E;
     const int tn = pairs ? pair_grouped_tokens(A, E) : grouped_tile_tokens(A, E);
     cudaError_t err;
-    {   // programmatic dependent launch, as the two kernels behind it: each waits before its first read
+    // programmatic dependent launch, as the kernel behind them: each is resident early and waits before its first read
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    auto config = [&](int64_t blocks, int threads) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1, 1, 1);
-        cfg.blockDim = dim3(kRouteThreads, 1, 1);
+        cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+        cfg.blockDim = dim3((unsigned)threads, 1, 1);
         cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        err = cudaLaunchKernelEx(&cfg, moe_route_kernel, token_of_row, expert_of_row, (int)A, (int)T, (int)E, tn, w.counts,
+        return cfg;
+    };
+    const uint4* rows_in = static_cast<const uint4*>(x);
+    uint4* rows_out = reinterpret_cast<uint4*>(w.x_sorted);
+    if (A <= kRankRows) {
+        const cudaLaunchConfig_t cfg = config(A + 1, kRankThreads);
+        err = cudaLaunchKernelEx(&cfg, moe_rank_gather_kernel, rows_in, token_of_row, expert_of_row, (int)A, (int)T, (int)E, tn,
+                                 w.counts, w.offsets, w.sorted_rows, w.num_tiles, w.tiles, rows_out, (int64_t)(K / 8), status);
+        count_launch();
+        if (err != cudaSuccess) return err;
+    } else {
+        const cudaLaunchConfig_t route = config(1, kRouteThreads), gather = config(A < 4096 ? A : 4096, 256);
+        err = cudaLaunchKernelEx(&route, moe_route_kernel, token_of_row, expert_of_row, (int)A, (int)T, (int)E, tn, w.counts,
                                  w.offsets, w.sorted_rows, w.num_tiles, w.tiles, status);
         count_launch();
         if (err != cudaSuccess) return err;
-    }
-    const int gather_grid = (int)(A < 4096 ? A : 4096);
-    {   // programmatic dependent launch: resident while the routing kernel runs, waits before its first read
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)gather_grid, 1, 1);
-        cfg.blockDim = dim3(256, 1, 1);
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        err = cudaLaunchKernelEx(&cfg, moe_gather_kernel, static_cast<const uint4*>(x), token_of_row,
-                                 (const int32_t*)w.sorted_rows, (const int32_t*)w.num_tiles,
-                                 reinterpret_cast<uint4*>(w.x_sorted), (int64_t)(K / 8));
+        err = cudaLaunchKernelEx(&gather, moe_gather_kernel, rows_in, token_of_row, (const int32_t*)w.sorted_rows,
+                                 (const int32_t*)w.num_tiles, rows_out, (int64_t)(K / 8));
         count_launch();
         if (err != cudaSuccess) return err;
     }
