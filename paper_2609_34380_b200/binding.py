@@ -58,7 +58,9 @@ def fastcall_path() -> Path:
 
 FASTCALL_PATH = fastcall_path()
 
-_fast_linear = None     # native marshalling of dps_linear (csrc/fastcall.cpp); set when the library is loaded, if it was built
+# native marshalling (csrc/fastcall.cpp), set when the library is loaded, if it was built: dps_linear's, and the module with the others'
+_fast_linear = None
+_native = None
 
 
 class DpsError(RuntimeError):
@@ -87,7 +89,7 @@ def library() -> ctypes.CDLL:
 
 def _load_fastcall(lib: ctypes.CDLL) -> None:
     """The same call with less host work; without the module every call takes the ctypes path below."""
-    global _fast_linear
+    global _fast_linear, _native
     path = fastcall_path()
     if not path.exists():       # not built, or built for another PyTorch or Python
         return
@@ -98,7 +100,9 @@ def _load_fastcall(lib: ctypes.CDLL) -> None:
     except ImportError:
         return
     module.set_linear(ctypes.cast(lib.dps_linear, ctypes.c_void_p).value)
-    _fast_linear = module.linear
+    module.set_functions(*(ctypes.cast(fn, ctypes.c_void_p).value
+                           for fn in (lib.dps_split_weights, lib.dps_reconstruct, lib.dps_moe_linear)))
+    _fast_linear, _native = module.linear, module
 
 
 def status_string(status: int) -> str:
@@ -138,6 +142,12 @@ def _dev(t: Optional[torch.Tensor], dtype, what: str) -> Optional[int]:
 def dps_split_weights(w_fp16: torch.Tensor, enc: int = DPS_ENC_AUTO, w_persist: Optional[torch.Tensor] = None,
                       w_resid: Optional[torch.Tensor] = None, stream=None) -> Tuple[torch.Tensor, torch.Tensor, int]:
     """FP16 W[rows][cols] -> (persistent plane, residual plane, encoding used)."""
+    if stream is None and _native is not None:
+        out = _native.split_weights(w_fp16, enc, w_persist, w_resid)
+        if out.__class__ is int:
+            _check(out, "dps_split_weights")
+        if out is not None:
+            return out
     rows, cols = w_fp16.shape
     if w_persist is None:
         w_persist = torch.empty((rows, cols), dtype=torch.uint8, device=w_fp16.device)
@@ -154,6 +164,12 @@ def dps_split_weights(w_fp16: torch.Tensor, enc: int = DPS_ENC_AUTO, w_persist: 
 def dps_reconstruct(w_persist: torch.Tensor, w_resid: Optional[torch.Tensor], enc: int,
                     w_fp16_out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """(P, R) -> the original FP16 weights; R = None gives the fast-mode weights."""
+    if stream is None and _native is not None:
+        out = _native.reconstruct(w_persist, w_resid, enc, w_fp16_out)
+        if out.__class__ is int:
+            _check(out, "dps_reconstruct")
+        if out is not None:
+            return out
     rows, cols = w_persist.shape
     if w_fp16_out is None:
         w_fp16_out = torch.empty((rows, cols), dtype=torch.float16, device=w_persist.device)
@@ -195,6 +211,12 @@ def dps_moe_linear(mode: int, enc_per_expert: Sequence[int], x: torch.Tensor, to
                    y: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                    stream=None) -> torch.Tensor:
     """Grouped linear: y[a] = x[token_of_row[a]] * W_eff(expert_of_row[a])^T."""
+    if stream is None and _native is not None and workspace is not None:
+        out = _native.moe_linear(mode, enc_per_expert, x, token_of_row, expert_of_row, w_persist, w_resid, y, workspace)
+        if out.__class__ is int:
+            _check(out, "dps_moe_linear")
+        if out is not None:
+            return out
     E, N, K = w_persist.shape
     T, K2 = x.shape
     if K != K2:

@@ -130,3 +130,51 @@ def test_a_module_of_another_version_is_not_taken(monkeypatch):
     monkeypatch.undo()
     binding._load_fastcall(lib)
     assert binding._fast_linear is not None
+
+
+def test_other_entries_pass_on_what_they_do_not_take():
+    build.build_fastcall()
+    if binding._native is None:
+        binding._load_fastcall(binding.library())
+    native, h, b = binding._native, torch.zeros((8, 16), dtype=torch.float16), torch.zeros((8, 16), dtype=torch.uint8)
+    assert native.split_weights(h, 0, None, None) is None and native.split_weights("w", 0, None, None) is None
+    assert native.reconstruct(b, b, 1, None) is None and native.reconstruct(b, b, "1", None) is None
+    assert native.moe_linear(0, [1], h, None, h, b, None, None, None) is None
+    assert native.moe_linear(0, [1] * 2000, h, None, h, b, None, None, b) is None
+    with pytest.raises(ValueError):
+        dps.dps_split_weights(h)
+    with pytest.raises(ValueError):
+        dps.dps_reconstruct(b, None, 1)
+
+
+@pytest.mark.gpu
+def test_other_entries_answer_as_the_other_path_does():
+    w = workloads.weights(24, 144, 3, device="cuda:0")
+    stream = torch.cuda.current_stream()                  # an explicit stream: the ctypes way
+    p, r, enc = dps.dps_split_weights(w)
+    q, s, enc2 = dps.dps_split_weights(w, stream=stream)
+    assert isinstance(enc, int) and enc == enc2 and torch.equal(p, q) and torch.equal(r, s) and p.shape == w.shape
+    out = torch.empty_like(p)
+    assert dps.dps_split_weights(w, dps.DPS_ENC_E5M2, out, r)[0] is out
+    r = s
+    assert torch.equal(dps.dps_reconstruct(p, r, enc), w)
+    assert torch.equal(dps.dps_reconstruct(p, None, enc), dps.dps_reconstruct(p, None, enc, stream=stream))
+    bad = torch.full_like(w, 4.0)
+    with pytest.raises(dps.DpsError) as caught:
+        dps.dps_split_weights(bad, dps.DPS_ENC_E4M3)
+    assert caught.value.status == binding.DPS_ERR_DATA
+    x = workloads.activations(3, 144, 4, device="cuda:0")
+    tok, exp = (torch.tensor(v, dtype=torch.int32, device="cuda:0") for v in ([0, 0, 2, 1], [0, 1, 1, 0]))
+    planes, res = torch.stack([p, p]), torch.stack([r, r])
+    ws = torch.empty(dps.dps_moe_workspace_bytes(4, 2, 144), dtype=torch.uint8, device="cuda:0")
+    for mode in (dps.DPS_MODE_FAST, dps.DPS_MODE_FULL):
+        args = (mode, [enc, enc], x, tok, exp, planes, res if mode else None)
+        y = dps.dps_moe_linear(*args, workspace=ws)
+        assert torch.equal(y, dps.dps_moe_linear(*args, workspace=ws, stream=stream)) and torch.equal(y, dps.dps_moe_linear(*args))
+        mine = torch.empty_like(y)
+        assert dps.dps_moe_linear(*args, y=mine, workspace=ws) is mine and torch.equal(mine, y)
+    for wrong, error in [(dict(workspace=ws[:16]), dps.DpsError), (dict(workspace=ws.cpu()), ValueError)]:
+        with pytest.raises(error):
+            dps.dps_moe_linear(dps.DPS_MODE_FAST, [enc, enc], x, tok, exp, planes, None, **wrong)
+    with pytest.raises(dps.DpsError):
+        dps.dps_moe_linear(dps.DPS_MODE_FULL, [enc, 77], x, tok, exp, planes, res, workspace=ws)
