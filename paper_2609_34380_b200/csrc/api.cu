@@ -147,6 +147,12 @@ namespace {
 bool decode_tiles_for_128(bool full, int64_t M, int64_t N, int64_t K) {
     return M <= 128 && ((N <= 4096 && N * K <= ((int64_t)1 << (full ? 24 : 26))) || N * K <= ((int64_t)1 << 23));
 }
+// 33-64 tokens: CTA pairs instead of the 64-token decode tiles where K is long and the rows make at least twenty tiles of a pair.
+// There a split pair has many steps and its fixed costs, which exceed the tiles', are small.  Fast / full mode at 40-64 tokens, tiles
+// against pairs: 8192 x 28672 52.0 / 84.2 us against 46.8 / 81.7, 5120 x 25600 32.0 / 50.5 against 29.9 / 49.4, 16384 x 16384 60.6 / 98.2
+// against 51.6 / 93.2; but 4096 x 14336 17.1 / 25.5 against 19.6 / 27.8, 57344 x 8192 93.7 / 170 against 95.4 / 174, 10240 x 8192 24.3 /
+// 36.3 against 26.5 / 39.6.  At 20 tokens the 32-token tiles are faster here too: 43.0 / 78.0 against 45.0 / 80.2.
+bool pairs_for_64(int64_t M, int64_t N, int64_t K) { return M > 32 && K >= 16384 && N >= 5120; }
 bool known_encoding(int32_t enc) {
     return enc == DPS_ENC_E4M3 || enc == DPS_ENC_E5M2 || enc == DPS_ENC_E4M3_RN || enc == DPS_ENC_E5M2_RN;
 }
@@ -278,7 +284,7 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     // What the rule costs: a matrix beyond it that is called by itself.  2048 x 2048, 9 tokens, takes 4.5 us in fast and 5.4 in
     // full mode, the streaming kernel 3.4 and 3.9; 4096 x 4096 6.7 and 9.3 against 5.7 and 8.8.  With other programs' kernels
     // between the linears every launch of the tiles pays for the change of split, about 2 us: 2048 x 2048 7.0 against 4.2.
-    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens CTA pairs (four Llama-7B linears, fast / full mode: 64
+    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for long K) CTA pairs (four Llama-7B linears, fast / full mode: 64
     // tokens 62 / 97 us with the tiles, 75 / 109 with pairs; 96 tokens 84 / 134 against 74 / 107).  (The CUDA-core GEMV
     // is kept as a cross-check.)
     const bool stream_mid = (N < K ? N : K) <= 1536 && N * K < ((int64_t)1 << 25);
@@ -290,7 +296,7 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     else if (path == 3 || M <= 8 || (M <= 16 && stream_mid)) {
         if (M > 16) return DPS_ERR_UNSUPPORTED;      // (only reachable with DPS_FORCE_PATH=stream)
         err = launch_decode_mma(mode, enc, x, w_persist, r, y, M, N, K, stream);
-    } else if (M > 64 && !decode_tiles_for_128(mode == DPS_MODE_FULL, M, N, K))
+    } else if ((M > 64 && !decode_tiles_for_128(mode == DPS_MODE_FULL, M, N, K)) || pairs_for_64(M, N, K))
         err = launch_pair_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
     else err = launch_umma_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
     return err == cudaSuccess ? DPS_OK : DPS_ERR_CUDA;
