@@ -131,10 +131,6 @@ __host__ __device__ constexpr int x_slots_alone(bool full, int tn) {
     return 5;
 }
 __host__ __device__ constexpr int x_tile_bytes(bool full, int tn) { return tn * block_k(full, tn) * 2; }
-// Bytes of one ring stage: planes and activations, or planes alone when the activations have slots.
-__host__ __device__ constexpr int ring_stage_bytes(bool full, int tn, bool grouped) {
-    return stage_bytes(full, tn) - (x_slots(full, grouped, tn) ? x_tile_bytes(full, tn) : 0);
-}
 
 // Optional timeline trace (compile with -DDPS_TRACE): lane 0 of each role of CTA (0,0,0) stamps
 // the SM clock at pipeline events of every K block.  Read back with dps_debug_trace().
@@ -182,6 +178,7 @@ struct GroupedParams {
 struct UmmaParams {
     __half* y;
     int M, N, K;
+    int rows;        // LOW: weight rows of a tile (a multiple of 8)
     int num_stages;
     int split;       // K split = cluster size along z; partial tiles are summed through DSMEM
     int red_offset;  // byte offset (from the aligned base of dynamic smem) of the split-K mailbox
@@ -201,7 +198,7 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
 
 // What a zip warp needs to know about its CTA's pipeline.
 struct ZipCtx {
-    int group, warp, lane, row, num_kb, num_stages, stage_bytes;
+    int group, warp, lane, row, num_kb, num_stages, stage_bytes, plane_bytes;
     uint32_t smem_base, tmem_a, lane_base, sw;
     uint64_t *bar_full, *bar_empty, *bar_a_full, *bar_a_empty;
 };
@@ -215,7 +212,6 @@ template <int ENC, bool FULL, int TN, bool EARLY = false>
 __device__ __forceinline__ bool zip_blocks(const ZipCtx& z) {
     constexpr int kBlockK = block_k(FULL, TN);
     constexpr int kACols = kBlockK / 2;
-    constexpr int kPlaneStageBytes = plane_stage_bytes(FULL, TN);
     bool ok = true;
     // Ring positions are advanced incrementally (no division in the loop).  Every stage and every A
     // slot always belongs to the same zip group, so that each waiter sees every phase of the barriers
@@ -253,7 +249,7 @@ __device__ __forceinline__ bool zip_blocks(const ZipCtx& z) {
             if (FULL)
                 asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
                              : "=r"(rv.x), "=r"(rv.y), "=r"(rv.z), "=r"(rv.w)
-                             : "r"(prow + kPlaneStageBytes + off));
+                             : "r"(prow + z.plane_bytes + off));
             uint32_t h8[8];
             if (FULL) join16<ENC, FULL>(pv, rv, h8);
             else fast16<ENC>(pv, h8);   // E4M3: 2^8 times the weights, undone in the epilogue
@@ -290,19 +286,21 @@ __device__ __forceinline__ bool zip_blocks(const ZipCtx& z) {
 }
 
 // ENC == 0 (grouped launches only): the encoding is a per-expert run-time value.
-template <int ENC, bool FULL, int TN, bool GROUPED>
+// LOW: tiles of less than kTileRows rows (see low_rows), K not split; a template argument because the others take a run-time
+// height for 0.3 % of their time.
+template <int ENC, bool FULL, int TN, bool GROUPED, bool LOW>
 __global__ void __launch_bounds__(kThreads, 2)
 umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r,
                    const __grid_constant__ CUtensorMap map_x, const UmmaParams prm, const GroupedParams gp) {
     constexpr int kBlockK = block_k(FULL, TN);
     constexpr int kXAtoms = kBlockK / 64;    // the x tile is stored as 64-element (128-byte) swizzle atoms
     constexpr int kACols = kBlockK / 2;      // TMEM columns of one A slot (two FP16 per column)
-    constexpr int kPlaneStageBytes = plane_stage_bytes(FULL, TN);
-    constexpr int kStage = ring_stage_bytes(FULL, TN, GROUPED);
-    constexpr int kXOffset = kPlaneStageBytes * (FULL ? 2 : 1);
     constexpr bool kXS = x_slots(FULL, GROUPED, TN) > 0;   // the activations have slots of their own ...
     const int xs_n = prm.x_slots;                               // ... this many (chosen per launch: what fits)
     constexpr int kXBytes = x_tile_bytes(FULL, TN);
+    const int rows = LOW ? prm.rows : kTileRows, quarters = (rows + 31) / 32;   // quarters of the lanes that hold rows
+    const int plane_bytes = rows * kBlockK, x_offset = plane_bytes * (FULL ? 2 : 1);
+    const int stage = x_offset + (kXS ? 0 : kXBytes);
     constexpr uint32_t kCols = tmem_cols(FULL, TN);
     static_assert(kCols <= 256, "two CTAs share the tensor memory of an SM");
 
@@ -346,7 +344,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         row_tile = group * kRowGroup + within % rows_here;
         tok_tile = within / rows_here;
     }
-    const int n0 = row_tile * kTileRows;
+    const int n0 = row_tile * rows;
     int m0 = tok_tile * TN;          // first token (dense) / first sorted row (grouped) of the tile
     int tile_tokens = TN;            // valid token columns of the tile (grouped)
     int plane_row0 = n0;             // first plane row of the tile in the [E * N][K] view
@@ -377,12 +375,12 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     if (threadIdx.x == 0) {
         for (int s = 0; s < num_stages; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
-            // 4 zip warps per reader group + 1 tcgen05.commit; a stage that holds planes only (the activations
-            // have slots) is read by the zip warps alone
-            mbar_init(smem_u32(&bar_empty[s]), kXS ? 4 : 5);
+            // the zip warps of a reader group, one for each quarter, + 1 tcgen05.commit; a stage that holds planes
+            // only (the activations have slots) is read by the zip warps alone
+            mbar_init(smem_u32(&bar_empty[s]), kXS ? quarters : quarters + 1);
         }
         for (int a = 0; a < kMaxAStages; ++a) {
-            mbar_init(smem_u32(&bar_a_full[a]), 4);
+            mbar_init(smem_u32(&bar_a_full[a]), quarters);
             mbar_init(smem_u32(&bar_a_empty[a]), 1);
         }
         mbar_init(smem_u32(&bar_d_full), 1);
@@ -423,19 +421,19 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         const int first = num_kb < num_stages ? num_kb : num_stages;
         auto load_planes = [&](int i, int s) {
             const uint32_t full = smem_u32(&bar_full[s]);
-            const uint32_t dst = smem_base + (uint32_t)s * kStage;
+            const uint32_t dst = smem_base + (uint32_t)(s * stage);
             const int k = (rank + i * split) * kBlockK;
-            mbar_arrive_expect_tx(full, (uint32_t)kStage);
+            mbar_arrive_expect_tx(full, (uint32_t)stage);
             tma_load_2d(dst, &map_p, full, k, plane_row0);
-            if (FULL) tma_load_2d(dst + kPlaneStageBytes, &map_r, full, k, plane_row0);
+            if (FULL) tma_load_2d(dst + plane_bytes, &map_r, full, k, plane_row0);
         };
         auto load_x = [&](int i, int s) {       // activation tile of K block i, riding in stage s
             const uint32_t full = smem_u32(&bar_full[s]);
-            const uint32_t dst = smem_base + (uint32_t)s * kStage;
+            const uint32_t dst = smem_base + (uint32_t)(s * stage);
             const int k = (rank + i * split) * kBlockK;
 #pragma unroll
             for (int t = 0; t < kXAtoms; ++t)
-                tma_load_2d(dst + kXOffset + (uint32_t)(t * TN * 128), &map_x, full, k + t * 64, m0);
+                tma_load_2d(dst + x_offset + (uint32_t)(t * TN * 128), &map_x, full, k + t * 64, m0);
         };
         auto load_x_slot = [&](int j, int slot) {   // activation tile of K block j into its own slot
             const uint32_t full = smem_u32(&bar_x_full[slot]);
@@ -571,7 +569,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                     ++cnt1;
                 }
                 const uint32_t xbase = kXS ? smem_base + (uint32_t)prm.x_offset + (uint32_t)(xslot * kXBytes)
-                                           : smem_base + (uint32_t)s * kStage + kXOffset;
+                                           : smem_base + (uint32_t)(s * stage) + x_offset;
                 DPS_STAMP(1, i);
                 ok = mbar_wait(smem_u32(&bar_a_full[a]), a_parity);
                 if (i == 0) DPS_CTA_STAMP_T(11, 32);
@@ -610,14 +608,15 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
         const int group = (warp - 2) >> 2;
         const int q = warp & 3;                  // TMEM lane quarter this warp may touch
         const int row = q * 32 + lane;           // weight row inside the tile
+        const int zip_row = min(row, rows - 1);  // (lanes without a row repeat the last one: nobody reads theirs)
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         ZipCtx zc;
-        zc.group = group; zc.warp = warp; zc.lane = lane; zc.row = row;
-        zc.num_kb = num_kb; zc.num_stages = num_stages; zc.stage_bytes = kStage;
+        zc.group = group; zc.warp = warp; zc.lane = lane; zc.row = zip_row;
+        zc.num_kb = num_kb; zc.num_stages = num_stages; zc.stage_bytes = stage; zc.plane_bytes = plane_bytes;
         zc.smem_base = smem_base; zc.tmem_a = tmem_a; zc.lane_base = lane_base;
         // TMA swizzle of the plane tiles: 128-byte rows: 16-byte chunk index ^= row % 8;
         // 64-byte rows: chunk index ^= (row / 2) % 4
-        zc.sw = kBlockK == 128 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
+        zc.sw = kBlockK == 128 ? (uint32_t)(zip_row & 7) : (uint32_t)((zip_row >> 1) & 3);
         zc.bar_full = bar_full; zc.bar_empty = bar_empty; zc.bar_a_full = bar_a_full; zc.bar_a_empty = bar_a_empty;
         // grouped launches: the callers' row ids of the tile's tokens, fetched before the zip loop (which
         // hides the latency) rather than in front of every store of the epilogue
@@ -629,7 +628,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
             else
                 ok = e5m2 ? zip_blocks<kEncE5M2, FULL, TN>(zc) : zip_blocks<kEncE4M3, FULL, TN>(zc);
         } else {
-            ok = zip_blocks<ENC, FULL, TN, kXS>(zc);
+            if (q < quarters) ok = zip_blocks<ENC, FULL, TN, kXS>(zc);
         }
         // E4M3 fast mode multiplied with 2^8 times the weights (hardware FP8 conversion)
         const float out_scale = (!FULL && !e5m2) ? 0.00390625f : 1.0f;
@@ -673,7 +672,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 for (int item = zt; item < ncols * kChunks; item += kZipGroups * 128) {
                     const int c = item / kChunks, q = item % kChunks;
                     const int n = n0 + q * 8;
-                    if (n >= prm.N) continue;                     // N is a multiple of 8: a piece is in or out
+                    if (q * 8 >= rows || n >= prm.N) continue;    // both are multiples of 8: a piece is in or out
                     const int m = GROUPED ? s_rows[c] : m0 + c;
                     uint4 val;
                     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -786,10 +785,31 @@ int choose_split(int64_t tiles, int total_kb, const int* capacity, int min_kb) {
     return best;
 }
 
-template <int ENC, bool FULL, int TN>
+// Rows per tile where K is not split because there are more tiles of kTileRows rows than SMs.  Two CTAs fit an SM: as many tiles as
+// slots allow without another wave, and 5 % less, load the SMs evenly, where 172 tiles on 148 SMs leave one tile on most and two on
+// some.  Full mode, tiles of kTileRows rows against what this chooses, us: 10-16 tokens 22016 x 4096 (88 rows) 35.9 / 32.1, 27648 x
+// 5120 (104) 48.2 / 45.1, 32768 x 6144 (120) 63.5 / 60.4, 57344 x 8192 (104) 156.5 / 142.5, 128256 x 4096 166 / 156.5; 32 tokens, whose
+// activations cost an SM more per tile, only where the load is most uneven: 22016 x 4096 (88) 36.5 / 33.0, but 27648 x 5120 48.5 / 48.4,
+// 57344 x 8192 158.5 / 156.5, 128256 x 4096 170 / 172.7.  (Fast mode gains 2-5 % on some and loses as much on others; below 88
+// rows the K blocks' latencies show: 22016 x 4096 with 72 rows 44.)
+// DPS_TILE_ROWS=64..120 pins the height.
+constexpr int kLeastRows = 88;
+int low_rows(int64_t N, int tn) {
+    static const int forced = [] { const char* e = getenv("DPS_TILE_ROWS"); return e ? atoi(e) / 8 * 8 : 0; }();
+    if (forced >= 64 && forced < kTileRows) return forced;
+    const int64_t sms = sm_count(), slots = 2 * sms, tiles = (N + kTileRows - 1) / kTileRows;
+    if (tiles <= sms) return kTileRows;
+    const int64_t waves = (tiles + slots - 1) / slots;
+    int64_t rows = (N * 20 + waves * slots * 19 - 1) / (waves * slots * 19);   // N / (0.95 of the slots)
+    rows = (rows + 7) / 8 * 8;
+    if (rows < kLeastRows) rows = kLeastRows;
+    if (rows >= kTileRows || (tn > 16 && rows > kLeastRows)) return kTileRows;
+    return (int)rows;
+}
+
+template <int ENC, bool FULL, int TN, bool LOW = false>
 cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
-                      int* status, cudaStream_t stream) {
-    constexpr int kStage = ring_stage_bytes(FULL, TN, false);   // planes only when the activations have slots
+                      int* status, cudaStream_t stream, int rows = kTileRows) {
     constexpr int kXSlots = x_slots(FULL, false, TN);            // with a split-K mailbox in shared memory
     constexpr int kXSlotsAlone = x_slots_alone(FULL, TN);           // without one (K not split)
     constexpr int kXTile = x_tile_bytes(FULL, TN);
@@ -798,15 +818,14 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     constexpr int kMailMax = (TN + kMaxSplit) * kTileRows * 4;  // mailbox, worst case
     // Ring depth for a given mailbox size: whatever fits (stage s is rebuilt by zip group s % 2, so
     // odd depths work; they just give the first group one stage more).
-    auto ring_depth = [&](int mail_bytes) {
+    auto stage_of = [](int tile_rows) { return tile_rows * block_k(FULL, TN) * (FULL ? 2 : 1) + (kXSlots ? 0 : kXTile); };
+    auto ring_depth = [&](int mail_bytes, int tile_rows) {
         const int x_ring = (mail_bytes > 0 ? kXSlots : kXSlotsAlone) * kXTile;
-        int d = (kSmemTotal - mail_bytes - x_ring) / kStage;
-        if (d > 8) d = 8;
-        if (d < 2) d = 2;
-        return d;
+        const int d = (kSmemTotal - mail_bytes - x_ring) / stage_of(tile_rows);
+        return d > 8 ? 8 : d < 2 ? 2 : d;
     };
-    const size_t smem_query = (size_t)ring_depth(kMailMax) * kStage + kXSlots * kXTile + kMailMax + 1024;
-    auto kernel = umma_linear_kernel<ENC, FULL, TN, false>;
+    const size_t smem_query = (size_t)ring_depth(kMailMax, kTileRows) * stage_of(kTileRows) + kXSlots * kXTile + kMailMax + 1024;
+    auto kernel = umma_linear_kernel<ENC, FULL, TN, false, LOW>;
     // CTAs that can be resident at once for each cluster size: per instantiation and per device, filled by
     // the first call on that device and read only after that set-up has returned.
     static int capacity_of[kMaxDevices][kMaxSplit + 1] = {};
@@ -858,15 +877,21 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
         if (e0 != cudaSuccess) return e0;
     }
     const int* capacity = capacity_of[dev];
-    CUtensorMap mp, mr, mx;
     constexpr int kBlockK = block_k(FULL, TN);
+    const int64_t tok_tiles = (M + TN - 1) / TN;
+    const int total_kb = (int)((K + kBlockK - 1) / kBlockK);
+    int split = LOW ? 1 : forced_split();
+    if (split <= 0) split = choose_split((N + rows - 1) / rows * tok_tiles, total_kb, capacity, FULL ? 5 : 4);
+    if (split > total_kb) split = total_kb;
+    if (split > kMaxSplit) split = kMaxSplit;
+    CUtensorMap mp, mr, mx;
     constexpr CUtensorMapSwizzle kPlaneSwizzle = kBlockK == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     constexpr CUtensorMapL2promotion kPromotion = CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
-    if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kTileRows, kBlockK,
+    if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, (uint32_t)rows, kBlockK,
                      kPlaneSwizzle, kPromotion))
         return cudaErrorInvalidValue;
     if (FULL) {
-        if (!make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kTileRows, kBlockK,
+        if (!make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, (uint32_t)rows, kBlockK,
                          kPlaneSwizzle, kPromotion))
             return cudaErrorInvalidValue;
     } else {
@@ -875,19 +900,14 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     if (!make_map_2d(&mx, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K, TN, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
-    const int64_t row_tiles = (N + kTileRows - 1) / kTileRows, tok_tiles = (M + TN - 1) / TN;
-    const int total_kb = (int)((K + kBlockK - 1) / kBlockK);
-    int split = forced_split();
-    if (split <= 0) split = choose_split(row_tiles * tok_tiles, total_kb, capacity, FULL ? 5 : 4);
-    if (split > total_kb) split = total_kb;
-    if (split > kMaxSplit) split = kMaxSplit;
+    const int64_t row_tiles = (N + rows - 1) / rows;
     // the mailbox exists only when K is split, and then has its exact size
     const int slots = split > 1 ? (TN + split - 1) / split : 0;
     const int mail_bytes = (split > 1 && kMailMax > 0) ? split * slots * kTileRows * 4 : 0;
-    const int stages = ring_depth(mail_bytes);
+    const int stages = ring_depth(mail_bytes, rows), stage = stage_of(rows);
     const int xs_n = mail_bytes > 0 ? kXSlots : kXSlotsAlone;
     const int x_ring = xs_n * kXTile;
-    const size_t smem = (size_t)stages * kStage + x_ring + mail_bytes + 1024;
+    const size_t smem = (size_t)stages * stage + x_ring + mail_bytes + 1024;
     if (getenv("DPS_DEBUG"))
         fprintf(stderr, "[dps] umma TN=%d full=%d N=%lld K=%lld M=%lld stages=%d split=%d capacity=%d,%d,%d,%d,%d,%d,%d,%d\n",
                 TN, (int)FULL, (long long)N, (long long)K, (long long)M, stages, split, capacity[1], capacity[2],
@@ -900,9 +920,10 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     prm.status = status;
     prm.num_stages = stages;
     prm.split = split;
-    prm.x_offset = stages * kStage;
+    prm.rows = rows;
+    prm.x_offset = stages * stage;
     prm.x_slots = xs_n;
-    prm.red_offset = stages * kStage + x_ring;
+    prm.red_offset = stages * stage + x_ring;
     prm.status = status;
 #ifdef DPS_TRACE
     static int trace_launches = 0;
@@ -934,6 +955,12 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
                        int* status, cudaStream_t stream) {
+    if constexpr (FULL) {
+        const int rows = M <= 32 && forced_split() <= 1 ? low_rows(N, M <= 16 ? 16 : 32) : kTileRows;
+        if (rows < kTileRows)
+            return M <= 16 ? launch_tn<ENC, FULL, 16, true>(x, p, r, y, M, N, K, status, stream, rows)
+                           : launch_tn<ENC, FULL, 32, true>(x, p, r, y, M, N, K, status, stream, rows);
+    }
     if (M <= 16) return launch_tn<ENC, FULL, 16>(x, p, r, y, M, N, K, status, stream);
     if (M <= 32) return launch_tn<ENC, FULL, 32>(x, p, r, y, M, N, K, status, stream);
     // 33 tokens and more (beyond 64 only where the dispatcher prefers two 64-token tiles per 128 rows to CTA pairs)
@@ -971,7 +998,7 @@ cudaError_t launch_grouped_tn(const uint32_t* e5m2_mask, const void* x_sorted, c
     if (stages > 8) stages = 8;
     if (stages < 2) stages = 2;
     const size_t smem = (size_t)stages * kStage + 1024;
-    auto kernel = umma_linear_kernel<0, FULL, TN, true>;
+    auto kernel = umma_linear_kernel<0, FULL, TN, true, false>;
     static PerDeviceOnce setup;     // per instantiation and per device
     {
         const cudaError_t e = setup.run([&] {

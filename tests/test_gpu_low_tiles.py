@@ -1,0 +1,41 @@
+"""GPU: full mode, 9 to 32 tokens, more 128-row tiles than SMs: lower tiles.  The matrix heights on both sides of the rule's edges (one
+wave of tiles and two), a last tile of few rows, K below and beyond the ring; and pinned heights that end inside every quarter of the
+lanes, in child processes, since the library reads the knob once."""
+import os
+import subprocess
+import sys
+
+import pytest
+import torch
+
+import oracle
+import paper_2609_34380_b200 as dps
+from paper_2609_34380_b200 import workloads
+from tests import test_gpu_pair_linear as checks
+from tests.helpers import assert_close_to_oracle, split_both, to_np_words
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("M,N,K,enc", [(13, 18944, 48, dps.DPS_ENC_E5M2), (16, 18952, 2064, dps.DPS_ENC_AUTO), (32, 22024, 272, dps.DPS_ENC_E4M3_RN),
+                                       (17, 27648, 144, dps.DPS_ENC_E5M2_RN), (9, 37896, 2064, dps.DPS_ENC_E5M2), (24, 40008, 16, dps.DPS_ENC_AUTO)])
+def test_heights_around_the_rule(M, N, K, enc):
+    p, r, enc, p_ref, r_ref = split_both(workloads.weights(N, K, 5, device=DEV), enc, DEV)
+    x = workloads.activations(M, K, 6, device=DEV)
+    guard = torch.full((M + 2, N), 7.0, dtype=torch.float16, device=DEV)
+    y = guard[1:M + 1]
+    dps.dps_linear(dps.DPS_MODE_FULL, enc, x, p, r, y)
+    assert_close_to_oracle(y, oracle.linear(dps.DPS_MODE_FULL, enc, to_np_words(x), p_ref, r_ref, threads=8), f"M={M} N={N} K={K} enc={enc}")
+    assert bool((guard[0] == 7.0).all()) and bool((guard[M + 1] == 7.0).all())
+    assert torch.equal(y, dps.dps_linear(dps.DPS_MODE_FULL, enc, x, p, r))
+    assert dps.dps_stream_status() == dps.DPS_OK
+
+
+@pytest.mark.parametrize("rows", [64, 72, 104, 120])
+def test_pinned_heights_in_child_process(rows):
+    env = dict(os.environ, DPS_FORCE_PATH="umma", DPS_TILE_ROWS=str(rows), PYTHONPATH=checks.REPO)
+    shapes = ["8,16,1", "136,80,17", "264,1040,25", "1032,2720,32", "1032,272,16"]
+    out = subprocess.run([sys.executable, os.path.abspath(checks.__file__), *shapes], cwd=checks.REPO, env=env, capture_output=True, text=True, timeout=900)
+    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
+    assert "all 30 cases passed" in out.stdout
