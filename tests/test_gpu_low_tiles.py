@@ -1,4 +1,4 @@
-"""GPU: full mode, 9 to 32 tokens, more 128-row tiles than SMs: lower tiles.  The matrix heights on both sides of the rule's edges (one
+"""GPU: 9 to 32 tokens, more 128-row tiles than SMs: lower tiles.  The matrix heights on both sides of the rule's edges (one
 wave of tiles and two), a last tile of few rows, K below and beyond the ring; and pinned heights that end inside every quarter of the
 lanes, in child processes, since the library reads the knob once."""
 import os
@@ -19,16 +19,19 @@ DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("M,N,K,enc", [(13, 18944, 48, dps.DPS_ENC_E5M2), (16, 18952, 2064, dps.DPS_ENC_AUTO), (32, 22024, 272, dps.DPS_ENC_E4M3_RN),
-                                       (17, 27648, 144, dps.DPS_ENC_E5M2_RN), (9, 37896, 2064, dps.DPS_ENC_E5M2), (24, 40008, 16, dps.DPS_ENC_AUTO)])
+                                       (17, 27648, 144, dps.DPS_ENC_E5M2_RN), (9, 37896, 2064, dps.DPS_ENC_E5M2), (24, 40008, 16, dps.DPS_ENC_AUTO),
+                                       (12, 20008, 6720, dps.DPS_ENC_AUTO)])
 def test_heights_around_the_rule(M, N, K, enc):
     p, r, enc, p_ref, r_ref = split_both(workloads.weights(N, K, 5, device=DEV), enc, DEV)
     x = workloads.activations(M, K, 6, device=DEV)
-    guard = torch.full((M + 2, N), 7.0, dtype=torch.float16, device=DEV)
-    y = guard[1:M + 1]
-    dps.dps_linear(dps.DPS_MODE_FULL, enc, x, p, r, y)
-    assert_close_to_oracle(y, oracle.linear(dps.DPS_MODE_FULL, enc, to_np_words(x), p_ref, r_ref, threads=8), f"M={M} N={N} K={K} enc={enc}")
-    assert bool((guard[0] == 7.0).all()) and bool((guard[M + 1] == 7.0).all())
-    assert torch.equal(y, dps.dps_linear(dps.DPS_MODE_FULL, enc, x, p, r))
+    for mode in (dps.DPS_MODE_FAST, dps.DPS_MODE_FULL):
+        guard = torch.full((M + 2, N), 7.0, dtype=torch.float16, device=DEV)
+        y = guard[1:M + 1]
+        dps.dps_linear(mode, enc, x, p, r if mode else None, y)
+        ref = oracle.linear(mode, enc, to_np_words(x), p_ref, r_ref, threads=8)
+        assert_close_to_oracle(y, ref, f"M={M} N={N} K={K} enc={enc} mode={mode}")
+        assert bool((guard[0] == 7.0).all()) and bool((guard[M + 1] == 7.0).all())
+        assert torch.equal(y, dps.dps_linear(mode, enc, x, p, r if mode else None))
     assert dps.dps_stream_status() == dps.DPS_OK
 
 
