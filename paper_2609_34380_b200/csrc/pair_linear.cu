@@ -222,10 +222,15 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             fence_async_proxy();
         }
         __syncwarp();
-        // The planes are model state, and their barriers this CTA's own: the ring fills while tensor memory is allocated and the
-        // pair meets.  With the divisions left to the host, four linears in a chain, fast / full mode: Llama-7B 64
-        // tokens 67.6 / 98.8 -> 65.1 / 95.5 us, 128 80.3 / 108.5 -> 76.5 / 104.9, 256 103.3 / 139.8 -> 100.8 / 138; 2048-wide layers, 128
-        // tokens, 42.1 / 49.3 -> 40.7 / 46.9 (the split's sum, 1-3 % of launches that have one, is in these).
+        // the others need the barriers only: they do not wait for the requests below (130 cycles each, twelve in fast mode)
+        named_barrier_arrive(1, kThreads);
+        cluster_arrive();
+        // The planes are model state, and their barriers this CTA's own: the ring fills while tensor memory is allocated and the pair
+        // meets.  Four linears in a chain, fast / full mode, loads by the role after the meeting (and quotients computed on the device)
+        // -> loads here with the block waiting for this warp -> as it is, us: Llama-7B 72 tokens 72.3 / 102.8 -> 71.3 / 100.4 -> 70.7 /
+        // 100.4, 512 168.6 / 213.9 -> 167.0 / 207.2 -> 164.5 / 201.2; 2048-wide layers, 256 tokens, 50.6 / 60.5 -> 50.0 / 56.0 -> 47.3 /
+        // 53.5; 1264-wide, 1189 tokens, planes out of L2, 61.7 / 71.2 -> 63.3 / 72.3 -> 59.6 / 67.2.  (The step between holds the L2
+        // requests in full mode and the sum over a K split as well.)
         if (work(0, w)) {
             loaded = min(units, steps_k);
             if (elect_one()) {
@@ -247,9 +252,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         prefetch_tensormap(&map_x);
     }
     if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_slot), 512);
-    tc_fence_before_sync();
-    __syncthreads();
-    cluster_sync_all();           // the other CTA's barriers exist
+    if (warp != 0) {
+        tc_fence_before_sync();
+        named_barrier_sync(1, kThreads);
+        cluster_arrive();
+    }
+    cluster_wait();               // the other CTA's barriers exist
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
     const uint32_t tmem_a = tmem_base + kAccCols;
