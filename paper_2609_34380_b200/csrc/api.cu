@@ -147,12 +147,19 @@ namespace {
 bool decode_tiles_for_128(bool full, int64_t M, int64_t N, int64_t K) {
     return M <= 128 && ((N <= 4096 && N * K <= ((int64_t)1 << (full ? 24 : 26))) || N * K <= ((int64_t)1 << 23));
 }
-// 33-64 tokens: CTA pairs instead of the 64-token decode tiles where K is long and the rows make at least twenty tiles of a pair.
-// There a split pair has many steps and its fixed costs, which exceed the tiles', are small.  Fast / full mode at 40-64 tokens, tiles
-// against pairs: 8192 x 28672 52.0 / 84.2 us against 46.8 / 81.7, 5120 x 25600 32.0 / 50.5 against 29.9 / 49.4, 16384 x 16384 60.6 / 98.2
-// against 51.6 / 93.2; but 4096 x 14336 17.1 / 25.5 against 19.6 / 27.8, 57344 x 8192 93.7 / 170 against 95.4 / 174, 10240 x 8192 24.3 /
-// 36.3 against 26.5 / 39.6.  At 20 tokens the 32-token tiles are faster here too: 43.0 / 78.0 against 45.0 / 80.2.
-bool pairs_for_64(int64_t M, int64_t N, int64_t K) { return M > 32 && K >= 16384 && N >= 5120; }
+// 33-64 tokens: CTA pairs instead of the 64-token decode tiles where K is long and the pairs take no more turns over the chip
+// (tile_plan.h: pairs_for_long_k, with what both sides take).  Fast / full mode, 64 tokens, tiles against pairs, us: 8192 x 28672 52.4 / 84.9 against 46.6 / 82.9,
+// 12288 x 16384 54.7 / 85.8 against 47.1 / 75.8, 38144 x 16384 147.5 / 277.8 against 132.2 / 242.5; but 6144 x 16384 27.0 / 40.2 against
+// 28.1 / 42.8, 8704 x 16384 32.8 / 51.6 against 44.7 / 66.0, 19200 x 16384 75.1 / 147.3 against 86.3 / 150.0.  With a shorter K the pairs' fixed
+// costs show: 4096 x 14336 17.1 / 25.5 against 19.6 / 27.8, 57344 x 8192 93.7 / 170 against 95.4 / 174, 10240 x 8192 24.3 / 36.3 against
+// 26.5 / 39.6; at 20 tokens the 32-token tiles are faster here too: 43.0 / 78.0 against 45.0 / 80.2.  A pair sums a longer range of K in one
+// accumulator: at 8192 x 28672 the error against 64 bits is 2.074e-4 of the output instead of 2.070e-4, of which the rounding to FP16 is 2.068e-4.
+bool pairs_for_64(int32_t mode, int32_t enc, int64_t M, int64_t N, int64_t K) {
+    if (M <= 32 || M > 64 || K < 16384 || N < 5120) return false;
+    tile_plan::Turns pairs, tiles;
+    return pair_turns(mode, enc, M, N, K, &pairs) == cudaSuccess && tile_turns_64(mode, enc, M, N, K, &tiles) == cudaSuccess &&
+           tile_plan::pairs_for_long_k(pairs, tiles);
+}
 bool known_encoding(int32_t enc) {
     return enc == DPS_ENC_E4M3 || enc == DPS_ENC_E5M2 || enc == DPS_ENC_E4M3_RN || enc == DPS_ENC_E5M2_RN;
 }
@@ -296,7 +303,7 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     else if (path == 3 || M <= 8 || (M <= 16 && stream_mid)) {
         if (M > 16) return DPS_ERR_UNSUPPORTED;      // (only reachable with DPS_FORCE_PATH=stream)
         err = launch_decode_mma(mode, enc, x, w_persist, r, y, M, N, K, stream);
-    } else if ((M > 64 && !decode_tiles_for_128(mode == DPS_MODE_FULL, M, N, K)) || pairs_for_64(M, N, K))
+    } else if ((M > 64 && !decode_tiles_for_128(mode == DPS_MODE_FULL, M, N, K)) || pairs_for_64(mode, enc, M, N, K))
         err = launch_pair_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
     else err = launch_umma_linear(mode, enc, x, w_persist, r, y, M, N, K, d->status, stream);
     return err == cudaSuccess ? DPS_OK : DPS_ERR_CUDA;

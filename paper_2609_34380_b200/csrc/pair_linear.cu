@@ -540,9 +540,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 
 // ---- host side ---------------------------------------------------------------------------------
 
+// `turns`, where not null: nothing is launched, *turns receives the turns the launch would take.
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K, int* status,
-                       cudaStream_t stream) {
+                       cudaStream_t stream, tile_plan::Turns* turns = nullptr) {
     auto kernel = umma_pair_kernel<ENC, FULL, false>;
     // Clusters of s pairs that are resident at once, per device (they must fit inside a GPC): filled by the first call on a
     // device, read only after that set-up has returned.
@@ -579,6 +580,12 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     }
     const Plan plan = make_plan(FULL, M, N, K, capacity_of[dev]);
     const int pairs = capacity_of[dev][1];
+    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
+    const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
+    if (turns != nullptr) {
+        *turns = tile_plan::turns(tiles, plan.split, pairs);
+        return cudaSuccess;
+    }
     CUtensorMap mp, mr, mx, mxt;
     if (!make_map_2d(&mp, p, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kRows, kUnitK,
                      CU_TENSOR_MAP_SWIZZLE_128B))
@@ -608,8 +615,6 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     prm.units = rings.units;
     prm.x_slots = rings.x_slots;
     prm.ahead = ahead_units(FULL, M, rings);
-    const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
-    const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
     const int64_t steps = (K + kUnitK - 1) / kUnitK;
     prm.pairs = (int)grid_pairs;
     prm.row_tiles = (int)row_tiles;
@@ -725,17 +730,28 @@ cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_s
                                                          max_tiles, status, stream);
 }
 
-cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
-                               int64_t N, int64_t K, int* status, cudaStream_t stream) {
+namespace {
+cudaError_t launch_or_plan(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N,
+                           int64_t K, int* status, cudaStream_t stream, tile_plan::Turns* turns) {
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);   // fast mode reads the persistent byte of a rounded nest like any other
-    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, M, N, K, status, stream);
-    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, M, N, K, status, stream);
+    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, M, N, K, status, stream, turns);
+    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, M, N, K, status, stream, turns);
     if (enc == kEncE4M3)
-        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, M, N, K, status, stream)
-                    : launch_enc<kEncE4M3, false>(x, p, r, y, M, N, K, status, stream);
-    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, M, N, K, status, stream)
-                : launch_enc<kEncE5M2, false>(x, p, r, y, M, N, K, status, stream);
+        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, M, N, K, status, stream, turns)
+                    : launch_enc<kEncE4M3, false>(x, p, r, y, M, N, K, status, stream, turns);
+    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, M, N, K, status, stream, turns)
+                : launch_enc<kEncE5M2, false>(x, p, r, y, M, N, K, status, stream, turns);
+}
+}  // namespace
+
+cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
+                               int64_t N, int64_t K, int* status, cudaStream_t stream) {
+    return launch_or_plan(mode, enc, x, p, r, y, M, N, K, status, stream, nullptr);
+}
+
+cudaError_t pair_turns(int mode, int enc, int64_t M, int64_t N, int64_t K, tile_plan::Turns* turns) {
+    return launch_or_plan(mode, enc, nullptr, nullptr, nullptr, nullptr, M, N, K, nullptr, nullptr, turns);
 }
 
 }  // namespace dps

@@ -42,8 +42,8 @@ namespace dps {
 namespace {
 
 using namespace sm100;
+using namespace tile_plan;
 
-constexpr int kTileRows = 128;   // weight rows per CTA (UMMA M)
 // K elements per pipeline stage: 128 (128-byte plane rows, the widest swizzled TMA box) where it still leaves a ring of
 // at least three or four stages, i.e. in fast mode; 64 in full mode (two planes per stage) with 64 tokens.  A ring of
 // two stages cannot cover the 1600-2150 cycles a stage load takes; halving the stage doubles the ring depth.
@@ -66,7 +66,6 @@ constexpr int kMaxAStages = 4;   // barrier array size for the A ring in tensor 
 constexpr int kZipGroups = 2;
 constexpr int kThreads = 64 + kZipGroups * 128;
 constexpr int kMaxStages = 12;
-constexpr int kMaxSplit = 8;     // portable cluster size
 
 __host__ __device__ constexpr int plane_stage_bytes(bool full, int tn) { return kTileRows * block_k(full, tn); }
 __host__ __device__ constexpr int stage_bytes(bool full, int tn) {
@@ -769,22 +768,6 @@ int forced_split() {
     return v;
 }
 
-// K split for a launch of `tiles` output tiles.  capacity[s] = CTAs that can be resident at once
-// when launched as clusters of s (clusters must fit inside one GPC, so this is not a multiple of
-// the SM count).  Measured on B200: a second wave costs more than it buys, so take the largest
-// factor (<= 8, a portable cluster) whose CTAs are all resident at once, keeping at least min_kb K
-// blocks per CTA: 4 in fast mode, 5 in full mode (4096 x 4096 at 32-64 tokens in full mode: 6 CTAs per
-// tile are 3-5 % faster than 8 with 4 blocks each, alone and inside the decode graphs; in fast mode they
-// are as fast alone and 4 % slower inside the graphs).
-int choose_split(int64_t tiles, int total_kb, const int* capacity, int min_kb) {
-    int best = 1;
-    for (int s = 2; s <= kMaxSplit; ++s) {
-        if (total_kb / s < min_kb) break;
-        if (tiles * s <= capacity[s]) best = s;
-    }
-    return best;
-}
-
 // Rows per tile where K is not split because there are more tiles of kTileRows rows than SMs.  Two CTAs fit an SM: as many tiles as
 // slots allow without another wave, and 5 % less, load the SMs evenly, where 172 tiles on 148 SMs leave one tile on most and two on
 // some.  Full mode, tiles of kTileRows rows against what this chooses, us: 10-16 tokens 22016 x 4096 (88 rows) 35.9 / 32.1, 27648 x
@@ -811,9 +794,10 @@ int low_rows(bool full, int64_t N, int64_t K, int tn) {
     return (int)rows;
 }
 
+// `plan`, where not null: nothing is launched, *plan receives the turns the launch would take.
 template <int ENC, bool FULL, int TN, bool LOW = false>
 cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
-                      int* status, cudaStream_t stream, int rows = kTileRows) {
+                      int* status, cudaStream_t stream, int rows = kTileRows, Turns* plan = nullptr) {
     constexpr int kXSlots = x_slots(FULL, false, TN);            // with a split-K mailbox in shared memory
     constexpr int kXSlotsAlone = x_slots_alone(FULL, TN);           // without one (K not split)
     constexpr int kXTile = x_tile_bytes(FULL, TN);
@@ -888,6 +872,10 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     if (split <= 0) split = choose_split((N + rows - 1) / rows * tok_tiles, total_kb, capacity, FULL ? 5 : 4);
     if (split > total_kb) split = total_kb;
     if (split > kMaxSplit) split = kMaxSplit;
+    if (plan != nullptr) {
+        *plan = turns((N + rows - 1) / rows * tok_tiles, split, capacity[1]);
+        return cudaSuccess;
+    }
     CUtensorMap mp, mr, mx;
     constexpr CUtensorMapSwizzle kPlaneSwizzle = kBlockK == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     constexpr CUtensorMapL2promotion kPromotion = CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
@@ -1099,6 +1087,16 @@ cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* 
                     : launch_enc<kEncE4M3, false>(x, p, r, y, M, N, K, status, stream);
     return full ? launch_enc<kEncE5M2, true>(x, p, r, y, M, N, K, status, stream)
                 : launch_enc<kEncE5M2, false>(x, p, r, y, M, N, K, status, stream);
+}
+
+cudaError_t tile_turns_64(int mode, int enc, int64_t M, int64_t N, int64_t K, Turns* plan) {
+    auto ask = [&](auto launch) { return launch(nullptr, nullptr, nullptr, nullptr, M, N, K, nullptr, nullptr, kTileRows, plan); };
+    const bool full = mode == DPS_MODE_FULL;
+    if (!full) enc = base_enc(enc);
+    if (enc == kEncE4M3R) return ask(launch_tn<kEncE4M3R, true, 64>);
+    if (enc == kEncE5M2R) return ask(launch_tn<kEncE5M2R, true, 64>);
+    if (enc == kEncE4M3) return full ? ask(launch_tn<kEncE4M3, true, 64>) : ask(launch_tn<kEncE4M3, false, 64>);
+    return full ? ask(launch_tn<kEncE5M2, true, 64>) : ask(launch_tn<kEncE5M2, false, 64>);
 }
 
 }  // namespace dps

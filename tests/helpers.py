@@ -1,4 +1,8 @@
 """Shared helpers for the GPU parity tests (host <-> device shuttling and the error bound)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import torch
 
@@ -49,3 +53,26 @@ def split_both(w: torch.Tensor, enc_req: int, device="cuda:0", p_out=None, r_out
 def split_on_host(w: torch.Tensor, enc: int):
     """Oracle split of a (possibly device) FP16 tensor -> numpy planes."""
     return oracle.split(to_np_words(w), enc)
+
+
+_LAUNCHES = """
+import sys, torch
+import paper_2609_34380_b200 as dps
+for case in sys.argv[1:]:
+    mode, M, N, K = map(int, case.split(","))
+    p = torch.zeros((N, K), dtype=torch.uint8, device="cuda:0")
+    x = torch.zeros((M, K), dtype=torch.float16, device="cuda:0")
+    y = dps.dps_linear(mode, dps.DPS_ENC_E4M3, x, p, p if mode else None)
+    assert dps.dps_stream_status() == dps.DPS_OK and not bool(y.any())
+    del p, x, y
+"""
+
+
+def launch_lines(cases, **env):
+    """What the library launched for dense linears of these (mode, M, N, K): the lines it prints on request, one per call
+    that the tensor-core tiles or the CTA pairs serve.  In a child process, since the library reads its knobs once."""
+    repo = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", _LAUNCHES, *(",".join(map(str, c)) for c in cases)], cwd=repo,
+                         env=dict(os.environ, DPS_DEBUG="1", PYTHONPATH=repo, **env), capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
+    return [line for line in out.stderr.splitlines() if line.startswith("[dps] ")]

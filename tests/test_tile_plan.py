@@ -1,0 +1,59 @@
+"""The border between the 64-token decode tiles and the CTA pairs on matrices with a long K, evaluated on the host with the capacities
+of a B200: the pairs serve what they were measured to be faster on, and the sizes at which they would leave much of the chip idle,
+or take a whole round for a few tiles, stay with the tiles."""
+import shutil
+import subprocess
+from pathlib import Path
+
+import pytest
+
+CSRC = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
+PROGRAM = r"""
+#include "pair_plan.h"
+#include "tile_plan.h"
+#include <cstdio>
+int main() {
+    const int pair_capacity[] = {0, 74, 33, 22, 15}, tile_capacity[] = {0, 296, 296, 270, 296, 260, 270, 210, 264};
+    long long M, N, K; int full;
+    while (scanf("%d %lld %lld %lld", &full, &M, &N, &K) == 4) {
+        const auto p = dps::pair_plan::make_plan(full, M, N, K, pair_capacity);
+        const long long pair_tiles = (N + 255) / 256 * ((M + p.tokens - 1) / p.tokens), tiles = (N + 127) / 128;
+        const int kb = full ? 64 : 128, split = dps::tile_plan::choose_split(tiles, (int)((K + kb - 1) / kb), tile_capacity, full ? 5 : 4);
+        const auto pairs = dps::tile_plan::turns(pair_tiles, p.split, pair_capacity[1]);
+        const auto alone = dps::tile_plan::turns(tiles, split, tile_capacity[1]);
+        printf("%d\n", (int)dps::tile_plan::pairs_for_long_k(pairs, alone));
+    }
+}
+"""
+# 256-row tiles: where the pairs are the faster ones
+FASTER = [*range(20, 23), *range(27, 34), *range(46, 75), *range(149, 223), *range(297, 371)]
+
+
+@pytest.fixture(scope="module")
+def ask(tmp_path_factory):
+    gxx = shutil.which("g++")
+    assert gxx
+    where = tmp_path_factory.mktemp("plan")
+    (where / "plan.cpp").write_text(PROGRAM)
+    subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "plan.cpp"), "-o", str(where / "plan")], check=True)
+
+    def run(cases):
+        out = subprocess.run([str(where / "plan")], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True)
+        return [int(v) for v in out.stdout.split()]
+    return run
+
+
+@pytest.mark.parametrize("K", [16384, 17920, 28672, 53248])
+def test_pairs_serve_a_long_k_where_they_fill_the_chip(ask, K):
+    for full in (0, 1):
+        for M in (33, 48, 64):
+            tiles = range(20, 371)
+            got = ask([(full, M, 256 * t, K) for t in tiles] + [(full, M, 256 * t - 248, K) for t in tiles])   # (8 rows in the last tile)
+            assert [t for t, g in zip(tiles, got) if g] == FASTER
+            short = [t for t, g in zip(tiles, got[len(tiles):]) if g]
+            assert set(short) <= set(FASTER) and set(range(28, 33)) | set(range(48, 73)) <= set(short)
+
+
+def test_sizes_that_lost(ask):
+    lost = [(f, 64, n, k) for f in (0, 1) for n in (8456, 10240, 11264, 19200, 20480, 28672) for k in (16384, 28672)]
+    assert not any(ask(lost))
