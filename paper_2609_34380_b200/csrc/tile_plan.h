@@ -25,6 +25,32 @@ inline int choose_split(int64_t tiles, int total_kb, const int* capacity, int mi
     return best;
 }
 
+// Rows per tile where K is not split because there are more tiles of kTileRows rows than SMs.  Two CTAs fit an SM: as many tiles as
+// slots allow without another wave, and 5 % less, load the SMs evenly, where 172 tiles on 148 SMs leave one tile on most and two on
+// some.  Full mode, tiles of kTileRows rows against what this chooses, us: 10-16 tokens 22016 x 4096 (88 rows) 35.9 / 32.1, 27648 x
+// 5120 (104) 48.2 / 45.1, 32768 x 6144 (120) 63.5 / 60.4, 57344 x 8192 (104) 156.5 / 142.5, 128256 x 4096 166 / 156.5; 32 tokens, whose
+// activations cost an SM more per tile, only where the load is most uneven: 22016 x 4096 (88) 36.5 / 33.0, but 27648 x 5120 48.5 / 48.4,
+// 57344 x 8192 158.5 / 156.5, 128256 x 4096 170 / 172.7.  Below 88 rows the K blocks' latencies show: 22016 x 4096 with 72 rows 44.
+// Fast mode, half the bytes per K block and so latencies earlier, only for 10-16 tokens, up to two waves, 96 or 104 rows and matrices
+// of 2^27 weights and more: 40000 x 4096 (96) 37.9 / 34.4, 20000 x 8192 (96) 36.5 / 35.0, 57344 x 8192 (104) 81.2 / 78.2, a layer with
+// the last of them 152.9 / 149.3; but 32768 x 6144 (120) 34.6 / 34.8, 128256 x 4096 (120) 88.3 / 93.2, and 22016 x 4096 (96), 21.0 /
+// 20.0 by itself, leaves its layer at 50.3 / 50.4.  At 32 tokens, with 96 rows: 40.3 / 37.9, 38.1 / 38.2 on the first two, 22016 x 4096
+// 21.0 / 21.4.  64-token tiles, which carry twice the activations again, lose in both modes.
+// From K = 1536 on: a shorter K is over before the even load shows, and more tiles are more fixed costs.  Full mode, 128 rows / lower, us: 24
+// tokens 22016 x 512 6.1 / 6.7, x 1024 9.5 / 10.2, x 1536 14.7 / 14.1, 41472 x 256 7.4 / 8.9, x 1536 29.4 / 26.1; 12 tokens 57344 x 768 17.3 / 19.5,
+// x 1024 21.7 / 23.7, x 1536 32.4 / 30.6, 128256 x 1024 46.0 / 47.8, x 1536 66.0 / 62.3.  (In between, 38016 x 1024 18.6 / 17.3 at 24 tokens.)
+inline int low_rows(bool full, int64_t N, int64_t K, int tn, int64_t sms) {
+    const int64_t slots = 2 * sms, tiles = (N + kTileRows - 1) / kTileRows;
+    if (tiles <= sms || K < 1536 || (!full && N * K < ((int64_t)1 << 27))) return kTileRows;
+    const int64_t waves = (tiles + slots - 1) / slots;
+    int64_t rows = (N * 20 + waves * slots * 19 - 1) / (waves * slots * 19);   // N / (0.95 of the slots)
+    rows = (rows + 7) / 8 * 8;
+    const int64_t least = full ? 88 : 96, most = full ? (tn > 16 ? 88 : 120) : 104;
+    if (rows < least) rows = least;
+    if (rows > most || (!full && (tn > 16 || waves > 2))) return kTileRows;
+    return (int)rows;
+}
+
 // A launch in turns: `rounds` times over the chip, a `split`-th of K each time.
 struct Turns {
     int64_t rounds;

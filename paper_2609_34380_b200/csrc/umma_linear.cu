@@ -768,30 +768,10 @@ int forced_split() {
     return v;
 }
 
-// Rows per tile where K is not split because there are more tiles of kTileRows rows than SMs.  Two CTAs fit an SM: as many tiles as
-// slots allow without another wave, and 5 % less, load the SMs evenly, where 172 tiles on 148 SMs leave one tile on most and two on
-// some.  Full mode, tiles of kTileRows rows against what this chooses, us: 10-16 tokens 22016 x 4096 (88 rows) 35.9 / 32.1, 27648 x
-// 5120 (104) 48.2 / 45.1, 32768 x 6144 (120) 63.5 / 60.4, 57344 x 8192 (104) 156.5 / 142.5, 128256 x 4096 166 / 156.5; 32 tokens, whose
-// activations cost an SM more per tile, only where the load is most uneven: 22016 x 4096 (88) 36.5 / 33.0, but 27648 x 5120 48.5 / 48.4,
-// 57344 x 8192 158.5 / 156.5, 128256 x 4096 170 / 172.7.  Below 88 rows the K blocks' latencies show: 22016 x 4096 with 72 rows 44.
-// Fast mode, half the bytes per K block and so latencies earlier, only for 10-16 tokens, up to two waves, 96 or 104 rows and matrices
-// of 2^27 weights and more: 40000 x 4096 (96) 37.9 / 34.4, 20000 x 8192 (96) 36.5 / 35.0, 57344 x 8192 (104) 81.2 / 78.2, a layer with
-// the last of them 152.9 / 149.3; but 32768 x 6144 (120) 34.6 / 34.8, 128256 x 4096 (120) 88.3 / 93.2, and 22016 x 4096 (96), 21.0 /
-// 20.0 by itself, leaves its layer at 50.3 / 50.4.  At 32 tokens, with 96 rows: 40.3 / 37.9, 38.1 / 38.2 on the first two, 22016 x 4096
-// 21.0 / 21.4.  64-token tiles, which carry twice the activations again, lose in both modes.
 // DPS_TILE_ROWS=64..120 pins the height.
-int low_rows(bool full, int64_t N, int64_t K, int tn) {
+int rows_of_tiles(bool full, int64_t N, int64_t K, int tn) {
     static const int forced = [] { const char* e = getenv("DPS_TILE_ROWS"); return e ? atoi(e) / 8 * 8 : 0; }();
-    if (forced >= 64 && forced < kTileRows) return forced;
-    const int64_t sms = sm_count(), slots = 2 * sms, tiles = (N + kTileRows - 1) / kTileRows;
-    if (tiles <= sms || (!full && N * K < ((int64_t)1 << 27))) return kTileRows;
-    const int64_t waves = (tiles + slots - 1) / slots;
-    int64_t rows = (N * 20 + waves * slots * 19 - 1) / (waves * slots * 19);   // N / (0.95 of the slots)
-    rows = (rows + 7) / 8 * 8;
-    const int64_t least = full ? 88 : 96, most = full ? (tn > 16 ? 88 : 120) : 104;
-    if (rows < least) rows = least;
-    if (rows > most || (!full && (tn > 16 || waves > 2))) return kTileRows;
-    return (int)rows;
+    return forced >= 64 && forced < kTileRows ? forced : low_rows(full, N, K, tn, sm_count());
 }
 
 // `plan`, where not null: nothing is launched, *plan receives the turns the launch would take.
@@ -901,8 +881,8 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     const int x_ring = xs_n * kXTile;
     const size_t smem = (size_t)stages * stage + x_ring + mail_bytes + 1024;
     if (getenv("DPS_DEBUG"))
-        fprintf(stderr, "[dps] umma TN=%d full=%d N=%lld K=%lld M=%lld stages=%d split=%d capacity=%d,%d,%d,%d,%d,%d,%d,%d\n",
-                TN, (int)FULL, (long long)N, (long long)K, (long long)M, stages, split, capacity[1], capacity[2],
+        fprintf(stderr, "[dps] umma TN=%d full=%d N=%lld K=%lld M=%lld rows=%d stages=%d split=%d capacity=%d,%d,%d,%d,%d,%d,%d,%d\n",
+                TN, (int)FULL, (long long)N, (long long)K, (long long)M, rows, stages, split, capacity[1], capacity[2],
                 capacity[3], capacity[4], capacity[5], capacity[6], capacity[7], capacity[8]);
     UmmaParams prm = {};
     prm.y = static_cast<__half*>(y);
@@ -948,7 +928,7 @@ template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
                        int* status, cudaStream_t stream) {
     if (M <= 32 && forced_split() <= 1) {
-        const int rows = low_rows(FULL, N, K, M <= 16 ? 16 : 32);
+        const int rows = rows_of_tiles(FULL, N, K, M <= 16 ? 16 : 32);
         if (rows < kTileRows && M <= 16) return launch_tn<ENC, FULL, 16, true>(x, p, r, y, M, N, K, status, stream, rows);
         if (rows < kTileRows) return launch_tn<ENC, FULL, 32, true>(x, p, r, y, M, N, K, status, stream, rows);
     }
