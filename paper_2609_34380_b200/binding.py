@@ -7,6 +7,7 @@ no CPU or PyTorch fallback.
 from __future__ import annotations
 
 import ctypes
+import hashlib
 import importlib.util
 import sysconfig
 from pathlib import Path
@@ -49,16 +50,22 @@ ABI = {
 _lib = None
 
 
+FASTCALL_SOURCE = Path(__file__).resolve().parent / "csrc" / "fastcall.cpp"
+
+
 def fastcall_path() -> Path:
     """Where the native marshalling for the PyTorch and Python of this process lives: it reads tensors by their C++
-    layout, so a binary built against another version must not be taken for it."""
-    return Path(__file__).resolve().parent / (f"_fastcall-{torch.__version__}-{str(torch.version.git_version)[:8]}-"
+    layout, so a binary built against another version must not be taken for it, nor one built from another source, whose
+    entries may be others."""
+    source = hashlib.sha256(FASTCALL_SOURCE.read_bytes()).hexdigest()[:8] if FASTCALL_SOURCE.exists() else "unknown"
+    return Path(__file__).resolve().parent / (f"_fastcall-{source}-{torch.__version__}-{str(torch.version.git_version)[:8]}-"
                                               f"{sysconfig.get_config_var('SOABI')}.so")
 
 
 FASTCALL_PATH = fastcall_path()
 
 # native marshalling (csrc/fastcall.cpp), set when the library is loaded, if it was built: dps_linear's, and the module with the others'
+_FASTCALL_ENTRIES = ("set_linear", "set_functions", "linear", "split_weights", "reconstruct", "moe_linear")
 _fast_linear = None
 _native = None
 
@@ -98,6 +105,8 @@ def _load_fastcall(lib: ctypes.CDLL) -> None:
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)
     except ImportError:
+        return
+    if not all(hasattr(module, entry) for entry in _FASTCALL_ENTRIES):      # built from an older source
         return
     module.set_linear(ctypes.cast(lib.dps_linear, ctypes.c_void_p).value)
     module.set_functions(*(ctypes.cast(fn, ctypes.c_void_p).value

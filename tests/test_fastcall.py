@@ -1,5 +1,7 @@
 """The native marshalling of dps_linear: what it does not take goes the ctypes way and is refused there as before."""
 import ctypes
+import subprocess
+import sysconfig
 import threading
 import time
 
@@ -130,6 +132,34 @@ def test_a_module_of_another_version_is_not_taken(monkeypatch):
     monkeypatch.undo()
     binding._load_fastcall(lib)
     assert binding._fast_linear is not None
+
+
+OLDER = r"""
+#include <Python.h>
+static PyObject* nothing(PyObject* self, PyObject* arg) { Py_RETURN_NONE; }
+static PyMethodDef methods[] = {{"set_linear", nothing, METH_O, 0}, {"linear", nothing, METH_O, 0}, {0, 0, 0, 0}};
+static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fastcall", 0, -1, methods};
+PyMODINIT_FUNC PyInit__fastcall(void) { return PyModule_Create(&module); }
+"""
+
+
+def test_a_module_that_lacks_an_entry_is_not_taken(monkeypatch, tmp_path):
+    lib = binding.library()
+    (tmp_path / "older.c").write_text(OLDER)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], str(tmp_path / "older.c"), "-o", str(tmp_path / "older.so")], check=True)
+    monkeypatch.setattr(binding, "_fast_linear", None)
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(binding, "fastcall_path", lambda: tmp_path / "older.so")
+    binding._load_fastcall(lib)
+    assert binding._fast_linear is None and binding._native is None
+
+
+def test_the_module_is_named_by_its_source(monkeypatch, tmp_path):
+    here = binding.fastcall_path()
+    other = tmp_path / "fastcall.cpp"
+    other.write_bytes(binding.FASTCALL_SOURCE.read_bytes() + b"\n")
+    monkeypatch.setattr(binding, "FASTCALL_SOURCE", other)
+    assert binding.fastcall_path() != here and binding.fastcall_path().parent == here.parent
 
 
 def test_other_entries_pass_on_what_they_do_not_take():
