@@ -240,16 +240,19 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             }
             __syncwarp();
         }
-    } else if (warp == 2 && lane == 0) {
-        for (int s = 0; s < x_slots; ++s) mbar_init(smem_u32(&bar_x_full[s]), 1);
-        for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 8 + 1);   // both CTAs' eight zip warps, warp 3
-        for (int a = 0; a < kDone; ++a) mbar_init(smem_u32(&bar_done[a]), 1);
-        for (int a = 0; a < 2; ++a) {
-            mbar_init(smem_u32(&bar_d_full[a]), 1);
-            mbar_init(smem_u32(&bar_d_empty[a]), 8);            // the epilogue warps of both CTAs
+    } else if (warp == 2) {
+        if (lane == 0) {
+            for (int s = 0; s < x_slots; ++s) mbar_init(smem_u32(&bar_x_full[s]), 1);
+            for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 8 + 1);   // both CTAs' eight zip warps, warp 3
+            for (int a = 0; a < kDone; ++a) mbar_init(smem_u32(&bar_done[a]), 1);
+            for (int a = 0; a < 2; ++a) {
+                mbar_init(smem_u32(&bar_d_full[a]), 1);
+                mbar_init(smem_u32(&bar_d_empty[a]), 8);            // the epilogue warps of both CTAs
+            }
+            fence_barrier_init();
+            prefetch_tensormap(&map_x);
         }
-        fence_barrier_init();
-        prefetch_tensormap(&map_x);
+        __syncwarp();             // the barriers below are .aligned: the whole warp arrives at once
     }
     if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_slot), 512);
     if (warp != 0) {

@@ -21,3 +21,18 @@ def test_only_planes_are_restrict_in_early_launched_kernels():
         marked = set(re.findall(r"__restrict__\s+(\w+)", head))
         allowed = {"P", "Rp", "x", "y"} if file == "decode_mma.cu" else {"P", "Rp"}
         assert marked <= allowed, f"{file}: {marked} in {head}"
+
+
+def test_pair_set_up_meets_again_before_its_aligned_barriers():
+    """Lane 0 of a warp initialises barriers alone; what follows (bar.sync, barrier.cluster.arrive.aligned, tcgen05.alloc) is for whole warps."""
+    text = (CSRC / "pair_linear.cu").read_text()
+    set_up = text[text.index("if (warp == 0) {\n        if (lane == 0) {"):text.index("    cluster_wait();")]
+    parted = [m.start() for m in re.finditer(r"lane == 0\)", set_up)]
+    assert len(parted) == 2
+    for at in parted:
+        after = set_up[at:]
+        meets = after.index("__syncwarp()")
+        assert all(meets < after.index(b) for b in ("named_barrier", "cluster_arrive") if b in after), after[:meets]
+    # between the second warp's set-up and the block's barrier
+    tail = set_up[parted[1]:]
+    assert tail.index("__syncwarp()") < tail.index("tmem_alloc_pair")
