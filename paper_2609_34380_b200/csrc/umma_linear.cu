@@ -365,7 +365,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     const int mma_n = GROUPED ? min(TN, (tile_tokens + 15) & ~15) : TN;
     const uint32_t idesc = umma_idesc_f16(kTileRows, mma_n);
     const int total_kb = (prm.K + kBlockK - 1) / kBlockK;
-    const int split = prm.split;
+    const int split = LOW ? 1 : prm.split;
     const int rank = (split > 1) ? (int)cluster_ctarank() : 0;   // == blockIdx.z
     // K blocks are dealt round-robin to the CTAs of the cluster: at any moment the cluster reads
     // `split` adjacent 64-byte pieces of each weight row, which DRAM serves as one longer burst.
@@ -811,6 +811,7 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
             e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
             if (e != cudaSuccess) return e;
+            if constexpr (LOW) return cudaSuccess;       // never split over K: nobody asks
             for (int s = 1; s <= kMaxSplit; ++s) {
                 cudaLaunchConfig_t q = {};
                 q.gridDim = dim3(1, 1, (unsigned)s);

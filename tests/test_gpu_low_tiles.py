@@ -51,7 +51,11 @@ def test_heights_launched():
     cases = {(1, 12, 18944, 2048): 128, (1, 12, 18952, 2048): 88, (1, 32, 22016, 1536): 88, (1, 32, 22016, 1520): 128, (1, 24, 22016, 768): 128,
              (1, 16, 57344, 1536): 104, (1, 17, 57344, 1536): 128, (1, 33, 22016, 2048): 128, (0, 13, 40000, 4096): 96, (0, 17, 40000, 4096): 128,
              (0, 13, 32760, 4096): 128, (0, 13, 38016, 3520): 128, (0, 13, 38016, 3536): 96}
-    assert heights(launch_lines(list(cases))) == list(cases.values())
+    lines = launch_lines(list(cases))
+    assert heights(lines) == list(cases.values())
+    # lower tiles never split K, so their set-up makes no occupancy queries
+    for line, rows in zip(lines, cases.values()):
+        assert line.endswith(" split=1 capacity=" + ",".join("0" * 8)) == (rows < 128), line
     assert heights(launch_lines([(1, 32, 1032, 272), (0, 16, 1032, 272)], DPS_FORCE_PATH="umma", DPS_TILE_ROWS="104")) == [104, 104]
 
 
