@@ -72,12 +72,13 @@ constexpr int kTableExperts = 256;
 
 // By the whole block: rows per expert (s_cnt, E entries, zero on entry), then by its first warp the first position and the
 // first tile of every expert, the tile list and the totals.  s_off (where not null): the first positions.
+template <int THREADS>
 __device__ __forceinline__ void list_tiles(const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E,
                                            int tile_tokens, int* s_cnt, int* s_off, int32_t* counts, int32_t* offsets,
                                            int32_t* num_tiles, int4* tiles, int* status) {
     const int tid = threadIdx.x, lane = tid & 31;
     int bad = 0;
-    for (int a = tid; a < A; a += (int)blockDim.x) {
+    for (int a = tid; a < A; a += THREADS) {
         if (row_valid(token_of_row, expert_of_row, a, T, E)) atomicAdd(&s_cnt[expert_of_row[a]], 1);
         else bad = 1;
     }
@@ -128,7 +129,7 @@ moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int 
     for (int e = tid; e < E; e += kRouteThreads) s_cnt[e] = 0;
     __syncthreads();
     sm100::grid_dependency_wait();      // the routing and, through an earlier call, the workspace are earlier kernels'
-    list_tiles(token_of_row, expert_of_row, A, T, E, tile_tokens, s_cnt, s_off, counts, offsets, num_tiles, tiles, status);
+    list_tiles<kRouteThreads>(token_of_row, expert_of_row, A, T, E, tile_tokens, s_cnt, s_off, counts, offsets, num_tiles, tiles, status);
     __syncthreads();
     if (E <= kTableExperts) {
         for (int base = 0; base < A; base += kRouteThreads) {
@@ -208,7 +209,7 @@ moe_rank_gather_kernel(const uint4* x, const int32_t* token_of_row, const int32_
         for (int e = tid; e < E; e += kRankThreads) s_cnt[e] = 0;
         __syncthreads();
         sm100::grid_dependency_wait();
-        list_tiles(token_of_row, expert_of_row, A, T, E, tile_tokens, s_cnt, nullptr, counts, offsets, num_tiles, tiles, status);
+        list_tiles<kRankThreads>(token_of_row, expert_of_row, A, T, E, tile_tokens, s_cnt, nullptr, counts, offsets, num_tiles, tiles, status);
         return;
     }
     const int a = (int)blockIdx.x - 1;
