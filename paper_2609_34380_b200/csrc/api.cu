@@ -141,9 +141,10 @@ using namespace dps;
 namespace {
 // 65-128 tokens: two 64-token decode tiles per 128 weight rows (K split over a cluster) instead of CTA pairs with 256-row
 // tiles, where the latter would leave most SMs idle and the weights are few enough to be streamed out of L2 and rebuilt
-// twice.  Measured, fast / full mode, 96-128 tokens: 4096 x 4096 10.4 / 14.1 us against 12.8 / 14.1-15.9, 2048 x 2048
-// 6.9 / 7.4 against 9.3 / 10.7, 6144 x 1024 6.9 / 8.2 against 7.9 / 9.1; 3088 x 8336 in full mode 25.2 against 20.0,
-// 4632 x 3088 16.6 / 23.1 against 12.4 / 14.5, 12288 x 4096 20.2 / 39.9 against 16.2 / 24.1.
+// twice.  Fast / full mode, tiles against pairs, us: 96 tokens 4096 x 4096 10.3 / 13.9 against 11.1 / 12.7, 2048 x 2048 6.3 / 7.4 against
+// 7.7 / 8.3, 6144 x 1024 6.6 / 8.0 against 6.7 / 7.8; 128 tokens 10.5 / 14.1 against 11.8 / 14.0, 6.4 / 7.5 against 8.3 / 9.2, 6.8 / 8.1
+// against 6.4 / 7.1 (where the tiles are a little behind the line is older than the pairs' present start); beyond the line, 96 tokens, 3088 x
+// 8336 in full mode 24.7 against 18.0, 4632 x 3088 15.4 / 22.4 against 10.8 / 12.6, 12288 x 4096 20.9 / 40.2 against 16.0 / 22.9.
 bool decode_tiles_for_128(bool full, int64_t M, int64_t N, int64_t K) {
     return M <= 128 && ((N <= 4096 && N * K <= ((int64_t)1 << (full ? 24 : 26))) || N * K <= ((int64_t)1 << 23));
 }
@@ -291,9 +292,9 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     // What the rule costs: a matrix beyond it that is called by itself.  2048 x 2048, 9 tokens, takes 4.5 us in fast and 5.4 in
     // full mode, the streaming kernel 3.4 and 3.9; 4096 x 4096 6.7 and 9.3 against 5.7 and 8.8.  With other programs' kernels
     // between the linears every launch of the tiles pays for the change of split, about 2 us: 2048 x 2048 7.0 against 4.2.
-    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for long K) CTA pairs (four Llama-7B linears, fast / full mode: 64
-    // tokens 62 / 97 us with the tiles, 75 / 109 with pairs; 96 tokens 84 / 134 against 74 / 107).  (The CUDA-core GEMV
-    // is kept as a cross-check.)
+    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for a long K, see pairs_for_64) CTA pairs.  Four linears of a layer,
+    // fast / full mode, tiles against pairs, us: Llama-7B 64 tokens 61.8 / 96.5 against 66.7 / 95.1, 96 tokens 89.0 / 147.4 against 69.6 / 98.8;
+    // hidden size 2048, 64 tokens, 29.7 / 39.8 against 35.6 / 40.8, 96 tokens 37.8 / 53.7 against 37.9 / 46.1.  (The CUDA-core GEMV is kept as a cross-check.)
     const bool stream_mid = (N < K ? N : K) <= 1536 && N * K < ((int64_t)1 << 25);
     const int path = forced_path();
     cudaError_t err;

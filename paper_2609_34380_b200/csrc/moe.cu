@@ -63,12 +63,7 @@ __device__ __forceinline__ bool row_valid(const int32_t* token_of_row, const int
     return e >= 0 && e < E && t >= 0 && t < T;
 }
 
-// One CTA.  Invalid rows belong to no group and raise the status word.  Rows are counted per expert with integer atomics
-// (the counts do not depend on their order); the grouping itself is stable without any: rows are placed 1024 at a time, a
-// row's position among its expert's rows being that of the rows placed before, of the warps before its own (a table of
-// counts per warp and expert, scanned by one thread per expert) and of the lanes before its own.  Latency-bound, one SM:
-// 4.7 us for 32 rows of 32 experts.  More than kTableExperts experts (the table's size): one warp per expert walks all rows.
-constexpr int kTableExperts = 256;
+constexpr int kTableExperts = 256;   // of the routing kernel's table
 
 // By the whole block: rows per expert (s_cnt, E entries, zero on entry), then by its first warp the first position and the
 // first tile of every expert, the tile list and the totals.  s_off (where not null): the first positions.
@@ -116,6 +111,11 @@ __device__ __forceinline__ void list_tiles(const int32_t* token_of_row, const in
     }
 }
 
+// One CTA.  Invalid rows belong to no group and raise the status word.  Rows are counted per expert with integer atomics
+// (the counts do not depend on their order); the grouping itself is stable without any: rows are placed 1024 at a time, a
+// row's position among its expert's rows being that of the rows placed before, of the warps before its own (a table of
+// counts per warp and expert, scanned by one thread per expert) and of the lanes before its own.  Latency-bound, one SM:
+// 4.7 us for 32 rows of 32 experts.  More than kTableExperts experts (the table's size): one warp per expert walks all rows.
 __global__ void __launch_bounds__(kRouteThreads)
 moe_route_kernel(const int32_t* token_of_row, const int32_t* expert_of_row, int A, int T, int E, int tile_tokens,
                  int32_t* counts, int32_t* offsets, int32_t* sorted_rows, int32_t* num_tiles, int4* tiles, int* status) {

@@ -65,7 +65,8 @@ struct PairParams {
     int ahead;         // plane units asked of L2 in front of their loads
     int split;         // K split: pairs of a cluster that share a tile, each a range of its K steps (then one tile per cluster)
     // What every warp would have to divide for in front of the first load: pairs in the grid (with a split, clusters), row tiles,
-    // (not grouped) token tiles and the tiles of whole rounds, and the K steps' quotient and remainder by the split.
+    // (not grouped) token tiles and the tiles of whole rounds, and the K steps' quotient and remainder by the split (the first
+    // ranges are a step longer).  With several token tiles, with pieces and in grouped launches an item still takes a division or two.
     int pairs, row_tiles, tok_tiles, t_main, steps_each, steps_over;
     int* status;
 };
@@ -273,9 +274,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 
     bool ok = true;
     if (warp == 0) {
-        // ---------------- plane producer (model state: does not wait for the preceding kernel) ----------------
-        // Four Llama-7B linears in a chain, fast / full mode, against a producer that waits first: 72 tokens 74.1 / 105 us
-        // against 75.6 / 109, 128 tokens 82.0 / 111.8 against 82.3 / 113.7, 512 tokens 167.5 / 215 against 167.9 / 217.
+        // ---------------- plane producer (model state: does not wait for the preceding kernel): what follows the ring above ----------------
         int s = 0;
         uint32_t ph = 1;          // a fresh barrier passes a wait for the phase before its first
         uint32_t issued = 0;

@@ -34,7 +34,9 @@ struct Plan {
 };
 
 // Time of one K step of a tile in ns, all pairs at work: measured with 74 and 148 tiles of one width (18944 and 37888 rows,
-// 8192 columns; in full mode, up to 128 tokens, on planes that come out of L2) every 32 tokens, between them in proportion.
+// 8192 columns; in full mode, up to 128 tokens, on planes that come out of L2) every 32 tokens, between them in proportion.  Measured
+// before the ring was filled ahead of the roles and, for full mode from 192 tokens on, without the L2 requests of ahead_units: it ranks
+// widths and splits, it does not predict a launch (four Llama-7B linears, 64 tokens, full mode: 72 us by it, 95 measured).
 inline double step_ns(bool full, int tokens) {
     static const double fast_ns[9] = {370, 370, 415, 480, 535, 610, 685, 750, 850};
     static const double full_ns[9] = {500, 500, 520, 600, 680, 800, 1000, 1040, 1100};
@@ -70,7 +72,7 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
             const double cost1 = step_ns(full, (int)tokens);
             p.cost = (double)rounds * ((double)steps * cost1 + drain) + 4.0 * (double)tokens;
             if (split > 1) {
-                // the sum over the cluster, measured: 1 us + 30 ns per token
+                // the sum over the cluster: 1 us + 30 ns per token (measured with a loop over the parts; it is about 0.4 us less now)
                 p.cost = (double)((steps + split - 1) / split) * cost1 + 1000.0 + 30.0 * (double)tokens;
             } else if (tail > 0) {
                 double last = (double)steps * cost1;
@@ -100,8 +102,8 @@ inline Rings size_rings(bool full, int tokens) {
 }
 
 // Plane units asked of L2 ahead of their loads.  A ring of two units (full mode, tiles of 192 tokens and more) has 64 KB per SM in
-// flight at best, and memory's latency takes more: the three units behind it are asked for too.  Up to 512 tokens, where every pair
-// streams planes of its own; with more token tiles several pairs read the same planes and it gained nothing.  Four linears in a
+// flight at best, and memory's latency takes more: the three units behind it are asked for too.  Up to 512 tokens: up to 256 every pair streams
+// planes of its own; with two token tiles two pairs read, and ask for, the same planes and it still gains, with more it gained nothing.  Four linears in a
 // chain, full mode, without / with 3 / 4 / 6 units, us: Llama-7B 192 tokens 132.8 / 121.5 / 122.2 / 124.2, 256 141 / 133.9 / 134.2 /
 // 135.8, 512 222 / 216.8 / 216.7 / 217.1; 8192-wide 256 tokens 481 / 434 / 443 / 456.  Rings of four units lose by it: 12288 x 4096 at
 // 128 tokens 24.7 / - / 25.5 in full mode, 256 tokens in fast mode 26.8 / - / 27.3.

@@ -5,12 +5,13 @@
 // residual tensor into the original FP16 values *during computation*; fast mode uses the FP8
 // tensor alone.  Here that combination happens on the way from shared memory to tensor memory.
 //
-// Tile: 128 weight rows (UMMA M) x TN tokens (UMMA N), K walked in blocks of 128 or 64.  The problem
+// Tile: 128 weight rows (UMMA M; 88 to 120 of them hold weights in the lower tiles, see low_rows in tile_plan.h) x TN tokens (UMMA N),
+// K walked in blocks of 128 or 64.  The problem
 // is "swapped": D[row][token] = sum_k W[row][k] * x[token][k], so that even a handful of decode
 // tokens fills the 128-lane datapath with weight rows and every weight byte is fetched once.
 //
 // Roles (10 warps):
-//   warp 0     TMA producer: P tile (128 rows x 128 or 64 bytes), R tile (full mode), x tile (TN rows
+//   warp 0     TMA producer: P tile (a tile's rows x 128 or 64 bytes), R tile (full mode), x tile (TN rows
 //              of 64-element swizzle atoms) into a ring of shared-memory stages, completion
 //              counted on mbarriers.  Dense tiles keep x in slots of their own, a second stream with its
 //              own barriers (see x_slots below).

@@ -1,4 +1,4 @@
-"""The native marshalling of dps_linear: what it does not take goes the ctypes way and is refused there as before."""
+"""The native marshalling: what it does not take goes the ctypes way and is refused there as before."""
 import ctypes
 import subprocess
 import sysconfig
@@ -208,3 +208,34 @@ def test_other_entries_answer_as_the_other_path_does():
             dps.dps_moe_linear(dps.DPS_MODE_FAST, [enc, enc], x, tok, exp, planes, None, **wrong)
     with pytest.raises(dps.DpsError):
         dps.dps_moe_linear(dps.DPS_MODE_FULL, [enc, 77], x, tok, exp, planes, res, workspace=ws)
+
+
+@pytest.mark.gpu
+def test_other_entries_take_the_current_stream():
+    """All three beside a busy default stream: their answers are there once their own stream is through, and they wait for what is on it."""
+    w = workloads.weights(64, 272, 3, device="cuda:0")
+    p0, r0, enc = dps.dps_split_weights(w)
+    x, token, expert = workloads.activations(5, 272, 4, device="cuda:0"), None, torch.tensor([1, 0, 1, 0, 0], dtype=torch.int32, device="cuda:0")
+    planes, res = torch.stack([p0, p0]), torch.stack([r0, r0])
+    ws = torch.empty(dps.dps_moe_workspace_bytes(5, 2, 272), dtype=torch.uint8, device="cuda:0")
+    want = dps.dps_moe_linear(dps.DPS_MODE_FULL, [enc, enc], x, token, expert, planes, res, workspace=ws)
+    side, done = torch.cuda.Stream(), torch.cuda.Event()
+    source, late, answers = torch.zeros_like(w), torch.zeros_like(x), {}
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)                    # 10 ms in front of the inputs: a call on another stream would read the zeros
+        source.copy_(w)
+        late.copy_(x)
+        answers["reconstruct"] = dps.dps_reconstruct(p0, r0, enc)
+        answers["moe"] = dps.dps_moe_linear(dps.DPS_MODE_FULL, [enc, enc], late, token, expert, planes, res, workspace=ws)
+        started = not side.query()
+        done.record()
+        p, r, got = dps.dps_split_weights(source, dps.DPS_ENC_E5M2)
+    torch.cuda._sleep(2_000_000_000)                     # a second on the default stream, which none of the answers waits for
+    side.synchronize()
+    assert started and done.query() and not torch.cuda.default_stream().query()
+    with torch.cuda.stream(side):
+        q, s, _ = dps.dps_split_weights(w, dps.DPS_ENC_E5M2, stream=side)
+        assert got == dps.DPS_ENC_E5M2 and torch.equal(p, q) and torch.equal(r, s)
+        assert torch.equal(answers["reconstruct"], w) and torch.equal(answers["moe"], want)
+    torch.cuda.synchronize()
