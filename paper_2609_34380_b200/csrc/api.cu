@@ -149,7 +149,7 @@ bool decode_tiles_for_128(bool full, int64_t M, int64_t N, int64_t K) {
     return M <= 128 && ((N <= 4096 && N * K <= ((int64_t)1 << (full ? 24 : 26))) || N * K <= ((int64_t)1 << 23));
 }
 // 33-64 tokens: CTA pairs instead of the 64-token decode tiles where K is long and the pairs take no more turns over the chip
-// (tile_plan.h: pairs_for_long_k, with what both sides take).  Fast / full mode, 64 tokens, tiles against pairs, us: 8192 x 28672 52.4 / 84.9 against 46.6 / 82.9,
+// (tile_plan.h: pairs_for_long_k, with what both sides take).  Fast / full mode, 64 tokens, tiles against pairs, us: 8192 x 28672 53.6 / 85.8 against 46.1 / 82.2,
 // 12288 x 16384 54.7 / 85.8 against 47.1 / 75.8, 38144 x 16384 147.5 / 277.8 against 132.2 / 242.5; but 6144 x 16384 27.0 / 40.2 against
 // 28.1 / 42.8, 8704 x 16384 32.8 / 51.6 against 44.7 / 66.0, 19200 x 16384 75.1 / 147.3 against 86.3 / 150.0.  With a shorter K the pairs' fixed
 // costs show: 4096 x 14336 17.1 / 25.5 against 19.6 / 27.8, 57344 x 8192 93.7 / 170 against 95.4 / 174, 10240 x 8192 24.3 / 36.3 against

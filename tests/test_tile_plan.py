@@ -1,6 +1,7 @@
-"""The height of the decode tiles, and the border between the 64-token tiles and the CTA pairs on matrices with a long K, evaluated on
-the host with the capacities of a B200.  Lower tiles only where K is long enough for their even load to show; the pairs serve what they were measured to be faster on, and the sizes at which they would leave much of the chip idle,
-or take a whole round for a few tiles, stay with the tiles."""
+"""The height of the decode tiles, and the border between the 64-token tiles and the CTA pairs on matrices with a long K, evaluated
+on the host with the capacities of a B200.  Lower tiles only where K is long enough for their even load to show; the pairs serve what
+they were measured to be faster on, and the sizes at which they would leave much of the chip idle, or take a whole round for a few
+tiles, stay with the tiles."""
 import shutil
 import subprocess
 from pathlib import Path
