@@ -192,7 +192,7 @@ moe_gather_kernel(const uint4* x, const int32_t* token_of_row, const int32_t* so
 // copies the activations there; one more block makes the tile list.  Two launches, each a chain of latencies that the next waits
 // for, become one.  The positions cost A comparisons per row, which is the longer way for many rows.  A whole call with hardly any
 // weights (256 rows x 4096, 8 experts / 256 x 2048, 64 experts), two launches against one, us: 2 rows 16.8 / 12.2 against 14.4 / 9.8,
-// 128 rows 17.1 / 13.6 against 15.0 / 11.0, 512 20.6 / 14.6 against 20.4 / 12.6, 1024 23.8 / 15.4 against 24.0 / 14.2, 2048 27.1 / 20.8
+// 128 rows 17.1 / 13.6 against 15.0 / 11.0, 512 20.6 / 14.8 against 19.2 / 12.9, 1024 23.5 / 15.6 against 23.4 / 14.4, 2048 27.1 / 20.8
 // against 31.2 / 23.3, 4096 37.6 / 28.2 against 56.7 / 47.0.
 constexpr int kRankRows = 1024;
 constexpr int kRankThreads = 256;
