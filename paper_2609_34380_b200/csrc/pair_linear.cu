@@ -125,7 +125,11 @@ __device__ __forceinline__ void rebuild(uint32_t prow, int half, uint32_t sw, ui
 }
 
 // GROUPED: a work item is a row tile of one expert x one of its token tiles; ENC is not used, the encoding is the expert's.
-template <int ENC, bool FULL, bool GROUPED>
+// WIDE: tiles of 320 or 384 tokens in two halves, an accumulator and MMAs each: what is fetched, rebuilt and stored of the weights serves half
+// as many tokens more.  74 row tiles of 8192 columns, short of the power cap, 256 -> 384 tokens, us: fast 56.8 -> 79.5, full 70.7 -> 93.0, 7 and
+// 12 % less per token.  Under the cap, where the MMAs' energy is most of it: 8192 tokens on a Llama-7B layer, full mode, tiles of 256 -> these,
+// 2973 -> 2893.  (A template argument: with the halves counted at run time in the issuer's loop 512 tokens took 2 % longer.)
+template <int ENC, bool FULL, bool GROUPED, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r,
                  const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_xt, const PairParams prm,
@@ -147,7 +151,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     const int rank = (int)(cluster_ctarank() & 1u), ks = (int)(first >> 1);
     const int pair = (int)cluster_id(), pairs = prm.pairs;      // (split > 1: the cluster)
     const int units = prm.units, x_slots = prm.x_slots;
-    const int x_atom = prm.tokens / 2 * 128, x_bytes = 2 * x_atom;   // 64 columns of K; a slot, 128
+    constexpr int kHalves = WIDE ? 2 : 1, kRing = WIDE ? kWideASteps : kASteps;
+    const int x_atom = prm.tokens / (2 * kHalves) * 128, x_bytes = prm.tokens * 128;   // 64 columns of K of a half; a slot, 128 of all
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t x_base = smem_base + (uint32_t)(units * kUnit);
     const uint32_t epi_base = x_base + (uint32_t)(x_slots * x_bytes);
@@ -244,7 +249,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     } else if (warp == 2) {
         if (lane == 0) {
             for (int s = 0; s < x_slots; ++s) mbar_init(smem_u32(&bar_x_full[s]), 1);
-            for (int a = 0; a < kASteps; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 8 + 1);   // both CTAs' eight zip warps, warp 3
+            for (int a = 0; a < kRing; ++a) mbar_init(smem_u32(&bar_a_full[a]), 2 * 8 + 1);   // both CTAs' eight zip warps, warp 3
             for (int a = 0; a < kDone; ++a) mbar_init(smem_u32(&bar_done[a]), 1);
             for (int a = 0; a < 2; ++a) {
                 mbar_init(smem_u32(&bar_d_full[a]), 1);
@@ -264,7 +269,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
     cluster_wait();               // the other CTA's barriers exist
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
-    const uint32_t tmem_a = tmem_base + kAccCols;
+    const uint32_t tmem_a = tmem_base + 512u - kRing * kACols;
     // accumulators: one or two tiles' worth
     const int accs = 2 * prm.tokens <= kAccCols ? 2 : 1;
 
@@ -306,7 +311,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         int s = 0;
         uint32_t t = 0;
         for (int i = 0; ok && work(i, w); ++i) {
-            const int half = w.tokens / 2;
+            const int halves = WIDE && !w.piece ? 2 : 1, half = w.tokens / (2 * halves);   // this CTA's share of an MMA's tokens
             const int m0 = w.m0 + rank * half;
             // (grouped: boxes of a quarter of the tile's tokens when they do)
             const bool small = GROUPED ? 4 * half <= prm.tokens : w.piece;
@@ -319,9 +324,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 if (elect_one()) {
                     const uint32_t full = map_to_cta(smem_u32(&bar_x_full[s]), first), dst = x_base + (uint32_t)(s * x_bytes);
                     // (the second CTA's bytes may land before this: the phase still waits for the one arrival)
-                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_x_full[s]), (uint32_t)(2 * 2 * box * 128));
-                    tma_load_2d_pair(dst, map, full, (step0 + j) * kUnitK, m0);
-                    tma_load_2d_pair(dst + (uint32_t)x_atom, map, full, (step0 + j) * kUnitK + 64, m0);
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_x_full[s]), (uint32_t)(2 * 2 * box * 128 * halves));
+                    for (int h = 0; h < halves; ++h) {
+                        const uint32_t to = dst + (uint32_t)(2 * h * x_atom);
+                        tma_load_2d_pair(to, map, full, (step0 + j) * kUnitK, m0 + 2 * h * half);
+                        tma_load_2d_pair(to + (uint32_t)x_atom, map, full, (step0 + j) * kUnitK + 64, m0 + 2 * h * half);
+                    }
                 }
                 __syncwarp();
             }
@@ -334,10 +342,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         uint32_t ph = 0, t = 0;
         for (int i = 0; rank == 0 && ok && work(i, w); ++i) {
             for (int j = 0; j < steps_k && ok; ++j, ++t, s = (s + 1 == x_slots) ? 0 : s + 1, ph ^= (s == 0)) {
-                if (t >= kASteps) ok = wait_done(t - kASteps);    // else the arrival might count for that step
+                if (t >= kRing) ok = wait_done(t - kRing);    // else the arrival might count for that step
                 if (ok) ok = mbar_wait(smem_u32(&bar_x_full[s]), ph);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                if (ok && lane == 0) mbar_arrive(smem_u32(&bar_a_full[t % kASteps]));
+                if (ok && lane == 0) mbar_arrive(smem_u32(&bar_a_full[t % kRing]));
             }
         }
     } else if (warp == 1) {
@@ -345,37 +353,45 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
         int xs = 0;
         uint32_t t = 0;
         for (int i = 0; rank == 0 && ok && work(i, w); ++i) {
-            const uint32_t idesc = umma_idesc_f16(2 * kRows, w.tokens);
+            const int halves = WIDE && !w.piece ? 2 : 1, n = w.tokens / halves;
+            const uint32_t idesc = umma_idesc_f16(2 * kRows, n);
             const int acc = accs == 2 ? i & 1 : 0, use = accs == 2 ? i >> 1 : i;
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * prm.tokens);
-            if (use > 0) {   // the tile before must have been read out of the accumulator by both CTAs
-                ok = mbar_wait(smem_u32(&bar_d_empty[acc]), (uint32_t)(use - 1) & 1u);
-                ok = __all_sync(0xFFFFFFFFu, ok);
-                if (!ok) break;
-                tc_fence_after_sync();
-            }
-            for (int j = 0; j < steps_k && ok; ++j, ++t) {
-                const uint32_t a = t % kASteps;
-                const uint64_t bdesc0 = umma_desc_k_sw128(x_base + (uint32_t)(xs * x_bytes));
-                const uint64_t bdesc1 = bdesc0 + (uint64_t)(x_atom >> 4);
-                const bool second = (step0 + j) * kUnitK + 64 < prm.K;        // (behind the end of K both operands are zero)
-                ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bar_a_full[a]), (t / kASteps) & 1u));
-                if (!ok) break;
-                tc_fence_after_sync();
-                if (elect_one()) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)                     // 16 columns of K = 32 bytes of the 128-byte swizzle atom
-                        umma_f16_ts_pair(tmem_d, tmem_a + a * kACols + q * 8, bdesc0 + (uint64_t)(q * 2), idesc,
-                                         (j > 0 || q > 0) ? 1u : 0u);
-                    if (second) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            umma_f16_ts_pair(tmem_d, tmem_a + a * kACols + 32 + q * 8, bdesc1 + (uint64_t)(q * 2), idesc, 1u);
-                    }
-                    umma_commit_pair(smem_u32(&bar_done[t % kDone]), first);
-                    if (j == steps_k - 1) umma_commit_pair(smem_u32(&bar_d_full[acc]), first);
+            // the tile before must have been read out of the accumulator by both CTAs
+            auto wait_empty = [&](int a) {
+                if (use > 0) {
+                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bar_d_empty[a]), (uint32_t)(use - 1) & 1u));
+                    tc_fence_after_sync();
                 }
-                __syncwarp();
+                return ok;
+            };
+            if (!wait_empty(acc)) break;
+            for (int j = 0; j < steps_k && ok; ++j, ++t) {
+                const uint32_t a = t % kRing;
+                const bool second = (step0 + j) * kUnitK + 64 < prm.K;        // (behind the end of K both operands are zero)
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bar_a_full[a]), (t / kRing) & 1u));
+                if (!ok) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int h = 0; h < kHalves; ++h) {
+                    if (h == 1 && (halves == 1 || (j == 0 && !wait_empty(1)))) break;
+                    const uint64_t bdesc0 = umma_desc_k_sw128(x_base + (uint32_t)(xs * x_bytes + 2 * h * x_atom));
+                    const uint64_t bdesc1 = bdesc0 + (uint64_t)(x_atom >> 4);
+                    const uint32_t d = tmem_d + (uint32_t)(h * n);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)                 // 16 columns of K = 32 bytes of the 128-byte swizzle atom
+                            umma_f16_ts_pair(d, tmem_a + a * kACols + q * 8, bdesc0 + (uint64_t)(q * 2), idesc, (j > 0 || q > 0) ? 1u : 0u);
+                        if (second) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                umma_f16_ts_pair(d, tmem_a + a * kACols + 32 + q * 8, bdesc1 + (uint64_t)(q * 2), idesc, 1u);
+                        }
+                        if (h == halves - 1) umma_commit_pair(smem_u32(&bar_done[t % kDone]), first);
+                        if (j == steps_k - 1) umma_commit_pair(smem_u32(&bar_d_full[acc + h]), first);
+                    }
+                    __syncwarp();
+                }
                 xs = xs + 1 == x_slots ? 0 : xs + 1;
             }
         }
@@ -407,8 +423,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                 if (lane == 0) mbar_arrive(smem_u32(&bar_p_empty[s]));
                 s += 2;
                 if (s >= (uint32_t)units) s -= (uint32_t)units, ph ^= 1u;
-                const uint32_t a = t % kASteps;
-                if (t >= kASteps) ok = __all_sync(0xFFFFFFFFu, wait_done(t - kASteps));  // the MMAs that read the slot before
+                const uint32_t a = t % kRing;
+                if (t >= kRing) ok = __all_sync(0xFFFFFFFFu, wait_done(t - kRing));  // the MMAs that read the slot before
                 if (!ok) break;
                 tc_fence_after_sync();
                 tmem_st_32x32b_x32(tmem_a + lane_base + a * kACols + (uint32_t)(half * 32), h);
@@ -428,46 +444,54 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             // grouped: the callers' row ids of the chunk's tokens, one per lane, a chunk ahead of their use
             int32_t ids = GROUPED && lane < w.ncols ? gp.sorted_rows[w.m0 + lane] : 0;
             const int acc = accs == 2 ? i & 1 : 0, use = accs == 2 ? i >> 1 : i;
-            ok = mbar_wait(smem_u32(&bar_d_full[acc]), (uint32_t)use & 1u);
-            ok = __all_sync(0xFFFFFFFFu, ok);
-            if (!ok) break;
-            tc_fence_after_sync();
+            const int halves = WIDE && !w.piece ? 2 : 1, per = w.tokens / halves;
             const uint32_t tmem_d = tmem_base + lane_base + (uint32_t)(acc * prm.tokens);
             const int n = (2 * w.row_tile + rank) * kRows + q * 32 + (lane & 3) * 8;
             __half* yrow = prm.y + (GROUPED ? (int64_t)n : (int64_t)(w.m0 + (lane >> 2)) * prm.N + n);
-            for (int c0 = 0; c0 < w.ncols; c0 += kEpiCols) {
-                uint32_t v[32];
-                tmem_ld_32x32b_x32(tmem_d + (uint32_t)c0, v);
-                int32_t next_ids = 0;
-                if (GROUPED && c0 + kEpiCols + lane < w.ncols) next_ids = gp.sorted_rows[w.m0 + c0 + kEpiCols + lane];
-                tmem_wait_ld();
-                if (c0 + kEpiCols >= w.ncols) {          // last chunk read: the accumulator is free again
+            for (int h = 0, c0 = 0; h < kHalves; ++h) {
+                if (h == halves) break;
+                ok = mbar_wait(smem_u32(&bar_d_full[acc + h]), (uint32_t)use & 1u);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                tc_fence_after_sync();
+                const int end = min(w.ncols, (h + 1) * per);
+                auto read_out = [&] {                        // the accumulator is free again
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_d_empty[acc]), first));
-                }
+                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_d_empty[acc + h]), first));
+                };
+                if (c0 >= end) read_out();                   // no token reaches this half
+                for (; c0 < end; c0 += kEpiCols) {
+                    uint32_t v[32];
+                    tmem_ld_32x32b_x32(tmem_d + (uint32_t)c0, v);
+                    int32_t next_ids = 0;
+                    if (GROUPED && c0 + kEpiCols + lane < w.ncols) next_ids = gp.sorted_rows[w.m0 + c0 + kEpiCols + lane];
+                    tmem_wait_ld();
+                    if (c0 + kEpiCols >= end) read_out();    // last chunk read
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const __half hv = __float2half_rn(__uint_as_float(v[j]) * out_scale);
-                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(buf + (uint32_t)(j * 64 + lane * 2)),
-                                 "h"(__half_as_ushort(hv))
-                                 : "memory");
-                }
-                __syncwarp();
+                    for (int j = 0; j < 32; ++j) {
+                        const __half hv = __float2half_rn(__uint_as_float(v[j]) * out_scale);
+                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(buf + (uint32_t)(j * 64 + lane * 2)),
+                                     "h"(__half_as_ushort(hv))
+                                     : "memory");
+                    }
+                    __syncwarp();
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {            // 8 tokens x 64 bytes per instruction; N is a multiple of 8
-                    const uint4 val = lds128(buf + (uint32_t)(t * 512 + lane * 16));
-                    const int64_t m = GROUPED ? __shfl_sync(0xFFFFFFFFu, ids, 8 * t + (lane >> 2)) : c0 + 8 * t;
-                    if (n < prm.N && c0 + 8 * t + (lane >> 2) < w.ncols)
-                        *reinterpret_cast<uint4*>(yrow + m * prm.N) = val;
+                    for (int t = 0; t < 4; ++t) {            // 8 tokens x 64 bytes per instruction; N is a multiple of 8
+                        const uint4 val = lds128(buf + (uint32_t)(t * 512 + lane * 16));
+                        const int64_t m = GROUPED ? __shfl_sync(0xFFFFFFFFu, ids, 8 * t + (lane >> 2)) : c0 + 8 * t;
+                        if (n < prm.N && c0 + 8 * t + (lane >> 2) < w.ncols)
+                            *reinterpret_cast<uint4*>(yrow + m * prm.N) = val;
+                    }
+                    ids = next_ids;
+                    __syncwarp();                            // the buffer is free for the next chunk
                 }
-                ids = next_ids;
-                __syncwarp();                            // the buffer is free for the next chunk
             }
+            if (!ok) break;
         }
     }
     if (!ok) atomicExch(prm.status, (int)DPS_ERR_CUDA);
-    if (split > 1) {
+    if (!WIDE && split > 1) {
         // A range of K each: the FP32 partial tile goes to shared memory, [token][row], over the rings -- the tile's MMAs are complete,
         // nothing is in flight any more.  Five warps share a quarter's columns (the epilogue's and its four zip warps).
         const bool tile = work(0, w);
@@ -546,7 +570,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K, int* status,
                        cudaStream_t stream, tile_plan::Turns* turns = nullptr) {
-    auto kernel = umma_pair_kernel<ENC, FULL, false>;
+    auto kernel = umma_pair_kernel<ENC, FULL, false, false>, wide_kernel = umma_pair_kernel<ENC, FULL, false, true>;
     // Clusters of s pairs that are resident at once, per device (they must fit inside a GPC): filled by the first call on a
     // device, read only after that set-up has returned.
     static int capacity_of[kMaxDevices][kMaxSplit + 1] = {};
@@ -556,7 +580,8 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
         const cudaError_t e = setup.run([&] {
             int d = 0;
             cudaGetDevice(&d);
-            const cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+            cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+            if (a == cudaSuccess) a = cudaFuncSetAttribute(wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
             if (a != cudaSuccess) return a;
             for (int s = 1; s <= kMaxSplit; ++s) {
                 cudaLaunchConfig_t q = {};
@@ -580,7 +605,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
         }, &dev);
         if (e != cudaSuccess) return e;
     }
-    const Plan plan = make_plan(FULL, M, N, K, capacity_of[dev]);
+    const Plan plan = make_plan(FULL, M, N, K, capacity_of[dev], true);
     const int pairs = capacity_of[dev][1];
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
     const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
@@ -596,7 +621,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     if (FULL && !make_map_2d(&mr, r, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, (uint64_t)K, kRows, kUnitK,
                              CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
-    if (!make_map_2d(&mx, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K, (uint32_t)plan.tokens / 2, 64,
+    if (!make_map_2d(&mx, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K, (uint32_t)mma_tokens(plan.tokens) / 2, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
     mxt = mx;
@@ -642,7 +667,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mp, mr, mx, mxt, prm, PairGroups{});
+    cudaError_t e = cudaLaunchKernelEx(&cfg, plan.tokens > kMaxTokens ? wide_kernel : kernel, mp, mr, mx, mxt, prm, PairGroups{});
     count_launch();
     return e;
 }
@@ -651,7 +676,7 @@ template <bool FULL>
 cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y, int64_t A,
                            int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,
                            const int32_t* sorted_rows, int max_tiles, int* status, cudaStream_t stream) {
-    auto kernel = umma_pair_kernel<0, FULL, true>;
+    auto kernel = umma_pair_kernel<0, FULL, true, false>;
     static PerDeviceOnce setup;     // per instantiation and per device
     {
         const cudaError_t e = setup.run(

@@ -20,7 +20,13 @@ constexpr int kSmemBytes = 222 * 1024;     // ring + slots + epilogue chunks + a
 // Token widths are multiples of 32: CUTLASS's atom for this instruction, SM100_MMA_F16BF16_2x1SM_TS (A in tensor memory, two
 // CTAs), admits N = 32, 64 .. 256 and nothing between; only the form with A in shared memory goes in steps of 16.
 constexpr int kTokenStep = 32;
-constexpr int kMaxTokens = 256;
+constexpr int kMaxTokens = 256;            // of one MMA
+
+// Wide tiles, two MMAs of half the tokens each per step of A: what is rebuilt and stored to tensor memory, and fetched of the planes,
+// serves half as many tokens more.  Their accumulators leave the A ring two steps.
+constexpr int kWideTokens[] = {320, 384};
+constexpr int kWideASteps = 2;
+constexpr int mma_tokens(int tokens) { return tokens > kMaxTokens ? tokens / 2 : tokens; }
 
 constexpr int unit_bytes(bool full) { return kRows * kUnitK * (full ? 2 : 1); }
 
@@ -38,65 +44,71 @@ struct Plan {
 // before the ring was filled ahead of the roles and, for full mode from 192 tokens on, without the L2 requests of ahead_units: it ranks
 // widths and splits, it does not predict a launch (four Llama-7B linears, 64 tokens, full mode: 72 us by it, 95 measured).
 inline double step_ns(bool full, int tokens) {
-    static const double fast_ns[9] = {370, 370, 415, 480, 535, 610, 685, 750, 850};
-    static const double full_ns[9] = {500, 500, 520, 600, 680, 800, 1000, 1040, 1100};
+    static const double fast_ns[13] = {370, 370, 415, 480, 535, 610, 685, 750, 850, 940, 1030, 1115, 1200};
+    static const double full_ns[13] = {500, 500, 520, 600, 680, 800, 1000, 1040, 1100, 1175, 1250, 1330, 1415};
     const double* t = full ? full_ns : fast_ns;
-    const int i = tokens >= 256 ? 7 : tokens / 32;
+    const int i = tokens >= 384 ? 11 : tokens / 32;
     return t[i] + (t[i + 1] - t[i]) * (tokens - 32 * i) / 32.0;
 }
 
 // A round of tiles over the pairs takes as long as one tile, so the number of token tiles is chosen to make the sum over the
 // rounds small; the tiles of a last, partial round are cut into pieces of the tokens if that shortens it.  Few tiles: up to
 // four pairs share each, a range of K each; capacity[s] = clusters of s pairs that are resident at once.
-// DPS_PAIR_TOKENS=1..256 (rounded up to a width there is) and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
-inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) {
+// `wide`: with tiles of kWideTokens.  DPS_PAIR_TOKENS=1..384 (rounded up to a width there is) and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
+inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity, bool wide = false) {
     static const int forced = [] { const char* e = getenv("DPS_PAIR_TOKENS"); return e ? (atoi(e) + kTokenStep - 1) / kTokenStep * kTokenStep : 0; }();
     static const int forced_split = [] { const char* e = getenv("DPS_PAIR_SPLIT"); return e ? atoi(e) : 0; }();
     const int64_t steps = (K + kUnitK - 1) / kUnitK, pairs = capacity[1];
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), t0 = (M + 255) / 256;
     Plan best;
+    auto consider = [&](int64_t tokens, int split) {
+        const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens);
+        if (split > 1 && (tiles > capacity[split] || steps < 2 * split)) return;
+        if (forced_split && split != forced_split && !(split == 1 && (tiles > capacity[forced_split] || steps < 2 * forced_split))) return;
+        const int64_t rounds = tiles / pairs, tail = split > 1 ? 1 : tiles % pairs;
+        Plan p;
+        p.split = split;
+        p.tokens = p.tail_tokens = (int)tokens;
+        // between tiles: with one accumulator the MMAs wait until it has been read out
+        const double drain = 2 * tokens <= kAccCols ? 100.0 : 3.0 * (double)mma_tokens((int)tokens);
+        const double cost1 = step_ns(full, (int)tokens);
+        p.cost = (double)rounds * ((double)steps * cost1 + drain) + 4.0 * (double)tokens;
+        if (split > 1) {
+            // the sum over the cluster: 1 us + 30 ns per token (measured with a loop over the parts; it is about 0.4 us less now)
+            p.cost = (double)((steps + split - 1) / split) * cost1 + 1000.0 + 30.0 * (double)tokens;
+        } else if (tail > 0) {
+            double last = (double)steps * cost1;
+            for (int parts = 2; rounds > 0 && parts <= 8 && parts * tail <= pairs && kTokenStep * parts <= tokens; ++parts) {
+                const int tt = (int)(((tokens + parts - 1) / parts + kTokenStep - 1) / kTokenStep * kTokenStep);
+                const double c = 1.2 * (double)steps * step_ns(full, tt) + drain;   // (the pieces stream the planes again)
+                if (c < 0.9 * last) { last = c; p.tail_parts = parts; p.tail_tokens = tt; }
+            }
+            p.cost += last;
+        }
+        if (best.cost == 0 || p.cost < best.cost) best = p;
+    };
     for (int64_t t = t0, end = t0 + (t0 < 12 ? t0 + 4 : 16); t <= end; ++t) {
         int64_t tokens = ((M + t - 1) / t + kTokenStep - 1) / kTokenStep * kTokenStep;
         if (forced >= kTokenStep && forced <= kMaxTokens) tokens = forced;
-        const int64_t tiles = row_tiles * ((M + tokens - 1) / tokens);
-        for (int split = 1; split <= kMaxSplit; ++split) {
-            if (split > 1 && (tiles > capacity[split] || steps < 2 * split)) continue;
-            if (forced_split && split != forced_split && !(split == 1 && (tiles > capacity[forced_split] || steps < 2 * forced_split)))
-                continue;
-            const int64_t rounds = tiles / pairs, tail = split > 1 ? 1 : tiles % pairs;
-            Plan p;
-            p.split = split;
-            p.tokens = p.tail_tokens = (int)tokens;
-            // between tiles: with one accumulator the MMAs wait until it has been read out
-            const double drain = 2 * tokens <= kAccCols ? 100.0 : 3.0 * (double)tokens;
-            const double cost1 = step_ns(full, (int)tokens);
-            p.cost = (double)rounds * ((double)steps * cost1 + drain) + 4.0 * (double)tokens;
-            if (split > 1) {
-                // the sum over the cluster: 1 us + 30 ns per token (measured with a loop over the parts; it is about 0.4 us less now)
-                p.cost = (double)((steps + split - 1) / split) * cost1 + 1000.0 + 30.0 * (double)tokens;
-            } else if (tail > 0) {
-                double last = (double)steps * cost1;
-                for (int parts = 2; rounds > 0 && parts <= 8 && parts * tail <= pairs && kTokenStep * parts <= tokens; ++parts) {
-                    const int tt = (int)(((tokens + parts - 1) / parts + kTokenStep - 1) / kTokenStep * kTokenStep);
-                    const double c = 1.2 * (double)steps * step_ns(full, tt) + drain;   // (the pieces stream the planes again)
-                    if (c < 0.9 * last) { last = c; p.tail_parts = parts; p.tail_tokens = tt; }
-                }
-                p.cost += last;
-            }
-            if (best.cost == 0 || p.cost < best.cost) best = p;
-        }
+        for (int split = 1; split <= kMaxSplit; ++split) consider(tokens, split);
+    }
+    if (wide && M > kMaxTokens && (forced == 0 || forced > kMaxTokens)) {
+        if (forced > kMaxTokens) best = Plan();
+        for (int tokens : kWideTokens)
+            if (forced == 0 || (forced <= 320) == (tokens == 320)) consider(tokens, 1);
     }
     return best;
 }
 
 // Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
-// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024), more if four plane units still fit; the
+// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024; three of a wide tile, whose steps are longer), more if four plane units still fit; the
 // planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen
 // by the same zip warps.
 inline Rings size_rings(bool full, int tokens) {
     const int x_bytes = tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
     int xs = (room - 4 * unit_bytes(full)) / x_bytes;
-    xs = xs < 4 ? 4 : xs > kMaxXSlots ? kMaxXSlots : xs;
+    const int least = tokens > kMaxTokens ? 3 : 4;
+    xs = xs < least ? least : xs > kMaxXSlots ? kMaxXSlots : xs;
     const int units = (room - xs * x_bytes) / unit_bytes(full);
     return {units > kMaxUnits ? kMaxUnits : units & ~1, xs};
 }
