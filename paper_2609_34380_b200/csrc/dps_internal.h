@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "../../include/dps.h"
+#include "pair_plan.h"
 #include "tile_plan.h"
 
 namespace dps {
@@ -55,16 +56,20 @@ cudaError_t launch_decode_mma(int mode, int enc, const void* x, const uint8_t* p
 
 // Dense linear, tensor-core path (tcgen05 + TMEM).  `status` receives DPS_ERR_CUDA if a bounded
 // wait inside the kernel ever gives up.
-cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y,
+cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy,
                                int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream);
 
 // Dense linear on CTA pairs (any M; meant for many tokens).
-cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
+cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M,
                                int64_t N, int64_t K, int* status, cudaStream_t stream);
 
 // What the launch of the 64-token decode tiles, of the CTA pairs, would take for this layer: for the choice between them.
 cudaError_t tile_turns_64(int mode, int enc, int64_t M, int64_t N, int64_t K, tile_plan::Turns* plan);
-cudaError_t pair_turns(int mode, int enc, int64_t M, int64_t N, int64_t K, tile_plan::Turns* turns);
+struct PairQuery {
+    tile_plan::Turns* turns;       // (each may be null)
+    pair_plan::RowShare* share;    // the rows that whole rounds of them serve
+};
+cudaError_t ask_pair_plan(int mode, int enc, int64_t M, int64_t N, int64_t K, const PairQuery& query);
 
 // Grouped linear on CTA pairs: arguments as below, `masks` the e5m2_mask array; pair_grouped_tokens: its token-tile width.
 int pair_grouped_tokens(int64_t A, int32_t E);

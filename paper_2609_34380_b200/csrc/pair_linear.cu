@@ -58,6 +58,7 @@ constexpr int kThreads = 768;
 struct PairParams {
     __half* y;
     int M, N, K;
+    int64_t ldy;       // elements from one token's row of y to the next
     int tokens;        // per tile
     int tail_tokens;   // per piece of a tile of the last, partial round
     int tail_parts;    // pieces such a tile is cut into (1: not cut)
@@ -447,7 +448,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
             const int halves = WIDE && !w.piece ? 2 : 1, per = w.tokens / halves;
             const uint32_t tmem_d = tmem_base + lane_base + (uint32_t)(acc * prm.tokens);
             const int n = (2 * w.row_tile + rank) * kRows + q * 32 + (lane & 3) * 8;
-            __half* yrow = prm.y + (GROUPED ? (int64_t)n : (int64_t)(w.m0 + (lane >> 2)) * prm.N + n);
+            __half* yrow = prm.y + (GROUPED ? (int64_t)n : (int64_t)(w.m0 + (lane >> 2)) * prm.ldy + n);
             for (int h = 0, c0 = 0; h < kHalves; ++h) {
                 if (h == halves) break;
                 ok = mbar_wait(smem_u32(&bar_d_full[acc + h]), (uint32_t)use & 1u);
@@ -481,7 +482,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                         const uint4 val = lds128(buf + (uint32_t)(t * 512 + lane * 16));
                         const int64_t m = GROUPED ? __shfl_sync(0xFFFFFFFFu, ids, 8 * t + (lane >> 2)) : c0 + 8 * t;
                         if (n < prm.N && c0 + 8 * t + (lane >> 2) < w.ncols)
-                            *reinterpret_cast<uint4*>(yrow + m * prm.N) = val;
+                            *reinterpret_cast<uint4*>(yrow + m * prm.ldy) = val;
                     }
                     ids = next_ids;
                     __syncwarp();                            // the buffer is free for the next chunk
@@ -546,7 +547,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
                     const __half2 h = __floats2half2_rn(t[2 * k], t[2 * k + 1]);
                     out[k] = *reinterpret_cast<const uint32_t*>(&h);
                 }
-                *reinterpret_cast<uint4*>(prm.y + (int64_t)(w.m0 + c) * prm.N + n) = make_uint4(out[0], out[1], out[2], out[3]);
+                *reinterpret_cast<uint4*>(prm.y + (int64_t)(w.m0 + c) * prm.ldy + n) = make_uint4(out[0], out[1], out[2], out[3]);
             }
         };
         if (tile) {
@@ -566,10 +567,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 
 // ---- host side ---------------------------------------------------------------------------------
 
-// `turns`, where not null: nothing is launched, *turns receives the turns the launch would take.
+// `query`, where not null: nothing is launched, its answers are filled in.
 template <int ENC, bool FULL>
-cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K, int* status,
-                       cudaStream_t stream, tile_plan::Turns* turns = nullptr) {
+cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N, int64_t K, int* status,
+                       cudaStream_t stream, const PairQuery* query) {
     auto kernel = umma_pair_kernel<ENC, FULL, false, false>, wide_kernel = umma_pair_kernel<ENC, FULL, false, true>;
     // Clusters of s pairs that are resident at once, per device (they must fit inside a GPC): filled by the first call on a
     // device, read only after that set-up has returned.
@@ -609,8 +610,9 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     const int pairs = capacity_of[dev][1];
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
     const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
-    if (turns != nullptr) {
-        *turns = tile_plan::turns(tiles, plan.split, pairs);
+    if (query != nullptr) {
+        if (query->turns != nullptr) *query->turns = tile_plan::turns(tiles, plan.split, pairs);
+        if (query->share != nullptr) *query->share = share_rows(FULL, M, N, K, pairs);
         return cudaSuccess;
     }
     CUtensorMap mp, mr, mx, mxt;
@@ -633,6 +635,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     prm.M = (int)M;
     prm.N = (int)N;
     prm.K = (int)K;
+    prm.ldy = ldy;
     prm.tokens = plan.tokens;
     prm.tail_tokens = plan.tail_tokens;
     prm.tail_parts = plan.tail_parts;
@@ -702,6 +705,7 @@ cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const ui
     prm.M = (int)A;
     prm.N = (int)N;
     prm.K = (int)K;
+    prm.ldy = N;
     prm.tokens = prm.tail_tokens = tn;
     prm.tail_parts = 1;
     prm.split = 1;
@@ -758,27 +762,25 @@ cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_s
 }
 
 namespace {
-cudaError_t launch_or_plan(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N,
-                           int64_t K, int* status, cudaStream_t stream, tile_plan::Turns* turns) {
+cudaError_t launch_or_plan(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N,
+                           int64_t K, int* status, cudaStream_t stream, const PairQuery* query) {
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);   // fast mode reads the persistent byte of a rounded nest like any other
-    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, M, N, K, status, stream, turns);
-    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, M, N, K, status, stream, turns);
-    if (enc == kEncE4M3)
-        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, M, N, K, status, stream, turns)
-                    : launch_enc<kEncE4M3, false>(x, p, r, y, M, N, K, status, stream, turns);
-    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, M, N, K, status, stream, turns)
-                : launch_enc<kEncE5M2, false>(x, p, r, y, M, N, K, status, stream, turns);
+    auto go = [&](auto launch) { return launch(x, p, r, y, ldy, M, N, K, status, stream, query); };
+    if (enc == kEncE4M3R) return go(launch_enc<kEncE4M3R, true>);
+    if (enc == kEncE5M2R) return go(launch_enc<kEncE5M2R, true>);
+    if (enc == kEncE4M3) return full ? go(launch_enc<kEncE4M3, true>) : go(launch_enc<kEncE4M3, false>);
+    return full ? go(launch_enc<kEncE5M2, true>) : go(launch_enc<kEncE5M2, false>);
 }
 }  // namespace
 
-cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M,
+cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M,
                                int64_t N, int64_t K, int* status, cudaStream_t stream) {
-    return launch_or_plan(mode, enc, x, p, r, y, M, N, K, status, stream, nullptr);
+    return launch_or_plan(mode, enc, x, p, r, y, ldy, M, N, K, status, stream, nullptr);
 }
 
-cudaError_t pair_turns(int mode, int enc, int64_t M, int64_t N, int64_t K, tile_plan::Turns* turns) {
-    return launch_or_plan(mode, enc, nullptr, nullptr, nullptr, nullptr, M, N, K, nullptr, nullptr, turns);
+cudaError_t ask_pair_plan(int mode, int enc, int64_t M, int64_t N, int64_t K, const PairQuery& query) {
+    return launch_or_plan(mode, enc, nullptr, nullptr, nullptr, nullptr, N, M, N, K, nullptr, nullptr, &query);
 }
 
 }  // namespace dps

@@ -100,6 +100,54 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
     return best;
 }
 
+// 17 to 128 tokens on a matrix with at least a row tile per pair: whether the pairs take it, and how many of its rows, where the rest is
+// better off as a launch of its own (decode tiles or pairs, K shared out over clusters) than as a last round that leaves most pairs idle.
+//
+// All figures are us per launch in loops of half a second, i.e. under the 1000 W cap, which is where a server runs; tiles / pairs / pairs and
+// a launch for the rest.  In T row tiles of 256 (74 pairs); what the cut gains is fitted by `cut_gain` (the round's memory time by its K
+// steps, against a launch's fixed costs and the rest's own time):
+// 33-64 tokens, full mode: T 76 K 2048 21.2 / 19.8 / 20.7, 4096 41.6 / 40.0 / 37.1, 8192 80.0 / 78.3 / 67.8; 90 (rest 16) 23.0 / 21.8 / 24.9,
+//   45.2 / 43.6 / 43.4, 87.0 / 84.4 / 78.8; 100 (26) 24.6 / 22.9 / 27.6, 47.5 / 45.3 / 46.8, 92.0 / 88.2 / 85.1; 150 40.7 / 34.4 / 35.6,
+//   76.7 / 67.7 / 64.9, 148 / 132 / 122; 190 (42) 46.1 / 40.0 / 45.4, 86.0 / 76.9 / 81.2, 168 / 149 / 149; 226 51.7 / 47.8 / 50.3, 100 / 94.7 /
+//   93.1, 193 / 186 / 178.
+// 33-64 tokens, fast mode: a wave of the tiles is 148 T, and they are the faster ones where their waves are as full as the pairs' rounds: T 76
+//   K 4096 22.2 / 23.6 / 23.2, 8192 44.0 / 46.8 / 42.0; 84 24.2 / 25.5 / 25.7, 46.5 / 49.4 / 45.4; 150 43.8 / 39.6 / 39.7, 83.4 / 77.5 / 72.6; 158
+//   45.2 / 41.7 / 42.1, 84.4 / 80.2 / 76.5; 226 56.4 / 56.9 / 56.7, 108 / 108 / 107; 296 68.4 / 67.1 / -, 133 / 136 / -; 501 119 / 118 / 119.
+// 17-32 tokens, full mode: T 76 K 4096 34.1 / 38.2 / 34.2, 8192 66.6 / 74.7 / 61.5; 90 38.0 / 40.9 / 38.1, 73.7 / 80.0 / 71.0; 100 80.5 / 83.4 / 78.3;
+//   150 61.9 / 63.3 / 60.3, 118 / 125 / 112; 158 35.9 / 33.3 / 34.7 (K 2048), 68.2 / 65.8 / 62.0, 136 / 128 / 117; 190 40.8 / 37.1 / 40.2, 78.2 /
+//   71.4 / 73.9; 226 46.5 / 45.2 / 46.9, 88.4 / 89.2 / 86.2, 173 / 173 / 163; 501 183 / 176 / 179.
+// 96 tokens, pairs / cut (a last round there is cut into pieces of the tokens): full T 76 41.7 / 39.1, 81.7 / 72.0; 84 44.7 / 45.4, 84.6 / 78.1; 158 73.3 /
+//   75.0, 142 / 136; 226 99.8 / 99.2, 197 / 193; fast 76 25.8 / 25.7, 50.3 / 46.0; 84 27.8 / 29.8, 54.1 / 52.2; 158 45.8 / 48.1, 89.2 / 86.3.
+struct RowShare {
+    bool pairs = false;      // false: as if there were no such rule
+    int64_t rows = 0;        // of y that whole rounds serve; 0: all of them, in one launch
+};
+inline double cut_gain(bool full, int64_t steps, int64_t rest) {
+    return full ? 0.244 * (double)steps - 4.5 - (double)rest * (0.10 + 0.0033 * (double)steps) : 0.15 * (double)steps - 5.0 - 0.1 * (double)rest;
+}
+// DPS_ROW_CUT=0: never, 1: wherever there is a whole round and a rest, up to 256 tokens (tuning knob).
+inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t pairs) {
+    static const int knob = [] { const char* e = getenv("DPS_ROW_CUT"); return e ? atoi(e) : -1; }();
+    const int64_t tiles = (N + 2 * kRows - 1) / (2 * kRows), steps = (K + kUnitK - 1) / kUnitK;
+    const int64_t rounds = tiles / pairs, rest = tiles % pairs, rows = rest > 0 ? rounds * pairs * 2 * kRows : 0;
+    if (knob == 0 || rounds == 0 || M <= 16 || M > kMaxTokens) return {};
+    if (knob == 1) return {true, rows};
+    const bool cut = rest > 0 && cut_gain(full, steps, rest) > 0;
+    if (M <= 64 && K >= 16384) return {};        // (a rule of its own: tile_plan.h)
+    if (M > 128) return {};
+    if (M > 64) return (rest > 0 && ((steps >= 64 && rest <= 10) || (full && steps >= 32 && rest <= 4))) ? RowShare{true, rows} : RowShare{};
+    if (rounds == 1) {
+        if (full && M > 32 && K > 2048) return {true, cut ? rows : 0};
+        const int64_t most = full ? 26 : 10;     // (fast mode: from 33 tokens on)
+        return (full || M > 32) && cut && steps >= 64 && rest <= most ? RowShare{true, rows} : RowShare{};
+    }
+    if (steps < 16) return {};
+    if (full) return {true, cut ? rows : 0};
+    if (M <= 32) return {};
+    const int64_t waves = (tiles + 2 * pairs - 1) / (2 * pairs);
+    return rounds + (rest > 0) < 2 * waves ? RowShare{true, cut ? rows : 0} : RowShare{};
+}
+
 // Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
 // (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024; three of a wide tile, whose steps are longer), more if four plane units still fit; the
 // planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen

@@ -178,6 +178,7 @@ struct GroupedParams {
 struct UmmaParams {
     __half* y;
     int M, N, K;
+    int64_t ldy;     // elements from one token's row of y to the next
     int rows;        // LOW: weight rows of a tile (a multiple of 8)
     int num_stages;
     int split;       // K split = cluster size along z; partial tiles are summed through DSMEM
@@ -678,7 +679,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
                                  : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
                                  : "r"(smem_base + (uint32_t)((c * kTileRows + q * 8) * 2)));
-                    *reinterpret_cast<uint4*>(prm.y + (int64_t)m * prm.N + n) = val;
+                    *reinterpret_cast<uint4*>(prm.y + m * prm.ldy + n) = val;
                 }
             }
         } else if (group == 0 || TN >= 32) {
@@ -745,7 +746,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
             out.y = pack_half2(acc[2], acc[3]);
             out.z = pack_half2(acc[4], acc[5]);
             out.w = pack_half2(acc[6], acc[7]);
-            *reinterpret_cast<uint4*>(prm.y + (int64_t)m * prm.N + n) = out;
+            *reinterpret_cast<uint4*>(prm.y + m * prm.ldy + n) = out;
         }
     }
     DPS_CTA_STAMP(6);
@@ -777,7 +778,7 @@ int rows_of_tiles(bool full, int64_t N, int64_t K, int tn) {
 
 // `plan`, where not null: nothing is launched, *plan receives the turns the launch would take.
 template <int ENC, bool FULL, int TN, bool LOW = false>
-cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
+cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N, int64_t K,
                       int* status, cudaStream_t stream, int rows = kTileRows, Turns* plan = nullptr) {
     constexpr int kXSlots = x_slots(FULL, false, TN);            // with a split-K mailbox in shared memory
     constexpr int kXSlotsAlone = x_slots_alone(FULL, TN);           // without one (K not split)
@@ -891,6 +892,7 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     prm.M = (int)M;
     prm.N = (int)N;
     prm.K = (int)K;
+    prm.ldy = ldy;
     prm.status = status;
     prm.num_stages = stages;
     prm.split = split;
@@ -927,17 +929,17 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
 }
 
 template <int ENC, bool FULL>
-cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
+cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N, int64_t K,
                        int* status, cudaStream_t stream) {
     if (M <= 32 && forced_split() <= 1) {
         const int rows = rows_of_tiles(FULL, N, K, M <= 16 ? 16 : 32);
-        if (rows < kTileRows && M <= 16) return launch_tn<ENC, FULL, 16, true>(x, p, r, y, M, N, K, status, stream, rows);
-        if (rows < kTileRows) return launch_tn<ENC, FULL, 32, true>(x, p, r, y, M, N, K, status, stream, rows);
+        if (rows < kTileRows && M <= 16) return launch_tn<ENC, FULL, 16, true>(x, p, r, y, ldy, M, N, K, status, stream, rows);
+        if (rows < kTileRows) return launch_tn<ENC, FULL, 32, true>(x, p, r, y, ldy, M, N, K, status, stream, rows);
     }
-    if (M <= 16) return launch_tn<ENC, FULL, 16>(x, p, r, y, M, N, K, status, stream);
-    if (M <= 32) return launch_tn<ENC, FULL, 32>(x, p, r, y, M, N, K, status, stream);
+    if (M <= 16) return launch_tn<ENC, FULL, 16>(x, p, r, y, ldy, M, N, K, status, stream);
+    if (M <= 32) return launch_tn<ENC, FULL, 32>(x, p, r, y, ldy, M, N, K, status, stream);
     // 33 tokens and more (beyond 64 only where the dispatcher prefers two 64-token tiles per 128 rows to CTA pairs)
-    return launch_tn<ENC, FULL, 64>(x, p, r, y, M, N, K, status, stream);
+    return launch_tn<ENC, FULL, 64>(x, p, r, y, ldy, M, N, K, status, stream);
 }
 
 }  // namespace
@@ -1003,6 +1005,7 @@ cudaError_t launch_grouped_tn(const uint32_t* e5m2_mask, const void* x_sorted, c
     prm.M = (int)A;
     prm.N = (int)N;
     prm.K = (int)K;
+    prm.ldy = N;
     prm.num_stages = stages;
     prm.split = 1;
     prm.red_offset = 0;
@@ -1058,21 +1061,21 @@ cudaError_t launch_umma_grouped(int mode, const uint32_t* e5m2_mask, const void*
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y,
+cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy,
                                int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream) {
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);   // fast mode reads the persistent byte of a rounded nest like any other
-    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, M, N, K, status, stream);
-    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, M, N, K, status, stream);
+    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, ldy, M, N, K, status, stream);
+    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, ldy, M, N, K, status, stream);
     if (enc == kEncE4M3)
-        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, M, N, K, status, stream)
-                    : launch_enc<kEncE4M3, false>(x, p, r, y, M, N, K, status, stream);
-    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, M, N, K, status, stream)
-                : launch_enc<kEncE5M2, false>(x, p, r, y, M, N, K, status, stream);
+        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, ldy, M, N, K, status, stream)
+                    : launch_enc<kEncE4M3, false>(x, p, r, y, ldy, M, N, K, status, stream);
+    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, ldy, M, N, K, status, stream)
+                : launch_enc<kEncE5M2, false>(x, p, r, y, ldy, M, N, K, status, stream);
 }
 
 cudaError_t tile_turns_64(int mode, int enc, int64_t M, int64_t N, int64_t K, Turns* plan) {
-    auto ask = [&](auto launch) { return launch(nullptr, nullptr, nullptr, nullptr, M, N, K, nullptr, nullptr, kTileRows, plan); };
+    auto ask = [&](auto launch) { return launch(nullptr, nullptr, nullptr, nullptr, N, M, N, K, nullptr, nullptr, kTileRows, plan); };
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);
     if (enc == kEncE4M3R) return ask(launch_tn<kEncE4M3R, true, 64>);

@@ -1,0 +1,59 @@
+"""Which rows of a matrix the CTA pairs take at 17 to 128 tokens (pair_plan.h): the rule's edges, and that a cut leaves whole tiles on one side."""
+import random
+import shutil
+import subprocess
+from pathlib import Path
+
+import pytest
+
+CSRC = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
+PROGRAM = r"""
+#include "pair_plan.h"
+#include <cstdio>
+int main() {
+    long long M, N, K; int full, pairs;
+    while (scanf("%d %lld %lld %lld %d", &full, &M, &N, &K, &pairs) == 5) {
+        const auto s = dps::pair_plan::share_rows(full, M, N, K, pairs);
+        printf("%d %lld\n", (int)s.pairs, (long long)s.rows);
+    }
+}
+"""
+ROUND = 74 * 256
+# (full, M, N, K): None: the other rules decide; 0: pairs, one launch; n: pairs up to there, the rest by itself
+EDGES = {(1, 64, ROUND - 256, 8192): None, (1, 64, ROUND, 8192): 0, (1, 64, ROUND + 8, 8192): ROUND, (1, 33, 86 * 256, 2048): None, (1, 33, 86 * 256, 2064): 0,
+         (1, 64, 86 * 256, 4096): ROUND, (1, 64, 112 * 256, 4096): 0, (1, 64, 224 * 256, 8192): 3 * ROUND, (1, 64, 75 * 256, 16384): None,
+         (1, 16, 224 * 256, 8192): None, (1, 17, 224 * 256, 8192): 3 * ROUND, (1, 17, 224 * 256, 1536): None, (1, 32, 86 * 256, 4096): None,
+         (1, 32, 86 * 256, 8192): ROUND, (0, 64, 86 * 256, 4096): None, (0, 64, 76 * 256, 8192): ROUND, (0, 64, 150 * 256, 4096): 0, (0, 64, 224 * 256, 8192): None, (0, 64, 296 * 256, 8192): None,
+         (0, 32, 224 * 256, 8192): None, (1, 96, 76 * 256, 4096): ROUND, (1, 96, 86 * 256, 4096): None, (0, 128, 224 * 256, 8192): 3 * ROUND,
+         (1, 129, 224 * 256, 8192): None}
+
+
+@pytest.fixture(scope="module")
+def ask(tmp_path_factory):
+    gxx = shutil.which("g++")
+    assert gxx
+    where = tmp_path_factory.mktemp("rows")
+    (where / "rows.cpp").write_text(PROGRAM)
+    subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "rows.cpp"), "-o", str(where / "rows")], check=True)
+
+    def run(cases, **env):
+        out = subprocess.run([str(where / "rows")], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True, env=env)
+        return [tuple(map(int, line.split())) for line in out.stdout.splitlines()]
+    return run
+
+
+def test_edges(ask):
+    for (case, want), (pairs, rows) in zip(EDGES.items(), ask([(*c, 74) for c in EDGES])):
+        assert (None if not pairs else rows) == want, case
+
+
+def test_a_cut_is_whole_rounds_and_a_rest(ask):
+    rng = random.Random(4)
+    cases = [(rng.randrange(2), int(2 ** rng.uniform(0, 10)), 8 * int(2 ** rng.uniform(0, 14.5)), 16 * int(2 ** rng.uniform(0, 11)), rng.choice((74, 66, 9))) for _ in range(4000)]
+    for env in ({}, {"DPS_ROW_CUT": "1"}):
+        cuts = 0
+        for (full, M, N, K, pairs), (taken, rows) in zip(cases, ask(cases, **env)):
+            assert not rows or (taken and 0 < rows < N and rows % (256 * pairs) == 0 and N - rows < 256 * pairs and 16 < M <= 256)
+            cuts += rows > 0
+        assert cuts > 20
+    assert all(answer == (0, 0) for answer in ask(cases, DPS_ROW_CUT="0"))
