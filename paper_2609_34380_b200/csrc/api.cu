@@ -174,7 +174,8 @@ cudaError_t launch_tensor(int32_t mode, int32_t enc, const void* x, const uint8_
 cudaError_t launch_rows(int32_t mode, int32_t enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
                         int* status, cudaStream_t stream) {
     pair_plan::RowShare share;
-    if (M > 16 && M <= pair_plan::kMaxTokens) {
+    // (a matrix of less than half a row tile per pair is never among them, and its calls are host time: they do not ask)
+    if (M > 16 && M <= pair_plan::kMaxTokens && N * 4 >= (int64_t)sm_count() * 2 * pair_plan::kRows) {
         const cudaError_t e = ask_pair_plan(mode, enc, M, N, K, {nullptr, &share});
         if (e != cudaSuccess) return e;
     }
@@ -316,7 +317,7 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     // What the rule costs: a matrix beyond it that is called by itself.  2048 x 2048, 9 tokens, takes 4.5 us in fast and 5.4 in
     // full mode, the streaming kernel 3.4 and 3.9; 4096 x 4096 6.7 and 9.3 against 5.7 and 8.8.  With other programs' kernels
     // between the linears every launch of the tiles pays for the change of split, about 2 us: 2048 x 2048 7.0 against 4.2.
-    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for a long K, see pairs_for_64) CTA pairs.  Four linears of a layer,
+    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for a long K, see pairs_for_64, from 17 on for tall matrices, see launch_rows) CTA pairs.  Four linears of a layer,
     // fast / full mode, tiles against pairs, us: Llama-7B 64 tokens 61.8 / 96.5 against 66.7 / 95.1, 96 tokens 89.0 / 147.4 against 69.6 / 98.8;
     // hidden size 2048, 64 tokens, 29.7 / 39.8 against 35.6 / 40.8, 96 tokens 37.8 / 53.7 against 37.9 / 46.1.  (The CUDA-core GEMV is kept as a cross-check.)
     const bool stream_mid = (N < K ? N : K) <= 1536 && N * K < ((int64_t)1 << 25);

@@ -100,7 +100,7 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
     return best;
 }
 
-// 17 to 128 tokens on a matrix with at least a row tile per pair: whether the pairs take it, and how many of its rows, where the rest is
+// 17 to 128 tokens: whether the pairs take a matrix, and, where it has a row tile per pair and more, how many of its rows, the rest being
 // better off as a launch of its own (decode tiles or pairs, K shared out over clusters) than as a last round that leaves most pairs idle.
 //
 // All figures are us per launch in loops of half a second, i.e. under the 1000 W cap, which is where a server runs; tiles / pairs / pairs and
@@ -109,13 +109,20 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
 // 33-64 tokens, full mode: T 76 K 2048 21.2 / 19.8 / 20.7, 4096 41.6 / 40.0 / 37.1, 8192 80.0 / 78.3 / 67.8; 90 (rest 16) 23.0 / 21.8 / 24.9,
 //   45.2 / 43.6 / 43.4, 87.0 / 84.4 / 78.8; 100 (26) 24.6 / 22.9 / 27.6, 47.5 / 45.3 / 46.8, 92.0 / 88.2 / 85.1; 150 40.7 / 34.4 / 35.6,
 //   76.7 / 67.7 / 64.9, 148 / 132 / 122; 190 (42) 46.1 / 40.0 / 45.4, 86.0 / 76.9 / 81.2, 168 / 149 / 149; 226 51.7 / 47.8 / 50.3, 100 / 94.7 /
-//   93.1, 193 / 186 / 178.
+//   93.1, 193 / 186 / 178.  With linears between them that the tiles serve, two changes of the family and a launch more cost some 3.5 us: a Llama-7B
+//   layer, T 86 and K 4096 on the pairs, 102.7 / 103.6, so one round and a rest only from K = 5120 on.
+// 33-64 tokens, less than a tile per pair, tiles / pairs, fast | full mode: T 46 K 3072 12.6 / 12.2 | 18.9 / 17.8, 8192 30.5 / 27.8 | 47.7 / 42.4; 58 14.3 /
+//   13.2 | 22.6 / 20.5, 33.1 / 31.1 | 54.2 / 47.7; 73 16.6 / 15.3 | 25.5 / 24.5, 37.3 / 35.5 | 63.1 / 57.3; but 40 11.1 / 12.0 | 16.7 / 16.7, 24.5 / 25.8 | 37.9 /
+//   39.4, and with other linears between them, which the tiles serve, each change of the family costs: with T 48 on the pairs a Llama-7B layer
+//   took 63.5 / 64.3 us in fast mode and 102.2 / 101.5 in full mode, with T 60 one of hidden size 5120 86.5 / 84.8 and 142 / 137, with T 66 one of 3088
+//   43.1 / 42.0 and 63.1 / 62.4.  So: from 0.8 of the pairs on.
 // 33-64 tokens, fast mode: a wave of the tiles is 148 T, and they are the faster ones where their waves are as full as the pairs' rounds: T 76
 //   K 4096 22.2 / 23.6 / 23.2, 8192 44.0 / 46.8 / 42.0; 84 24.2 / 25.5 / 25.7, 46.5 / 49.4 / 45.4; 150 43.8 / 39.6 / 39.7, 83.4 / 77.5 / 72.6; 158
 //   45.2 / 41.7 / 42.1, 84.4 / 80.2 / 76.5; 226 56.4 / 56.9 / 56.7, 108 / 108 / 107; 296 68.4 / 67.1 / -, 133 / 136 / -; 501 119 / 118 / 119.
 // 17-32 tokens, full mode: T 76 K 4096 34.1 / 38.2 / 34.2, 8192 66.6 / 74.7 / 61.5; 90 38.0 / 40.9 / 38.1, 73.7 / 80.0 / 71.0; 100 80.5 / 83.4 / 78.3;
 //   150 61.9 / 63.3 / 60.3, 118 / 125 / 112; 158 35.9 / 33.3 / 34.7 (K 2048), 68.2 / 65.8 / 62.0, 136 / 128 / 117; 190 40.8 / 37.1 / 40.2, 78.2 /
-//   71.4 / 73.9; 226 46.5 / 45.2 / 46.9, 88.4 / 89.2 / 86.2, 173 / 173 / 163; 501 183 / 176 / 179.
+//   71.4 / 73.9; 226 46.5 / 45.2 / 46.9, 88.4 / 89.2 / 86.2, 173 / 173 / 163; 501 183 / 176 / 179.  (In a layer of hidden size 6144, T 150 and K 6144,
+//   190 / 185; gains of less than the change of family are left.)
 // 96 tokens, pairs / cut (a last round there is cut into pieces of the tokens): full T 76 41.7 / 39.1, 81.7 / 72.0; 84 44.7 / 45.4, 84.6 / 78.1; 158 73.3 /
 //   75.0, 142 / 136; 226 99.8 / 99.2, 197 / 193; fast 76 25.8 / 25.7, 50.3 / 46.0; 84 27.8 / 29.8, 54.1 / 52.2; 158 45.8 / 48.1, 89.2 / 86.3.
 struct RowShare {
@@ -130,22 +137,27 @@ inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t p
     static const int knob = [] { const char* e = getenv("DPS_ROW_CUT"); return e ? atoi(e) : -1; }();
     const int64_t tiles = (N + 2 * kRows - 1) / (2 * kRows), steps = (K + kUnitK - 1) / kUnitK;
     const int64_t rounds = tiles / pairs, rest = tiles % pairs, rows = rest > 0 ? rounds * pairs * 2 * kRows : 0;
-    if (knob == 0 || rounds == 0 || M <= 16 || M > kMaxTokens) return {};
+    if (knob == 0 || M <= 16 || M > kMaxTokens) return {};
+    if (rounds == 0) {
+        if (M <= 32 || M > 64 || K >= 16384) return {};
+        return {5 * tiles >= 4 * pairs && K >= 3072, 0};
+    }
     if (knob == 1) return {true, rows};
     const bool cut = rest > 0 && cut_gain(full, steps, rest) > 0;
     if (M <= 64 && K >= 16384) return {};        // (a rule of its own: tile_plan.h)
     if (M > 128) return {};
     if (M > 64) return (rest > 0 && ((steps >= 64 && rest <= 10) || (full && steps >= 32 && rest <= 4))) ? RowShare{true, rows} : RowShare{};
     if (rounds == 1) {
-        if (full && M > 32 && K > 2048) return {true, cut ? rows : 0};
+        if (full && M > 32 && K >= 5120) return {true, cut ? rows : 0};
         const int64_t most = full ? 26 : 10;     // (fast mode: from 33 tokens on)
         return (full || M > 32) && cut && steps >= 64 && rest <= most ? RowShare{true, rows} : RowShare{};
     }
-    if (steps < 16) return {};
-    if (full) return {true, cut ? rows : 0};
-    if (M <= 32) return {};
-    const int64_t waves = (tiles + 2 * pairs - 1) / (2 * pairs);
-    return rounds + (rest > 0) < 2 * waves ? RowShare{true, cut ? rows : 0} : RowShare{};
+    // two rounds and more; `even`: the tiles' waves are as full as the pairs' rounds
+    const bool even = rounds + (rest > 0) >= 2 * ((tiles + 2 * pairs - 1) / (2 * pairs));
+    if (steps < (full && M > 32 ? 16 : 32)) return {};
+    if (M <= 32 && (!full || (steps < 48 && (even || rest <= 4)))) return {};
+    if (!full && even) return {};
+    return {true, cut ? rows : 0};
 }
 
 // Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least

@@ -31,8 +31,10 @@ def test_launches_at_the_edges():
     def families(mode, M, N, K):
         return [(line.split()[1], int(line.split(" N=")[1].split()[0])) for line in launch_lines([(mode, M, N, K)])]
 
-    assert families(1, 64, 86 * 256, 4096) == [("pair", ROUND), ("umma", 12 * 256)]
-    assert families(1, 64, 112 * 256, 4096) == [("pair", 112 * 256)]
+    assert families(1, 64, 86 * 256, 5120) == [("pair", ROUND), ("umma", 12 * 256)]
+    assert families(1, 64, 112 * 256, 5120) == [("pair", 112 * 256)]
     assert families(0, 64, 86 * 256, 4096) == [("umma", 86 * 256)]
     assert families(1, 24, 75 * 256, 8192) == [("pair", ROUND), ("umma", 256)]
     assert families(1, 16, 75 * 256, 8192) == [("umma", 75 * 256)]
+    assert families(0, 48, 60 * 256, 4096) == [("pair", 60 * 256)]
+    assert families(0, 48, 48 * 256, 4096) == [("umma", 48 * 256)]

@@ -20,9 +20,10 @@ int main() {
 """
 ROUND = 74 * 256
 # (full, M, N, K): None: the other rules decide; 0: pairs, one launch; n: pairs up to there, the rest by itself
-EDGES = {(1, 64, ROUND - 256, 8192): None, (1, 64, ROUND, 8192): 0, (1, 64, ROUND + 8, 8192): ROUND, (1, 33, 86 * 256, 2048): None, (1, 33, 86 * 256, 2064): 0,
-         (1, 64, 86 * 256, 4096): ROUND, (1, 64, 112 * 256, 4096): 0, (1, 64, 224 * 256, 8192): 3 * ROUND, (1, 64, 75 * 256, 16384): None,
-         (1, 16, 224 * 256, 8192): None, (1, 17, 224 * 256, 8192): 3 * ROUND, (1, 17, 224 * 256, 1536): None, (1, 32, 86 * 256, 4096): None,
+EDGES = {(1, 64, ROUND - 256, 8192): 0, (0, 33, 60 * 256, 3072): 0, (0, 33, 59 * 256, 3072): None, (1, 64, 60 * 256, 3056): None, (1, 32, 60 * 256, 8192): None,
+         (1, 65, 60 * 256, 8192): None, (0, 64, 60 * 256, 16384): None, (1, 64, ROUND, 8192): 0, (1, 64, ROUND + 8, 8192): ROUND, (1, 33, 86 * 256, 2048): None, (1, 33, 86 * 256, 4096): None,
+         (1, 64, 86 * 256, 5120): ROUND, (1, 64, 112 * 256, 5120): 0, (1, 64, 224 * 256, 8192): 3 * ROUND, (1, 64, 75 * 256, 16384): None,
+         (1, 16, 224 * 256, 8192): None, (1, 17, 224 * 256, 8192): 3 * ROUND, (1, 17, 224 * 256, 1536): None, (1, 32, 226 * 256, 4096): None, (1, 32, 158 * 256, 4096): 2 * ROUND, (1, 33, 158 * 256, 2048): 0, (0, 33, 158 * 256, 2048): None, (1, 32, 86 * 256, 4096): None,
          (1, 32, 86 * 256, 8192): ROUND, (0, 64, 86 * 256, 4096): None, (0, 64, 76 * 256, 8192): ROUND, (0, 64, 150 * 256, 4096): 0, (0, 64, 224 * 256, 8192): None, (0, 64, 296 * 256, 8192): None,
          (0, 32, 224 * 256, 8192): None, (1, 96, 76 * 256, 4096): ROUND, (1, 96, 86 * 256, 4096): None, (0, 128, 224 * 256, 8192): 3 * ROUND,
          (1, 129, 224 * 256, 8192): None}
