@@ -255,11 +255,8 @@ cudaError_t launch_moe(int mode, const int32_t* enc_host, const void* x, const i
                        int64_t T, int64_t N, int64_t K, int32_t E, void* workspace, int* status,
                        cudaStream_t stream) {
     const Workspace w = carve(workspace, A, E, K);
-    // CTA pairs from 48 rows per expert on; below, 128-row tiles of two CTAs per SM, which divide few experts' rows more
-    // evenly (measured per call, gate/up + down: Mixtral experts, 64 tokens, fast mode 284 us with the tiles against 290 with
-    // pairs, 4 tokens in full mode 219 / 229; 256 tokens 314 / 309 in fast and 532 / 512 in full mode, 1024 tokens 758 / 675,
-    // 2048 in full mode 2167 / 1969).
-    const bool pairs = A >= 48 * (int64_t)E;
+    // CTA pairs or 128-row tiles, two CTAs per SM: pair_plan.h
+    const bool pairs = pair_plan::grouped_on_pairs(mode == DPS_MODE_FULL, A, N, K, E, sm_count() / 2);
     const int tn = pairs ? pair_grouped_tokens(A, E) : grouped_tile_tokens(A, E);
     cudaError_t err;
     // programmatic dependent launch, as the kernel behind them: each is resident early and waits before its first read

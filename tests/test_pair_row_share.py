@@ -10,8 +10,11 @@ CSRC = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
 PROGRAM = r"""
 #include "pair_plan.h"
 #include <cstdio>
-int main() {
+int main(int argc, char**) {
     long long M, N, K; int full, pairs;
+    int E;
+    while (argc > 1 && scanf("%d %lld %lld %lld %d %d", &full, &M, &N, &K, &E, &pairs) == 6)      // (M rows over E experts)
+        printf("%d 0\n", (int)dps::pair_plan::grouped_on_pairs(full, M, N, K, E, pairs));
     while (scanf("%d %lld %lld %lld %d", &full, &M, &N, &K, &pairs) == 5) {
         const auto s = dps::pair_plan::share_rows(full, M, N, K, pairs);
         printf("%d %lld\n", (int)s.pairs, (long long)s.rows);
@@ -37,8 +40,8 @@ def ask(tmp_path_factory):
     (where / "rows.cpp").write_text(PROGRAM)
     subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "rows.cpp"), "-o", str(where / "rows")], check=True)
 
-    def run(cases, **env):
-        out = subprocess.run([str(where / "rows")], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True, env=env)
+    def run(cases, *argv, **env):
+        out = subprocess.run([str(where / "rows"), *argv], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True, env=env)
         return [tuple(map(int, line.split())) for line in out.stdout.splitlines()]
     return run
 
@@ -58,3 +61,11 @@ def test_a_cut_is_whole_rounds_and_a_rest(ask):
             cuts += rows > 0
         assert cuts > 20
     assert all(answer == (0, 0) for answer in ask(cases, DPS_ROW_CUT="0"))
+
+
+def test_grouped_launches_on_pairs(ask):
+    # (full, rows, N, K, experts)
+    edges = {(0, 48 * 8, 4096, 64, 8): 1, (0, 47 * 8, 4096, 14336, 8): 0, (0, 20 * 8, 28672, 4096, 8): 1, (0, 20 * 8 - 1, 28672, 4096, 8): 0,
+             (1, 12 * 8, 28672, 4096, 8): 1, (1, 12 * 8 - 1, 28672, 4096, 8): 0, (1, 30 * 8, 4096, 14336, 8): 0, (0, 30 * 4, 4096, 8192, 4): 1,
+             (0, 30 * 4, 4096, 3056, 4): 0, (0, 30 * 8, 264, 8192, 8): 0, (0, 30 * 64, 2816, 2048, 64): 1, (1, 30 * 8, 2816, 8192, 8): 0, (1, 30 * 4, 16384, 4096, 4): 0}
+    assert [pairs for pairs, _ in ask([(*c, 74) for c in edges], "grouped")] == list(edges.values())
