@@ -85,7 +85,9 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
             }
             p.cost += last;
         }
-        if (best.cost == 0 || p.cost < best.cost) best = p;
+        // (wide tiles instead of others only for 3 % and more: four Llama-7B linears, 2048 tokens, fast mode, 0.6 % by this, 647 -> 661 us measured)
+        const bool first_wide = tokens > kMaxTokens && best.tokens <= kMaxTokens;
+        if (best.cost == 0 || p.cost < (first_wide ? 0.97 : 1.0) * best.cost) best = p;
     };
     for (int64_t t = t0, end = t0 + (t0 < 12 ? t0 + 4 : 16); t <= end; ++t) {
         int64_t tokens = ((M + t - 1) / t + kTokenStep - 1) / kTokenStep * kTokenStep;
