@@ -193,23 +193,37 @@ inline int grouped_tokens(int64_t A, int32_t E) {
     return tokens < kTokenStep ? kTokenStep : tokens > kMaxTokens ? kMaxTokens : tokens;
 }
 
-// Grouped launches: CTA pairs or 128-row tiles, two CTAs per SM.  From 48 rows per expert on pairs, whose tiles are wide enough for an expert's rows.  Below,
-// with a token tile per expert, it is turns over the chip again: a wave of the tiles is two rounds of the pairs, T row tiles of 256 over all
-// experts, and the pairs win where fewer rounds do, or as many of them as make fixed costs small.  Tiles / pairs, us per call under the power cap,
-// 16 / 24 / 40 rows per expert, fast | full mode (full mode at 12 rows):
-//   T 896 (8 x 28672 x 4096) 178 / 186, 194 / 188, 209 / 208 | 335 / 322, 340 / 328, 350 / 330, 357 / 349; 768 (16 x 12288 x 2048) 85.9 / 82.9, 93.3 / 85.8,
-//   104 / 92.9 | 151 / 144, 155 / 142, 158 / 146, 164 / 159; 512 (64 x 2048 x 1408) 47.3 / 45.5, 53.2 / 46.6, 59.0 / 53.4 | 78.6 / 71.1, 81.6 / 72.6, 83.5 /
-//   74.8, 90.9 / 82.4; 64 (4 x 4096 x 8192) 38.3 / 36.1, 42.7 / 36.9, 44.0 / 38.2 | 75.1 / 57.0, 76.5 / 57.1, 70.3 / 57.7, 71.5 / 59.1;
-//   as many rounds: 704 (64 x 2816 x 2048, ten) 83.0 / 81.3, 92.0 / 83.3, 99.5 / 96.4 | 143 / 136, 143 / 137, 149 / 140, 158 / 151; but 128 (8 x 4096 x 14336, two)
-//   91.5 / 100, 99.6 / 105, 114 / 115 | 174 / 173, 174 / 174, 181 / 176, 189 / 187; 256 (4 x 16384 x 4096, four) 53.6 / 59.5, 59.6 / 59.8, 65.2 / 67.4 | 102 / 101,
-//   101 / 102, 102 / 103, 107 / 110; 88 (8 x 2816 x 8192, two, the second nearly empty) 43.7 / 57.6, 49.8 / 56.7, 53.4 / 59.4 | 85.4 / 91.5, 86.5 / 91.9, 83.0 / 92.3,
-//   88.0 / 94.9.  Fast mode with fewer than 20 rows: 12 rows 168 / 176, 83.8 / 84.7, 46.5 / 44.3; eight rows lose in both modes.
+// Grouped launches: CTA pairs or 128-row tiles, two CTAs per SM.  From 48 rows per expert on pairs, whose tiles are wide enough for an expert's rows.
+// Below, with a token tile per expert, it is turns over the chip: the pairs go in rounds of a 256-row tile each; a wave of the other tiles, as many
+// as CTA slots, takes as long as two rounds and counts for two turns.  (An expert whose rows end in the first half of a 256-row tile is half a tile
+// more work for the pairs: 32 experts of 1152 rows are three rounds of 160 tiles, or one wave of 288.)  The pairs win where rounds are fewer than
+// turns, and from eight rounds on, which make fixed costs small, whatever the turns, that are then an eighth fewer at most.
+// Tiles / pairs, us per call in loops, i.e. under the power cap, by rows per expert:
+//   experts x N x K  rounds turns | fast mode: 16         24          40          | full mode: 12 or 13  16          24          40
+//    8 x 28672 x 4096    13    14 |    178 / 186    194 / 188   209 / 208   |     335 / 322   340 / 328   350 / 330   357 / 349
+//   16 x 12288 x 2048    11    12 |   85.9 / 82.9  93.3 / 85.8   104 / 92.9 |     151 / 144   155 / 142   158 / 146   164 / 159
+//   64 x 2048 x 1408      7     8 |   47.3 / 45.5  53.2 / 46.6  59.0 / 53.4 |    78.6 / 71.1 81.6 / 72.6 83.5 / 74.8 90.9 / 82.4
+//    4 x 4096 x 8192      1     2 |   38.3 / 36.1  42.7 / 36.9  44.0 / 38.2 |    75.1 / 57.0 76.5 / 57.1 70.3 / 57.7 71.5 / 59.1
+//    8 x 4096 x 14336     2     2 |   91.5 / 100   99.6 / 105    114 / 115  |     174 / 173   174 / 174   181 / 176   189 / 187
+//    8 x 2816 x 8192      2     2 |   43.7 / 57.6  49.8 / 56.7  53.4 / 59.4 |    85.4 / 91.5 86.5 / 91.9 83.0 / 92.3 88.0 / 94.9
+//    4 x 16384 x 4096     4     4 |   53.6 / 59.5  59.6 / 59.8  65.2 / 67.4 |     102 / 101   101 / 102   102 / 103   107 / 110
+//   64 x 2816 x 2048     10    10 |   83.0 / 81.3  92.0 / 83.3  99.5 / 96.4 |     143 / 136   143 / 137   149 / 140   158 / 151
+//   32 x 1152 x 2048      3     2 |                24.6 / 28.8  26.4 / 31.8 |    37.0 / 42.7             39.8 / 44.4 41.2 / 46.5
+//    8 x 4736 x 4096      3     2 |                38.0 / 45.1  39.5 / 47.9 |    60.0 / 73.2             61.4 / 73.7 64.8 / 76.8
+//   64 x 1152 x 2048      5     4 |                43.8 / 44.6  49.8 / 52.6 |    68.4 / 69.9             71.3 / 72.5 77.4 / 80.0
+//   16 x 6976 x 1024      7     6 |                33.0 / 32.0  36.5 / 36.9 |    48.6 / 49.3             51.6 / 49.7 54.3 / 54.1
+//   64 x 1664 x 2048      7     6 |                59.2 / 58.4  66.3 / 67.4 |    91.8 / 94.6             96.8 / 97.6  103 / 105
+//   32 x 4736 x 1024      9     8 |                44.4 / 41.5  49.4 / 47.2 |    65.0 / 62.8             69.2 / 65.7 72.6 / 70.1
+//   64 x 2880 x 2048     11    10 |                94.2 / 90.0   105 / 104  |     151 / 149               154 / 151   164 / 163
+//   256 x 1152 x 1024    18    16 |                 103 / 91.0   124 / 111  |     130 / 123               141 / 134   157 / 156
+// Fast mode with fewer than 20 rows: 12 rows on the first three 168 / 176, 83.8 / 84.7, 46.5 / 44.3; eight rows lose in both modes.
 inline bool grouped_on_pairs(bool full, int64_t A, int64_t N, int64_t K, int32_t E, int64_t pairs) {
     if (A >= 48 * (int64_t)E) return true;
     if (A < (full ? 12 : 20) * (int64_t)E) return false;
-    const int64_t tiles = E * ((N + 2 * kRows - 1) / (2 * kRows)), rounds = (tiles + pairs - 1) / pairs, waves = (tiles + 2 * pairs - 1) / (2 * pairs);
+    const int64_t tiles = E * ((N + 2 * kRows - 1) / (2 * kRows)), rounds = (tiles + pairs - 1) / pairs;
+    const int64_t half_tiles = E * ((N + kRows - 1) / kRows), turns = 2 * ((half_tiles + 4 * pairs - 1) / (4 * pairs));
     if (rounds == 1) return 5 * tiles >= 4 * pairs && K >= 3072;      // (as dense launches: share_rows)
-    return rounds < 2 * waves || rounds >= 8;
+    return rounds < turns || rounds >= 8;
 }
 
 }  // namespace pair_plan

@@ -69,3 +69,17 @@ def test_grouped_launches_on_pairs(ask):
              (1, 12 * 8, 28672, 4096, 8): 1, (1, 12 * 8 - 1, 28672, 4096, 8): 0, (1, 30 * 8, 4096, 14336, 8): 0, (0, 30 * 4, 4096, 8192, 4): 1,
              (0, 30 * 4, 4096, 3056, 4): 0, (0, 30 * 8, 264, 8192, 8): 0, (0, 30 * 64, 2816, 2048, 64): 1, (1, 30 * 8, 2816, 8192, 8): 0, (1, 30 * 4, 16384, 4096, 4): 0}
     assert [pairs for pairs, _ in ask([(*c, 74) for c in edges], "grouped")] == list(edges.values())
+
+
+def test_grouped_launches_count_the_turns_of_either_kernel(ask):
+    """Below eight rounds no shape goes to the pairs that the tiles of 128 rows serve in as many turns or fewer, each counted as its kernel cuts the rows."""
+    cases = [(full, 30 * E, N, K, E) for full in (0, 1) for E in (4, 8, 12, 16, 32, 64, 100, 256) for N in [*range(8, 512, 56), *range(512, 8193, 32)] for K in (1024, 8192)]
+    given = 0
+    for (full, A, N, K, E), (pairs, _) in zip(cases, ask([(*c, 74) for c in cases], "grouped"), strict=True):
+        rounds, turns = -(-E * -(-N // 256) // 74), 2 * -(-E * -(-N // 128) // (4 * 74))
+        assert rounds == 1 or rounds >= 8 or pairs == (rounds < turns), (full, A, N, K, E)
+        given += pairs
+    assert given > len(cases) // 4
+    # three rounds against a wave; seven against three; the same with a shape that fills its tiles; eleven against five waves
+    edges = {(0, 24 * 32, 1152, 2048, 32): 0, (1, 13 * 8, 4736, 4096, 8): 0, (1, 24 * 16, 6976, 1024, 16): 0, (1, 24 * 16, 7168, 1024, 16): 1, (0, 24 * 64, 2880, 2048, 64): 1}
+    assert [pairs for pairs, _ in ask([(*c, 74) for c in edges], "grouped")] == list(edges.values())
