@@ -63,7 +63,7 @@ __device__ __forceinline__ bool row_valid(const int32_t* token_of_row, const int
     return e >= 0 && e < E && t >= 0 && t < T;
 }
 
-constexpr int kTableExperts = 256;   // of the routing kernel's table
+constexpr int kTableExperts = pair_plan::kRoutedByTable;   // of the routing kernel's table
 
 // By the whole block: rows per expert (s_cnt, E entries, zero on entry), then by its first warp the first position and the
 // first tile of every expert, the tile list and the totals.  s_off (where not null): the first positions.

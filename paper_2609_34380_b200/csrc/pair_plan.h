@@ -217,9 +217,14 @@ inline int grouped_tokens(int64_t A, int32_t E) {
 //   64 x 2880 x 2048     11    10 |                94.2 / 90.0   105 / 104  |     151 / 149               154 / 151   164 / 163
 //   256 x 1152 x 1024    18    16 |                 103 / 91.0   124 / 111  |     130 / 123               141 / 134   157 / 156
 // Fast mode with fewer than 20 rows: 12 rows on the first three 168 / 176, 83.8 / 84.7, 46.5 / 44.3; eight rows lose in both modes.
+// More than kRoutedByTable experts: the routing kernel, which then has a warp walk all rows for each expert, is most of a call, and lives on the L1
+// cache.  A launch of pairs leaves the SMs split for its 222 KB of shared memory, and the next call's routing reads through what is left: 512 experts of
+// 384 x 1024 with 24 rows each, fast mode, calls back to back, 799 / 1372 (routing alone 800 / 1270, calls with waits between them 830 / 830); 1024 of 128 x 1024
+// 3742 / 5260; 13 rows, full mode, 481 / 777 and 1600 / 2820.
+constexpr int kRoutedByTable = 256;
 inline bool grouped_on_pairs(bool full, int64_t A, int64_t N, int64_t K, int32_t E, int64_t pairs) {
     if (A >= 48 * (int64_t)E) return true;
-    if (A < (full ? 12 : 20) * (int64_t)E) return false;
+    if (A < (full ? 12 : 20) * (int64_t)E || E > kRoutedByTable) return false;
     const int64_t tiles = E * ((N + 2 * kRows - 1) / (2 * kRows)), rounds = (tiles + pairs - 1) / pairs;
     const int64_t half_tiles = E * ((N + kRows - 1) / kRows), turns = 2 * ((half_tiles + 4 * pairs - 1) / (4 * pairs));
     if (rounds == 1) return 5 * tiles >= 4 * pairs && K >= 3072;      // (as dense launches: share_rows)

@@ -83,3 +83,8 @@ def test_grouped_launches_count_the_turns_of_either_kernel(ask):
     # three rounds against a wave; seven against three; the same with a shape that fills its tiles; eleven against five waves
     edges = {(0, 24 * 32, 1152, 2048, 32): 0, (1, 13 * 8, 4736, 4096, 8): 0, (1, 24 * 16, 6976, 1024, 16): 0, (1, 24 * 16, 7168, 1024, 16): 1, (0, 24 * 64, 2880, 2048, 64): 1}
     assert [pairs for pairs, _ in ask([(*c, 74) for c in edges], "grouped")] == list(edges.values())
+
+
+def test_grouped_launches_with_a_long_routing_stay_on_the_tiles(ask):
+    edges = {(0, 24 * 256, 1152, 1024, 256): 1, (0, 24 * 257, 1152, 1024, 257): 0, (1, 13 * 512, 384, 1024, 512): 0, (0, 47 * 1024, 128, 1024, 1024): 0, (0, 48 * 512, 384, 1024, 512): 1}
+    assert [pairs for pairs, _ in ask([(*c, 74) for c in edges], "grouped")] == list(edges.values())
