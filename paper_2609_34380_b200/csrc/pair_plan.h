@@ -105,35 +105,77 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
 // 17 to 128 tokens: whether the pairs take a matrix, and, where it has a row tile per pair and more, how many of its rows, the rest being
 // better off as a launch of its own (decode tiles or pairs, K shared out over clusters) than as a last round that leaves most pairs idle.
 //
-// All figures are us per launch in loops of half a second, i.e. under the 1000 W cap, which is where a server runs; tiles / pairs / pairs and
-// a launch for the rest.  In T row tiles of 256 (74 pairs); what the cut gains is fitted by `cut_gain` (the round's memory time by its K
-// steps, against a launch's fixed costs and the rest's own time):
-// 33-64 tokens, full mode: T 76 K 2048 21.2 / 19.8 / 20.7, 4096 41.6 / 40.0 / 37.1, 8192 80.0 / 78.3 / 67.8; 90 (rest 16) 23.0 / 21.8 / 24.9,
-//   45.2 / 43.6 / 43.4, 87.0 / 84.4 / 78.8; 100 (26) 24.6 / 22.9 / 27.6, 47.5 / 45.3 / 46.8, 92.0 / 88.2 / 85.1; 150 40.7 / 34.4 / 35.6,
-//   76.7 / 67.7 / 64.9, 148 / 132 / 122; 190 (42) 46.1 / 40.0 / 45.4, 86.0 / 76.9 / 81.2, 168 / 149 / 149; 226 51.7 / 47.8 / 50.3, 100 / 94.7 /
-//   93.1, 193 / 186 / 178.  With linears between them that the tiles serve, two changes of the family and a launch more cost some 3.5 us: a Llama-7B
-//   layer, T 86 and K 4096 on the pairs, 102.7 / 103.6, so one round and a rest only from K = 5120 on.
-// 33-64 tokens, less than a tile per pair, tiles / pairs, fast | full mode: T 46 K 3072 12.6 / 12.2 | 18.9 / 17.8, 8192 30.5 / 27.8 | 47.7 / 42.4; 58 14.3 /
-//   13.2 | 22.6 / 20.5, 33.1 / 31.1 | 54.2 / 47.7; 73 16.6 / 15.3 | 25.5 / 24.5, 37.3 / 35.5 | 63.1 / 57.3; but 40 11.1 / 12.0 | 16.7 / 16.7, 24.5 / 25.8 | 37.9 /
-//   39.4, and with other linears between them, which the tiles serve, each change of the family costs: with T 48 on the pairs a Llama-7B layer
-//   took 63.5 / 64.3 us in fast mode and 102.2 / 101.5 in full mode, with T 60 one of hidden size 5120 86.5 / 84.8 and 142 / 137, with T 66 one of 3088
-//   43.1 / 42.0 and 63.1 / 62.4.  So: from 0.8 of the pairs on.
-// 33-64 tokens, fast mode: a wave of the tiles is 148 T, and they are the faster ones where their waves are as full as the pairs' rounds: T 76
-//   K 4096 22.2 / 23.6 / 23.2, 8192 44.0 / 46.8 / 42.0; 84 24.2 / 25.5 / 25.7, 46.5 / 49.4 / 45.4; 150 43.8 / 39.6 / 39.7, 83.4 / 77.5 / 72.6; 158
-//   45.2 / 41.7 / 42.1, 84.4 / 80.2 / 76.5; 226 56.4 / 56.9 / 56.7, 108 / 108 / 107; 296 68.4 / 67.1 / -, 133 / 136 / -; 501 119 / 118 / 119.
-// 17-32 tokens, full mode: T 76 K 4096 34.1 / 38.2 / 34.2, 8192 66.6 / 74.7 / 61.5; 90 38.0 / 40.9 / 38.1, 73.7 / 80.0 / 71.0; 100 80.5 / 83.4 / 78.3;
-//   150 61.9 / 63.3 / 60.3, 118 / 125 / 112; 158 35.9 / 33.3 / 34.7 (K 2048), 68.2 / 65.8 / 62.0, 136 / 128 / 117; 190 40.8 / 37.1 / 40.2, 78.2 /
-//   71.4 / 73.9; 226 46.5 / 45.2 / 46.9, 88.4 / 89.2 / 86.2, 173 / 173 / 163; 501 183 / 176 / 179.  (In a layer of hidden size 6144, T 150 and K 6144,
-//   190 / 185; gains of less than the change of family are left.)
-// 96 tokens, pairs / cut (a last round there is cut into pieces of the tokens): full T 76 41.7 / 39.1, 81.7 / 72.0; 84 44.7 / 45.4, 84.6 / 78.1; 158 73.3 /
-//   75.0, 142 / 136; 226 99.8 / 99.2, 197 / 193; fast 76 25.8 / 25.7, 50.3 / 46.0; 84 27.8 / 29.8, 54.1 / 52.2; 158 45.8 / 48.1, 89.2 / 86.3.
+// All figures are us per launch in loops of a third of a second, i.e. under the 1000 W cap, which is where a server runs; T: row tiles of 256 (74
+// pairs), (r): of them behind whole rounds; tiles / pairs / pairs and a launch for the rest (the cut).
+//
+// 33-64 tokens, full mode          K = 2048               4096                 8192                 14336
+//   T  76  (2)             21.2 / 19.8 / 20.7   41.6 / 40.0 / 37.1   80.0 / 78.3 / 67.8
+//   T  78  (4)                                                       81.2 / 78.9 / 69.0    146 /  139 /  118
+//   T  90 (16)             23.0 / 21.8 / 24.9   45.2 / 43.6 / 43.4   87.0 / 84.4 / 78.8    156 /  146 /  134
+//   T 100 (26)             24.6 / 22.9 / 27.6   47.5 / 45.3 / 46.8   92.0 / 88.2 / 85.1    165 /  152 /  143
+//   T 109 (35)                                                       99.0 / 92.4 / 95.2    172 /  159 /  163
+//   T 119 (45)                                                        104 / 95.3 / 99.0    180 /  167 /  168
+//   T 125 (51)                                                        106 / 98.2 /  108    185 /  173 /  188
+//   T 150  (2)             40.7 / 34.4 / 35.6   76.7 / 67.7 / 64.9    148 /  132 /  122
+//   T 152  (4)                                                        150 /  134 /  123    265 /  232 /  212
+//   T 164 (16)                                                        156 /  140 /  134    284 /  241 /  228
+//   T 174 (26)                                                        160 /  141 /  140    282 /  244 /  245
+//   T 183 (35)                                                        163 /  144 /  152    286 /  254 /  258
+//   T 190 (42)             46.1 / 40.0 / 45.4   86.0 / 76.9 / 81.2    168 /  149 /  149
+//   T 199 (51)                                                        170 /  152 /  163    301 /  276 /  283
+//   T 226  (4)             51.7 / 47.8 / 50.3    100 / 94.7 / 93.1    193 /  186 /  178
+//   With linears between them that the tiles serve, two changes of the family and a launch more cost some 3.5 us: a Llama-7B layer, T 86 and
+//   K 4096 on the pairs, 102.7 / 103.6, so one round and a rest only from K = 5120 on.
+// 33-64 tokens, fast mode; a wave of the tiles is 148 T, and they are the faster ones where their waves are as full as the pairs' rounds
+//   T  76  (2)                                  22.2 / 23.6 / 23.2   44.0 / 46.8 / 42.0
+//   T  84 (10)                                  24.2 / 25.5 / 25.7   46.5 / 49.4 / 45.4
+//   T 152  (4)                                  43.8 / 40.0 / 40.0   84.9 / 80.1 / 74.2    143 /  135 /  125
+//   T 159 (11)                                  45.8 / 42.0 / 42.7   86.7 / 83.2 / 79.0    147 /  138 /  129
+//   T 168 (20)                                  47.0 / 43.2 / 45.0   88.6 / 85.0 / 83.1    150 /  146 /  136
+//   T 178 (30)                                  49.0 / 45.7 / 47.2   92.1 / 87.9 / 87.8    156 /  151 /  144
+//   T 188 (40)                                  50.3 / 46.8 / 50.0   95.0 / 90.9 / 93.5    160 /  156 /  157
+//   T 198 (50)                                  51.4 / 49.0 / 53.8   97.5 / 94.0 /  101    159 /  160 /  168
+//   T 208 (60)                                  53.6 / 50.8 / 55.2    104 / 98.2 /  103    174 /  169 /  175
+//   T 221 (73)                                  56.0 / 52.4 / 57.0    108 /  103 /  106    180 /  178 /  183
+//   T 226  (4)                                  56.4 / 56.9 / 56.7    108 /  108 /  107
+//   T 296  (0)                                  68.4 / 67.1           133 /  136
+// 17-32 tokens, full mode
+//   T  76  (2)                                  34.1 / 38.2 / 34.2   66.6 / 74.7 / 61.5
+//   T  90 (16)                                  38.0 / 40.9 / 38.1   73.7 / 80.0 / 71.0
+//   T 100 (26)                                                       80.5 / 83.4 / 78.3
+//   T 150  (2)                                  61.9 / 63.3 / 60.3    118 /  125 /  112
+//   T 158 (10)             35.9 / 33.3 / 34.7   68.2 / 65.8 / 62.0    136 /  128 /  116    238 /  223 /  198
+//   T 178 (30)                                                        143 /  135 /  131    254 /  229 /  220
+//   T 190 (42)             40.8 / 37.1 / 40.2   78.2 / 71.4 / 73.9
+//   T 193 (45)                                                        154 /  142 /  142    266 /  241 /  243
+//   T 226  (4)             46.5 / 45.2 / 46.9   88.4 / 89.2 / 86.2    173 /  173 /  163
+//   (In a layer of hidden size 6144, T 150 and K 6144, 190 / 185.)
+// 33-64 tokens, less than a tile per pair, tiles / pairs: fast mode       full mode
+//   T 40                    K = 3072 11.1 / 12.0, 8192 24.5 / 25.8    3072 16.7 / 16.7, 8192 37.9 / 39.4
+//   T 46                             12.6 / 12.2       30.5 / 27.8         18.9 / 17.8       47.7 / 42.4
+//   T 58                             14.3 / 13.2       33.1 / 31.1         22.6 / 20.5       54.2 / 47.7
+//   T 73                             16.6 / 15.3       37.3 / 35.5         25.5 / 24.5       63.1 / 57.3
+//   With other linears between them, which the tiles serve, each change of the family costs: with T 48 on the pairs a Llama-7B layer took 63.5 / 64.3
+//   in fast mode and 102.2 / 101.5 in full mode, with T 60 one of hidden size 5120 86.5 / 84.8 and 142 / 137, with T 66 one of 3088 43.1 / 42.0 and
+//   63.1 / 62.4.  So: from 0.8 of the pairs on.
+// 96 tokens, pairs / cut (a last round there is cut into pieces of the tokens), K 4096, 8192: full mode T 76 41.7 / 39.1, 81.7 / 72.0; 84 44.7 /
+//   45.4, 84.6 / 78.1; 158 73.3 / 75.0, 142 / 136; 226 99.8 / 99.2, 197 / 193; fast mode 76 25.8 / 25.7, 50.3 / 46.0; 84 27.8 / 29.8, 54.1 / 52.2;
+//   158 45.8 / 48.1, 89.2 / 86.3.
 struct RowShare {
     bool pairs = false;      // false: as if there were no such rule
     int64_t rows = 0;        // of y that whole rounds serve; 0: all of them, in one launch
 };
-inline double cut_gain(bool full, int64_t steps, int64_t rest) {
-    return full ? 0.244 * (double)steps - 4.5 - (double)rest * (0.10 + 0.0033 * (double)steps) : 0.15 * (double)steps - 5.0 - 0.1 * (double)rest;
+// What the cut gains over one launch of pairs, us, fitted to the tables: a round's memory time by its K steps, less a launch's fixed costs and the
+// rest's own time, which grows with the K steps as well.  The fits are off by a microsecond or two, so a gain of less is none.
+constexpr double kLeastGain = 1.5;
+inline double cut_gain(bool full, int64_t M, int64_t steps, int64_t rest) {
+    const double s = (double)steps, r = (double)rest;
+    if (!full) return 0.15 * s - 3.5 - r * 0.0033 * s;
+    return M > 32 ? 0.244 * s - 4.5 - r * (0.10 + 0.0033 * s) : 0.35 * s - 7.0 - r * 0.006 * s;
 }
+// The rest's row tiles at most (of 74 pairs): beyond, its decode tiles are too many to share K out over clusters five ways (33-64 tokens, full mode)
+// or four ways, and a round of the pairs is as good.
+inline int64_t most_rest(bool full, int64_t M) { return full && M > 32 ? 26 : 37; }
 // DPS_ROW_CUT=0: never, 1: wherever there is a whole round and a rest, up to 256 tokens (tuning knob).
 inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t pairs) {
     static const int knob = [] { const char* e = getenv("DPS_ROW_CUT"); return e ? atoi(e) : -1; }();
@@ -145,14 +187,14 @@ inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t p
         return {5 * tiles >= 4 * pairs && K >= 3072, 0};
     }
     if (knob == 1) return {true, rows};
-    const bool cut = rest > 0 && cut_gain(full, steps, rest) > 0;
+    const bool cut = rest > 0 && rest <= most_rest(full, M) && cut_gain(full, M, steps, rest) > kLeastGain;
     if (M <= 64 && K >= 16384) return {};        // (a rule of its own: tile_plan.h)
     if (M > 128) return {};
     if (M > 64) return (rest > 0 && ((steps >= 64 && rest <= 10) || (full && steps >= 32 && rest <= 4))) ? RowShare{true, rows} : RowShare{};
     if (rounds == 1) {
         if (full && M > 32 && K >= 5120) return {true, cut ? rows : 0};
-        const int64_t most = full ? 26 : 10;     // (fast mode: from 33 tokens on)
-        return (full || M > 32) && cut && steps >= 64 && rest <= most ? RowShare{true, rows} : RowShare{};
+        // (fast mode: from 33 tokens on, and against the tiles, which are the faster ones here)
+        return (full || M > 32) && cut && steps >= 64 && rest <= (full ? 26 : 10) ? RowShare{true, rows} : RowShare{};
     }
     // two rounds and more; `even`: the tiles' waves are as full as the pairs' rounds
     const bool even = rounds + (rest > 0) >= 2 * ((tiles + 2 * pairs - 1) / (2 * pairs));

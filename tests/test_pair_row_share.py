@@ -88,3 +88,22 @@ def test_grouped_launches_count_the_turns_of_either_kernel(ask):
 def test_grouped_launches_with_a_long_routing_stay_on_the_tiles(ask):
     edges = {(0, 24 * 256, 1152, 1024, 256): 1, (0, 24 * 257, 1152, 1024, 257): 0, (1, 13 * 512, 384, 1024, 512): 0, (0, 47 * 1024, 128, 1024, 1024): 0, (0, 48 * 512, 384, 1024, 512): 1}
     assert [pairs for pairs, _ in ask([(*c, 74) for c in edges], "grouped")] == list(edges.values())
+
+
+def test_a_rest_is_cut_off_only_where_that_was_measured_to_pay(ask):
+    """As measured (the table beside the rule): the rests that a launch of their own makes slower stay, those that gain 2 us and more are cut off."""
+    pays = [(0, 64, 2, 4, 8192), (0, 64, 2, 4, 14336), (0, 64, 2, 11, 8192), (0, 64, 2, 20, 8192), (0, 64, 2, 20, 14336), (0, 64, 2, 30, 14336), (1, 64, 1, 4, 8192), (1, 64, 1, 16, 8192), (1, 64, 1, 26, 8192), (1, 64, 1, 26, 14336),
+            (1, 64, 2, 16, 14336), (1, 24, 2, 10, 8192), (1, 24, 2, 30, 8192), (1, 24, 2, 30, 14336)]
+    loses = [(0, 64, 2, r, K) for r in (40, 50, 60, 73) for K in (4096, 8192, 14336)] + [(0, 64, 2, r, 4096) for r in (4, 11, 20, 30)]
+    loses += [(1, 64, n, r, K) for n in (1, 2) for r in (35, 45, 51) for K in (8192, 14336)] + [(1, 24, 2, 45, K) for K in (8192, 14336)]
+    for cases, cut in ((pays, True), (loses, False)):
+        for (full, M, rounds, rest, K), (pairs, rows) in zip(cases, ask([(f, M, (74 * n + r) * 256 - 96, K, 74) for f, M, n, r, K in cases])):
+            assert pairs and (rows > 0) == cut, (full, M, rounds, rest, K)
+    # anywhere else: never most of a round, and with as many K steps never a longer rest where a shorter one stays
+    for full in (0, 1):
+        for M in (17, 32, 33, 64):
+            for n in (1, 2, 5):
+                for K in (2048, 4096, 8192, 12288, 16368):
+                    rows = [r for taken, r in ask([(full, M, (74 * n + rest) * 256, K, 74) for rest in range(1, 74)]) if taken]
+                    longest = sum(r > 0 for r in rows)
+                    assert all(r > 0 for r in rows[:longest]) and longest <= 37, (full, M, n, K, longest)
