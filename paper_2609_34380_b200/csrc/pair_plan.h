@@ -150,11 +150,12 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
 //   T 193 (45)                                                        154 /  142 /  142    266 /  241 /  243
 //   T 226  (4)             46.5 / 45.2 / 46.9   88.4 / 89.2 / 86.2    173 /  173 /  163
 //   (In a layer of hidden size 6144, T 150 and K 6144, 190 / 185.)
-// 33-64 tokens, less than a tile per pair, tiles / pairs: fast mode       full mode
+// 33-64 tokens, a tile per pair at most, tiles / pairs: fast mode       full mode
 //   T 40                    K = 3072 11.1 / 12.0, 8192 24.5 / 25.8    3072 16.7 / 16.7, 8192 37.9 / 39.4
 //   T 46                             12.6 / 12.2       30.5 / 27.8         18.9 / 17.8       47.7 / 42.4
 //   T 58                             14.3 / 13.2       33.1 / 31.1         22.6 / 20.5       54.2 / 47.7
 //   T 73                             16.6 / 15.3       37.3 / 35.5         25.5 / 24.5       63.1 / 57.3
+//   T 74                             16.9 / 15.7       39.1 / 36.3         26.6 / 24.8  5104 49.4 / 40.5
 //   With other linears between them, which the tiles serve, each change of the family costs: with T 48 on the pairs a Llama-7B layer took 63.5 / 64.3
 //   in fast mode and 102.2 / 101.5 in full mode, with T 60 one of hidden size 5120 86.5 / 84.8 and 142 / 137, with T 66 one of 3088 43.1 / 42.0 and
 //   63.1 / 62.4.  So: from 0.8 of the pairs on.
@@ -182,7 +183,7 @@ inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t p
     const int64_t tiles = (N + 2 * kRows - 1) / (2 * kRows), steps = (K + kUnitK - 1) / kUnitK;
     const int64_t rounds = tiles / pairs, rest = tiles % pairs, rows = rest > 0 ? rounds * pairs * 2 * kRows : 0;
     if (knob == 0 || M <= 16 || M > kMaxTokens) return {};
-    if (rounds == 0) {
+    if (tiles <= pairs) {
         if (M <= 32 || M > 64 || K >= 16384) return {};
         return {5 * tiles >= 4 * pairs && K >= 3072, 0};
     }

@@ -107,3 +107,13 @@ def test_a_rest_is_cut_off_only_where_that_was_measured_to_pay(ask):
                     rows = [r for taken, r in ask([(full, M, (74 * n + rest) * 256, K, 74) for rest in range(1, 74)]) if taken]
                     longest = sum(r > 0 for r in rows)
                     assert all(r > 0 for r in rows[:longest]) and longest <= 37, (full, M, n, K, longest)
+
+
+def test_a_tile_for_every_pair_is_one_round(ask):
+    """74 row tiles, every pair busy: the rule of 60 to 73, not that of a round and a rest."""
+    for full in (0, 1):
+        for M in (33, 64):
+            for N in (ROUND - 248, ROUND - 96, ROUND):
+                cases = [(full, M, N, K, 74) for K in (3056, 3072, 4096, 5104, 8192, 14336)]
+                assert ask(cases) == [(0, 0)] + [(1, 0)] * 5, (full, M, N)
+    assert ask([(f, M, ROUND, K, 74) for f in (0, 1) for M in (17, 32, 65, 128) for K in (4096, 8192)]) == [(0, 0)] * 16
