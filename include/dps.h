@@ -37,7 +37,8 @@
  *   - Every device base pointer must be 16-byte aligned; K must be a multiple of 16 and
  *     N a multiple of 8.  Violations return DPS_ERR_ALIGN / DPS_ERR_SHAPE.
  *   - The return value reports host-detectable errors only; on error nothing has been
- *     enqueued.  Data-dependent problems found on the device (an expert or token index
+ *     enqueued (DPS_ERR_CUDA from a call that is several launches: what the CUDA runtime
+ *     accepted before it refused a later launch has been).  Data-dependent problems found on the device (an expert or token index
  *     out of range) set a per-device status word: the offending row is skipped, its
  *     output row is left untouched, and dps_stream_status() reports DPS_ERR_DATA.
  *   - No exception crosses this boundary.  Calls on distinct streams are thread-safe.

@@ -9,6 +9,7 @@
 
 #include "bits.cuh"
 #include "dps_internal.h"
+#include "two_launches.h"
 
 namespace dps {
 
@@ -163,10 +164,10 @@ bool pairs_for_64(int32_t mode, int32_t enc, int64_t M, int64_t N, int64_t K) {
 }
 // More than a handful of tokens on rows of one matrix: decode tiles or CTA pairs.
 cudaError_t launch_tensor(int32_t mode, int32_t enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N,
-                          int64_t K, int* status, cudaStream_t stream) {
+                          int64_t K, int* status, cudaStream_t stream, bool prepare_only = false) {
     const bool pairs = M > 64 ? !decode_tiles_for_128(mode == DPS_MODE_FULL, M, N, K) : pairs_for_64(mode, enc, M, N, K);
-    return pairs ? launch_pair_linear(mode, enc, x, p, r, y, ldy, M, N, K, status, stream)
-                 : launch_umma_linear(mode, enc, x, p, r, y, ldy, M, N, K, status, stream);
+    return pairs ? launch_pair_linear(mode, enc, x, p, r, y, ldy, M, N, K, status, stream, prepare_only)
+                 : launch_umma_linear(mode, enc, x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
 }
 // The same for a whole matrix: the rows of whole rounds of pairs first, where the rest is better off by itself (pair_plan.h: share_rows).  The
 // second launch depends on the first for nothing but the order; its planes are on their way while the first drains.  Two layers of hidden
@@ -181,10 +182,12 @@ cudaError_t launch_rows(int32_t mode, int32_t enc, const void* x, const uint8_t*
     }
     if (!share.pairs) return launch_tensor(mode, enc, x, p, r, y, N, M, N, K, status, stream);
     const int64_t rows = share.rows > 0 ? share.rows : N;
-    const cudaError_t e = launch_pair_linear(mode, enc, x, p, r, y, N, M, rows, K, status, stream);
-    if (e != cudaSuccess || rows == N) return e;
-    return launch_tensor(mode, enc, x, p + rows * K, r != nullptr ? r + rows * K : nullptr, static_cast<uint16_t*>(y) + rows, N, M, N - rows, K, status,
-                         stream);
+    auto whole_rounds = [&] { return launch_pair_linear(mode, enc, x, p, r, y, N, M, rows, K, status, stream); };
+    if (rows == N) return whole_rounds();
+    return launch_two(whole_rounds, [&](bool prepare_only) {
+        return launch_tensor(mode, enc, x, p + rows * K, r != nullptr ? r + rows * K : nullptr, static_cast<uint16_t*>(y) + rows, N, M, N - rows, K, status,
+                             stream, prepare_only);
+    });
 }
 bool known_encoding(int32_t enc) {
     return enc == DPS_ENC_E4M3 || enc == DPS_ENC_E5M2 || enc == DPS_ENC_E4M3_RN || enc == DPS_ENC_E5M2_RN;

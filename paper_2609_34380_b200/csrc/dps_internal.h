@@ -56,12 +56,13 @@ cudaError_t launch_decode_mma(int mode, int enc, const void* x, const uint8_t* p
 
 // Dense linear, tensor-core path (tcgen05 + TMEM).  `status` receives DPS_ERR_CUDA if a bounded
 // wait inside the kernel ever gives up.
+// prepare_only: all that can fail in front of the launch, and no launch.
 cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy,
-                               int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream);
+                               int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream, bool prepare_only = false);
 
 // Dense linear on CTA pairs (any M; meant for many tokens).
 cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M,
-                               int64_t N, int64_t K, int* status, cudaStream_t stream);
+                               int64_t N, int64_t K, int* status, cudaStream_t stream, bool prepare_only = false);
 
 // What the launch of the 64-token decode tiles, of the CTA pairs, would take for this layer: for the choice between them.
 cudaError_t tile_turns_64(int mode, int enc, int64_t M, int64_t N, int64_t K, tile_plan::Turns* plan);

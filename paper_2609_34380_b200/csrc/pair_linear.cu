@@ -567,10 +567,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constan
 
 // ---- host side ---------------------------------------------------------------------------------
 
-// `query`, where not null: nothing is launched, its answers are filled in.
+// `query`, where not null: nothing is launched, its answers are filled in.  prepare_only: all but the launch.
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N, int64_t K, int* status,
-                       cudaStream_t stream, const PairQuery* query) {
+                       cudaStream_t stream, const PairQuery* query, bool prepare_only) {
     auto kernel = umma_pair_kernel<ENC, FULL, false, false>, wide_kernel = umma_pair_kernel<ENC, FULL, false, true>;
     // Clusters of s pairs that are resident at once, per device (they must fit inside a GPC): filled by the first call on a
     // device, read only after that set-up has returned.
@@ -631,6 +631,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     if (plan.tail_parts > 1 && !make_map_2d(&mxt, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K,
                                             (uint32_t)plan.tail_tokens / 2, 64, CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
+    if (prepare_only) return cudaSuccess;
     PairParams prm = {};
     prm.y = static_cast<__half*>(y);
     prm.M = (int)M;
@@ -764,10 +765,10 @@ cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_s
 
 namespace {
 cudaError_t launch_or_plan(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N,
-                           int64_t K, int* status, cudaStream_t stream, const PairQuery* query) {
+                           int64_t K, int* status, cudaStream_t stream, const PairQuery* query, bool prepare_only) {
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);   // fast mode reads the persistent byte of a rounded nest like any other
-    auto go = [&](auto launch) { return launch(x, p, r, y, ldy, M, N, K, status, stream, query); };
+    auto go = [&](auto launch) { return launch(x, p, r, y, ldy, M, N, K, status, stream, query, prepare_only); };
     if (enc == kEncE4M3R) return go(launch_enc<kEncE4M3R, true>);
     if (enc == kEncE5M2R) return go(launch_enc<kEncE5M2R, true>);
     if (enc == kEncE4M3) return full ? go(launch_enc<kEncE4M3, true>) : go(launch_enc<kEncE4M3, false>);
@@ -776,12 +777,12 @@ cudaError_t launch_or_plan(int mode, int enc, const void* x, const uint8_t* p, c
 }  // namespace
 
 cudaError_t launch_pair_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M,
-                               int64_t N, int64_t K, int* status, cudaStream_t stream) {
-    return launch_or_plan(mode, enc, x, p, r, y, ldy, M, N, K, status, stream, nullptr);
+                               int64_t N, int64_t K, int* status, cudaStream_t stream, bool prepare_only) {
+    return launch_or_plan(mode, enc, x, p, r, y, ldy, M, N, K, status, stream, nullptr, prepare_only);
 }
 
 cudaError_t ask_pair_plan(int mode, int enc, int64_t M, int64_t N, int64_t K, const PairQuery& query) {
-    return launch_or_plan(mode, enc, nullptr, nullptr, nullptr, nullptr, N, M, N, K, nullptr, nullptr, &query);
+    return launch_or_plan(mode, enc, nullptr, nullptr, nullptr, nullptr, N, M, N, K, nullptr, nullptr, &query, false);
 }
 
 }  // namespace dps

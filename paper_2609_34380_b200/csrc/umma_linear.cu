@@ -776,10 +776,10 @@ int rows_of_tiles(bool full, int64_t N, int64_t K, int tn) {
     return forced >= 64 && forced < kTileRows ? forced : low_rows(full, N, K, tn, sm_count());
 }
 
-// `plan`, where not null: nothing is launched, *plan receives the turns the launch would take.
+// `plan`, where not null: nothing is launched, *plan receives the turns the launch would take.  prepare_only: all but the launch.
 template <int ENC, bool FULL, int TN, bool LOW = false>
 cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N, int64_t K,
-                      int* status, cudaStream_t stream, int rows = kTileRows, Turns* plan = nullptr) {
+                      int* status, cudaStream_t stream, bool prepare_only, int rows = kTileRows, Turns* plan = nullptr) {
     constexpr int kXSlots = x_slots(FULL, false, TN);            // with a split-K mailbox in shared memory
     constexpr int kXSlotsAlone = x_slots_alone(FULL, TN);           // without one (K not split)
     constexpr int kXTile = x_tile_bytes(FULL, TN);
@@ -875,6 +875,7 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
     if (!make_map_2d(&mx, x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (uint64_t)M, (uint64_t)K, TN, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
+    if (prepare_only) return cudaSuccess;
     const int64_t row_tiles = (N + rows - 1) / rows;
     // the mailbox exists only when K is split, and then has its exact size
     const int slots = split > 1 ? (TN + split - 1) / split : 0;
@@ -930,16 +931,16 @@ cudaError_t launch_tn(const void* x, const uint8_t* p, const uint8_t* r, void* y
 
 template <int ENC, bool FULL>
 cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy, int64_t M, int64_t N, int64_t K,
-                       int* status, cudaStream_t stream) {
+                       int* status, cudaStream_t stream, bool prepare_only) {
     if (M <= 32 && forced_split() <= 1) {
         const int rows = rows_of_tiles(FULL, N, K, M <= 16 ? 16 : 32);
-        if (rows < kTileRows && M <= 16) return launch_tn<ENC, FULL, 16, true>(x, p, r, y, ldy, M, N, K, status, stream, rows);
-        if (rows < kTileRows) return launch_tn<ENC, FULL, 32, true>(x, p, r, y, ldy, M, N, K, status, stream, rows);
+        if (rows < kTileRows && M <= 16) return launch_tn<ENC, FULL, 16, true>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only, rows);
+        if (rows < kTileRows) return launch_tn<ENC, FULL, 32, true>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only, rows);
     }
-    if (M <= 16) return launch_tn<ENC, FULL, 16>(x, p, r, y, ldy, M, N, K, status, stream);
-    if (M <= 32) return launch_tn<ENC, FULL, 32>(x, p, r, y, ldy, M, N, K, status, stream);
+    if (M <= 16) return launch_tn<ENC, FULL, 16>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
+    if (M <= 32) return launch_tn<ENC, FULL, 32>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
     // 33 tokens and more (beyond 64 only where the dispatcher prefers two 64-token tiles per 128 rows to CTA pairs)
-    return launch_tn<ENC, FULL, 64>(x, p, r, y, ldy, M, N, K, status, stream);
+    return launch_tn<ENC, FULL, 64>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
 }
 
 }  // namespace
@@ -1062,20 +1063,20 @@ cudaError_t launch_umma_grouped(int mode, const uint32_t* e5m2_mask, const void*
 }
 
 cudaError_t launch_umma_linear(int mode, int enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t ldy,
-                               int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream) {
+                               int64_t M, int64_t N, int64_t K, int* status, cudaStream_t stream, bool prepare_only) {
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);   // fast mode reads the persistent byte of a rounded nest like any other
-    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, ldy, M, N, K, status, stream);
-    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, ldy, M, N, K, status, stream);
+    if (enc == kEncE4M3R) return launch_enc<kEncE4M3R, true>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
+    if (enc == kEncE5M2R) return launch_enc<kEncE5M2R, true>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
     if (enc == kEncE4M3)
-        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, ldy, M, N, K, status, stream)
-                    : launch_enc<kEncE4M3, false>(x, p, r, y, ldy, M, N, K, status, stream);
-    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, ldy, M, N, K, status, stream)
-                : launch_enc<kEncE5M2, false>(x, p, r, y, ldy, M, N, K, status, stream);
+        return full ? launch_enc<kEncE4M3, true>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only)
+                    : launch_enc<kEncE4M3, false>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
+    return full ? launch_enc<kEncE5M2, true>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only)
+                : launch_enc<kEncE5M2, false>(x, p, r, y, ldy, M, N, K, status, stream, prepare_only);
 }
 
 cudaError_t tile_turns_64(int mode, int enc, int64_t M, int64_t N, int64_t K, Turns* plan) {
-    auto ask = [&](auto launch) { return launch(nullptr, nullptr, nullptr, nullptr, N, M, N, K, nullptr, nullptr, kTileRows, plan); };
+    auto ask = [&](auto launch) { return launch(nullptr, nullptr, nullptr, nullptr, N, M, N, K, nullptr, nullptr, false, kTileRows, plan); };
     const bool full = mode == DPS_MODE_FULL;
     if (!full) enc = base_enc(enc);
     if (enc == kEncE4M3R) return ask(launch_tn<kEncE4M3R, true, 64>);
