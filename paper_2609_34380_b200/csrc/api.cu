@@ -175,8 +175,7 @@ cudaError_t launch_tensor(int32_t mode, int32_t enc, const void* x, const uint8_
 cudaError_t launch_rows(int32_t mode, int32_t enc, const void* x, const uint8_t* p, const uint8_t* r, void* y, int64_t M, int64_t N, int64_t K,
                         int* status, cudaStream_t stream) {
     pair_plan::RowShare share;
-    // (a matrix of less than half a row tile per pair is never among them, and its calls are host time: they do not ask)
-    if (M > 16 && M <= pair_plan::kMaxTokens && N * 4 >= (int64_t)sm_count() * 2 * pair_plan::kRows) {
+    if (pair_plan::may_share_rows(M, N, sm_count())) {
         const cudaError_t e = ask_pair_plan(mode, enc, M, N, K, {nullptr, &share});
         if (e != cudaSuccess) return e;
     }

@@ -178,8 +178,14 @@ inline double cut_gain(bool full, int64_t M, int64_t steps, int64_t rest) {
 // or four ways, and a round of the pairs is as good.
 inline int64_t most_rest(bool full, int64_t M) { return full && M > 32 ? 26 : 37; }
 // DPS_ROW_CUT=0: never, 1: wherever there is a whole round and a rest, up to 256 tokens (tuning knob).
-inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t pairs) {
+inline int row_cut_knob() {
     static const int knob = [] { const char* e = getenv("DPS_ROW_CUT"); return e ? atoi(e) : -1; }();
+    return knob;
+}
+// Whether share_rows can answer anything but no: small matrices and other numbers of tokens, whose calls are host time, do not ask.
+inline bool may_share_rows(int64_t M, int64_t N, int64_t sms) { return M > 16 && M <= (row_cut_knob() == 1 ? kMaxTokens : 128) && N * 4 >= sms * 2 * kRows; }
+inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t pairs) {
+    const int knob = row_cut_knob();
     const int64_t tiles = (N + 2 * kRows - 1) / (2 * kRows), steps = (K + kUnitK - 1) / kUnitK;
     const int64_t rounds = tiles / pairs, rest = tiles % pairs, rows = rest > 0 ? rounds * pairs * 2 * kRows : 0;
     if (knob == 0 || M <= 16 || M > kMaxTokens) return {};

@@ -17,7 +17,7 @@ int main(int argc, char**) {
         printf("%d 0\n", (int)dps::pair_plan::grouped_on_pairs(full, M, N, K, E, pairs));
     while (scanf("%d %lld %lld %lld %d", &full, &M, &N, &K, &pairs) == 5) {
         const auto s = dps::pair_plan::share_rows(full, M, N, K, pairs);
-        printf("%d %lld\n", (int)s.pairs, (long long)s.rows);
+        printf("%d %lld %d\n", (int)s.pairs, (long long)s.rows, (int)dps::pair_plan::may_share_rows(M, N, 2 * pairs));
     }
 }
 """
@@ -40,9 +40,9 @@ def ask(tmp_path_factory):
     (where / "rows.cpp").write_text(PROGRAM)
     subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "rows.cpp"), "-o", str(where / "rows")], check=True)
 
-    def run(cases, *argv, **env):
+    def run(cases, *argv, whole=False, **env):
         out = subprocess.run([str(where / "rows"), *argv], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True, env=env)
-        return [tuple(map(int, line.split())) for line in out.stdout.splitlines()]
+        return [tuple(map(int, line.split()[:4 if whole else 2])) for line in out.stdout.splitlines()]
     return run
 
 
@@ -117,3 +117,10 @@ def test_a_tile_for_every_pair_is_one_round(ask):
                 cases = [(full, M, N, K, 74) for K in (3056, 3072, 4096, 5104, 8192, 14336)]
                 assert ask(cases) == [(0, 0)] + [(1, 0)] * 5, (full, M, N)
     assert ask([(f, M, ROUND, K, 74) for f in (0, 1) for M in (17, 32, 65, 128) for K in (4096, 8192)]) == [(0, 0)] * 16
+
+
+def test_calls_that_cannot_share_do_not_ask(ask):
+    cases = [(full, M, N, K, 74) for full in (0, 1) for M in (8, 16, 17, 33, 64, 65, 128, 129, 200, 256, 257) for N in (4096, 9464, 9472, 15112, 18944, 22016, 57344) for K in (2048, 8192, 16384)]
+    for env, most in (({}, 128), ({"DPS_ROW_CUT": "1"}, 256)):
+        for (full, M, N, K, _), (pairs, rows, asked) in zip(cases, ask(cases, whole=True, **env), strict=True):
+            assert asked == (16 < M <= most and N >= 9472) and (asked or not pairs), (full, M, N, K)
