@@ -287,6 +287,7 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
         const float wscale = prm.e5m2 ? 1.0f : 0.00390625f;   // E4M3 bytes read as FP8 are 2^8 times the weights
         const uint32_t buf = epi_base + (uint32_t)(q * kEpiCols * 64);
         float* scales = reinterpret_cast<float*>(smem_raw + (epi_base - smem_u32(smem_raw)) + 4 * kEpiCols * 64) + q * kMaxTokens;
+        grid_dependency_wait();   // the scales come from the quantisation kernel, as the codes do
         int it = 0;
         for (int lin = pair; lin < total; lin += pairs, ++it) {
             int n0, m0;
@@ -298,7 +299,6 @@ fp8act_linear_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_con
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after_sync();
-            // (written by the preceding kernel; the accumulator could not be complete before it was)
             for (int c = lane; c < ncols; c += 32) scales[c] = prm.scale[m0 + c] * wscale;
             __syncwarp();
             const int row0 = n0 + q * 32;                // this warp's first row

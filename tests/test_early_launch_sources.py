@@ -36,3 +36,14 @@ def test_pair_set_up_meets_again_before_its_aligned_barriers():
     # between the second warp's set-up and the block's barrier
     tail = set_up[parted[1]:]
     assert tail.index("__syncwarp()") < tail.index("tmem_alloc_pair")
+
+
+def test_fp8_epilogue_waits_itself_for_the_scales_it_reads():
+    """The scales are the preceding kernel's output, read with ordinary loads: the warps that read them wait for that kernel, not another warp for them."""
+    text = (CSRC / "fp8act.cu").read_text()
+    kernel = text[text.index("fp8act_linear_kernel("):]
+    kernel = kernel[:kernel.index("\n}\n")]
+    reads = [m.start() for m in re.finditer(r"prm\.scale\[", kernel)]
+    role = kernel.index("// ---------------- epilogue")
+    assert reads and all(role < at for at in reads)
+    assert "grid_dependency_wait()" in kernel[role:reads[0]]
