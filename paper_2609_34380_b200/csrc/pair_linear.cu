@@ -609,7 +609,7 @@ cudaError_t launch_enc(const void* x, const uint8_t* p, const uint8_t* r, void* 
     const int pairs = capacity_of[dev][1];
     if (query != nullptr && query->share != nullptr) *query->share = share_rows(FULL, M, N, K, pairs);
     if (query != nullptr && query->turns == nullptr) return cudaSuccess;
-    const Plan plan = make_plan(FULL, M, N, K, capacity_of[dev], true);
+    const Plan plan = make_plan(FULL, M, N, K, capacity_of[dev]);
     const int64_t row_tiles = (N + 2 * kRows - 1) / (2 * kRows), tok_tiles = (M + plan.tokens - 1) / plan.tokens;
     const int64_t tiles = row_tiles * tok_tiles, grid_pairs = plan.split > 1 ? tiles : tiles < pairs ? tiles : pairs;
     if (query != nullptr) {

@@ -54,8 +54,8 @@ inline double step_ns(bool full, int tokens) {
 // A round of tiles over the pairs takes as long as one tile, so the number of token tiles is chosen to make the sum over the
 // rounds small; the tiles of a last, partial round are cut into pieces of the tokens if that shortens it.  Few tiles: up to
 // four pairs share each, a range of K each; capacity[s] = clusters of s pairs that are resident at once.
-// `wide`: with tiles of kWideTokens.  DPS_PAIR_TOKENS=1..384 (rounded up to a width there is) and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
-inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity, bool wide = false) {
+// DPS_PAIR_TOKENS=1..384 (rounded up to a width there is) and DPS_PAIR_SPLIT=1..4 override (tuning knobs).
+inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* capacity) {
     static const int forced = [] { const char* e = getenv("DPS_PAIR_TOKENS"); return e ? (atoi(e) + kTokenStep - 1) / kTokenStep * kTokenStep : 0; }();
     static const int forced_split = [] { const char* e = getenv("DPS_PAIR_SPLIT"); return e ? atoi(e) : 0; }();
     const int64_t steps = (K + kUnitK - 1) / kUnitK, pairs = capacity[1];
@@ -94,7 +94,7 @@ inline Plan make_plan(bool full, int64_t M, int64_t N, int64_t K, const int* cap
         if (forced >= kTokenStep && forced <= kMaxTokens) tokens = forced;
         for (int split = 1; split <= kMaxSplit; ++split) consider(tokens, split);
     }
-    if (wide && M > kMaxTokens && (forced == 0 || forced > kMaxTokens)) {
+    if (M > kMaxTokens && (forced == 0 || forced > kMaxTokens)) {
         if (forced > kMaxTokens) best = Plan();
         for (int tokens : kWideTokens)
             if (forced == 0 || (forced <= 320) == (tokens == 320)) consider(tokens, 1);

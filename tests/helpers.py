@@ -1,7 +1,9 @@
 """Shared helpers for the GPU parity tests (host <-> device shuttling and the error bound)."""
 import os
+import shutil
 import subprocess
 import sys
+from pathlib import Path
 
 import numpy as np
 import torch
@@ -55,6 +57,21 @@ def split_on_host(w: torch.Tensor, enc: int):
     return oracle.split(to_np_words(w), enc)
 
 
+def host_program(where: Path, source: str):
+    """A host program against the library's own headers.  Returns run(lines, *argv, **env): a tuple of whole numbers for each line that it prints."""
+    gxx = shutil.which("g++")
+    assert gxx
+    csrc = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
+    (where / "program.cpp").write_text(source)
+    subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(csrc), str(where / "program.cpp"), "-o", str(where / "program")], check=True)
+
+    def run(lines, *argv, **env):
+        text = "\n".join(line if isinstance(line, str) else " ".join(map(str, line)) for line in lines)
+        out = subprocess.run([str(where / "program"), *argv], input=text, text=True, capture_output=True, check=True, env=env)
+        return [tuple(map(int, line.split())) for line in out.stdout.splitlines()]
+    return run
+
+
 _LAUNCHES = """
 import sys, torch
 import paper_2609_34380_b200 as dps
@@ -69,8 +86,8 @@ for case in sys.argv[1:]:
 
 
 def launch_lines(cases, **env):
-    """What the library launched for dense linears of these (mode, M, N, K): the lines it prints on request, one per call
-    that the tensor-core tiles or the CTA pairs serve.  In a child process, since the library reads its knobs once."""
+    """What the library launched for dense linears of these (mode, M, N, K): the lines it prints on request, one per launch of the tensor-core
+    tiles or the CTA pairs (a call is one, or two where rows are cut off).  In a child process, since the library reads its knobs once."""
     repo = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     out = subprocess.run([sys.executable, "-c", _LAUNCHES, *(",".join(map(str, c)) for c in cases)], cwd=repo,
                          env=dict(os.environ, DPS_DEBUG="1", PYTHONPATH=repo, **env), capture_output=True, text=True, timeout=600)

@@ -1,13 +1,11 @@
 """The tile plan of the CTA-pair linear, evaluated on the host over its whole range of sizes: every width is one that the
 instruction has, the rings fit shared memory, and the tiles and pieces cover every token exactly once."""
 import random
-import shutil
-import subprocess
-from pathlib import Path
 
 import pytest
 
-CSRC = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
+from tests.helpers import host_program
+
 PROGRAM = r"""
 #include "pair_plan.h"
 #include <cstdio>
@@ -37,27 +35,20 @@ CAPACITIES = [(0, 74, 33, 16, 16), (0, 66, 30, 14, 14), (0, 9, 4, 2, 2), (0, 3, 
 
 @pytest.fixture(scope="module")
 def plan(tmp_path_factory):
-    gxx = shutil.which("g++")
-    assert gxx
-    where = tmp_path_factory.mktemp("plan")
-    (where / "plan.cpp").write_text(PROGRAM)
-    subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "plan.cpp"), "-o", str(where / "plan")], check=True)
-
-    def ask(lines, **env):
-        out = subprocess.run([str(where / "plan")], input="\n".join(lines), text=True, capture_output=True, check=True, env=env)
-        return [tuple(map(int, line.split())) for line in out.stdout.splitlines()]
-    return ask
+    return host_program(tmp_path_factory.mktemp("plan"), PROGRAM)
 
 
 def check_rings(full, tokens, units, x_slots):
     unit = 128 * 128 * (2 if full else 1)
-    assert units >= 2 and units % 2 == 0 and units <= 12 and 4 <= x_slots <= 8
+    assert units >= 2 and units % 2 == 0 and units <= 12 and (4 if tokens <= 256 else 3) <= x_slots <= 8
     assert units * unit + x_slots * tokens * 128 + 4 * 32 * 64 + 1024 <= 222 * 1024
 
 
 def check_dense(full, M, N, K, cap, answer):
     tokens, parts, tail_tokens, split, units, x_slots = answer
-    assert tokens % 32 == 0 and 32 <= tokens <= 256 and tail_tokens % 32 == 0 and 32 <= tail_tokens <= tokens
+    assert tokens % 32 == 0 and tail_tokens % 32 == 0 and 32 <= tail_tokens <= tokens
+    # wide tiles: two MMAs each, which a piece must do with one of; K is not split
+    assert 32 <= tokens <= 256 or (tokens in (320, 384) and M > 256 and split == 1 and (parts == 1 or tail_tokens <= tokens // 2))
     check_rings(full, tokens, units, x_slots)
     row_tiles, tok_tiles = -(-N // 256), -(-M // tokens)
     tiles, pairs = row_tiles * tok_tiles, cap[1]
@@ -81,17 +72,20 @@ def test_dense_plans_over_the_range(plan):
         K = 16 * int(2 ** rng.uniform(0, 11))
         cases.append((rng.randrange(2), M, N, K, rng.choice(CAPACITIES)))
     cases += [(f, M, N, 4096, CAPACITIES[0]) for f in (0, 1) for M in range(1, 700) for N in (4096, 18944)]
+    cases += [(f, M, N, 4096, c) for f in (0, 1) for M in (257, 320, 384, 700, 1100, 1536, 2999, 8192) for N in range(256, 24000, 744) for c in CAPACITIES]
     answers = plan([f"d {f} {M} {N} {K} {c[1]} {c[2]} {c[3]} {c[4]}" for f, M, N, K, c in cases])
     assert len(answers) == len(cases)
     for case, answer in zip(cases, answers):
         check_dense(*case, answer)
     assert any(a[1] > 1 for a in answers) and any(a[3] > 1 for a in answers)
+    # wide tiles, whole and in pieces, with every number of pairs
+    assert {(c[4], a[1] > 1) for c, a in zip(cases, answers) if a[0] > 256} == {(c, cut) for c in CAPACITIES for cut in (False, True)}
 
 
-@pytest.mark.parametrize("tokens", ["16", "48", "112", "256", "300"])
+@pytest.mark.parametrize("tokens", ["16", "48", "112", "256", "300", "384"])
 def test_forced_widths_are_widths_there_are(plan, tokens):
-    for answer in plan(["d 0 500 4096 4096 74 33 16 16", "d 1 31 512 2064 74 33 16 16"], DPS_PAIR_TOKENS=tokens):
-        assert answer[0] % 32 == 0 and 32 <= answer[0] <= 256 and answer[2] % 32 == 0
+    for M, answer in zip((500, 31), plan(["d 0 500 4096 4096 74 33 16 16", "d 1 31 512 2064 74 33 16 16"], DPS_PAIR_TOKENS=tokens), strict=True):
+        assert answer[0] % 32 == 0 and (32 <= answer[0] <= 256 or (M > 256 and answer[0] == max(320, int(tokens)))) and answer[2] % 32 == 0
 
 
 def test_grouped_widths(plan):

@@ -1,12 +1,10 @@
 """Which rows of a matrix the CTA pairs take at 17 to 128 tokens (pair_plan.h): the rule's edges, and that a cut leaves whole tiles on one side."""
 import random
-import shutil
-import subprocess
-from pathlib import Path
 
 import pytest
 
-CSRC = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
+from tests.helpers import host_program
+
 PROGRAM = r"""
 #include "pair_plan.h"
 #include <cstdio>
@@ -34,16 +32,8 @@ EDGES = {(1, 64, ROUND - 256, 8192): 0, (0, 33, 60 * 256, 3072): 0, (0, 33, 59 *
 
 @pytest.fixture(scope="module")
 def ask(tmp_path_factory):
-    gxx = shutil.which("g++")
-    assert gxx
-    where = tmp_path_factory.mktemp("rows")
-    (where / "rows.cpp").write_text(PROGRAM)
-    subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "rows.cpp"), "-o", str(where / "rows")], check=True)
-
-    def run(cases, *argv, whole=False, **env):
-        out = subprocess.run([str(where / "rows"), *argv], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True, env=env)
-        return [tuple(map(int, line.split()[:4 if whole else 2])) for line in out.stdout.splitlines()]
-    return run
+    run = host_program(tmp_path_factory.mktemp("rows"), PROGRAM)
+    return lambda cases, *argv, whole=False, **env: [answer[:None if whole else 2] for answer in run(cases, *argv, **env)]
 
 
 def test_edges(ask):

@@ -2,13 +2,10 @@
 on the host with the capacities of a B200.  Lower tiles only where K is long enough for their even load to show; the pairs serve what
 they were measured to be faster on, and the sizes at which they would leave much of the chip idle, or take a whole round for a few
 tiles, stay with the tiles."""
-import shutil
-import subprocess
-from pathlib import Path
-
 import pytest
 
-CSRC = Path(__file__).resolve().parents[1] / "paper_2609_34380_b200" / "csrc"
+from tests.helpers import host_program
+
 PROGRAM = r"""
 #include "pair_plan.h"
 #include "tile_plan.h"
@@ -36,16 +33,8 @@ FASTER = [*range(20, 23), *range(27, 34), *range(46, 75), *range(149, 223), *ran
 
 @pytest.fixture(scope="module")
 def ask(tmp_path_factory):
-    gxx = shutil.which("g++")
-    assert gxx
-    where = tmp_path_factory.mktemp("plan")
-    (where / "plan.cpp").write_text(PROGRAM)
-    subprocess.run([gxx, "-std=c++17", "-O1", "-I", str(CSRC), str(where / "plan.cpp"), "-o", str(where / "plan")], check=True)
-
-    def run(cases):
-        out = subprocess.run([str(where / "plan")], input="\n".join(" ".join(map(str, c)) for c in cases), text=True, capture_output=True, check=True)
-        return [int(v) for v in out.stdout.split()]
-    return run
+    run = host_program(tmp_path_factory.mktemp("plan"), PROGRAM)
+    return lambda cases: [answer for (answer,) in run(cases)]
 
 
 @pytest.mark.parametrize("K", [16384, 17920, 28672, 53248])
