@@ -72,8 +72,7 @@ struct PairQuery {
 };
 cudaError_t ask_pair_plan(int mode, int enc, int64_t M, int64_t N, int64_t K, const PairQuery& query);
 
-// Grouped linear on CTA pairs: arguments as below, `masks` the e5m2_mask array; pair_grouped_tokens: its token-tile width.
-int pair_grouped_tokens(int64_t A, int32_t E);
+// Grouped linear on CTA pairs: arguments as below, `masks` the e5m2_mask array; tn: pair_plan::grouped_width.
 cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y,
                                 int64_t A, int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,
                                 const int32_t* sorted_rows, int max_tiles, int* status, cudaStream_t stream);

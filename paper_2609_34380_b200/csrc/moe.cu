@@ -257,7 +257,7 @@ cudaError_t launch_moe(int mode, const int32_t* enc_host, const void* x, const i
     const Workspace w = carve(workspace, A, E, K);
     // CTA pairs or 128-row tiles, two CTAs per SM: pair_plan.h
     const bool pairs = pair_plan::grouped_on_pairs(mode == DPS_MODE_FULL, A, N, K, E, sm_count() / 2);
-    const int tn = pairs ? pair_grouped_tokens(A, E) : grouped_tile_tokens(A, E);
+    const int tn = pairs ? pair_plan::grouped_width(mode == DPS_MODE_FULL, A, N, E, sm_count() / 2) : grouped_tile_tokens(A, E);
     cudaError_t err;
     // programmatic dependent launch, as the kernel behind them: each is resident early and waits before its first read
     cudaLaunchAttribute attr[1];

@@ -752,8 +752,6 @@ cudaError_t launch_grouped(const uint32_t* masks, const void* x_sorted, const ui
 
 }  // namespace
 
-int pair_grouped_tokens(int64_t A, int32_t E) { return grouped_tokens(A, E); }
-
 cudaError_t launch_pair_grouped(int mode, const uint32_t* masks, const void* x_sorted, const uint8_t* p, const uint8_t* r, void* y,
                                 int64_t A, int64_t N, int64_t K, int32_t E, int tn, const void* tiles, const int32_t* num_tiles,
                                 const int32_t* sorted_rows, int max_tiles, int* status, cudaStream_t stream) {

@@ -280,5 +280,22 @@ inline bool grouped_on_pairs(bool full, int64_t A, int64_t N, int64_t K, int32_t
     return rounds < turns || rounds >= 8;
 }
 
+// The token-tile width of a grouped launch.  Below 48 rows per expert an uneven routing must not undo what grouped_on_pairs counted: an expert with more rows than a
+// tile is another row of items, and one round of the pairs becomes two where the other kernel's wave has room.  A wider tile costs the ring's depth only (an
+// item multiplies the columns it has): nothing in full mode up to 128 tokens in one round and 96 in more, 0-2 % in fast mode for 96.  128-row tiles / pairs by the
+// average's width / as it is, us, 40 rows per expert, an even routing and one that gives an expert 30 % of the rows on top, fast | full mode:
+//   4 x 4096 x 8192 (one round)     44.1 / 38.9 / 39.8, 46.0 / 53.3 / 38.7 | 71.9 / 60.7 / 61.8, 76.7 / 85.1 / 61.5
+//   8 x 2304 x 8192 (one)           47.4 / 42.6 / 43.4, 49.5 / 56.0 / 56.7 | 76.4 / 67.1 / 67.2, 81.9 / 89.8 / 66.8     (128 in fast mode: 44.8, 45.2)
+//   16 x 1024 x 4096 (one)          28.5 / 24.3 / 24.2, 30.3 / 33.2 / 24.2 | 43.7 / 36.8 / 37.1, 46.3 / 49.0 / 36.7
+//   3 x 15496 x 4096 (three)        51.6 / 49.4 / 49.4, 55.5 / 55.4 / 55.4 | 87.3 / 83.2 / 82.1, 90.7 / 98.5 / 81.1
+//   8 x 14336 x 4096 (seven)         114 /  115 /  115,  118 /  110 /  110 |  189 /  184 /  186,  200 /  204 /  185
+inline int grouped_width(bool full, int64_t A, int64_t N, int32_t E, int64_t pairs) {
+    const int tokens = grouped_tokens(A, E);
+    if (A >= 48 * (int64_t)E) return tokens;
+    const bool one_round = E * ((N + 2 * kRows - 1) / (2 * kRows)) <= pairs;
+    const int least = one_round ? (full ? 128 : 96) : full ? 96 : kTokenStep;
+    return tokens < least ? least : tokens;
+}
+
 }  // namespace pair_plan
 }  // namespace dps

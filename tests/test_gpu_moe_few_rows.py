@@ -1,5 +1,5 @@
 """GPU: grouped launches of 12 to 47 rows per expert on either side of the border between CTA pairs and 128-row tiles (row tiles over the experts),
-against the oracle: mixed encodings, rounded nests, skewed routing (an expert with several token tiles, one without rows), token tiles of 32 and 64.
+against the oracle: mixed encodings, rounded nests, skewed routing (an expert with several token tiles, one without rows), token tiles of 64 to 128.
 Which kernel ran is read off the lines that the library prints on request; it reads its knobs once per process, so a case is a child
 process: this file executed as a script."""
 import os
@@ -14,11 +14,12 @@ REPO = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 # 128-row tiles (two per wave of 296):
 CASES = [(2, 37 * 256 + 8, 80, 13, 0, 0),         # 76, two against two
          (2, 112 * 256 + 136, 48, 25, 0, 0),      # 226, four against four
-         (2, 80 * 256 + 8, 80, 13, 0, 32),        # 162, three against four; fast mode has too few rows
-         (3, 60 * 256 + 136, 48, 25, 64, 64),     # 183, three against four
+         (2, 80 * 256 + 8, 80, 13, 0, 96),        # 162, three against four; fast mode has too few rows
+         (3, 60 * 256 + 136, 48, 25, 64, 96),     # 183, three against four
          (8, 18 * 256 + 8, 80, 25, 0, 0),         # 152, three against two: 37 tiles of 128 rows an expert are one wave
-         (12, 49 * 256 + 520, 144, 46, 64, 64),   # 624, nine
-         (24, 25 * 256 + 8, 144, 13, 0, 32)]      # 624, nine
+         (12, 49 * 256 + 520, 144, 46, 64, 96),   # 624, nine
+         (24, 25 * 256 + 8, 144, 13, 0, 96),      # 624, nine
+         (4, 16 * 256 - 8, 3088, 30, 96, 128)]    # 64, one against two
 
 
 def _run(E, N, K, rows, skewed):

@@ -21,8 +21,8 @@ int main() {
             const Rings r = size_rings(full, p.tokens);
             printf("%d %d %d %d %d %d\n", p.tokens, p.tail_parts, p.tail_tokens, p.split, r.units, r.x_slots);
         } else {
-            if (scanf("%lld %d", &A, &E) != 2) return 1;
-            const int t = grouped_tokens(A, E);
+            if (scanf("%d %lld %lld %d", &full, &A, &N, &E) != 4) return 1;
+            const int t = grouped_width(full, A, N, E, 74);
             const Rings f = size_rings(false, t), g = size_rings(true, t);
             printf("%d %d %d %d %d\n", t, f.units, f.x_slots, g.units, g.x_slots);
         }
@@ -89,8 +89,16 @@ def test_forced_widths_are_widths_there_are(plan, tokens):
 
 
 def test_grouped_widths(plan):
-    cases = [(A, E) for E in (1, 3, 8, 64, 1024) for A in sorted({1, 47 * E, 48 * E, 49 * E, 100 * E + 7, 200 * E, 256 * E, 257 * E, 5000 * E})]
-    for (A, E), (tokens, *rings) in zip(cases, plan([f"g {A} {E}" for A, E in cases])):
+    cases = [(f, A, N, E) for f in (0, 1) for N in (8, 4096, 40000) for E in (1, 3, 8, 64, 1024)
+             for A in sorted({1, 47 * E, 48 * E, 49 * E, 100 * E + 7, 200 * E, 256 * E, 257 * E, 5000 * E})]
+    for (f, A, N, E), (tokens, *rings) in zip(cases, plan([f"g {f} {A} {N} {E}" for f, A, N, E in cases]), strict=True):
         assert tokens % 32 == 0 and 32 <= tokens <= 256, (A, E)
         check_rings(False, tokens, *rings[:2])
         check_rings(True, tokens, *rings[2:])
+
+
+def test_an_uneven_routing_does_not_add_a_round(plan):
+    """Few rows per expert: an expert with a good part of all rows still has one token tile, so that the one round that the border counted stays one; wider tiles only below 48 rows."""
+    for full, E, N, rows, share in ((0, 4, 4096, 40, 0.47), (1, 4, 4096, 40, 0.47), (1, 8, 2304, 40, 0.38), (0, 16, 1024, 40, 0.15), (1, 3, 15496, 40, 0.53), (1, 64, 256, 47, 0.04)):
+        assert plan([f"g {full} {rows * E} {N} {E}"])[0][0] >= share * rows * E, (full, E, N, rows)
+    assert [plan([f"g {f} {rows * 8} {N} 8"])[0][0] for f, rows, N in ((0, 24, 14336), (1, 24, 14336), (0, 24, 2304), (1, 24, 2304), (0, 48, 2304), (1, 48, 2304))] == [64, 96, 96, 128, 96, 96]
