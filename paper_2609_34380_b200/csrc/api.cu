@@ -153,8 +153,9 @@ bool decode_tiles_for_128(bool full, int64_t M, int64_t N, int64_t K) {
 // (tile_plan.h: pairs_for_long_k, with what both sides take).  Fast / full mode, 64 tokens, tiles against pairs, us: 8192 x 28672 53.6 / 85.8 against 46.1 / 82.2,
 // 12288 x 16384 54.7 / 85.8 against 47.1 / 75.8, 38144 x 16384 147.5 / 277.8 against 132.2 / 242.5; but 6144 x 16384 27.0 / 40.2 against
 // 28.1 / 42.8, 8704 x 16384 32.8 / 51.6 against 44.7 / 66.0, 19200 x 16384 75.1 / 147.3 against 86.3 / 150.0.  With a shorter K the pairs' fixed
-// costs show: 4096 x 14336 17.1 / 25.5 against 19.6 / 27.8, 57344 x 8192 93.7 / 170 against 95.4 / 174, 10240 x 8192 24.3 / 36.3 against
-// 26.5 / 39.6; at 20 tokens the 32-token tiles are faster here too: 43.0 / 78.0 against 45.0 / 80.2.  A pair sums a longer range of K in one
+// costs show: 4096 x 14336 17.1 / 25.5 against 19.6 / 27.8, 10240 x 8192 24.3 / 36.3 against 26.5 / 39.6; at 20 tokens the 32-token tiles are
+// faster here too: 43.0 / 78.0 against 45.0 / 80.2.  (All of these in bursts.  57344 x 8192, 93.7 / 170 against 95.4 / 174 so, takes 193 against 186 in
+// full mode under the power cap, which is where the rule for tall matrices, share_rows, was measured.)  A pair sums a longer range of K in one
 // accumulator: at 8192 x 28672 the error against 64 bits is 2.074e-4 of the output instead of 2.070e-4, of which the rounding to FP16 is 2.068e-4.
 bool pairs_for_64(int32_t mode, int32_t enc, int64_t M, int64_t N, int64_t K) {
     if (M <= 32 || M > 64 || K < 16384 || N < 5120) return false;
@@ -319,8 +320,9 @@ dps_status dps_linear(int32_t mode, int32_t enc, const void* x, const uint8_t* w
     // What the rule costs: a matrix beyond it that is called by itself.  2048 x 2048, 9 tokens, takes 4.5 us in fast and 5.4 in
     // full mode, the streaming kernel 3.4 and 3.9; 4096 x 4096 6.7 and 9.3 against 5.7 and 8.8.  With other programs' kernels
     // between the linears every launch of the tiles pays for the change of split, about 2 us: 2048 x 2048 7.0 against 4.2.
-    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for a long K, see pairs_for_64, from 17 on for tall matrices, see launch_rows) CTA pairs.  Four linears of a layer,
-    // fast / full mode, tiles against pairs, us: Llama-7B 64 tokens 61.8 / 96.5 against 66.7 / 95.1, 96 tokens 89.0 / 147.4 against 69.6 / 98.8;
+    // Beyond 16 tokens the tcgen05 tiles take over, beyond 64 tokens (33 for a long K, see pairs_for_64, from 17 on for tall matrices, see launch_rows) CTA
+    // pairs.  Four linears of a layer, fast / full mode, tiles against pairs, us, in bursts: Llama-7B 64 tokens 61.8 / 96.5 against 66.7 / 95.1,
+    // 96 tokens 89.0 / 147.4 against 69.6 / 98.8;
     // hidden size 2048, 64 tokens, 29.7 / 39.8 against 35.6 / 40.8, 96 tokens 37.8 / 53.7 against 37.9 / 46.1.  (The CUDA-core GEMV is kept as a cross-check.)
     const bool stream_mid = (N < K ? N : K) <= 1536 && N * K < ((int64_t)1 << 25);
     const int path = forced_path();

@@ -128,8 +128,9 @@ __device__ __forceinline__ void rebuild(uint32_t prow, int half, uint32_t sw, ui
 // GROUPED: a work item is a row tile of one expert x one of its token tiles; ENC is not used, the encoding is the expert's.
 // WIDE: tiles of 320 or 384 tokens in two halves, an accumulator and MMAs each: what is fetched, rebuilt and stored of the weights serves half
 // as many tokens more.  74 row tiles of 8192 columns, short of the power cap, 256 -> 384 tokens, us: fast 56.8 -> 79.5, full 70.7 -> 93.0, 7 and
-// 12 % less per token.  Under the cap, where the MMAs' energy is most of it: 8192 tokens on a Llama-7B layer, full mode, tiles of 256 -> these,
-// 2973 -> 2893.  (A template argument: with the halves counted at run time in the issuer's loop 512 tokens took 2 % longer.)
+// 12 % less per token.  Under the cap, where the MMAs' energy is most of it: a Llama-7B layer, full mode, tiles of 256 -> these, 1536 tokens 630 -> 566,
+// 4096 1525 -> 1466, 8192 2950 -> 2866 (two runs a side, 3 % apart).  (A template argument: with the halves counted at run time in the issuer's
+// loop 512 tokens took 2 % longer.)
 template <int ENC, bool FULL, bool GROUPED, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r,

@@ -212,8 +212,8 @@ inline RowShare share_rows(bool full, int64_t M, int64_t N, int64_t K, int64_t p
 }
 
 // Shared memory: activations take 2000 cycles and more out of L2, so four K steps of them are kept in flight at least
-// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024; three of a wide tile, whose steps are longer), more if four plane units still fit; the
-// planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen
+// (2.5 steps: 1250 cycles per step of 256 tokens in full mode instead of 1024; three of a wide tile, whose steps are longer), more if four plane
+// units still fit; the planes have the A ring as a second buffer, two units do.  An even number of units, so that a unit's phases are all seen
 // by the same zip warps.
 inline Rings size_rings(bool full, int tokens) {
     const int x_bytes = tokens * 128, room = kSmemBytes - 1024 - kEpiBytes;
@@ -280,10 +280,11 @@ inline bool grouped_on_pairs(bool full, int64_t A, int64_t N, int64_t K, int32_t
     return rounds < turns || rounds >= 8;
 }
 
-// The token-tile width of a grouped launch.  Below 48 rows per expert an uneven routing must not undo what grouped_on_pairs counted: an expert with more rows than a
-// tile is another row of items, and one round of the pairs becomes two where the other kernel's wave has room.  A wider tile costs the ring's depth only (an
-// item multiplies the columns it has): nothing in full mode up to 128 tokens in one round and 96 in more, 0-2 % in fast mode for 96.  128-row tiles / pairs by the
-// average's width / as it is, us, 40 rows per expert, an even routing and one that gives an expert 30 % of the rows on top, fast | full mode:
+// The token-tile width of a grouped launch.  Below 48 rows per expert an uneven routing must not undo what grouped_on_pairs counted: an expert with
+// more rows than a tile is another row of items, and one round of the pairs becomes two where the other kernel's wave has room.  A wider tile costs
+// the ring's depth only (an item multiplies the columns it has): nothing in full mode up to 128 tokens in one round and 96 in more, 0-2 % in fast
+// mode for 96.  128-row tiles / pairs by the average's width / as it is, us, 40 rows per expert, an even routing and one that gives an expert 30 %
+// of the rows on top, fast | full mode:
 //   4 x 4096 x 8192 (one round)     44.1 / 38.9 / 39.8, 46.0 / 53.3 / 38.7 | 71.9 / 60.7 / 61.8, 76.7 / 85.1 / 61.5
 //   8 x 2304 x 8192 (one)           47.4 / 42.6 / 43.4, 49.5 / 56.0 / 56.7 | 76.4 / 67.1 / 67.2, 81.9 / 89.8 / 66.8     (128 in fast mode: 44.8, 45.2)
 //   16 x 1024 x 4096 (one)          28.5 / 24.3 / 24.2, 30.3 / 33.2 / 24.2 | 43.7 / 36.8 / 37.1, 46.3 / 49.0 / 36.7
